@@ -130,6 +130,18 @@ static bool use_reslean(const wrnn_model *m, int batch)
     return reslean_supported(m, batch) == WRNN_OK;
 }
 
+// Rows of a dense bf16 H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
+// clusters of eight) and more in waves; the cluster-partitioned kernel takes all at once and costs almost the same whatever
+// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 10.1 / 25.2, 112: 20.2 / 25.8, 128: 26.3 /
+// 27.7, 150: 28.4 / 28.3, 256: 47 / 32.3.
+static bool use_rescl(const wrnn_model *m, int batch)
+{
+    if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
+    const char *off = getenv(batch == 1 ? "WRNN_RESIDENT_LEAN" : "WRNN_NO_MULTI");
+    if (off && off[0] == (batch == 1 ? '0' : '1')) return false;
+    return batch <= 128 && rescl_supported(m, batch) == WRNN_OK;
+}
+
 static bool use_resf32(const wrnn_model *m, int batch)
 {
     if (m->kernel == WRNN_KERNEL_GENERIC || m->kernel == WRNN_KERNEL_BATCHED || m->kernel == WRNN_KERNEL_BCLUSTER) return false;
@@ -226,6 +238,7 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     if (!ensure_g(m, (size_t)a.batch * nf * 3 * m->H)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
     int rc = cond_project(m, a.cond, a.batch, nf, s);
     if (rc != WRNN_OK) return fail(m, rc, "conditioning projection launch failed");
+    if (use_rescl(m, a.batch)) return rescl_run(m, a, s);
     // staggered rows: the cluster-partitioned kernel, else the any-shape kernel
     if (a.row_lag > 0) {
         if (a.batch >= 2 && use_multi(m, a.batch)) return resmulti_run(m, a, s);
@@ -434,6 +447,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
         if (m->dtype == WRNN_BF16 && m->variant == 0) reslean_prepare(m);                        // optional: the row-split resident kernel serves the stream without it
+        if (m->dtype == WRNN_BF16 && m->variant == 0 && !reslean_checked(m)) rescl_prepare(m);
         if (m->dtype == WRNN_BF16 && m->variant == 0 && max_batch >= 2) resmulti_prepare(m);   // optional: other kernels serve the batch without it
     }
     m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call
@@ -451,6 +465,7 @@ void wrnn_destroy(wrnn_model *m)
     reslean_destroy(m);
     resf32_destroy(m);
     resmulti_destroy(m);
+    rescl_destroy(m);
     batched_destroy(m);
     bcluster_destroy(m);
     sparse_destroy(m);
@@ -635,7 +650,7 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
         if (rc != WRNN_OK) return fail(m, rc, "conditioning launch failed");
         // rows advance together on the multi-stream resident kernel where the model has one; without it up to three rows go
         // one after the other through the single-stream kernel
-        const int group = (n_rows >= 2 && use_multi(m, n_rows)) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
+        const int group = (n_rows >= 2 && (use_rescl(m, n_rows) || use_multi(m, n_rows))) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
         for (int b0 = 0; b0 < n_rows; b0 += group) {
             const int r0 = r_a + b0;
             const long long p0 = p_lo - (long long)b0 * lag;
@@ -720,7 +735,7 @@ int wrnn_subscale_net_rows(wrnn_model *m, wrnn_subscale_net *net, const float *f
     float *v = reinterpret_cast<float *>(m->sub_scratch);
     int rc = subnet_run(net, hist, frames, n_frames, hop, L, r_lo, n_rows, p_lo, lag, n_steps, v, m->wait_limit_ns(), s);
     if (rc != WRNN_OK) return fail(m, rc, "conditioning launch failed");
-    const int group = (n_rows >= 2 && use_multi(m, n_rows)) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
+    const int group = (n_rows >= 2 && (use_rescl(m, n_rows) || use_multi(m, n_rows))) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
     for (int b0 = 0; b0 < n_rows; b0 += group) {
         const int r0 = r_lo + b0;
         const long long p0 = p_lo - (long long)b0 * lag;
@@ -834,6 +849,10 @@ int wrnn_launch_info(wrnn_model *m, int32_t batch, int32_t *kernel, int32_t *n_c
                      int64_t *weight_bytes_per_step, int32_t *smem_bytes)
 {
     if (!m || batch < 1 || batch > m->max_batch) return WRNN_ERR_INVALID_ARG;
+    if (use_rescl(m, batch)) {
+        if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
+        return rescl_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
+    }
     if (use_reslean(m, batch)) {
         if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
         return reslean_launch_info(m, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
@@ -900,7 +919,10 @@ int wrnn_phase_names(wrnn_model *m, char *buf, int32_t cap)
                         "F.hid_products,C.hid_products,F.log_products,C.log_products";
     const char *lean = "F.wait_y,F.hid_products,F.hid_sums_send,F.recurrent_products,F.rsums_gateprep,F.wait_logit_rows_send,F.wait_logits,F.draw_gates,"
                        "C.wait_y,C.hid_products,C.hid_sums_send,C.recurrent_products,C.rsums_gateprep,C.wait_logit_rows_send,C.wait_logits,C.draw_gates";
-    const char *src = (!m->resf32 && m->prof_multi) ? multi : (!m->resf32 && m->prof_lean) ? lean : first;
+    // per half: warp 0 of CTA 0 (wait, products, sums and sends), then its first drawing warp
+    const char *cl = "F.wait_y,F.hid_products,F.hid_sums_send,F.wait_q,F.log_products,F.log_sums_send,F.draw,F.gates,"
+                     "C.wait_y,C.hid_products,C.hid_sums_send,C.wait_q,C.log_products,C.log_sums_send,C.draw,C.gates";
+    const char *src = m->prof_cl ? cl : (!m->resf32 && m->prof_multi) ? multi : (!m->resf32 && m->prof_lean) ? lean : first;
     std::snprintf(buf, (size_t)cap, "%s", src);
     return WRNN_OK;
 }
@@ -909,6 +931,7 @@ int wrnn_phase_cycles(wrnn_model *m, int64_t *out16)
 {
     if (!m || !out16) return WRNN_ERR_INVALID_ARG;
     static_assert(sizeof(long long) == sizeof(int64_t), "");
+    if (m->prof_cl) return rescl_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->resf32) return resf32_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->prof_multi) return resmulti_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->prof_lean) return reslean_phase_cycles(m, reinterpret_cast<long long *>(out16));

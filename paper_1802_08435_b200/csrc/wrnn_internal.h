@@ -64,6 +64,7 @@ struct SparsePack;     // compressed block rows of the single-cluster block-spar
 struct ResF32Pack;     // per-CTA fp32 weight shards of the single-stream fp32 resident kernel (opaque here)
 struct ResLeanPack;      // per-CTA weights of the lean single-stream resident kernel (opaque here)
 struct ResMultiPack;  // per-CTA weights of the multi-stream resident kernel (opaque here)
+struct ResClPack;      // per-CTA weights of the cluster-resident kernel (opaque here)
 struct BcPack;         // per-CTA weight slices and stacked activation images of the cluster-partitioned multi-row kernel
 
 }  // namespace wrnn
@@ -104,6 +105,8 @@ struct wrnn_model {
     bool prof_lean = false;           // the last call with phase timing ran on the lean single-stream resident kernel
     wrnn::ResF32Pack *resf32 = nullptr;
     wrnn::ResMultiPack *resmulti = nullptr;
+    wrnn::ResClPack *rescl = nullptr;
+    bool prof_cl = false;             // the last call with phase timing ran on the cluster-resident kernel
     // wrnn_selftest_lost_word: bound of every device-side wait (0 = the default of two seconds) and the CTA / step whose
     // publication (or operand load) is withheld (-1 = none)
     unsigned long long dbg_limit_ns = 0;
@@ -176,6 +179,7 @@ void pack_tile(const std::vector<std::vector<uint16_t>> &rows, int K, uint16_t *
 
 // wrnn_reslean.cu: one stream of a dense bf16 H = 896 model, the row-split resident kernel with a shorter chain per half-step
 int reslean_supported(const wrnn_model *m, int batch);
+bool reslean_checked(const wrnn_model *m);      // the model was created for the checked build (WRNN_DEBUG=1)
 int reslean_prepare(wrnn_model *m);
 void reslean_destroy(wrnn_model *m);
 int reslean_launch_info(const wrnn_model *m, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
@@ -189,6 +193,14 @@ void resmulti_destroy(wrnn_model *m);
 int resmulti_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
 int resmulti_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int resmulti_phase_cycles(const wrnn_model *m, long long *out16);
+
+// wrnn_rescl.cu: rows of a dense bf16 H = 896 model, the whole model in one cluster (R in tensor memory)
+int rescl_supported(const wrnn_model *m, int batch);
+int rescl_prepare(wrnn_model *m);
+void rescl_destroy(wrnn_model *m);
+int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
+int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
+int rescl_phase_cycles(const wrnn_model *m, long long *out16);
 
 // wrnn_resf32.cu: the same role for dense fp32 models (every matrix sharded chip-wide, nothing replicated)
 int resf32_supported(const wrnn_model *m, int batch, std::string *why);

@@ -1,0 +1,878 @@
+// Cluster-resident persistent sampling kernel: the whole dense bf16 H = 896 model lives in ONE 16-CTA cluster -- the
+// recurrent matrix in tensor memory, everything else in shared memory -- and a cluster advances its own rows alone.
+//
+// A step of the sampler (Fig. 1 of the paper) is a chain of exchanges, not of arithmetic: what bounds it is how long it
+// takes to hand the state, the hidden layer and the logits from the SM that computed them to the SMs that need them.  The
+// model is 6.1 MB; the shared memory of a 16-CTA cluster is 3.6 MB, but its tensor memory is another 4.2 MB, and
+// tcgen05.mma takes its A operand from there.  With the model inside one cluster every exchange is an all-gather through
+// distributed shared memory (measured here: 420 cycles + bytes / 17.5 per SM, against 1,000 - 1,500 cycles for the same
+// through L2 and across the chip), clusters never meet, and seven of them advance seven times as many rows in the same time.
+//
+// Per CTA (rank r of its cluster): state units 28 r .. 28 r + 27 of both halves with their 168 rows of R, rows 28 r .. of O1
+// and O3, rows 16 r .. of O2 and O4.
+//   * R: 128 rows (all 84 coarse rows and 44 fine ones) in tensor memory, the other 40 fine rows in shared memory.  Both feed
+//     mma.sync: a TMEM column is one register of an A fragment for the warps of its lane quadrant, so tcgen05.ld brings four
+//     fragments per instruction and no shared-memory load is spent on them.  (tcgen05.mma takes 46 cycles per K = 16 whatever
+//     N is up to 64; at eight operand columns mma.sync at 8 cycles per sub-partition does three times as much per cycle, and
+//     needs no proxy fence and no read-back of accumulators: 6.4 us per step with tcgen05.mma.)  The products are needed by
+//     the gates at the end of the half-step (coarse rows x fine columns) or later, and run beside the head.
+//   * The heads are on the critical path: K split over 4 (hidden layer) and 7 (logits) groups of warps, whose weight
+//     fragments are loaded from shared memory before the wait for the input (the loads, 4 cycles of the load / store unit per
+//     fragment, are what took the time in the shared-memory-resident kernels, not the MMAs).
+//   * State halves and hidden layers cross the cluster as bf16 parts of their fp32 values -- three exact parts when a
+//     cluster has one row, high and low parts (residual 2^-18) when it has several, as in the other multi-row kernels --
+//     stored by their producers straight into every receiver's operand image of 8 x 16-byte matrices, as ldmatrix reads them.
+//   * Every CTA draws every row of its cluster (one warp per row) and computes the gates of its own 28 units in the same
+//     warp, so the drawn symbol never leaves the warp.
+// Every wait is bounded; a warp that gives up records where, skips its remaining waits and sends and keeps meeting its
+// barriers, and all CTAs leave through the final cluster barrier.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include <cstdlib>
+#include <cstring>
+
+#include "wrnn_cluster.cuh"
+#include "wrnn_internal.h"
+#include "wrnn_tc.cuh"
+
+namespace wrnn {
+
+namespace {
+constexpr int CK = 448;                  // H / 2
+constexpr int CU = 28;                   // state units of one half, hidden-layer rows per CTA
+constexpr int CL = 16;                   // logits rows per CTA
+constexpr int CCS = 16;                  // CTAs per cluster
+constexpr int CK8 = CK / 8;              // core matrices along K per half
+constexpr int CT2 = 6 * CU - 128;        // rows of R outside the TMEM tile
+constexpr int CMAXR = 8;                 // rows per cluster
+constexpr int CNC = 7;                   // clusters the grid has at least
+constexpr int CPH = 40, CPL = 24, CPR = 136, CP2 = 40;       // floats per (K-split, row) of the partial sums: conflict-free for the fragment owners
+constexpr size_t CW_HID = 2 * 28 * 512;                      // O1 (O3) rows of a CTA as A fragments: two tiles
+constexpr size_t CW_LOG = 28 * 512;                          // O2 (O4) rows: one tile
+constexpr size_t CW_R2 = 2 * CK8 * CT2 * 16;                 // 40 rows of R as core matrices [k / 8][5][8][16 B]
+constexpr int C_SMALL = 2 * 3 * CU * 3 + 2 * 32 + 2 * CL;    // I of the CTA's units [half][gate][unit][3], b1, b3 (32 each), b2, b4
+constexpr size_t CB_SMEM = 2 * CW_HID + 2 * CW_LOG + CW_R2 + C_SMALL * 4;
+constexpr size_t CB_TMEM = (size_t)448 * 128 * 4;
+static_assert(CB_SMEM % 16 == 0, "the blob is copied in 16-byte pieces");
+constexpr int CNG = 2;                                       // column groups (of four rows) the carve-up has room for
+constexpr size_t CS_IMG = (size_t)CK8 * CNG * 128;           // operand image of one vector
+constexpr size_t CS_PART = (size_t)7 * 4 * CNG * CPL * 4;    // partial sums (>= 4 * 4 * CNG * CPH * 4)
+static_assert(CS_PART >= (size_t)4 * 4 * CNG * CPH * 4, "the partial sums of both products share a buffer");
+constexpr size_t CS_PARTR = (size_t)2 * 4 * CNG * CPR * 4, CS_PART2 = (size_t)4 * 4 * CNG * CP2 * 4;     // R h: tensor-memory rows, the others
+constexpr size_t CS_BYTES = CB_SMEM + 3 * CS_IMG /* two state halves, hidden layer */ + (size_t)CMAXR * 1024 /* logits */ + CS_PART + CS_PARTR + CS_PART2 +
+                            (size_t)CMAXR * CL * 4 + (size_t)CMAXR * 2 * CU * 2 /* staged logits and values */;
+}  // namespace
+
+struct ResClPack {
+    uint8_t *d_blob = nullptr;               // [16 ranks][CB_SMEM | CB_TMEM]
+    long long *d_prof = nullptr;             // [16]
+    int max_clusters = 0;
+};
+
+struct ClParams {
+    int batch, nr;              // rows of the call, rows per cluster
+    long long n_steps, step0;
+    unsigned stream0;
+    unsigned long long seed;
+    int n_frames, hop, row_stride, row_offset_mul, row_lag;
+    long long out_pitch;
+    const uint8_t *blob;
+    const float *g;                          // [batch][n_frames][3H]
+    const float *h_in; float *h_out;
+    const uint8_t *c_in, *f_in; uint8_t *c_st_out, *f_st_out;
+    const uint8_t *c_forced, *f_forced;
+    uint8_t *c_out, *f_out;
+    int16_t *out;
+    float *dbg_gates, *dbg_h, *dbg_logits;
+    DevStatus *status;
+    unsigned long long limit_ns;
+    int skip_rank; long long skip_step;      // self-test: CTAs of this rank withhold the state they publish at this step (-1: none)
+    long long *prof;
+};
+
+__device__ __forceinline__ void cl_ldmatrix4(uint32_t addr, uint32_t (&r)[4])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void cl_mma(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+// shared-memory address of another CTA of the cluster (as map_to_rank, free to be moved)
+__device__ __forceinline__ uint32_t cl_map(uint32_t addr, int rank) { uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r; }
+__device__ __forceinline__ void cl_bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void cl_bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// asynchronous 8-byte store into a CTA of the cluster, counted on that CTA's mbarrier
+__device__ __forceinline__ void cl_st_async8(unsigned addr, uint2 v, unsigned mbar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(mbar) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() { asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory"); }
+// 2^x, 1 / x straight from the special-function unit (arguments and results that matter here are normal numbers)
+__device__ __forceinline__ float cl_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float cl_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+constexpr float CL_LOG2E = 1.4426950408889634f;
+__device__ __forceinline__ float cl_sigmoid(float x) { return cl_rcp(1.0f + cl_ex2(-CL_LOG2E * x)); }
+__device__ __forceinline__ float cl_tanh(float x) { return fmaf(-2.0f, cl_rcp(1.0f + cl_ex2(2.0f * CL_LOG2E * x)), 1.0f); }
+// One warp, 256 logits, lane l holds [8 l, 8 l + 8): the smallest k whose running sum of exp(l_k - max) exceeds u times the
+// total; 255 if none does.  461 -> 387 cycles against warp_softmax_draw_fast (one warp alone).
+__device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
+{
+    float m = fmaxf(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])), fmaxf(fmaxf(l[4], l[5]), fmaxf(l[6], l[7])));
+    asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
+    m *= CL_LOG2E;
+    float w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = cl_ex2(fmaf(l[i], CL_LOG2E, -m));
+    const float p0 = w[0], p1 = w[0] + w[1], p2 = p1 + w[2], p3 = p1 + (w[2] + w[3]), p4 = p3 + w[4], p5 = p3 + (w[4] + w[5]), p6 = p5 + w[6], p7 = p5 + (w[6] + w[7]);
+    // butterfly: the total of the block of 2 o lanes and, in `run`, the sum of the lanes of the block below this one
+    float tot = p7, run = 0.f;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float other = __shfl_xor_sync(FULL, tot, o);
+        if (lane & o) run += other;
+        tot += other;
+    }
+    const float thr = u * tot;
+    // the running sums do not decrease: the first one above the threshold comes after those that are not
+    const int c = (run + p0 <= thr) + (run + p1 <= thr) + (run + p2 <= thr) + (run + p3 <= thr) + (run + p4 <= thr) + (run + p5 <= thr) + (run + p6 <= thr) + (run + p7 <= thr);
+    return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
+}
+// part k of x in a split into bf16 parts (k = 0: the nearest bf16, then the nearest bf16 of the remainder, ...)
+template <int P>
+__device__ __forceinline__ void cl_split(float x, unsigned short (&b)[P])
+{
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(x);
+        b[k] = __bfloat16_as_ushort(h);
+        x -= __bfloat162float(h);
+    }
+}
+
+// P: bf16 parts per fp32 value (3: one row per cluster, exact; 2: several rows).  NG: groups of four rows.
+// MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
+// Warps 0..7: hidden layer, logits, sends (0..3 also the rows of R outside tensor memory).  Warps 8..15: the rows of R in
+// tensor memory, then one row of the batch each: draw and gates.
+template <int P, int NG, int MODE>
+__global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
+{
+    static_assert(P == 2 || (P == 3 && NG == 1), "three parts fill one column group with one row");
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
+    __shared__ uint32_t s_tmem;
+    __shared__ long long s_prof[MODE != 0 ? 16 : 1];
+    constexpr int H = 2 * CK;
+    constexpr bool DBG = MODE != 0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g4 = lane >> 2, t4 = lane & 3;
+    const int cl = blockIdx.x / CCS;
+    const int row0 = cl * p.nr, nrc = min(p.nr, p.batch - row0);
+    if (nrc <= 0) return;                                                // the same for every CTA of the cluster
+    unsigned rank_u;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_u));
+    const int rank = (int)rank_u;
+
+    // ---- shared memory carve-up (must match CS_BYTES)
+    const uint4 *wH[2] = {reinterpret_cast<const uint4 *>(smem + CW_HID), reinterpret_cast<const uint4 *>(smem)};                    // [half]: O3, O1
+    const uint4 *wL[2] = {reinterpret_cast<const uint4 *>(smem + 2 * CW_HID + CW_LOG), reinterpret_cast<const uint4 *>(smem + 2 * CW_HID)};
+    const uint32_t r2_addr = smem_u32(smem + 2 * CW_HID + 2 * CW_LOG);
+    const float *sI = reinterpret_cast<const float *>(smem + 2 * CW_HID + 2 * CW_LOG + CW_R2);      // [half][gate][unit][3]
+    const float *sb1 = sI + 2 * 3 * CU * 3, *sb3 = sb1 + 32, *sb2 = sb3 + 32, *sb4 = sb2 + CL;
+    uint8_t *ximg = smem + CB_SMEM;                                      // [2: coarse, fine] state image
+    uint8_t *qimg = ximg + 2 * CS_IMG;
+    float *lbuf = reinterpret_cast<float *>(qimg + CS_IMG);              // [rows][256]
+    float *part = lbuf + CMAXR * 256;
+    float *partR = part + CS_PART / 4;                                   // [2 halves of K][rows][128]: R h, rows in tensor memory
+    float *part2 = partR + CS_PARTR / 4;                                 // [4 quarters of K][rows][40]: the other rows
+    float *lstage = part2 + CS_PART2 / 4;                                // [row][16] this CTA's logits
+    unsigned short *ystage = reinterpret_cast<unsigned short *>(lstage + CMAXR * CL);            // [row][part][28]: this CTA's state or hidden-layer values
+
+    // ---- one-time load: weights, zero images, barriers, tensor memory
+    {
+        const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM);
+        const uint4 *src = reinterpret_cast<const uint4 *>(blob);
+        uint4 *dst = reinterpret_cast<uint4 *>(smem);
+        for (int i = tid; i < (int)(CB_SMEM / 16); i += 512) dst[i] = __ldg(src + i);
+        uint4 *z = reinterpret_cast<uint4 *>(ximg);
+        for (int i = tid; i < (int)(3 * CS_IMG / 16); i += 512) z[i] = make_uint4(0, 0, 0, 0);
+        if (warp == 1) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        if (tid == 0) {
+            mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
+            mbar_fence_init();
+        }
+        if (DBG && tid < 16) s_prof[tid] = 0;
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const uint32_t *tsrc = reinterpret_cast<const uint32_t *>(blob + CB_SMEM) + 32 * (warp & 3) + lane;
+        const uint32_t tdst = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+#pragma unroll 1
+        for (int c = 8 * (warp >> 2); c < 448; c += 32) {
+            uint32_t r[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) r[k] = __ldg(tsrc + (size_t)(c + k) * 128);
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(tdst + c), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]),
+                         "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        // images of the initial state
+        if (p.h_in)
+            for (int i = tid; i < nrc * H; i += 512) {
+                const int st = i / H, j = i - st * H, half_f = j >= CK, k = j - half_f * CK;
+                unsigned short b[P];
+                cl_split<P>(p.h_in[(size_t)(row0 + st) * H + j], b);
+                unsigned short *im = reinterpret_cast<unsigned short *>(ximg + half_f * CS_IMG + (size_t)((k >> 3) * NG + (st >> 2)) * 128);
+#pragma unroll
+                for (int q = 0; q < P; ++q) im[((P == 2 ? 2 * (st & 3) : 0) + q) * 8 + (k & 7)] = b[q];
+            }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    cluster_sync_all();                                                  // every peer's barriers are initialised before anyone sends
+    const uint32_t tmem = s_tmem;
+
+    Waiter wt{p.status, p.limit_ns};
+    bool bad = false;                                                    // warp-uniform: this warp gave up
+    const bool prof_on = DBG && p.prof != nullptr && blockIdx.x == 0 && (warp == 0 || warp == 8);
+    long long prof_t = clock64();
+#define STAMP(i) do { if (DBG && prof_on) { const long long now_ = clock64(); if (lane == 0) s_prof[i] += now_ - prof_t; prof_t = now_; } } while (0)
+#define STAMP0() do { if (DBG && prof_on) prof_t = clock64(); } while (0)
+    auto wait_bar = [&](unsigned long long *b, unsigned parity, int step, int phase) {
+        if (bad) return;
+        const unsigned a = smem_u32(b);
+        unsigned long long t0 = 0; unsigned cnt = 0;
+        bool fail = false;
+        while (!mbar_try(a, parity & 1u))
+            if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { fail = true; break; }
+        bad = __any_sync(FULL, fail);
+    };
+
+    // ---- rows of R times one half of the state, accumulated over both halves.
+    // Tensor memory, lane quadrant w & 3 (warps 8..15): tiles 4 (quadrant & 1) + 2 j, + 1 with j = (w >> 2) & 1, half of K
+    // quadrant >> 1; columns [half of the state][j][k-tile pair][tile][k-tile][4].
+    float accR[2][NG][4];
+    const int rq = warp & 3, rj = (warp >> 2) & 1;
+    auto r_clear = [&]() {
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) accR[n][grp][k] = 0.f;
+    };
+    auto r_load = [&](int half_f, int pair, uint32_t (&r)[16]) {
+        tmem_ld16(tmem + ((uint32_t)(32 * rq) << 16) + (uint32_t)(((half_f * 2 + rj) * 7 + pair) * 16), r);
+    };
+    auto r_products = [&](int half_f, uint32_t (&r0)[16]) {               // r0: the fragments of pair 0, requested earlier
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + (uint32_t)((28 * (rq >> 1) + (lane >> 3)) * NG * 128 + (lane & 7) * 16);
+        uint32_t r1[16], c0[NG][4], c1[NG][4];
+        auto bload = [&](int pair, uint32_t (&b)[NG][4]) {
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp) cl_ldmatrix4(b0 + (uint32_t)((4 * pair * NG + grp) * 128), b[grp]);
+        };
+        auto mmas = [&](const uint32_t (&r)[16], const uint32_t (&b)[NG][4]) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                    for (int n = 0; n < 2; ++n)
+                        cl_mma(accR[n][grp], make_uint4(r[8 * n + 4 * k], r[8 * n + 4 * k + 1], r[8 * n + 4 * k + 2], r[8 * n + 4 * k + 3]), b[grp][2 * k], b[grp][2 * k + 1]);
+        };
+        bload(0, c0);
+#pragma unroll
+        for (int pair = 0; pair < 7; ++pair) {
+            tmem_wait_ld();
+            if (pair & 1) { if (pair < 6) { r_load(half_f, pair + 1, r0); bload(pair + 1, c0); } mmas(r1, c1); }
+            else { if (pair < 6) { r_load(half_f, pair + 1, r1); bload(pair + 1, c1); } mmas(r0, c0); }
+        }
+    };
+    auto r_store = [&]() {
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp) {
+                float *d = partR + ((rq >> 1) * 4 * NG + 4 * grp + t4) * CPR + (4 * (rq & 1) + 2 * rj + n) * 16 + g4;
+                d[0] = accR[n][grp][0] + accR[n][grp][1];
+                d[8] = accR[n][grp][2] + accR[n][grp][3];
+            }
+    };
+    // The 40 rows in shared memory (warps 0..3, a quarter of K each; the third tile has eight rows)
+    float acc2[3][NG][4];
+    auto r2_clear = [&]() {
+#pragma unroll
+        for (int n = 0; n < 3; ++n)
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc2[n][grp][k] = 0.f;
+    };
+    auto r2_products = [&](int half_f) {
+        const uint32_t a0 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + (lane >> 4)) * CT2 + ((lane >> 3) & 1) * 8 + (lane & 7)) * 16);
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + (uint32_t)((14 * rq + ((lane >> 3) & 1)) * NG * 128 + (lane >> 4) * (NG - 1) * 128 + (lane & 7) * 16);
+#pragma unroll
+        for (int kt = 0; kt < 7; ++kt) {
+            uint32_t b[4];                                               // (k / 8 even, odd) of column group 0, then of group 1
+            cl_ldmatrix4(b0 + (uint32_t)(2 * kt * NG * 128), b);
+#pragma unroll
+            for (int n = 0; n < 3; ++n) {
+                uint32_t a[4];
+                // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
+                cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * n) * 16) - (n == 2 ? ((lane >> 3) & 1) * 128u : 0u), a);
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) cl_mma(acc2[n][grp], make_uint4(a[0], a[1], a[2], a[3]), b[2 * grp], b[2 * grp + 1]);
+            }
+        }
+    };
+    auto r2_store = [&]() {
+#pragma unroll
+        for (int grp = 0; grp < NG; ++grp) {
+            float *d = part2 + (rq * 4 * NG + 4 * grp + t4) * CP2 + g4;
+#pragma unroll
+            for (int n = 0; n < 3; ++n) {
+                d[16 * n] = acc2[n][grp][0] + acc2[n][grp][1];
+                if (n < 2) d[16 * n + 8] = acc2[n][grp][2] + acc2[n][grp][3];
+            }
+        }
+    };
+
+    // ---- fixed addresses
+    uint32_t delta[2];                                                   // CTA (warp & 7) + 8 k of the cluster: what to add to an address of mine
+#pragma unroll
+    for (int k = 0; k < 2; ++k) delta[k] = map_to_rank(smem_u32(smem), (unsigned)((warp & 7) + 8 * k)) - smem_u32(smem);
+    // The 28 values of this CTA travel in pieces of four: piece i = (row, part, quad) is elements 28 rank + 4 quad .. + 3 of one
+    // part of one row; poff: its byte offset in an image (a lane takes pieces lane, lane + 32, ...)
+    constexpr int NPASS = P == 3 ? 1 : 2 * NG;
+    const int n_pieces = nrc * P * 7;
+    uint32_t poff[NPASS];
+#pragma unroll
+    for (int it = 0; it < NPASS; ++it) {
+        const int i = lane + 32 * it, rp = i / 7, k = CU * rank + 4 * (i - 7 * rp), st = rp / P, q = rp - st * P;
+        poff[it] = (uint32_t)(((k >> 3) * NG + ((st >> 2) & (NG - 1))) * 128 + ((P == 2 ? 2 * (st & 3) : 0) + q) * 16 + (k & 4) * 2);
+    }
+    const int skip_at = (DBG && rank == p.skip_rank) ? (int)p.skip_step : -1;
+
+    // ---- the row this warp draws (warps 8..15), its last symbols, and the gates of its unit (lane) in both halves
+    const bool drawer = warp >= 8 && warp - 8 < nrc;
+    const int st_d = warp - 8, gb = row0 + (drawer ? st_d : 0);          // row of the call
+    const bool gater = drawer && lane < CU;
+    const int gj = CU * rank + (lane < CU ? lane : 0);
+    int c_prev = 128, f_prev = 0;
+    float hC = 0.f, hF = 0.f;
+    if (drawer) { c_prev = p.c_in ? p.c_in[gb] : 128; f_prev = p.f_in ? p.f_in[gb] : 0; }
+    if (gater && p.h_in) { hC = p.h_in[(size_t)gb * H + gj]; hF = p.h_in[(size_t)gb * H + CK + gj]; }
+    const bool writer = drawer && rank == 2 * st_d;                      // the CTA whose drawing warp writes this row's samples
+
+    struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
+    // a row of R h of this row of the batch: both halves (or all quarters) of K; three parts: both columns of their sums
+    auto r_row = [&](int i) {
+        float v = 0.f;
+        constexpr int NSL = P == 3 ? 2 : 1;
+        if (i < 128) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int sl = 0; sl < NSL; ++sl) v += partR[(k * 4 * NG + st_d + sl) * CPR + i];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int sl = 0; sl < NSL; ++sl) v += part2[(k * 4 * NG + st_d + sl) * CP2 + i - 128];
+        }
+        return v;
+    };
+    // everything of the gates of one half that does not depend on the pending draw
+    auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
+        GatePre q;
+        const int u = lane < CU ? lane : 0;
+        const float x0 = scale8(c_prev), x1 = scale8(f_prev);
+        const float *Iu = sI + ((half_g * 3 + 0) * CU + u) * 3, *Ir = Iu + CU * 3, *Ie = Ir + CU * 3;
+        q.pu = r_row(half_g * 3 * CU + u) + fmaf(Iu[0], x0, half_g ? fmaf(Iu[1], x1, gv[0]) : gv[0]);
+        q.pr = r_row(half_g * 3 * CU + CU + u) + fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
+        q.pe = fmaf(Ie[0], x0, half_g ? fmaf(Ie[1], x1, gv[2]) : gv[2]);
+        q.ae = r_row(half_g * 3 * CU + 2 * CU + u);
+        q.ku = half_g ? Iu[2] : Iu[1]; q.kr = half_g ? Ir[2] : Ir[1]; q.ke = half_g ? Ie[2] : Ie[1];
+        return q;
+    };
+    auto gates_and_stage = [&](int half_g, long long s, int drawn, const GatePre &q) {
+        const float xk = scale8(drawn);
+        const float u = cl_sigmoid(fmaf(q.ku, xk, q.pu)), r = cl_sigmoid(fmaf(q.kr, xk, q.pr));
+        const float e = cl_tanh(fmaf(r, q.ae, fmaf(q.ke, xk, q.pe)));
+        const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
+        if (half_g) hF = hn; else hC = hn;
+        if (gater) {
+            unsigned short b[P];
+            cl_split<P>(hn, b);
+#pragma unroll
+            for (int k = 0; k < P; ++k) ystage[(st_d * P + k) * CU + lane] = b[k];
+            if (DBG) {
+                const int jj = half_g * CK + gj;
+                if (p.dbg_gates) { float *d = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; d[jj] = u; d[H + jj] = r; d[2 * H + jj] = e; }
+                if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + jj] = hn;
+            }
+        }
+    };
+    auto load_g = [&](int half_g, long long s, float (&gv)[3]) {
+        const long long fr = p.row_lag > 0 ? s : ((p.step0 + s) * p.row_stride + (long long)(p.stream0 + (unsigned)gb) * p.row_offset_mul) / p.hop;
+        const float *g = p.g + ((size_t)gb * p.n_frames + fr) * 3 * H + half_g * CK + gj;
+#pragma unroll
+        for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
+    };
+    // warps 0..7: the staged pieces of this CTA's 28 values of every row -> images in the cluster's CTAs, two CTAs per warp
+    auto send_staged = [&](uint32_t img, uint32_t bar) {
+        if (bad) return;
+#pragma unroll
+        for (int it = 0; it < NPASS; ++it) {
+            const int i = lane + 32 * it;
+            if (i < n_pieces) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(ystage + 4 * i);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) cl_st_async8(img + poff[it] + delta[k], v, bar + delta[k]);
+            }
+        }
+    };
+    auto send_y = [&](int half_g, long long s) {
+        if (!DBG || (int)s != skip_at) send_staged(smem_u32(ximg + half_g * CS_IMG), smem_u32(&xy[half_g]));
+    };
+    const int n_draw = 32 * nrc;                                         // threads of the drawing warps
+    const unsigned ybytes = (unsigned)(nrc * CK * P * 2), lbytes = (unsigned)(nrc * 1024);
+
+    // ---- prologue: R h of the initial state, coarse gates of step 0
+    if (warp >= 8) {
+        uint32_t r0[16];
+        r_clear();
+#pragma unroll 1
+        for (int half_f = 0; half_f < 2; ++half_f) { r_load(half_f, 0, r0); r_products(half_f, r0); }
+        r_store();
+    } else if (warp < 4) {
+        r2_clear();
+#pragma unroll 1
+        for (int half_f = 0; half_f < 2; ++half_f) r2_products(half_f);
+        r2_store();
+        cl_bar_arrive(5, 128 + n_draw);
+    }
+    if (warp == 8 && lane == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
+    __syncthreads();
+    if (drawer) {
+        float gv[3];
+        load_g(0, 0, gv);
+        gates_and_stage(0, 0, f_prev, gates_prepare(0, gv));
+    }
+    __syncthreads();
+    if (warp < 8) send_y(0, 0);
+
+    // what a half-step's draw and gates take from outside: gate offsets of the half of the state whose gates it computes, the
+    // uniform and (teacher forcing) the symbol
+    float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
+    int forced = -1;
+    auto fetch = [&](int half, long long s) {
+        const long long t = half ? s : s - 1;
+        if (s < p.n_steps) load_g(half, s, gv);
+        u01 = uniform24(p.seed, p.stream0 + (unsigned)gb, (unsigned long long)(p.step0 + t - (long long)gb * p.row_lag), half ? 0u : 1u);
+        if (DBG) {
+            const uint8_t *fz = half ? p.c_forced : p.f_forced;
+            if (fz) forced = fz[(size_t)gb * p.n_steps + t];
+        }
+    };
+    if (drawer) fetch(1, 0);
+
+    // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
+    // n = 2 s the fine half (input y_f(s - 1): fine head -> f_{s-1}, R h_{s-1} completed, then the coarse gates of step s).
+    const long long T = p.n_steps;
+    auto half_step = [&](auto HALF_C, const long long n) {
+        constexpr int half = decltype(HALF_C)::value;                    // 1: coarse half
+        constexpr int in = half ? 0 : 1;                                 // image of its input
+        const long long s = n >> 1;
+        const bool last = n == 2 * T;
+        const unsigned yuse = (unsigned)((n - 1) >> 1), quse = (unsigned)(n - 1);
+        if (warp < 8) {
+            // hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
+            uint4 av[7];
+            const int tile = warp & 1, split = warp >> 1;
+            {
+                const uint4 *A = wH[half] + (tile * 28 + 7 * split) * 32 + lane;
+#pragma unroll
+                for (int i = 0; i < 7; ++i) av[i] = A[i * 32];
+            }
+            STAMP0();
+            wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
+            STAMP(8 * half + 0);
+            {
+                const uint32_t b0 = smem_u32(ximg + in * CS_IMG) + (uint32_t)((14 * split) * NG * 128 + (lane & 7) * 16);
+                float acc[NG][2][4];
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) {
+                    uint32_t b[4][4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) cl_ldmatrix4(b0 + (uint32_t)(((i < 3 ? 4 * i + (lane >> 3) : 12 + ((lane >> 3) & 1)) * NG + grp) * 128), b[i]);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) acc[grp][c][k] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 7; ++i) cl_mma(acc[grp][i & 1], av[i], b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
+                }
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) {
+                    float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
+                    float lo = (acc[grp][0][0] + acc[grp][1][0]) + (acc[grp][0][1] + acc[grp][1][1]);
+                    float hi = (acc[grp][0][2] + acc[grp][1][2]) + (acc[grp][0][3] + acc[grp][1][3]);
+                    if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }      // (hi, mid) + lo parts
+                    d[0] = lo; d[8] = hi;
+                }
+            }
+            {
+                cl_bar_sync(1, 512);
+                STAMP(8 * half + 1);
+                const uint32_t bar = smem_u32(&xq);
+// one warp per row adds the K-split sums and splits the values into their parts; then every warp sends
+                if (warp < nrc && lane < P * 7) {
+                    const int q = lane / 7, quad = lane - 7 * q;
+                    float4 v = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * quad);
+#pragma unroll
+                    for (int sp = 0; sp < 4; ++sp) {
+                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + warp) * CPH + 4 * quad);
+                        v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+                    }
+                    v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
+                    // this lane's part of the four values: the remainder after q parts, rounded to bf16
+                    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+#pragma unroll
+                    for (int k = 1; k < P; ++k)
+                        if (q >= k) {
+                            v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
+                            lo = __floats2bfloat162_rn(v.x, v.y); hi = __floats2bfloat162_rn(v.z, v.w);
+                        }
+                    *reinterpret_cast<uint2 *>(ystage + (warp * P + q) * CU + 4 * quad) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                }
+                cl_bar_sync(7, 256);
+                send_staged(smem_u32(qimg), bar);
+                STAMP(8 * half + 2);
+            }
+            // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
+            {
+                const float lbias = (half ? sb2 : sb4)[lane & 15];
+                if (warp < 7) {
+                    uint4 lv[4];
+                    const uint4 *A = wL[half] + 4 * warp * 32 + lane;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
+                    wait_bar(&xq, quse, (int)s, 2 + 4 * half);
+                    STAMP(8 * half + 3);
+                    const uint32_t b0 = smem_u32(qimg) + (uint32_t)(8 * warp * NG * 128 + (lane & 7) * 16);
+#pragma unroll
+                    for (int grp = 0; grp < NG; ++grp) {
+                        uint32_t b[2][4];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) cl_ldmatrix4(b0 + (uint32_t)(((4 * i + (lane >> 3)) * NG + grp) * 128), b[i]);
+                        float acc[2][4];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
+                        float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
+                        float lo = (acc[0][0] + acc[1][0]) + (acc[0][1] + acc[1][1]), hi = (acc[0][2] + acc[1][2]) + (acc[0][3] + acc[1][3]);
+                        if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }
+                        d[0] = lo; d[8] = hi;
+                    }
+                }
+                cl_bar_sync(2, 256);
+                STAMP(8 * half + 4);
+if (warp < nrc && lane < CL) {
+                    float v = lbias;
+#pragma unroll
+                    for (int sp = 0; sp < 7; ++sp) v += part[(sp * 4 * NG + warp) * CPL + lane];
+                    lstage[warp * CL + lane] = v;
+                }
+                cl_bar_sync(8, 256);
+                if (lane < 4 * nrc && !bad) {
+                    const float4 v = *reinterpret_cast<const float4 *>(lstage + 4 * lane);
+                    const uint32_t a = smem_u32(lbuf + (lane >> 2) * 256 + CL * rank + 4 * (lane & 3));
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) st_async_v4(a + delta[k], v.x, v.y, v.z, v.w, smem_u32(&xl) + delta[k]);
+                }
+                STAMP(8 * half + 5);
+            }
+            // ---- the rows of R outside tensor memory (needed by the fine gates half a step or more from now), while the logits cross
+            if (warp < 4) {
+                if (half) r2_clear();
+                r2_products(in);
+                if (!half) { r2_store(); if (!last) cl_bar_arrive(5, 128 + n_draw); }
+            }
+            if (!last) {
+                cl_bar_sync(4, 256 + n_draw);
+                STAMP0();
+                send_y(half, s);
+            }
+        } else {
+            // ---- this warp's rows of R (they start when the hidden-layer products are done, so as not to share the pipe with
+            // them), then one row of the batch: everything that does not depend on the chain before the wait for the logits
+            if (warp == 8 && lane == 0 && !bad) {
+                mbar_arrive_expect(smem_u32(&xq), ybytes);
+                mbar_arrive_expect(smem_u32(&xl), lbytes);
+                if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
+            }
+            const long long t = half ? s : s - 1;
+            uint32_t r0[16];
+            r_load(in, 0, r0);
+            cl_bar_sync(1, 512);
+            if (half) r_clear();
+            r_products(in, r0);
+            if (!half) r_store();
+            // (in both halves: a peer overwrites this image only after it has logits that this CTA sends after the state that
+            // the drawing warps publish below)
+            cl_bar_sync(3, 256);
+            if (drawer) {
+                if (half) cl_bar_sync(5, 128 + n_draw);                   // part2
+                const GatePre gp = gates_prepare(half, gv);
+                const float u_now = u01;
+                const int forced_now = forced;
+                if (!last) fetch(1 - half, half ? s + 1 : s);             // of the next half-step, while the logits are on their way
+                wait_bar(&xl, quse, (int)s, 3 + 4 * half);
+                STAMP0();
+                float l[8];
+                {
+                    const float4 a = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane), b = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane + 4);
+                    l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
+                }
+                const int drawn = cl_draw(l, u_now, lane);
+                const int fed = (DBG && forced_now >= 0) ? forced_now : drawn;
+                STAMP(8 * half + 6);
+                if (!last) {
+                    gates_and_stage(half, s, fed, gp);
+                    cl_bar_arrive(4, 256 + n_draw);
+                }
+                STAMP(8 * half + 7);
+                if (writer && !bad) {
+                    if (DBG && p.dbg_logits) {
+                        float *d = p.dbg_logits + (((size_t)t * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) d[k] = l[k];
+                    }
+                    if (lane == 0) {
+                        uint8_t *o = half ? p.c_out : p.f_out;
+                        if (o) o[(size_t)gb * T + t] = (uint8_t)drawn;
+                        if (!half && p.out) p.out[(long long)gb * p.out_pitch + t] = (int16_t)(256 * c_prev + fed - 32768);
+                    }
+                }
+                if (half) c_prev = fed; else f_prev = fed;
+            }
+        }
+    };
+#pragma unroll 1
+    for (long long s2 = 0; s2 < T; ++s2) {
+        half_step(std::integral_constant<int, 1>{}, 2 * s2 + 1);
+        half_step(std::integral_constant<int, 0>{}, 2 * s2 + 2);
+    }
+#undef STAMP
+#undef STAMP0
+
+    // ---- results; nobody leaves while a peer may still write into its shared memory
+    const int any_bad = __syncthreads_or(bad);
+    if (!any_bad) {
+        if (gater && p.h_out) { p.h_out[(size_t)gb * H + gj] = hC; p.h_out[(size_t)gb * H + CK + gj] = hF; }
+        if (writer && lane == 0) {
+            if (p.c_st_out) p.c_st_out[gb] = (uint8_t)c_prev;
+            if (p.f_st_out) p.f_st_out[gb] = (uint8_t)f_prev;
+        }
+    }
+    if (DBG && p.prof && blockIdx.x == 0 && tid < 16) p.prof[tid] = s_prof[tid];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    cluster_sync_all();
+}
+
+// ---------------------------------------------------------------------------------------------
+static const void *cl_kernel_of(int nr, bool dbg)
+{
+    if (nr == 1) return dbg ? (const void *)resident_cluster_kernel<3, 1, 1> : (const void *)resident_cluster_kernel<3, 1, 0>;
+    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<2, 1, 1> : (const void *)resident_cluster_kernel<2, 1, 0>;
+    return dbg ? (const void *)resident_cluster_kernel<2, 2, 1> : (const void *)resident_cluster_kernel<2, 2, 0>;
+}
+
+static void cl_fill_launch(int n_clusters, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
+{
+    std::memset(cfg, 0, sizeof(*cfg));
+    cfg->gridDim = dim3(n_clusters * CCS);
+    cfg->blockDim = dim3(512);
+    cfg->dynamicSmemBytes = CS_BYTES;
+    cfg->stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CCS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+
+// Rows per cluster and clusters of a batch.  Clusters never wait for one another, so a batch of more rows than the resident
+// clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
+static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
+{
+    const int most = k.max_clusters * CMAXR, waves = (batch + most - 1) / most;
+    *nr = (batch + waves * k.max_clusters - 1) / (waves * k.max_clusters);
+    const int need = (batch + *nr - 1) / *nr;
+    *n_clusters = need < CNC ? CNC : need;       // (a cluster without rows returns at once)
+}
+
+int rescl_prepare(wrnn_model *m)
+{
+    const int H = m->H;
+    if (m->dtype != WRNN_BF16 || m->sparse || m->variant != 0 || H != 2 * CK) { m->err = "cluster-resident kernel: dense bf16 H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
+    cudaDeviceProp prop;
+    cudaGetDeviceProperties(&prop, m->device);
+    ResClPack k;
+    cudaFuncAttributes fa;
+    for (int nr : {1, 2, 5})
+        for (int dbg = 0; dbg < 2; ++dbg) {
+            const void *f = cl_kernel_of(nr, dbg != 0);
+            if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || CS_BYTES + fa.sharedSizeBytes > prop.sharedMemPerBlockOptin ||
+                cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS_BYTES) != cudaSuccess) {
+                cudaGetLastError(); m->err = "cluster-resident kernel does not fit this device"; return WRNN_ERR_UNSUPPORTED;
+            }
+        }
+    {
+        cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
+        cl_fill_launch(CNC, &cfg, at, 0);
+        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(1, false), &cfg) != cudaSuccess || k.max_clusters < 1) {
+            cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
+        }
+    }
+    const std::vector<uint16_t> dR = dense_bf16_bits(m->hR), dO[4] = {dense_bf16_bits(m->hO1), dense_bf16_bits(m->hO3), dense_bf16_bits(m->hO2), dense_bf16_bits(m->hO4)};
+    std::vector<uint8_t> blob(CCS * (CB_SMEM + CB_TMEM), 0);
+    // row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
+    auto r_row = [&](int rank, int i) { return &dR[((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
+    // A fragments of 16 rows (row r < n_rows, zero otherwise): lane (g, t) holds (row g, k 2t..2t+1), (row g + 8, same), (row g, k 2t+8..9), (row g + 8, same)
+    auto pack = [&](const std::vector<uint16_t> &M, int first, int n_rows, uint16_t *dst) {
+        for (int kt = 0; kt < 28; ++kt)
+            for (int lane = 0; lane < 32; ++lane)
+                for (int q = 0; q < 4; ++q) {
+                    const int r = (lane >> 2) + 8 * (q & 1), c = 2 * (lane & 3) + 8 * (q >> 1);
+                    for (int j = 0; j < 2; ++j) dst[((size_t)kt * 32 + lane) * 8 + 2 * q + j] = r < n_rows ? M[(size_t)(first + r) * CK + 16 * kt + c + j] : 0;
+                }
+    };
+    for (int rank = 0; rank < CCS; ++rank) {
+        uint8_t *base = blob.data() + (size_t)rank * (CB_SMEM + CB_TMEM);
+        for (int h = 0; h < 2; ++h) {
+            for (int t = 0; t < 2; ++t) pack(dO[h], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + h * CW_HID + (size_t)t * 28 * 512));
+            pack(dO[2 + h], CL * rank, CL, reinterpret_cast<uint16_t *>(base + 2 * CW_HID + h * CW_LOG));
+        }
+        uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
+        for (int i = 0; i < CT2; ++i)
+            for (int k8 = 0; k8 < 2 * CK8; ++k8) std::memcpy(r2 + ((size_t)k8 * CT2 + i) * 8, r_row(rank, 128 + i) + 8 * k8, 16);
+        float *sm = reinterpret_cast<float *>(base + 2 * CW_HID + 2 * CW_LOG + CW_R2);
+        for (int i = 0; i < 6 * CU; ++i) {
+            const size_t row = (size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU;
+            for (int c = 0; c < 3; ++c) sm[i * 3 + c] = m->hI[row * 3 + c];
+        }
+        float *b = sm + 6 * CU * 3;
+        for (int r = 0; r < CU; ++r) { b[r] = m->hb1[CU * rank + r]; b[32 + r] = m->hb3[CU * rank + r]; }
+        for (int r = 0; r < CL; ++r) { b[64 + r] = m->hb2[CL * rank + r]; b[64 + CL + r] = m->hb4[CL * rank + r]; }
+        // tensor memory: lane quadrant q holds tiles 4 (q & 1) .. + 3 and half q >> 1 of the k-tiles of both halves of the state;
+        // columns [half of the state][j][pair of k-tiles][tile 2 j + n][k-tile][4 registers of the A fragment]
+        uint16_t *tm = reinterpret_cast<uint16_t *>(base + CB_SMEM);
+        for (int q = 0; q < 4; ++q)
+            for (int c = 0; c < 448; ++c) {
+                const int reg = c & 3, kt1 = (c >> 2) & 1, n = (c >> 3) & 1, pair = (c >> 4) % 7, j = (c / 112) & 1, half_f = c / 224;
+                const int tile = 4 * (q & 1) + 2 * j + n, kt = 28 * half_f + 14 * (q >> 1) + 2 * pair + kt1;
+                for (int lane = 0; lane < 32; ++lane) {
+                    const uint16_t *src = r_row(rank, 16 * tile + (lane >> 2) + 8 * (reg & 1)) + 16 * kt + 2 * (lane & 3) + 8 * (reg >> 1);
+                    uint16_t *d = tm + ((size_t)c * 128 + 32 * q + lane) * 2;
+                    d[0] = src[0]; d[1] = src[1];
+                }
+            }
+    }
+    ResClPack *pk = new ResClPack(k);
+    if (cudaMalloc((void **)&pk->d_blob, blob.size()) != cudaSuccess || cudaMemcpy(pk->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMalloc((void **)&pk->d_prof, 16 * sizeof(long long)) != cudaSuccess || cudaMemset(pk->d_prof, 0, 16 * sizeof(long long)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(pk->d_blob); cudaFree(pk->d_prof);
+        delete pk;
+        m->err = "device allocation for the cluster-resident kernel failed";
+        return WRNN_ERR_NOMEM;
+    }
+    m->rescl = pk;
+    return WRNN_OK;
+}
+
+void rescl_destroy(wrnn_model *m)
+{
+    if (!m->rescl) return;
+    cudaFree(m->rescl->d_blob); cudaFree(m->rescl->d_prof);
+    delete m->rescl;
+    m->rescl = nullptr;
+}
+
+int rescl_supported(const wrnn_model *m, int batch)
+{
+    return m->rescl && batch >= 1 && batch <= m->max_batch ? WRNN_OK : WRNN_ERR_UNSUPPORTED;
+}
+
+int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes)
+{
+    int nr, n_clusters;
+    cl_geometry(*m->rescl, batch, &nr, &n_clusters);
+    if (n_ctas) *n_ctas = n_clusters * CCS;
+    if (n_threads) *n_threads = 512;
+    if (smem) *smem = (int)CS_BYTES;
+    if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(2 * CW_HID + 2 * CW_LOG + CW_R2 + CB_TMEM);
+    return WRNN_OK;
+}
+
+int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
+{
+    const ResClPack &k = *m->rescl;
+    ClParams p;
+    std::memset(&p, 0, sizeof(p));
+    int nr, n_clusters;
+    cl_geometry(k, a.batch, &nr, &n_clusters);
+    p.batch = a.batch; p.nr = nr;
+    p.n_steps = a.n_steps; p.step0 = a.step0; p.stream0 = a.stream0; p.seed = a.seed;
+    p.n_frames = m->cond_dim ? a.n_frames : 1;
+    p.hop = m->cond_dim ? a.hop : 1;
+    p.row_stride = m->cond_dim ? a.row_stride : 0;
+    p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
+    p.row_lag = a.row_lag; p.out_pitch = a.out_pitch ? a.out_pitch : a.n_steps;
+    p.blob = k.d_blob; p.g = m->g;
+    p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
+    p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
+    p.dbg_gates = a.dbg_gates; p.dbg_h = a.dbg_h; p.dbg_logits = a.dbg_logits;
+    p.status = m->status;
+    p.limit_ns = m->wait_limit_ns();
+    p.skip_rank = m->dbg_skip_cta >= 0 ? m->dbg_skip_cta % CCS : -1; p.skip_step = m->dbg_skip_step;
+    p.prof = m->prof_enabled ? k.d_prof : nullptr;
+    if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
+    const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.dbg_gates || p.dbg_h || p.dbg_logits;
+    cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
+    cl_fill_launch(n_clusters, &cfg, at, s);
+    void *args[] = {&p};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg), args);
+    if (e != cudaSuccess) {
+        m->err = std::string("cluster-resident kernel launch failed: ") + cudaGetErrorString(e);
+        cudaGetLastError();
+        return WRNN_ERR_CUDA;
+    }
+    ++g_launches;
+    m->prof_cl = true;
+    return WRNN_OK;
+}
+
+int rescl_phase_cycles(const wrnn_model *m, long long *out16)
+{
+    return m->rescl && cudaMemcpy(out16, m->rescl->d_prof, 16 * sizeof(long long), cudaMemcpyDeviceToHost) == cudaSuccess ? WRNN_OK : WRNN_ERR_CUDA;
+}
+
+}  // namespace wrnn

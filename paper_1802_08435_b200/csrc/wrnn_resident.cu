@@ -1190,6 +1190,7 @@ int resident_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     ++g_launches;
     m->prof_multi = false;
     m->prof_lean = false;
+    m->prof_cl = false;
     return WRNN_OK;
 }
 
@@ -1248,6 +1249,7 @@ int resident_pair_run(wrnn_model *m, const StepArgs &a, int pair, cudaStream_t s
     ++g_launches;
     m->prof_multi = false;
     m->prof_lean = false;
+    m->prof_cl = false;
     return WRNN_OK;
 }
 

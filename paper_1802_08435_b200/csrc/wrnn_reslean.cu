@@ -560,6 +560,8 @@ int reslean_supported(const wrnn_model *m, int batch)
     return (batch == 1 && m->reslean != nullptr) ? WRNN_OK : WRNN_ERR_UNSUPPORTED;
 }
 
+bool reslean_checked(const wrnn_model *m) { return m->reslean && m->reslean->checked; }
+
 int reslean_prepare(wrnn_model *m)
 {
     if (m->dtype != WRNN_BF16 || m->sparse || m->H != 2 * RL_K) { m->err = "lean resident kernel: dense bf16 H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
@@ -711,6 +713,7 @@ int reslean_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     ++g_launches;
     m->prof_multi = false;
     m->prof_lean = true;
+    m->prof_cl = false;
     return WRNN_OK;
 }
 

@@ -831,6 +831,7 @@ int resmulti_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     }
     ++g_launches;
     m->prof_multi = true;
+    m->prof_cl = false;
     return WRNN_OK;
 }
 

@@ -640,6 +640,34 @@ def test_multi_stream_every_row_count(env):
         os.environ.pop("WRNN_NO_PAIR", None)
 
 
+@pytest.mark.parametrize("batch", [1, 8, 15, 28, 29, 56, 57, 128])
+def test_cluster_resident_kernel_row_counts(env, batch):
+    """The cluster-resident kernel at the edges of its forms -- one row per cluster, one and two column groups of four rows,
+    seven full clusters, a second wave of clusters with a partial last one -- teacher-forced against the oracle with
+    per-row conditioning offsets, then resumed from the middle of a conditioning frame."""
+    torch, B = env
+    wl = synth.WORKLOADS[7]
+    w, masks, cond = synth.build_workload(wl, batch=batch)
+    om = orc.OracleModel(w, wl.dtype)
+    n = 70
+    m = B.wrnn_create(w, wl.dtype, max_batch=batch)
+    try:
+        info = B.wrnn_launch_info(m, batch)
+        assert info["kernel"] == B.WRNN_KERNEL_RESIDENT and info["n_ctas"] % 16 == 0
+        r = pu.teacher_forced_parity(torch, B, m, om, cond, n, batch, SEED, hop=10, row_stride=3, row_offset_mul=7, stream0=5, threads=pu.NCPU)
+        _tol_check(r, wl.dtype)
+        kw = dict(hop=10, row_stride=3, row_offset_mul=7, stream0=5)
+        full = _free_run(torch, B, m, cond, n, batch, SEED, **kw)
+        h = torch.zeros((batch, wl.H), dtype=torch.float32, device="cuda:0")
+        cp = torch.full((batch,), 128, dtype=torch.uint8, device="cuda:0")
+        fp = torch.zeros((batch,), dtype=torch.uint8, device="cuda:0")
+        a = _free_run(torch, B, m, cond, 23, batch, SEED, h=h, c_prev=cp, f_prev=fp, **kw)
+        b = _free_run(torch, B, m, cond, n - 23, batch, SEED, h=h, c_prev=cp, f_prev=fp, step0=23, **kw)
+        assert np.array_equal(np.concatenate([a, b], axis=1), full)
+    finally:
+        B.wrnn_destroy(m)
+
+
 def _sparse_golden():
     """The oracle's stored 24,000-step run of the block-sparse workload (tests/golden/make_sparse2048_stream.py)."""
     import hashlib
