@@ -45,7 +45,7 @@ constexpr int CK = 448;                  // H / 2
 constexpr int CU = 28;                   // state units of one half, hidden-layer rows per CTA
 constexpr int CL = 16;                   // logits rows per CTA
 constexpr int CCS = 16;                  // CTAs per cluster
-constexpr int CK8 = CK / 8;              // core matrices along K per half
+constexpr int CK8 = CK / 8, CQ = CK / 4; // groups of eight and of four values of a half
 constexpr int CT2 = 6 * CU - 128;        // rows of R outside the TMEM tile
 constexpr int CMAXR = 8;                 // rows per cluster
 constexpr int CNC = 7;                   // clusters the grid has at least
@@ -58,12 +58,12 @@ constexpr size_t CB_SMEM = 2 * CW_HID + 2 * CW_LOG + CW_R2 + C_SMALL * 4;
 constexpr size_t CB_TMEM = (size_t)448 * 128 * 4;
 static_assert(CB_SMEM % 16 == 0, "the blob is copied in 16-byte pieces");
 constexpr int CNG = 2;                                       // column groups (of four rows) the carve-up has room for
-constexpr size_t CS_IMG = (size_t)CK8 * CNG * 128;           // operand image of one vector
+constexpr size_t CS_IMG = (size_t)CQ * CNG * 64;            // operand image of one vector
 constexpr size_t CS_PART = (size_t)7 * 4 * CNG * CPL * 4;    // partial sums (>= 4 * 4 * CNG * CPH * 4)
 static_assert(CS_PART >= (size_t)4 * 4 * CNG * CPH * 4, "the partial sums of both products share a buffer");
 constexpr size_t CS_PARTR = (size_t)2 * 4 * CNG * CPR * 4, CS_PART2 = (size_t)4 * 4 * CNG * CP2 * 4;     // R h: tensor-memory rows, the others
 constexpr size_t CS_BYTES = CB_SMEM + 3 * CS_IMG /* two state halves, hidden layer */ + (size_t)CMAXR * 1024 /* logits */ + CS_PART + CS_PARTR + CS_PART2 +
-                            (size_t)CMAXR * CL * 4 + (size_t)CMAXR * 2 * CU * 2 /* staged logits and values */;
+                            (size_t)CMAXR * 2 * CU * 2 /* staged state */;
 }  // namespace
 
 struct ResClPack {
@@ -107,6 +107,10 @@ __device__ __forceinline__ void cl_mma(float (&c)[4], const uint4 &a, uint32_t b
 __device__ __forceinline__ uint32_t cl_map(uint32_t addr, int rank) { uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r; }
 __device__ __forceinline__ void cl_bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void cl_bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void cl_st_async16(unsigned addr, uint4 v, unsigned mbar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(mbar) : "memory");
+}
 // asynchronous 8-byte store into a CTA of the cluster, counted on that CTA's mbarrier
 __device__ __forceinline__ void cl_st_async8(unsigned addr, uint2 v, unsigned mbar)
 {
@@ -143,6 +147,7 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
     const int c = (run + p0 <= thr) + (run + p1 <= thr) + (run + p2 <= thr) + (run + p3 <= thr) + (run + p4 <= thr) + (run + p5 <= thr) + (run + p6 <= thr) + (run + p7 <= thr);
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
 }
+__device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
 // part k of x in a split into bf16 parts (k = 0: the nearest bf16, then the nearest bf16 of the remainder, ...)
 template <int P>
 __device__ __forceinline__ void cl_split(float x, unsigned short (&b)[P])
@@ -157,8 +162,8 @@ __device__ __forceinline__ void cl_split(float x, unsigned short (&b)[P])
 
 // P: bf16 parts per fp32 value (3: one row per cluster, exact; 2: several rows).  NG: groups of four rows.
 // MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
-// Warps 0..7: hidden layer, logits, sends (0..3 also the rows of R outside tensor memory).  Warps 8..15: the rows of R in
-// tensor memory, then one row of the batch each: draw and gates.
+// Warps 0..7: hidden layer, logits, their sends (4..7 also the rows of R outside tensor memory).  Warps 8..15: the rows of R in
+// tensor memory, then one row of the batch each: draw and gates.  All: sends of the state.
 template <int P, int NG, int MODE>
 __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
 {
@@ -166,6 +171,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
     __shared__ uint32_t s_tmem;
+    __shared__ float s_u[2][CMAXR];                                      // [coarse half?][row]: uniform, conditioning frame
+    __shared__ int s_fr[2][CMAXR];
     __shared__ long long s_prof[MODE != 0 ? 16 : 1];
     constexpr int H = 2 * CK;
     constexpr bool DBG = MODE != 0;
@@ -187,11 +194,18 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     uint8_t *ximg = smem + CB_SMEM;                                      // [2: coarse, fine] state image
     uint8_t *qimg = ximg + 2 * CS_IMG;
     float *lbuf = reinterpret_cast<float *>(qimg + CS_IMG);              // [rows][256]
-    float *part = lbuf + CMAXR * 256;
+    float *part = lbuf + CMAXR * 256;                                    // K-split sums of the hidden rows, then of the logits rows
     float *partR = part + CS_PART / 4;                                   // [2 halves of K][rows][128]: R h, rows in tensor memory
     float *part2 = partR + CS_PARTR / 4;                                 // [4 quarters of K][rows][40]: the other rows
-    float *lstage = part2 + CS_PART2 / 4;                                // [row][16] this CTA's logits
-    unsigned short *ystage = reinterpret_cast<unsigned short *>(lstage + CMAXR * CL);            // [row][part][28]: this CTA's state or hidden-layer values
+    uint8_t *ystage = reinterpret_cast<uint8_t *>(part2 + CS_PART2 / 4); // [row][quad][16 or 24 bytes]: new state values of this CTA's units
+
+    // Operand image of a vector: the four values of a quad are adjacent, part by part -- P = 2: [group][quad][4 rows][high x 4,
+    // low x 4]; P = 3: [quad][3 parts x 4, pad] -- so that a producer's four values of a row travel in one 16-byte (or three
+    // 8-byte) stores and the B fragment of lane (column g, t) of a k-tile (its quad t) is one 8-byte load.  The k order of a tile
+    // is permuted accordingly in all weights: slot c holds k = 4 ((c & 7) / 2) + 2 (c / 8) + (c & 1).
+    constexpr uint32_t QSTR = P == 2 ? 64 : 32, GSTR = CQ * 64;
+    auto img_off = [](int st, int quad) { return (uint32_t)(P == 2 ? (st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16 : quad * 32); };
+    const uint32_t frag = t4 * QSTR + (P == 2 ? g4 : (g4 & 3)) * 8;      // of k-tile 0, group 0 (P = 3: columns 4..7 repeat 0..3 and are not read)
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     {
@@ -230,9 +244,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 const int st = i / H, j = i - st * H, half_f = j >= CK, k = j - half_f * CK;
                 unsigned short b[P];
                 cl_split<P>(p.h_in[(size_t)(row0 + st) * H + j], b);
-                unsigned short *im = reinterpret_cast<unsigned short *>(ximg + half_f * CS_IMG + (size_t)((k >> 3) * NG + (st >> 2)) * 128);
+                unsigned short *im = reinterpret_cast<unsigned short *>(ximg + half_f * CS_IMG + img_off(st, k >> 2));
 #pragma unroll
-                for (int q = 0; q < P; ++q) im[((P == 2 ? 2 * (st & 3) : 0) + q) * 8 + (k & 7)] = b[q];
+                for (int q = 0; q < P; ++q) im[4 * q + (k & 3)] = b[q];
             }
     }
     tc_fence_before();
@@ -242,7 +256,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const uint32_t tmem = s_tmem;
 
     Waiter wt{p.status, p.limit_ns};
-    bool bad = false;                                                    // warp-uniform: this warp gave up
+    bool bad = false;                                                    // this thread gave up: it skips waits and sends from here on
     const bool prof_on = DBG && p.prof != nullptr && blockIdx.x == 0 && (warp == 0 || warp == 8);
     long long prof_t = clock64();
 #define STAMP(i) do { if (DBG && prof_on) { const long long now_ = clock64(); if (lane == 0) s_prof[i] += now_ - prof_t; prof_t = now_; } } while (0)
@@ -251,10 +265,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         if (bad) return;
         const unsigned a = smem_u32(b);
         unsigned long long t0 = 0; unsigned cnt = 0;
-        bool fail = false;
         while (!mbar_try(a, parity & 1u))
-            if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { fail = true; break; }
-        bad = __any_sync(FULL, fail);
+            if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { bad = true; break; }
     };
 
     // ---- rows of R times one half of the state, accumulated over both halves.
@@ -274,20 +286,23 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         tmem_ld16(tmem + ((uint32_t)(32 * rq) << 16) + (uint32_t)(((half_f * 2 + rj) * 7 + pair) * 16), r);
     };
     auto r_products = [&](int half_f, uint32_t (&r0)[16]) {               // r0: the fragments of pair 0, requested earlier
-        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + (uint32_t)((28 * (rq >> 1) + (lane >> 3)) * NG * 128 + (lane & 7) * 16);
-        uint32_t r1[16], c0[NG][4], c1[NG][4];
-        auto bload = [&](int pair, uint32_t (&b)[NG][4]) {
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 14 * (rq >> 1) * 4 * QSTR + frag;
+        uint32_t r1[16];
+        uint2 c0[NG][2], c1[NG][2];
+        auto bload = [&](int pair, uint2 (&b)[NG][2]) {
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp) cl_ldmatrix4(b0 + (uint32_t)((4 * pair * NG + grp) * 128), b[grp]);
+            for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                for (int k = 0; k < 2; ++k) b[grp][k] = cl_lds8(b0 + (2 * pair + k) * 4 * QSTR + grp * GSTR);
         };
-        auto mmas = [&](const uint32_t (&r)[16], const uint32_t (&b)[NG][4]) {
+        auto mmas = [&](const uint32_t (&r)[16], const uint2 (&b)[NG][2]) {
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
                 for (int grp = 0; grp < NG; ++grp)
 #pragma unroll
                     for (int n = 0; n < 2; ++n)
-                        cl_mma(accR[n][grp], make_uint4(r[8 * n + 4 * k], r[8 * n + 4 * k + 1], r[8 * n + 4 * k + 2], r[8 * n + 4 * k + 3]), b[grp][2 * k], b[grp][2 * k + 1]);
+                        cl_mma(accR[n][grp], make_uint4(r[8 * n + 4 * k], r[8 * n + 4 * k + 1], r[8 * n + 4 * k + 2], r[8 * n + 4 * k + 3]), b[grp][k].x, b[grp][k].y);
         };
         bload(0, c0);
 #pragma unroll
@@ -297,17 +312,21 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             else { if (pair < 6) { r_load(half_f, pair + 1, r1); bload(pair + 1, c1); } mmas(r0, c0); }
         }
     };
+    // K-split sums of a fragment: the parts of a value are adjacent columns (three parts: also those of the neighbouring lane)
+    auto part_sum = [&](const float (&c)[4], float &lo, float &hi) {
+        lo = c[0] + c[1]; hi = c[2] + c[3];
+        if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }
+    };
     auto r_store = [&]() {
 #pragma unroll
         for (int n = 0; n < 2; ++n)
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp) {
                 float *d = partR + ((rq >> 1) * 4 * NG + 4 * grp + t4) * CPR + (4 * (rq & 1) + 2 * rj + n) * 16 + g4;
-                d[0] = accR[n][grp][0] + accR[n][grp][1];
-                d[8] = accR[n][grp][2] + accR[n][grp][3];
+                part_sum(accR[n][grp], d[0], d[8]);
             }
     };
-    // The 40 rows in shared memory (warps 0..3, a quarter of K each; the third tile has eight rows)
+    // The 40 rows in shared memory (warps 4..7, a quarter of K each; the third tile has eight rows)
     float acc2[3][NG][4];
     auto r2_clear = [&]() {
 #pragma unroll
@@ -319,19 +338,25 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     };
     auto r2_products = [&](int half_f) {
         const uint32_t a0 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + (lane >> 4)) * CT2 + ((lane >> 3) & 1) * 8 + (lane & 7)) * 16);
-        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + (uint32_t)((14 * rq + ((lane >> 3) & 1)) * NG * 128 + (lane >> 4) * (NG - 1) * 128 + (lane & 7) * 16);
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
+        uint32_t a[2][3][4];
+        uint2 b[2][NG];
+        auto load = [&](int kt) {
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp) b[kt & 1][grp] = cl_lds8(b0 + kt * 4 * QSTR + grp * GSTR);
+            // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
+#pragma unroll
+            for (int n = 0; n < 3; ++n) cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * n) * 16) - (n == 2 ? ((lane >> 3) & 1) * 128u : 0u), a[kt & 1][n]);
+        };
+        load(0);
 #pragma unroll
         for (int kt = 0; kt < 7; ++kt) {
-            uint32_t b[4];                                               // (k / 8 even, odd) of column group 0, then of group 1
-            cl_ldmatrix4(b0 + (uint32_t)(2 * kt * NG * 128), b);
+            if (kt < 6) load(kt + 1);
 #pragma unroll
-            for (int n = 0; n < 3; ++n) {
-                uint32_t a[4];
-                // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
-                cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * n) * 16) - (n == 2 ? ((lane >> 3) & 1) * 128u : 0u), a);
+            for (int n = 0; n < 3; ++n)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) cl_mma(acc2[n][grp], make_uint4(a[0], a[1], a[2], a[3]), b[2 * grp], b[2 * grp + 1]);
-            }
+                for (int grp = 0; grp < NG; ++grp)
+                    cl_mma(acc2[n][grp], make_uint4(a[kt & 1][n][0], a[kt & 1][n][1], a[kt & 1][n][2], a[kt & 1][n][3]), b[kt & 1][grp].x, b[kt & 1][grp].y);
         }
     };
     auto r2_store = [&]() {
@@ -340,67 +365,59 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             float *d = part2 + (rq * 4 * NG + 4 * grp + t4) * CP2 + g4;
 #pragma unroll
             for (int n = 0; n < 3; ++n) {
-                d[16 * n] = acc2[n][grp][0] + acc2[n][grp][1];
-                if (n < 2) d[16 * n + 8] = acc2[n][grp][2] + acc2[n][grp][3];
+                float lo, hi;
+                part_sum(acc2[n][grp], lo, hi);
+                d[16 * n] = lo;
+                if (n < 2) d[16 * n + 8] = hi;
             }
         }
     };
 
     // ---- fixed addresses
-    uint32_t delta[2];                                                   // CTA (warp & 7) + 8 k of the cluster: what to add to an address of mine
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t dy = map_to_rank(sbase, (unsigned)warp) - sbase;      // CTA `warp` of the cluster: what to add to an address of mine
+    uint32_t delta4[4];                                                  // CTA (warp & 3) + 4 k
 #pragma unroll
-    for (int k = 0; k < 2; ++k) delta[k] = map_to_rank(smem_u32(smem), (unsigned)((warp & 7) + 8 * k)) - smem_u32(smem);
-    // The 28 values of this CTA travel in pieces of four: piece i = (row, part, quad) is elements 28 rank + 4 quad .. + 3 of one
-    // part of one row; poff: its byte offset in an image (a lane takes pieces lane, lane + 32, ...)
-    constexpr int NPASS = P == 3 ? 1 : 2 * NG;
-    const int n_pieces = nrc * P * 7;
-    uint32_t poff[NPASS];
-#pragma unroll
-    for (int it = 0; it < NPASS; ++it) {
-        const int i = lane + 32 * it, rp = i / 7, k = CU * rank + 4 * (i - 7 * rp), st = rp / P, q = rp - st * P;
-        poff[it] = (uint32_t)(((k >> 3) * NG + ((st >> 2) & (NG - 1))) * 128 + ((P == 2 ? 2 * (st & 3) : 0) + q) * 16 + (k & 4) * 2);
-    }
+    for (int k = 0; k < 4; ++k) delta4[k] = map_to_rank(sbase, (unsigned)((warp & 3) + 4 * k)) - sbase;
+    // A lane's piece of this CTA's 28 values: P = 2: four values of a row (both parts), lane = (row of a group of four, quad);
+    // P = 3: one part of four values of the row, lane = (part, quad)
+    const int pc_a = lane / 7, pc_quad = lane - 7 * pc_a;
+    const bool pc_on = P == 2 ? lane < 28 : lane < 21;
+    const uint32_t pc_off = P == 2 ? img_off(pc_a & 3, 7 * rank + pc_quad) : img_off(0, 7 * rank + pc_quad) + pc_a * 8;
     const int skip_at = (DBG && rank == p.skip_rank) ? (int)p.skip_step : -1;
 
     // ---- the row this warp draws (warps 8..15), its last symbols, and the gates of its unit (lane) in both halves
     const bool drawer = warp >= 8 && warp - 8 < nrc;
     const int st_d = warp - 8, gb = row0 + (drawer ? st_d : 0);          // row of the call
     const bool gater = drawer && lane < CU;
-    const int gj = CU * rank + (lane < CU ? lane : 0);
+    const int gu = lane < CU ? lane : 0, gj = CU * rank + gu;
     int c_prev = 128, f_prev = 0;
     float hC = 0.f, hF = 0.f;
     if (drawer) { c_prev = p.c_in ? p.c_in[gb] : 128; f_prev = p.f_in ? p.f_in[gb] : 0; }
     if (gater && p.h_in) { hC = p.h_in[(size_t)gb * H + gj]; hF = p.h_in[(size_t)gb * H + CK + gj]; }
     const bool writer = drawer && rank == 2 * st_d;                      // the CTA whose drawing warp writes this row's samples
+    const float *g_row = p.g + (size_t)gb * p.n_frames * 3 * H + gj;
 
     struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
-    // a row of R h of this row of the batch: both halves (or all quarters) of K; three parts: both columns of their sums
+    // a row of R h of this row of the batch: both halves (or all quarters) of K
     auto r_row = [&](int i) {
-        float v = 0.f;
-        constexpr int NSL = P == 3 ? 2 : 1;
-        if (i < 128) {
-#pragma unroll
-            for (int k = 0; k < 2; ++k)
-#pragma unroll
-                for (int sl = 0; sl < NSL; ++sl) v += partR[(k * 4 * NG + st_d + sl) * CPR + i];
-        } else {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int sl = 0; sl < NSL; ++sl) v += part2[(k * 4 * NG + st_d + sl) * CP2 + i - 128];
+        float v;
+        if (i < 128) v = partR[st_d * CPR + i] + partR[(4 * NG + st_d) * CPR + i];
+        else {
+            const float *q = part2 + st_d * CP2 + i - 128;
+            v = (q[0] + q[4 * NG * CP2]) + (q[8 * NG * CP2] + q[12 * NG * CP2]);
         }
         return v;
     };
     // everything of the gates of one half that does not depend on the pending draw
     auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
         GatePre q;
-        const int u = lane < CU ? lane : 0;
         const float x0 = scale8(c_prev), x1 = scale8(f_prev);
-        const float *Iu = sI + ((half_g * 3 + 0) * CU + u) * 3, *Ir = Iu + CU * 3, *Ie = Ir + CU * 3;
-        q.pu = r_row(half_g * 3 * CU + u) + fmaf(Iu[0], x0, half_g ? fmaf(Iu[1], x1, gv[0]) : gv[0]);
-        q.pr = r_row(half_g * 3 * CU + CU + u) + fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
+        const float *Iu = sI + ((half_g * 3 + 0) * CU + gu) * 3, *Ir = Iu + CU * 3, *Ie = Ir + CU * 3;
+        q.pu = r_row(half_g * 3 * CU + gu) + fmaf(Iu[0], x0, half_g ? fmaf(Iu[1], x1, gv[0]) : gv[0]);
+        q.pr = r_row(half_g * 3 * CU + CU + gu) + fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
         q.pe = fmaf(Ie[0], x0, half_g ? fmaf(Ie[1], x1, gv[2]) : gv[2]);
-        q.ae = r_row(half_g * 3 * CU + 2 * CU + u);
+        q.ae = r_row(half_g * 3 * CU + 2 * CU + gu);
         q.ku = half_g ? Iu[2] : Iu[1]; q.kr = half_g ? Ir[2] : Ir[1]; q.ke = half_g ? Ie[2] : Ie[1];
         return q;
     };
@@ -411,41 +428,52 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
         if (half_g) hF = hn; else hC = hn;
         if (gater) {
-            unsigned short b[P];
+            unsigned short b[P], *d = reinterpret_cast<unsigned short *>(ystage + (st_d * 7 + (lane >> 2)) * (8 * P)) + (lane & 3);
             cl_split<P>(hn, b);
 #pragma unroll
-            for (int k = 0; k < P; ++k) ystage[(st_d * P + k) * CU + lane] = b[k];
+            for (int k = 0; k < P; ++k) d[4 * k] = b[k];
             if (DBG) {
                 const int jj = half_g * CK + gj;
-                if (p.dbg_gates) { float *d = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; d[jj] = u; d[H + jj] = r; d[2 * H + jj] = e; }
+                if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[jj] = u; o[H + jj] = r; o[2 * H + jj] = e; }
                 if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + jj] = hn;
             }
         }
     };
-    auto load_g = [&](int half_g, long long s, float (&gv)[3]) {
-        const long long fr = p.row_lag > 0 ? s : ((p.step0 + s) * p.row_stride + (long long)(p.stream0 + (unsigned)gb) * p.row_offset_mul) / p.hop;
-        const float *g = p.g + ((size_t)gb * p.n_frames + fr) * 3 * H + half_g * CK + gj;
+    // warp w: the staged state values of this CTA's units -> image in CTA w of the cluster
+    auto send_y = [&](int half_g, long long s) {
+        if (bad || !pc_on || (DBG && (int)s == skip_at)) return;
+        const uint32_t a = sbase + (uint32_t)(CB_SMEM + half_g * CS_IMG) + pc_off + dy, bar = smem_u32(&xy[half_g]) + dy;
+        if (P == 3) cl_st_async8(a, *reinterpret_cast<const uint2 *>(ystage + pc_quad * 24 + pc_a * 8), bar);
+        else
 #pragma unroll
-        for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
+            for (int grp = 0; grp < NG; ++grp)
+                if (4 * grp + pc_a < nrc) cl_st_async16(a + grp * GSTR, *reinterpret_cast<const uint4 *>(ystage + ((4 * grp + pc_a) * 7 + pc_quad) * 16), bar);
     };
-    // warps 0..7: the staged pieces of this CTA's 28 values of every row -> images in the cluster's CTAs, two CTAs per warp
-    auto send_staged = [&](uint32_t img, uint32_t bar) {
-        if (bad) return;
-#pragma unroll
-        for (int it = 0; it < NPASS; ++it) {
-            const int i = lane + 32 * it;
-            if (i < n_pieces) {
-                const uint2 v = *reinterpret_cast<const uint2 *>(ystage + 4 * i);
-#pragma unroll
-                for (int k = 0; k < 2; ++k) cl_st_async8(img + poff[it] + delta[k], v, bar + delta[k]);
+    const unsigned ybytes = (unsigned)(nrc * CK * P * 2), lbytes = (unsigned)(nrc * 1024);
+
+    // ---- warp 7 prepares, one row per lane, what the draws of a half-step need: the uniform and the conditioning frame (the
+    // same for both halves of a step), tracked without a division per step
+    long long w_pos = 0;
+    int w_frame = 0, w_rem = 0;
+    const int w_q = p.row_stride / p.hop, w_r = p.row_stride - w_q * p.hop;
+    auto prepare_rows = [&](int half, long long s) {                     // of half-step 2 s + half
+        if (lane < nrc) {
+            const long long t = half ? s : s - 1;
+            s_u[half][lane] = uniform24(p.seed, p.stream0 + (unsigned)(row0 + lane), (unsigned long long)(w_pos + t), half ? 0u : 1u);
+            if (!half) {                                                 // the fine half computes the coarse gates of step s
+                w_frame += w_q; w_rem += w_r;
+                if (w_rem >= p.hop) { w_rem -= p.hop; ++w_frame; }
+                if (p.row_lag > 0) w_frame = (int)s;
             }
+            s_fr[half][lane] = w_frame;
         }
     };
-    auto send_y = [&](int half_g, long long s) {
-        if (!DBG || (int)s != skip_at) send_staged(smem_u32(ximg + half_g * CS_IMG), smem_u32(&xy[half_g]));
-    };
-    const int n_draw = 32 * nrc;                                         // threads of the drawing warps
-    const unsigned ybytes = (unsigned)(nrc * CK * P * 2), lbytes = (unsigned)(nrc * 1024);
+    if (warp == 7 && lane < nrc) {
+        const long long b = row0 + lane, pos = p.row_lag > 0 ? 0 : p.step0 * p.row_stride + ((long long)p.stream0 + b) * p.row_offset_mul;
+        w_pos = p.step0 - b * p.row_lag;
+        w_frame = (int)(pos / p.hop); w_rem = (int)(pos - (long long)w_frame * p.hop);
+        prepare_rows(1, 0);
+    }
 
     // ---- prologue: R h of the initial state, coarse gates of step 0
     if (warp >= 8) {
@@ -454,40 +482,27 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll 1
         for (int half_f = 0; half_f < 2; ++half_f) { r_load(half_f, 0, r0); r_products(half_f, r0); }
         r_store();
-    } else if (warp < 4) {
+    } else if (warp >= 4) {
         r2_clear();
 #pragma unroll 1
         for (int half_f = 0; half_f < 2; ++half_f) r2_products(half_f);
         r2_store();
-        cl_bar_arrive(5, 128 + n_draw);
     }
     if (warp == 8 && lane == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
     __syncthreads();
     if (drawer) {
         float gv[3];
-        load_g(0, 0, gv);
+        const float *g = g_row + (size_t)s_fr[1][st_d] * 3 * H;
+#pragma unroll
+        for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
         gates_and_stage(0, 0, f_prev, gates_prepare(0, gv));
     }
     __syncthreads();
-    if (warp < 8) send_y(0, 0);
-
-    // what a half-step's draw and gates take from outside: gate offsets of the half of the state whose gates it computes, the
-    // uniform and (teacher forcing) the symbol
-    float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
-    int forced = -1;
-    auto fetch = [&](int half, long long s) {
-        const long long t = half ? s : s - 1;
-        if (s < p.n_steps) load_g(half, s, gv);
-        u01 = uniform24(p.seed, p.stream0 + (unsigned)gb, (unsigned long long)(p.step0 + t - (long long)gb * p.row_lag), half ? 0u : 1u);
-        if (DBG) {
-            const uint8_t *fz = half ? p.c_forced : p.f_forced;
-            if (fz) forced = fz[(size_t)gb * p.n_steps + t];
-        }
-    };
-    if (drawer) fetch(1, 0);
+    send_y(0, 0);
 
     // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
     // n = 2 s the fine half (input y_f(s - 1): fine head -> f_{s-1}, R h_{s-1} completed, then the coarse gates of step s).
+    // A peer may overwrite an image, a sum or the logits only after it has received what this CTA sends after its last use.
     const long long T = p.n_steps;
     auto half_step = [&](auto HALF_C, const long long n) {
         constexpr int half = decltype(HALF_C)::value;                    // 1: coarse half
@@ -495,126 +510,119 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const long long s = n >> 1;
         const bool last = n == 2 * T;
         const unsigned yuse = (unsigned)((n - 1) >> 1), quse = (unsigned)(n - 1);
+        const uint32_t xin = sbase + (uint32_t)(CB_SMEM + in * CS_IMG), qin = sbase + (uint32_t)(CB_SMEM + 2 * CS_IMG);
         if (warp < 8) {
-            // hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
-            uint4 av[7];
-            const int tile = warp & 1, split = warp >> 1;
+            // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
             {
+                uint4 av[7];
+                const int tile = warp & 1, split = warp >> 1;
                 const uint4 *A = wH[half] + (tile * 28 + 7 * split) * 32 + lane;
 #pragma unroll
                 for (int i = 0; i < 7; ++i) av[i] = A[i * 32];
-            }
-            STAMP0();
-            wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
-            STAMP(8 * half + 0);
-            {
-                const uint32_t b0 = smem_u32(ximg + in * CS_IMG) + (uint32_t)((14 * split) * NG * 128 + (lane & 7) * 16);
-                float acc[NG][2][4];
+                STAMP0();
+                wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
+                STAMP(8 * half + 0);
+                const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
 #pragma unroll
                 for (int grp = 0; grp < NG; ++grp) {
-                    uint32_t b[4][4];
+                    uint2 b[7];
+                    float acc[2][4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) cl_ldmatrix4(b0 + (uint32_t)(((i < 3 ? 4 * i + (lane >> 3) : 12 + ((lane >> 3) & 1)) * NG + grp) * 128), b[i]);
+                    for (int i = 0; i < 7; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
 #pragma unroll
                     for (int c = 0; c < 2; ++c)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) acc[grp][c][k] = 0.f;
+                        for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) cl_mma(acc[grp][i & 1], av[i], b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
-                }
+                    for (int i = 0; i < 7; ++i) cl_mma(acc[i & 1], av[i], b[i].x, b[i].y);
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) {
+                    for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
                     float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
-                    float lo = (acc[grp][0][0] + acc[grp][1][0]) + (acc[grp][0][1] + acc[grp][1][1]);
-                    float hi = (acc[grp][0][2] + acc[grp][1][2]) + (acc[grp][0][3] + acc[grp][1][3]);
-                    if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }      // (hi, mid) + lo parts
-                    d[0] = lo; d[8] = hi;
+                    part_sum(acc[0], d[0], d[8]);
                 }
             }
-            {
-                cl_bar_sync(1, 512);
-                STAMP(8 * half + 1);
-                const uint32_t bar = smem_u32(&xq);
-// one warp per row adds the K-split sums and splits the values into their parts; then every warp sends
-                if (warp < nrc && lane < P * 7) {
-                    const int q = lane / 7, quad = lane - 7 * q;
-                    float4 v = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * quad);
+            cl_bar_arrive(2, 512);                                       // the rows of R may take the tensor pipe
+            cl_bar_sync(1, 256);
+            STAMP(8 * half + 1);
+            // ---- K-split sums, bias, relu, bf16 parts; every sending warp adds up the same sums (cheaper than a hand-over) and
+            // serves four CTAs: warps 0..3 the first group of rows, 4..7 the second
+            if ((NG == 2 || warp < 4) && pc_on) {
+                const int grp = NG == 2 ? warp >> 2 : 0, st = P == 2 ? 4 * grp + pc_a : 0;
+                if (st < nrc && !bad) {
+                    float4 v = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
 #pragma unroll
                     for (int sp = 0; sp < 4; ++sp) {
-                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + warp) * CPH + 4 * quad);
+                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
                     v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
-                    // this lane's part of the four values: the remainder after q parts, rounded to bf16
-                    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+                    uint2 w[P];                                          // parts: what is left after the earlier ones, rounded to bf16
 #pragma unroll
-                    for (int k = 1; k < P; ++k)
-                        if (q >= k) {
-                            v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
-                            lo = __floats2bfloat162_rn(v.x, v.y); hi = __floats2bfloat162_rn(v.z, v.w);
-                        }
-                    *reinterpret_cast<uint2 *>(ystage + (warp * P + q) * CU + 4 * quad) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
-                }
-                cl_bar_sync(7, 256);
-                send_staged(smem_u32(qimg), bar);
-                STAMP(8 * half + 2);
-            }
-            // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
-            {
-                const float lbias = (half ? sb2 : sb4)[lane & 15];
-                if (warp < 7) {
-                    uint4 lv[4];
-                    const uint4 *A = wL[half] + 4 * warp * 32 + lane;
+                    for (int k = 0; k < P; ++k) {
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+                        v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
+                        w[k] = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                    }
+                    const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
-                    wait_bar(&xq, quse, (int)s, 2 + 4 * half);
-                    STAMP(8 * half + 3);
-                    const uint32_t b0 = smem_u32(qimg) + (uint32_t)(8 * warp * NG * 128 + (lane & 7) * 16);
-#pragma unroll
-                    for (int grp = 0; grp < NG; ++grp) {
-                        uint32_t b[2][4];
-#pragma unroll
-                        for (int i = 0; i < 2; ++i) cl_ldmatrix4(b0 + (uint32_t)(((4 * i + (lane >> 3)) * NG + grp) * 128), b[i]);
-                        float acc[2][4];
-#pragma unroll
-                        for (int c = 0; c < 2; ++c)
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
-                        float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
-                        float lo = (acc[0][0] + acc[1][0]) + (acc[0][1] + acc[1][1]), hi = (acc[0][2] + acc[1][2]) + (acc[0][3] + acc[1][3]);
-                        if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }
-                        d[0] = lo; d[8] = hi;
+                    for (int k = 0; k < 4; ++k) {
+                        if (P == 3) cl_st_async8(a + delta4[k], pc_a == 0 ? w[0] : pc_a == 1 ? w[1] : w[P - 1], bar + delta4[k]);
+                        else cl_st_async16(a + delta4[k], make_uint4(w[0].x, w[0].y, w[1].x, w[1].y), bar + delta4[k]);
                     }
                 }
-                cl_bar_sync(2, 256);
-                STAMP(8 * half + 4);
-if (warp < nrc && lane < CL) {
-                    float v = lbias;
-#pragma unroll
-                    for (int sp = 0; sp < 7; ++sp) v += part[(sp * 4 * NG + warp) * CPL + lane];
-                    lstage[warp * CL + lane] = v;
-                }
-                cl_bar_sync(8, 256);
-                if (lane < 4 * nrc && !bad) {
-                    const float4 v = *reinterpret_cast<const float4 *>(lstage + 4 * lane);
-                    const uint32_t a = smem_u32(lbuf + (lane >> 2) * 256 + CL * rank + 4 * (lane & 3));
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) st_async_v4(a + delta[k], v.x, v.y, v.z, v.w, smem_u32(&xl) + delta[k]);
-                }
-                STAMP(8 * half + 5);
             }
-            // ---- the rows of R outside tensor memory (needed by the fine gates half a step or more from now), while the logits cross
-            if (warp < 4) {
+            STAMP(8 * half + 2);
+            // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
+            if (warp < 7) {
+                uint4 lv[4];
+                const uint4 *A = wL[half] + 4 * warp * 32 + lane;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
+                const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + 4 * (lane & 3));
+                wait_bar(&xq, quse, (int)s, 2 + 4 * half);
+                STAMP(8 * half + 3);
+                const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) {
+                    uint2 b[4];
+                    float acc[2][4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i].x, b[i].y);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
+                    float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
+                    part_sum(acc[0], d[0], d[8]);
+                }
+                if (warp >= 4) cl_bar_arrive(3, 224);
+                else {
+                    cl_bar_sync(3, 224);
+                    STAMP(8 * half + 4);
+                    if (lane < 4 * nrc && !bad) {
+                        const int st = lane >> 2;
+                        float4 v = lbias;
+#pragma unroll
+                        for (int sp = 0; sp < 7; ++sp) {
+                            const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + 4 * (lane & 3));
+                            v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+                        }
+                        const uint32_t a = smem_u32(lbuf + st * 256 + CL * rank + 4 * (lane & 3)), bar = smem_u32(&xl);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) st_async_v4(a + delta4[k], v.x, v.y, v.z, v.w, bar + delta4[k]);
+                    }
+                    STAMP(8 * half + 5);
+                }
+            } else if (!last) prepare_rows(1 - half, half ? s + 1 : s);
+            // ---- the rows of R outside tensor memory (needed by the fine gates half a step or more from now)
+            if (warp >= 4) {
                 if (half) r2_clear();
                 r2_products(in);
-                if (!half) { r2_store(); if (!last) cl_bar_arrive(5, 128 + n_draw); }
-            }
-            if (!last) {
-                cl_bar_sync(4, 256 + n_draw);
-                STAMP0();
-                send_y(half, s);
+                if (!half) r2_store();
             }
         } else {
             // ---- this warp's rows of R (they start when the hidden-layer products are done, so as not to share the pipe with
@@ -627,19 +635,25 @@ if (warp < nrc && lane < CL) {
             const long long t = half ? s : s - 1;
             uint32_t r0[16];
             r_load(in, 0, r0);
-            cl_bar_sync(1, 512);
+            float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
+            int forced = -1;
+            if (drawer) {
+                u01 = s_u[half][st_d];
+                const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
+                if (!last)
+#pragma unroll
+                    for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
+                if (DBG) {
+                    const uint8_t *fz = half ? p.c_forced : p.f_forced;
+                    if (fz) forced = fz[(size_t)gb * T + t];
+                }
+            }
+            cl_bar_sync(2, 512);
             if (half) r_clear();
             r_products(in, r0);
-            if (!half) r_store();
-            // (in both halves: a peer overwrites this image only after it has logits that this CTA sends after the state that
-            // the drawing warps publish below)
-            cl_bar_sync(3, 256);
+            if (!half) { r_store(); cl_bar_sync(4, 256); }
             if (drawer) {
-                if (half) cl_bar_sync(5, 128 + n_draw);                   // part2
                 const GatePre gp = gates_prepare(half, gv);
-                const float u_now = u01;
-                const int forced_now = forced;
-                if (!last) fetch(1 - half, half ? s + 1 : s);             // of the next half-step, while the logits are on their way
                 wait_bar(&xl, quse, (int)s, 3 + 4 * half);
                 STAMP0();
                 float l[8];
@@ -647,13 +661,10 @@ if (warp < nrc && lane < CL) {
                     const float4 a = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane), b = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane + 4);
                     l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
                 }
-                const int drawn = cl_draw(l, u_now, lane);
-                const int fed = (DBG && forced_now >= 0) ? forced_now : drawn;
+                const int drawn = cl_draw(l, u01, lane);
+                const int fed = (DBG && forced >= 0) ? forced : drawn;
                 STAMP(8 * half + 6);
-                if (!last) {
-                    gates_and_stage(half, s, fed, gp);
-                    cl_bar_arrive(4, 256 + n_draw);
-                }
+                if (!last) gates_and_stage(half, s, fed, gp);
                 STAMP(8 * half + 7);
                 if (writer && !bad) {
                     if (DBG && p.dbg_logits) {
@@ -663,12 +674,16 @@ if (warp < nrc && lane < CL) {
                     }
                     if (lane == 0) {
                         uint8_t *o = half ? p.c_out : p.f_out;
-                        if (o) o[(size_t)gb * T + t] = (uint8_t)drawn;
+                        if (DBG && o) o[(size_t)gb * T + t] = (uint8_t)drawn;
                         if (!half && p.out) p.out[(long long)gb * p.out_pitch + t] = (int16_t)(256 * c_prev + fed - 32768);
                     }
                 }
                 if (half) c_prev = fed; else f_prev = fed;
             }
+        }
+        if (!last) {
+            __syncthreads();
+            send_y(half, s);
         }
     };
 #pragma unroll 1
@@ -755,12 +770,12 @@ int rescl_prepare(wrnn_model *m)
     std::vector<uint8_t> blob(CCS * (CB_SMEM + CB_TMEM), 0);
     // row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
     auto r_row = [&](int rank, int i) { return &dR[((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
-    // A fragments of 16 rows (row r < n_rows, zero otherwise): lane (g, t) holds (row g, k 2t..2t+1), (row g + 8, same), (row g, k 2t+8..9), (row g + 8, same)
+    // A fragments of 16 rows (row r < n_rows, zero otherwise): lane (g, t) holds rows g, g + 8 at k 4t, 4t + 1, then at 4t + 2, 4t + 3 (the permuted k order)
     auto pack = [&](const std::vector<uint16_t> &M, int first, int n_rows, uint16_t *dst) {
         for (int kt = 0; kt < 28; ++kt)
             for (int lane = 0; lane < 32; ++lane)
                 for (int q = 0; q < 4; ++q) {
-                    const int r = (lane >> 2) + 8 * (q & 1), c = 2 * (lane & 3) + 8 * (q >> 1);
+                    const int r = (lane >> 2) + 8 * (q & 1), c = 4 * (lane & 3) + 2 * (q >> 1);
                     for (int j = 0; j < 2; ++j) dst[((size_t)kt * 32 + lane) * 8 + 2 * q + j] = r < n_rows ? M[(size_t)(first + r) * CK + 16 * kt + c + j] : 0;
                 }
     };
@@ -772,7 +787,10 @@ int rescl_prepare(wrnn_model *m)
         }
         uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
         for (int i = 0; i < CT2; ++i)
-            for (int k8 = 0; k8 < 2 * CK8; ++k8) std::memcpy(r2 + ((size_t)k8 * CT2 + i) * 8, r_row(rank, 128 + i) + 8 * k8, 16);
+            for (int k8 = 0; k8 < 2 * CK8; ++k8) {
+                const uint16_t *src = r_row(rank, 128 + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
+                for (int e = 0; e < 8; ++e) r2[((size_t)k8 * CT2 + i) * 8 + e] = src[4 * (e >> 1) + (e & 1)];
+            }
         float *sm = reinterpret_cast<float *>(base + 2 * CW_HID + 2 * CW_LOG + CW_R2);
         for (int i = 0; i < 6 * CU; ++i) {
             const size_t row = (size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU;
@@ -789,7 +807,7 @@ int rescl_prepare(wrnn_model *m)
                 const int reg = c & 3, kt1 = (c >> 2) & 1, n = (c >> 3) & 1, pair = (c >> 4) % 7, j = (c / 112) & 1, half_f = c / 224;
                 const int tile = 4 * (q & 1) + 2 * j + n, kt = 28 * half_f + 14 * (q >> 1) + 2 * pair + kt1;
                 for (int lane = 0; lane < 32; ++lane) {
-                    const uint16_t *src = r_row(rank, 16 * tile + (lane >> 2) + 8 * (reg & 1)) + 16 * kt + 2 * (lane & 3) + 8 * (reg >> 1);
+                    const uint16_t *src = r_row(rank, 16 * tile + (lane >> 2) + 8 * (reg & 1)) + 16 * kt + 4 * (lane & 3) + 2 * (reg >> 1);
                     uint16_t *d = tm + ((size_t)c * 128 + 32 * q + lane) * 2;
                     d[0] = src[0]; d[1] = src[1];
                 }
