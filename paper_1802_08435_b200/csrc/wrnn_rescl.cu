@@ -134,17 +134,23 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = cl_ex2(fmaf(l[i], CL_LOG2E, -m));
     const float p0 = w[0], p1 = w[0] + w[1], p2 = p1 + w[2], p3 = p1 + (w[2] + w[3]), p4 = p3 + w[4], p5 = p3 + (w[4] + w[5]), p6 = p5 + w[6], p7 = p5 + (w[6] + w[7]);
-    // butterfly: the total of the block of 2 o lanes and, in `run`, the sum of the lanes of the block below this one
+    // butterfly over groups of 4, 16 and 32 lanes: the total of the block and, in `run`, the sum of its lanes below this one
     float tot = p7, run = 0.f;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float other = __shfl_xor_sync(FULL, tot, o);
-        if (lane & o) run += other;
-        tot += other;
+    for (int o = 1; o < 16; o <<= 2) {
+        const float x1 = __shfl_xor_sync(FULL, tot, o), x2 = __shfl_xor_sync(FULL, tot, 2 * o), x3 = __shfl_xor_sync(FULL, tot, 3 * o);
+        const bool odd = lane & o, up = lane & (2 * o);
+        run += (odd ? x1 : 0.f) + (up ? x2 + x3 : 0.f);
+        tot = (tot + x1) + (x2 + x3);
     }
-    const float thr = u * tot;
+    {
+        const float x = __shfl_xor_sync(FULL, tot, 16);
+        if (lane & 16) run += x;
+        tot += x;
+    }
+    const float thr = fmaf(u, tot, -run);
     // the running sums do not decrease: the first one above the threshold comes after those that are not
-    const int c = (run + p0 <= thr) + (run + p1 <= thr) + (run + p2 <= thr) + (run + p3 <= thr) + (run + p4 <= thr) + (run + p5 <= thr) + (run + p6 <= thr) + (run + p7 <= thr);
+    const int c = ((p0 <= thr) + (p1 <= thr)) + ((p2 <= thr) + (p3 <= thr)) + (((p4 <= thr) + (p5 <= thr)) + ((p6 <= thr) + (p7 <= thr)));
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
 }
 __device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
@@ -396,6 +402,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     if (drawer) { c_prev = p.c_in ? p.c_in[gb] : 128; f_prev = p.f_in ? p.f_in[gb] : 0; }
     if (gater && p.h_in) { hC = p.h_in[(size_t)gb * H + gj]; hF = p.h_in[(size_t)gb * H + CK + gj]; }
     const bool writer = drawer && rank == 2 * st_d;                      // the CTA whose drawing warp writes this row's samples
+    int drawn_out = 0;
+    int16_t *out_row = p.out ? p.out + (long long)gb * p.out_pitch : nullptr;
     const float *g_row = p.g + (size_t)gb * p.n_frames * 3 * H + gj;
 
     struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
@@ -666,24 +674,26 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 STAMP(8 * half + 6);
                 if (!last) gates_and_stage(half, s, fed, gp);
                 STAMP(8 * half + 7);
-                if (writer && !bad) {
-                    if (DBG && p.dbg_logits) {
-                        float *d = p.dbg_logits + (((size_t)t * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) d[k] = l[k];
-                    }
-                    if (lane == 0) {
-                        uint8_t *o = half ? p.c_out : p.f_out;
-                        if (DBG && o) o[(size_t)gb * T + t] = (uint8_t)drawn;
-                        if (!half && p.out) p.out[(long long)gb * p.out_pitch + t] = (int16_t)(256 * c_prev + fed - 32768);
-                    }
-                }
                 if (half) c_prev = fed; else f_prev = fed;
+                drawn_out = drawn;
+                if (DBG && p.dbg_logits && writer && !bad) {
+                    float *d = p.dbg_logits + (((size_t)t * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) d[k] = l[k];
+                }
             }
         }
         if (!last) {
             __syncthreads();
             send_y(half, s);
+        }
+        // the samples leave when the state is on its way
+        if (writer && lane == 0 && !bad) {
+            if (DBG) {
+                uint8_t *o = half ? p.c_out : p.f_out;
+                if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
+            }
+            if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
         }
     };
 #pragma unroll 1
