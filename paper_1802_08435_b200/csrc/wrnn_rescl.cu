@@ -26,9 +26,10 @@
 //     warp, so the drawn symbol never leaves the warp.
 // Every wait is bounded; a warp that gives up records where, skips its remaining waits and sends and keeps meeting its
 // barriers, and all CTAs leave through the final cluster barrier.
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include <cstdlib>
@@ -70,6 +71,7 @@ struct ResClPack {
     uint8_t *d_blob = nullptr;               // [16 ranks][CB_SMEM | CB_TMEM]
     long long *d_prof = nullptr;             // [16]
     int max_clusters = 0;
+    float inv_R = 0.f, inv_O1[2] = {0.f, 0.f}, inv_O2[2] = {0.f, 0.f}, q_scale[2] = {0.f, 0.f};
 };
 
 struct ClParams {
@@ -81,6 +83,7 @@ struct ClParams {
     long long out_pitch;
     const uint8_t *blob;
     const float *g;                          // [batch][n_frames][3H]
+    float inv_R, inv_O1[2], inv_O2[2], q_scale[2];   // 2^-14 over the power of two in R, in the hidden layers and logits rows; the one of the hidden-layer values
     const float *h_in; float *h_out;
     const uint8_t *c_in, *f_in; uint8_t *c_st_out, *f_st_out;
     const uint8_t *c_forced, *f_forced;
@@ -99,7 +102,7 @@ __device__ __forceinline__ void cl_ldmatrix4(uint32_t addr, uint32_t (&r)[4])
 }
 __device__ __forceinline__ void cl_mma(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1)
 {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
@@ -154,29 +157,26 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
 }
 __device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
-// part k of x in a split into bf16 parts (k = 0: the nearest bf16, then the nearest bf16 of the remainder, ...)
-template <int P>
-__device__ __forceinline__ void cl_split(float x, unsigned short (&b)[P])
+// x (scaled by a power of two into the range of fp16) as high and low fp16 parts: x - high - low is at most 2^-24 |x|, half a
+// unit in the last place of fp32
+__device__ __forceinline__ uint2 cl_split4(float a, float b, float c, float d, uint2 &low)
 {
-#pragma unroll
-    for (int k = 0; k < P; ++k) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(x);
-        b[k] = __bfloat16_as_ushort(h);
-        x -= __bfloat162float(h);
-    }
+    const __half2 h0 = __floats2half2_rn(a, b), h1 = __floats2half2_rn(c, d);
+    const __half2 l0 = __floats2half2_rn(a - __low2float(h0), b - __high2float(h0)), l1 = __floats2half2_rn(c - __low2float(h1), d - __high2float(h1));
+    low = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+    return make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
 }
 
-// P: bf16 parts per fp32 value (3: one row per cluster, exact; 2: several rows).  NG: groups of four rows.
-// MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
-// Warps 0..7: hidden layer, logits, their sends (4..7 also the rows of R outside tensor memory).  Warps 8..15: the rows of R in
-// tensor memory, then one row of the batch each: draw and gates.  All: sends of the state.
-template <int P, int NG, int MODE>
+// NG: groups of four rows.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
+// Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
+// multiply the rows of R in the background, while the chain waits for exchanges.
+template <int NG, int MODE>
 __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
 {
-    static_assert(P == 2 || (P == 3 && NG == 1), "three parts fill one column group with one row");
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
     __shared__ uint32_t s_tmem;
+    __shared__ int s_hexp;
     __shared__ float s_u[2][CMAXR];                                      // [coarse half?][row]: uniform, conditioning frame
     __shared__ int s_fr[2][CMAXR];
     __shared__ long long s_prof[MODE != 0 ? 16 : 1];
@@ -205,13 +205,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     float *part2 = partR + CS_PARTR / 4;                                 // [4 quarters of K][rows][40]: the other rows
     uint8_t *ystage = reinterpret_cast<uint8_t *>(part2 + CS_PART2 / 4); // [row][quad][16 or 24 bytes]: new state values of this CTA's units
 
-    // Operand image of a vector: the four values of a quad are adjacent, part by part -- P = 2: [group][quad][4 rows][high x 4,
-    // low x 4]; P = 3: [quad][3 parts x 4, pad] -- so that a producer's four values of a row travel in one 16-byte (or three
-    // 8-byte) stores and the B fragment of lane (column g, t) of a k-tile (its quad t) is one 8-byte load.  The k order of a tile
+    // Operand image of a vector: [group][quad][4 rows][high x 4, low x 4] -- a producer's four values of a row travel in one 16-byte
+    // store, and the B fragment of lane (column g = row, part; t = quad of the k-tile) is one 8-byte load.  The k order of a tile
     // is permuted accordingly in all weights: slot c holds k = 4 ((c & 7) / 2) + 2 (c / 8) + (c & 1).
-    constexpr uint32_t QSTR = P == 2 ? 64 : 32, GSTR = CQ * 64;
-    auto img_off = [](int st, int quad) { return (uint32_t)(P == 2 ? (st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16 : quad * 32); };
-    const uint32_t frag = t4 * QSTR + (P == 2 ? g4 : (g4 & 3)) * 8;      // of k-tile 0, group 0 (P = 3: columns 4..7 repeat 0..3 and are not read)
+    constexpr uint32_t QSTR = 64, GSTR = CQ * 64;
+    auto img_off = [](int st, int quad) { return (uint32_t)((st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16); };
+    const uint32_t frag = t4 * QSTR + g4 * 8;                            // of k-tile 0, group 0
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     {
@@ -226,6 +225,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
         if (tid == 0) {
+            s_hexp = 0;
             mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
             mbar_fence_init();
         }
@@ -244,15 +244,22 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                          "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        // the power of two that takes the state (below one but for what the caller passes in) to at most 2^14
+        if (p.h_in) {
+            float m = 1.f;
+            for (int i = tid; i < nrc * H; i += 512) m = fmaxf(m, fabsf(p.h_in[(size_t)row0 * H + i]));
+            if (!(m <= 1.f)) atomicMax(&s_hexp, min(127, ilogbf(m) + 1));
+        }
+        __syncthreads();
+        const float scale = ldexpf(1.f, 14 - s_hexp);
         // images of the initial state
         if (p.h_in)
             for (int i = tid; i < nrc * H; i += 512) {
                 const int st = i / H, j = i - st * H, half_f = j >= CK, k = j - half_f * CK;
-                unsigned short b[P];
-                cl_split<P>(p.h_in[(size_t)(row0 + st) * H + j], b);
-                unsigned short *im = reinterpret_cast<unsigned short *>(ximg + half_f * CS_IMG + img_off(st, k >> 2));
-#pragma unroll
-                for (int q = 0; q < P; ++q) im[4 * q + (k & 3)] = b[q];
+                const float x = p.h_in[(size_t)(row0 + st) * H + j] * scale;
+                __half *im = reinterpret_cast<__half *>(ximg + half_f * CS_IMG + img_off(st, k >> 2)) + (k & 3);
+                im[0] = __float2half_rn(x);
+                im[4] = __float2half_rn(x - __half2float(im[0]));
             }
     }
     tc_fence_before();
@@ -260,10 +267,11 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     tc_fence_after();
     cluster_sync_all();                                                  // every peer's barriers are initialised before anyone sends
     const uint32_t tmem = s_tmem;
+    const float h_scale = ldexpf(1.f, 14 - s_hexp), h_inv = ldexpf(1.f, s_hexp);          // of the state; its inverse without the 2^-14 in inv_*
 
     Waiter wt{p.status, p.limit_ns};
     bool bad = false;                                                    // this thread gave up: it skips waits and sends from here on
-    const bool prof_on = DBG && p.prof != nullptr && blockIdx.x == 0 && (warp == 0 || warp == 8);
+    const bool prof_on = DBG && p.prof != nullptr && blockIdx.x == 0 && warp == 0;
     long long prof_t = clock64();
 #define STAMP(i) do { if (DBG && prof_on) { const long long now_ = clock64(); if (lane == 0) s_prof[i] += now_ - prof_t; prof_t = now_; } } while (0)
 #define STAMP0() do { if (DBG && prof_on) prof_t = clock64(); } while (0)
@@ -318,10 +326,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             else { if (pair < 6) { r_load(half_f, pair + 1, r1); bload(pair + 1, c1); } mmas(r0, c0); }
         }
     };
-    // K-split sums of a fragment: the parts of a value are adjacent columns (three parts: also those of the neighbouring lane)
+    // the parts of a value are adjacent columns
     auto part_sum = [&](const float (&c)[4], float &lo, float &hi) {
         lo = c[0] + c[1]; hi = c[2] + c[3];
-        if (P == 3) { lo += __shfl_xor_sync(FULL, lo, 1); hi += __shfl_xor_sync(FULL, hi, 1); }
     };
     auto r_store = [&]() {
 #pragma unroll
@@ -332,11 +339,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 part_sum(accR[n][grp], d[0], d[8]);
             }
     };
-    // The 40 rows in shared memory (warps 4..7, a quarter of K each; the third tile has eight rows)
-    float acc2[3][NG][4];
+    // The 40 rows in shared memory, a quarter of K per lane quadrant: the first two tiles on warps 12..15, the third (eight rows)
+    // on warps 8..11
+    float acc2[2][NG][4];
     auto r2_clear = [&]() {
 #pragma unroll
-        for (int n = 0; n < 3; ++n)
+        for (int n = 0; n < 2; ++n)
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp)
 #pragma unroll
@@ -345,56 +353,62 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     auto r2_products = [&](int half_f) {
         const uint32_t a0 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + (lane >> 4)) * CT2 + ((lane >> 3) & 1) * 8 + (lane & 7)) * 16);
         const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
-        uint32_t a[2][3][4];
-        uint2 b[2][NG];
-        auto load = [&](int kt) {
+        auto run = [&](auto NT_C) {
+            constexpr int NT = decltype(NT_C)::value, n0 = NT == 1 ? 2 : 0;
+            uint32_t a[2][NT][4];
+            uint2 b[2][NG];
+            auto load = [&](int kt) {
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp) b[kt & 1][grp] = cl_lds8(b0 + kt * 4 * QSTR + grp * GSTR);
-            // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
+                for (int grp = 0; grp < NG; ++grp) b[kt & 1][grp] = cl_lds8(b0 + kt * 4 * QSTR + grp * GSTR);
+                // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
 #pragma unroll
-            for (int n = 0; n < 3; ++n) cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * n) * 16) - (n == 2 ? ((lane >> 3) & 1) * 128u : 0u), a[kt & 1][n]);
+                for (int n = 0; n < NT; ++n) cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * (n0 + n)) * 16) - (NT == 1 ? ((lane >> 3) & 1) * 128u : 0u), a[kt & 1][n]);
+            };
+            load(0);
+#pragma unroll
+            for (int kt = 0; kt < 7; ++kt) {
+                if (kt < 6) load(kt + 1);
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int grp = 0; grp < NG; ++grp)
+                        cl_mma(acc2[n][grp], make_uint4(a[kt & 1][n][0], a[kt & 1][n][1], a[kt & 1][n][2], a[kt & 1][n][3]), b[kt & 1][grp].x, b[kt & 1][grp].y);
+            }
         };
-        load(0);
-#pragma unroll
-        for (int kt = 0; kt < 7; ++kt) {
-            if (kt < 6) load(kt + 1);
-#pragma unroll
-            for (int n = 0; n < 3; ++n)
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp)
-                    cl_mma(acc2[n][grp], make_uint4(a[kt & 1][n][0], a[kt & 1][n][1], a[kt & 1][n][2], a[kt & 1][n][3]), b[kt & 1][grp].x, b[kt & 1][grp].y);
-        }
+        if (rj) run(std::integral_constant<int, 2>{});
+        else run(std::integral_constant<int, 1>{});
     };
     auto r2_store = [&]() {
 #pragma unroll
         for (int grp = 0; grp < NG; ++grp) {
-            float *d = part2 + (rq * 4 * NG + 4 * grp + t4) * CP2 + g4;
+            float *d = part2 + (rq * 4 * NG + 4 * grp + t4) * CP2 + g4 + (rj ? 0 : 32);
 #pragma unroll
-            for (int n = 0; n < 3; ++n) {
+            for (int n = 0; n < 2; ++n) {
                 float lo, hi;
                 part_sum(acc2[n][grp], lo, hi);
-                d[16 * n] = lo;
-                if (n < 2) d[16 * n + 8] = hi;
+                if (rj || n == 0) d[16 * n] = lo;
+                if (rj) d[16 * n + 8] = hi;
             }
         }
     };
 
     // ---- fixed addresses
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t dy = map_to_rank(sbase, (unsigned)warp) - sbase;      // CTA `warp` of the cluster: what to add to an address of mine
+    uint32_t dy[2];                                                      // CTA (warp & 7) + 8 k of the cluster: what to add to an address of mine
+#pragma unroll
+    for (int k = 0; k < 2; ++k) dy[k] = map_to_rank(sbase, (unsigned)((warp & 7) + 8 * k)) - sbase;
     uint32_t delta4[4];                                                  // CTA (warp & 3) + 4 k
 #pragma unroll
     for (int k = 0; k < 4; ++k) delta4[k] = map_to_rank(sbase, (unsigned)((warp & 3) + 4 * k)) - sbase;
-    // A lane's piece of this CTA's 28 values: P = 2: four values of a row (both parts), lane = (row of a group of four, quad);
-    // P = 3: one part of four values of the row, lane = (part, quad)
+    // A lane's piece of this CTA's 28 values: four values of a row, lane = (row of a group of four, quad)
     const int pc_a = lane / 7, pc_quad = lane - 7 * pc_a;
-    const bool pc_on = P == 2 ? lane < 28 : lane < 21;
-    const uint32_t pc_off = P == 2 ? img_off(pc_a & 3, 7 * rank + pc_quad) : img_off(0, 7 * rank + pc_quad) + pc_a * 8;
+    const bool pc_on = lane < 28;
+    const uint32_t pc_off = img_off(pc_a & 3, 7 * rank + pc_quad);
     const int skip_at = (DBG && rank == p.skip_rank) ? (int)p.skip_step : -1;
 
-    // ---- the row this warp draws (warps 8..15), its last symbols, and the gates of its unit (lane) in both halves
-    const bool drawer = warp >= 8 && warp - 8 < nrc;
-    const int st_d = warp - 8, gb = row0 + (drawer ? st_d : 0);          // row of the call
+    // ---- the row this warp draws (warps 0..7), its last symbols, and the gates of its unit (lane) in both halves
+    const bool drawer = warp < nrc;
+    const int st_d = warp & 7, gb = row0 + (drawer ? st_d : 0);          // row of the call
     const bool gater = drawer && lane < CU;
     const int gu = lane < CU ? lane : 0, gj = CU * rank + gu;
     int c_prev = 128, f_prev = 0;
@@ -406,6 +420,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     int16_t *out_row = p.out ? p.out + (long long)gb * p.out_pitch : nullptr;
     const float *g_row = p.g + (size_t)gb * p.n_frames * 3 * H + gj;
 
+    const float r_inv = p.inv_R * h_inv;
     struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
     // a row of R h of this row of the batch: both halves (or all quarters) of K
     auto r_row = [&](int i) {
@@ -415,7 +430,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             const float *q = part2 + st_d * CP2 + i - 128;
             v = (q[0] + q[4 * NG * CP2]) + (q[8 * NG * CP2] + q[12 * NG * CP2]);
         }
-        return v;
+        return v * r_inv;
     };
     // everything of the gates of one half that does not depend on the pending draw
     auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
@@ -436,10 +451,11 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
         if (half_g) hF = hn; else hC = hn;
         if (gater) {
-            unsigned short b[P], *d = reinterpret_cast<unsigned short *>(ystage + (st_d * 7 + (lane >> 2)) * (8 * P)) + (lane & 3);
-            cl_split<P>(hn, b);
-#pragma unroll
-            for (int k = 0; k < P; ++k) d[4 * k] = b[k];
+            __half *d = reinterpret_cast<__half *>(ystage + (st_d * 7 + (lane >> 2)) * 16) + (lane & 3);
+            const float x = hn * h_scale;
+            const __half hi = __float2half_rn(x);
+            d[0] = hi;
+            d[4] = __float2half_rn(x - __half2float(hi));
             if (DBG) {
                 const int jj = half_g * CK + gj;
                 if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[jj] = u; o[H + jj] = r; o[2 * H + jj] = e; }
@@ -447,17 +463,22 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             }
         }
     };
-    // warp w: the staged state values of this CTA's units -> image in CTA w of the cluster
+    // warps 0..7: the staged state values of this CTA's units -> images in the cluster's CTAs, two each
     auto send_y = [&](int half_g, long long s) {
         if (bad || !pc_on || (DBG && (int)s == skip_at)) return;
-        const uint32_t a = sbase + (uint32_t)(CB_SMEM + half_g * CS_IMG) + pc_off + dy, bar = smem_u32(&xy[half_g]) + dy;
-        if (P == 3) cl_st_async8(a, *reinterpret_cast<const uint2 *>(ystage + pc_quad * 24 + pc_a * 8), bar);
-        else
+        const uint32_t a = sbase + (uint32_t)(CB_SMEM + half_g * CS_IMG) + pc_off, bar = smem_u32(&xy[half_g]);
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-                if (4 * grp + pc_a < nrc) cl_st_async16(a + grp * GSTR, *reinterpret_cast<const uint4 *>(ystage + ((4 * grp + pc_a) * 7 + pc_quad) * 16), bar);
+        for (int grp = 0; grp < NG; ++grp)
+            if (4 * grp + pc_a < nrc) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((4 * grp + pc_a) * 7 + pc_quad) * 16);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) cl_st_async16(a + grp * GSTR + dy[k], v, bar + dy[k]);
+            }
     };
-    const unsigned ybytes = (unsigned)(nrc * CK * P * 2), lbytes = (unsigned)(nrc * 1024);
+    const float inv_h0 = p.inv_O1[0] * h_inv, inv_h1 = p.inv_O1[1] * h_inv, inv_l0 = p.inv_O2[0] * h_inv, inv_l1 = p.inv_O2[1] * h_inv;
+    const float q_s0 = p.q_scale[0] * ldexpf(1.f, -s_hexp), q_s1 = p.q_scale[1] * ldexpf(1.f, -s_hexp);
+    const int n_draw = 32 * nrc;                                         // threads of the drawing warps
+    const unsigned ybytes = (unsigned)(nrc * CK * 4), lbytes = (unsigned)(nrc * 1024);
 
     // ---- warp 7 prepares, one row per lane, what the draws of a half-step need: the uniform and the conditioning frame (the
     // same for both halves of a step), tracked without a division per step
@@ -490,13 +511,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll 1
         for (int half_f = 0; half_f < 2; ++half_f) { r_load(half_f, 0, r0); r_products(half_f, r0); }
         r_store();
-    } else if (warp >= 4) {
         r2_clear();
 #pragma unroll 1
         for (int half_f = 0; half_f < 2; ++half_f) r2_products(half_f);
         r2_store();
     }
-    if (warp == 8 && lane == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
+    if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
     __syncthreads();
     if (drawer) {
         float gv[3];
@@ -506,7 +526,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         gates_and_stage(0, 0, f_prev, gates_prepare(0, gv));
     }
     __syncthreads();
-    send_y(0, 0);
+    if (warp < 8) send_y(0, 0);
 
     // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
     // n = 2 s the fine half (input y_f(s - 1): fine head -> f_{s-1}, R h_{s-1} completed, then the coarse gates of step s).
@@ -520,6 +540,24 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const unsigned yuse = (unsigned)((n - 1) >> 1), quse = (unsigned)(n - 1);
         const uint32_t xin = sbase + (uint32_t)(CB_SMEM + in * CS_IMG), qin = sbase + (uint32_t)(CB_SMEM + 2 * CS_IMG);
         if (warp < 8) {
+            if (tid == 0 && !bad) {
+                mbar_arrive_expect(smem_u32(&xq), ybytes);
+                mbar_arrive_expect(smem_u32(&xl), lbytes);
+                if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
+            }
+            float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
+            int forced = -1;
+            if (drawer) {
+                u01 = s_u[half][st_d];
+                const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
+                if (!last)
+#pragma unroll
+                    for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
+                if (DBG) {
+                    const uint8_t *fz = half ? p.c_forced : p.f_forced;
+                    if (fz) forced = fz[(size_t)gb * T + (half ? s : s - 1)];
+                }
+            }
             // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
             {
                 uint4 av[7];
@@ -549,36 +587,31 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                     part_sum(acc[0], d[0], d[8]);
                 }
             }
-            cl_bar_arrive(2, 512);                                       // the rows of R may take the tensor pipe
             cl_bar_sync(1, 256);
             STAMP(8 * half + 1);
-            // ---- K-split sums, bias, relu, bf16 parts; every sending warp adds up the same sums (cheaper than a hand-over) and
-            // serves four CTAs: warps 0..3 the first group of rows, 4..7 the second
+            // ---- K-split sums, bias, relu, parts; every sending warp adds up the same sums (cheaper than a hand-over) and serves
+            // four CTAs: warps 0..3 the first group of rows, 4..7 the second
             if ((NG == 2 || warp < 4) && pc_on) {
-                const int grp = NG == 2 ? warp >> 2 : 0, st = P == 2 ? 4 * grp + pc_a : 0;
+                const int grp = NG == 2 ? warp >> 2 : 0, st = 4 * grp + pc_a;
                 if (st < nrc && !bad) {
-                    float4 v = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
+                    const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
+                    float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int sp = 0; sp < 4; ++sp) {
                         const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
-                    v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f);
-                    uint2 w[P];                                          // parts: what is left after the earlier ones, rounded to bf16
-#pragma unroll
-                    for (int k = 0; k < P; ++k) {
-                        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-                        v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
-                        w[k] = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
-                    }
+                    const float inv = half ? inv_h0 : inv_h1;
+                    v.x = fmaxf(fmaf(v.x, inv, bias.x), 0.f) * (half ? q_s0 : q_s1); v.y = fmaxf(fmaf(v.y, inv, bias.y), 0.f) * (half ? q_s0 : q_s1);
+                    v.z = fmaxf(fmaf(v.z, inv, bias.z), 0.f) * (half ? q_s0 : q_s1); v.w = fmaxf(fmaf(v.w, inv, bias.w), 0.f) * (half ? q_s0 : q_s1);
+                    uint2 lo;
+                    const uint2 hi = cl_split4(v.x, v.y, v.z, v.w, lo);
                     const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (P == 3) cl_st_async8(a + delta4[k], pc_a == 0 ? w[0] : pc_a == 1 ? w[1] : w[P - 1], bar + delta4[k]);
-                        else cl_st_async16(a + delta4[k], make_uint4(w[0].x, w[0].y, w[1].x, w[1].y), bar + delta4[k]);
-                    }
+                    for (int k = 0; k < 4; ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
                 }
             }
+            cl_bar_sync(2, 512);                 // the background warps are done with the last half-step (and go on, in the fine half)
             STAMP(8 * half + 2);
             // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
             if (warp < 7) {
@@ -613,54 +646,25 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                     STAMP(8 * half + 4);
                     if (lane < 4 * nrc && !bad) {
                         const int st = lane >> 2;
-                        float4 v = lbias;
+                        float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int sp = 0; sp < 7; ++sp) {
                             const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + 4 * (lane & 3));
                             v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                         }
+                        const float inv = half ? inv_l0 : inv_l1;
                         const uint32_t a = smem_u32(lbuf + st * 256 + CL * rank + 4 * (lane & 3)), bar = smem_u32(&xl);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) st_async_v4(a + delta4[k], v.x, v.y, v.z, v.w, bar + delta4[k]);
+                        for (int k = 0; k < 4; ++k)
+                            st_async_v4(a + delta4[k], fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + delta4[k]);
                     }
                     STAMP(8 * half + 5);
                 }
             } else if (!last) prepare_rows(1 - half, half ? s + 1 : s);
-            // ---- the rows of R outside tensor memory (needed by the fine gates half a step or more from now)
-            if (warp >= 4) {
-                if (half) r2_clear();
-                r2_products(in);
-                if (!half) r2_store();
-            }
-        } else {
-            // ---- this warp's rows of R (they start when the hidden-layer products are done, so as not to share the pipe with
-            // them), then one row of the batch: everything that does not depend on the chain before the wait for the logits
-            if (warp == 8 && lane == 0 && !bad) {
-                mbar_arrive_expect(smem_u32(&xq), ybytes);
-                mbar_arrive_expect(smem_u32(&xl), lbytes);
-                if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
-            }
-            const long long t = half ? s : s - 1;
-            uint32_t r0[16];
-            r_load(in, 0, r0);
-            float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
-            int forced = -1;
+            if (half) cl_bar_arrive(5, 512);     // coarse half: the background warps go on
+            // ---- one row per warp: what does not depend on the draw, the draw, the gates
             if (drawer) {
-                u01 = s_u[half][st_d];
-                const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
-                if (!last)
-#pragma unroll
-                    for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
-                if (DBG) {
-                    const uint8_t *fz = half ? p.c_forced : p.f_forced;
-                    if (fz) forced = fz[(size_t)gb * T + t];
-                }
-            }
-            cl_bar_sync(2, 512);
-            if (half) r_clear();
-            r_products(in, r0);
-            if (!half) { r_store(); cl_bar_sync(4, 256); }
-            if (drawer) {
+                if (!half) cl_bar_sync(4, 256 + n_draw);                  // R h is complete
                 const GatePre gp = gates_prepare(half, gv);
                 wait_bar(&xl, quse, (int)s, 3 + 4 * half);
                 STAMP0();
@@ -677,23 +681,34 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 if (half) c_prev = fed; else f_prev = fed;
                 drawn_out = drawn;
                 if (DBG && p.dbg_logits && writer && !bad) {
-                    float *d = p.dbg_logits + (((size_t)t * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+                    float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) d[k] = l[k];
                 }
             }
-        }
-        if (!last) {
-            __syncthreads();
-            send_y(half, s);
-        }
-        // the samples leave when the state is on its way
-        if (writer && lane == 0 && !bad) {
-            if (DBG) {
-                uint8_t *o = half ? p.c_out : p.f_out;
-                if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
+            if (!last) {
+                cl_bar_sync(1, 256);
+                send_y(half, s);
             }
-            if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
+            // the samples leave when the state is on its way
+            if (writer && lane == 0 && !bad) {
+                if (DBG) {
+                    uint8_t *o = half ? p.c_out : p.f_out;
+                    if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
+                }
+                if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
+            }
+        } else {
+            // ---- the rows of R: in the fine half right after the hidden layer is sent (its coarse rows are needed by the gates at
+            // the end), in the coarse half when the logits are
+            uint32_t r0[16];
+            r_load(in, 0, r0);
+            cl_bar_sync(2, 512);
+            if (half) { cl_bar_sync(5, 512); r_clear(); r2_clear(); }
+            r_products(in, r0);
+            if (!half) { r_store(); cl_bar_arrive(4, 256 + n_draw); }
+            r2_products(in);
+            if (!half) r2_store();
         }
     };
 #pragma unroll 1
@@ -724,9 +739,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 // ---------------------------------------------------------------------------------------------
 static const void *cl_kernel_of(int nr, bool dbg)
 {
-    if (nr == 1) return dbg ? (const void *)resident_cluster_kernel<3, 1, 1> : (const void *)resident_cluster_kernel<3, 1, 0>;
-    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<2, 1, 1> : (const void *)resident_cluster_kernel<2, 1, 0>;
-    return dbg ? (const void *)resident_cluster_kernel<2, 2, 1> : (const void *)resident_cluster_kernel<2, 2, 0>;
+    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1> : (const void *)resident_cluster_kernel<1, 0>;
+    return dbg ? (const void *)resident_cluster_kernel<2, 1> : (const void *)resident_cluster_kernel<2, 0>;
 }
 
 static void cl_fill_launch(int n_clusters, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
@@ -760,7 +774,7 @@ int rescl_prepare(wrnn_model *m)
     cudaGetDeviceProperties(&prop, m->device);
     ResClPack k;
     cudaFuncAttributes fa;
-    for (int nr : {1, 2, 5})
+    for (int nr : {1, 5})
         for (int dbg = 0; dbg < 2; ++dbg) {
             const void *f = cl_kernel_of(nr, dbg != 0);
             if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || CS_BYTES + fa.sharedSizeBytes > prop.sharedMemPerBlockOptin ||
@@ -776,7 +790,40 @@ int rescl_prepare(wrnn_model *m)
             cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
         }
     }
-    const std::vector<uint16_t> dR = dense_bf16_bits(m->hR), dO[4] = {dense_bf16_bits(m->hO1), dense_bf16_bits(m->hO3), dense_bf16_bits(m->hO2), dense_bf16_bits(m->hO4)};
+    // fp16 weights, every matrix scaled by a power of two to at most 2^14: the eight bits of a bf16 weight are kept unless it is
+    // below 2^-28 of the largest one, where at most 2^-39 of that is lost
+    auto to_half = [](const BsrHost &M, int *exp) {
+        const std::vector<uint16_t> b = dense_bf16_bits(M);
+        auto value = [](uint16_t v) { const uint32_t u = (uint32_t)v << 16; float f; std::memcpy(&f, &u, 4); return f; };
+        float top = 0.f;
+        for (uint16_t v : b) top = std::max(top, std::fabs(value(v)));
+        *exp = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+        const float scale = std::ldexp(1.f, 14 - *exp);
+        std::vector<uint16_t> h(b.size());
+        for (size_t i = 0; i < b.size(); ++i) { const __half x = __float2half_rn(value(b[i]) * scale); std::memcpy(&h[i], &x, 2); }
+        return h;
+    };
+    int e[5];
+    const std::vector<uint16_t> dR = to_half(m->hR, &e[0]), dO[4] = {to_half(m->hO1, &e[1]), to_half(m->hO3, &e[2]), to_half(m->hO2, &e[3]), to_half(m->hO4, &e[4])};
+    // products of operands scaled by 2^(14 - exponent) each
+    k.inv_R = std::ldexp(1.f, e[0] - 28);
+    for (int h = 0; h < 2; ++h) {
+        // |hidden value| <= sum |O1 row| + |b1| for a state below one (the kernel takes a larger initial state into account)
+        const BsrHost &O = h ? m->hO3 : m->hO1;
+        const std::vector<float> &bias = h ? m->hb3 : m->hb1;
+        float top = 0.f;
+        for (int br = 0; br < O.rows4; ++br)
+            for (int r = 0; r < 4; ++r) {
+                float sum = std::fabs(bias[4 * br + r]);
+                for (int b = O.row_ptr[br]; b < O.row_ptr[br + 1]; ++b)
+                    for (int c = 0; c < 4; ++c) sum += std::fabs(O.vals[(size_t)b * 16 + 4 * r + c]);
+                top = std::max(top, sum);
+            }
+        const int eq = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+        k.inv_O1[h] = std::ldexp(1.f, e[1 + h] - 28);
+        k.q_scale[h] = std::ldexp(1.f, 14 - eq);
+        k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);
+    }
     std::vector<uint8_t> blob(CCS * (CB_SMEM + CB_TMEM), 0);
     // row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
     auto r_row = [&](int rank, int i) { return &dR[((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
@@ -875,6 +922,8 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
     p.row_lag = a.row_lag; p.out_pitch = a.out_pitch ? a.out_pitch : a.n_steps;
     p.blob = k.d_blob; p.g = m->g;
+    p.inv_R = k.inv_R;
+    for (int h = 0; h < 2; ++h) { p.inv_O1[h] = k.inv_O1[h]; p.inv_O2[h] = k.inv_O2[h]; p.q_scale[h] = k.q_scale[h]; }
     p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
     p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
     p.dbg_gates = a.dbg_gates; p.dbg_h = a.dbg_h; p.dbg_logits = a.dbg_logits;
