@@ -47,23 +47,24 @@ constexpr int CU = 28;                   // state units of one half, hidden-laye
 constexpr int CL = 16;                   // logits rows per CTA
 constexpr int CCS = 16;                  // CTAs per cluster
 constexpr int CK8 = CK / 8, CQ = CK / 4; // groups of eight and of four values of a half
-constexpr int CT2 = 6 * CU - 128;        // rows of R outside the TMEM tile
+constexpr int CRT = 9, CRS = 6 * CU - 16 * CRT;             // of the 168 rows of R: tiles of 16 in tensor memory, the 24 rows left in shared memory
 constexpr int CMAXR = 8;                 // rows per cluster
 constexpr int CNC = 7;                   // clusters the grid has at least
-constexpr int CPH = 40, CPL = 24, CPR = 136, CP2 = 40;       // floats per (K-split, row) of the partial sums: conflict-free for the fragment owners
+constexpr int CPH = 40, CPL = 24, CPR = 6 * CU;              // floats per (K-split, row) of the partial sums: conflict-free for the fragment owners
 constexpr size_t CW_HID = 2 * 28 * 512;                      // O1 (O3) rows of a CTA as A fragments: two tiles
 constexpr size_t CW_LOG = 28 * 512;                          // O2 (O4) rows: one tile
-constexpr size_t CW_R2 = 2 * CK8 * CT2 * 16;                 // 40 rows of R as core matrices [k / 8][5][8][16 B]
+constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
 constexpr int C_SMALL = 2 * 3 * CU * 3 + 2 * 32 + 2 * CL;    // I of the CTA's units [half][gate][unit][3], b1, b3 (32 each), b2, b4
 constexpr size_t CB_SMEM = 2 * CW_HID + 2 * CW_LOG + CW_R2 + C_SMALL * 4;
-constexpr size_t CB_TMEM = (size_t)448 * 128 * 4;
+constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: [2 halves][7 k-tiles][9 tiles][4 registers]
+constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
 static_assert(CB_SMEM % 16 == 0, "the blob is copied in 16-byte pieces");
 constexpr int CNG = 2;                                       // column groups (of four rows) the carve-up has room for
 constexpr size_t CS_IMG = (size_t)CQ * CNG * 64;            // operand image of one vector
 constexpr size_t CS_PART = (size_t)7 * 4 * CNG * CPL * 4;    // partial sums (>= 4 * 4 * CNG * CPH * 4)
 static_assert(CS_PART >= (size_t)4 * 4 * CNG * CPH * 4, "the partial sums of both products share a buffer");
-constexpr size_t CS_PARTR = (size_t)2 * 4 * CNG * CPR * 4, CS_PART2 = (size_t)4 * 4 * CNG * CP2 * 4;     // R h: tensor-memory rows, the others
-constexpr size_t CS_BYTES = CB_SMEM + 3 * CS_IMG /* two state halves, hidden layer */ + (size_t)CMAXR * 1024 /* logits */ + CS_PART + CS_PARTR + CS_PART2 +
+constexpr size_t CS_PARTR = (size_t)4 * 4 * CNG * CPR * 4;     // R h
+constexpr size_t CS_BYTES = CB_SMEM + 3 * CS_IMG /* two state halves, hidden layer */ + (size_t)CMAXR * 1024 /* logits */ + CS_PART + CS_PARTR +
                             (size_t)CMAXR * 2 * CU * 2 /* staged state */;
 }  // namespace
 
@@ -201,9 +202,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     uint8_t *qimg = ximg + 2 * CS_IMG;
     float *lbuf = reinterpret_cast<float *>(qimg + CS_IMG);              // [rows][256]
     float *part = lbuf + CMAXR * 256;                                    // K-split sums of the hidden rows, then of the logits rows
-    float *partR = part + CS_PART / 4;                                   // [2 halves of K][rows][128]: R h, rows in tensor memory
-    float *part2 = partR + CS_PARTR / 4;                                 // [4 quarters of K][rows][40]: the other rows
-    uint8_t *ystage = reinterpret_cast<uint8_t *>(part2 + CS_PART2 / 4); // [row][quad][16 or 24 bytes]: new state values of this CTA's units
+    float *partR = part + CS_PART / 4;                                   // [4 quarters of K][rows][168]: R h
+    uint8_t *ystage = reinterpret_cast<uint8_t *>(partR + CS_PARTR / 4); // [row][quad][16 or 24 bytes]: new state values of this CTA's units
 
     // Operand image of a vector: [group][quad][4 rows][high x 4, low x 4] -- a producer's four values of a row travel in one 16-byte
     // store, and the B fragment of lane (column g = row, part; t = quad of the k-tile) is one 8-byte load.  The k order of a tile
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const uint32_t *tsrc = reinterpret_cast<const uint32_t *>(blob + CB_SMEM) + 32 * (warp & 3) + lane;
         const uint32_t tdst = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16);
 #pragma unroll 1
-        for (int c = 8 * (warp >> 2); c < 448; c += 32) {
+        for (int c = 8 * (warp >> 2); c < CTC; c += 32) {
             uint32_t r[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) r[k] = __ldg(tsrc + (size_t)(c + k) * 128);
@@ -283,112 +283,83 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { bad = true; break; }
     };
 
-    // ---- rows of R times one half of the state, accumulated over both halves.
-    // Tensor memory, lane quadrant w & 3 (warps 8..15): tiles 4 (quadrant & 1) + 2 j, + 1 with j = (w >> 2) & 1, half of K
-    // quadrant >> 1; columns [half of the state][j][k-tile pair][tile][k-tile][4].
-    float accR[2][NG][4];
+    // ---- rows of R times one half of the state, accumulated over both halves (warps 8..15).  Lane quadrant w & 3 holds a quarter
+    // of K of all tiles in its tensor memory; of the two warps of a quadrant one takes tiles 0..3 and the rows in shared memory
+    // (a tile and a half), the other tiles 4..8, so that a B fragment is loaded once for five or six tiles (these loads and
+    // ldmatrix share the load / store pipe with the chain's shuffles).  Columns: [first warp: half][k-tile][4 tiles][4], then
+    // [second warp: half][k-tile][5 tiles][4].
+    float acc[6][NG][4];
     const int rq = warp & 3, rj = (warp >> 2) & 1;
+    const uint32_t r_col = tmem + ((uint32_t)(32 * rq) << 16) + (rj ? 2 * 7 * 16 : 0);
     auto r_clear = [&]() {
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
+        for (int n = 0; n < 6; ++n)
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) accR[n][grp][k] = 0.f;
+                for (int k = 0; k < 4; ++k) acc[n][grp][k] = 0.f;
     };
-    auto r_load = [&](int half_f, int pair, uint32_t (&r)[16]) {
-        tmem_ld16(tmem + ((uint32_t)(32 * rq) << 16) + (uint32_t)(((half_f * 2 + rj) * 7 + pair) * 16), r);
+    auto r_load = [&](int half_f, int kt, uint32_t (&r)[20]) {
+        const uint32_t c = r_col + (uint32_t)((half_f * 7 + kt) * (rj ? 20 : 16));
+        tmem_ld16(c, *reinterpret_cast<uint32_t (*)[16]>(&r));
+        if (rj) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]) : "r"(c + 16));
     };
-    auto r_products = [&](int half_f, uint32_t (&r0)[16]) {               // r0: the fragments of pair 0, requested earlier
-        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 14 * (rq >> 1) * 4 * QSTR + frag;
-        uint32_t r1[16];
-        uint2 c0[NG][2], c1[NG][2];
-        auto bload = [&](int pair, uint2 (&b)[NG][2]) {
+    auto r_products = [&](int half_f) {
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
+        const uint32_t a0 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + (lane >> 4)) * CRS + ((lane >> 3) & 1) * 8 + (lane & 7)) * 16);
+        const uint32_t a1 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + ((lane >> 3) & 1)) * CRS + 16 + (lane & 7)) * 16);
+        uint32_t r0[20], r1[20], t0[6], t1[6];
+        r_load(half_f, 0, r0);
+        uint2 c0[NG], c1[NG];
+        auto load = [&](int kt, uint2 (&b)[NG], uint32_t (&t)[6]) {
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                for (int k = 0; k < 2; ++k) b[grp][k] = cl_lds8(b0 + (2 * pair + k) * 4 * QSTR + grp * GSTR);
+            for (int grp = 0; grp < NG; ++grp) b[grp] = cl_lds8(b0 + kt * 4 * QSTR + grp * GSTR);
+            if (!rj) {
+                cl_ldmatrix4(a0 + kt * 2 * CRS * 16, *reinterpret_cast<uint32_t (*)[4]>(&t));
+                asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(t[4]), "=r"(t[5]) : "r"(a1 + kt * 2 * CRS * 16) : "memory");
+            }
         };
-        auto mmas = [&](const uint32_t (&r)[16], const uint2 (&b)[NG][2]) {
+        auto mmas = [&](const uint32_t (&r)[20], const uint2 (&b)[NG], const uint32_t (&t)[6]) {
 #pragma unroll
-            for (int k = 0; k < 2; ++k)
+            for (int n = 0; n < 4; ++n)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp)
+                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[n][grp], make_uint4(r[4 * n], r[4 * n + 1], r[4 * n + 2], r[4 * n + 3]), b[grp].x, b[grp].y);
 #pragma unroll
-                    for (int n = 0; n < 2; ++n)
-                        cl_mma(accR[n][grp], make_uint4(r[8 * n + 4 * k], r[8 * n + 4 * k + 1], r[8 * n + 4 * k + 2], r[8 * n + 4 * k + 3]), b[grp][k].x, b[grp][k].y);
+            for (int grp = 0; grp < NG; ++grp) {
+                if (rj) cl_mma(acc[4][grp], make_uint4(r[16], r[17], r[18], r[19]), b[grp].x, b[grp].y);
+                else {
+                    cl_mma(acc[4][grp], make_uint4(t[0], t[1], t[2], t[3]), b[grp].x, b[grp].y);
+                    cl_mma(acc[5][grp], make_uint4(t[4], 0, t[5], 0), b[grp].x, b[grp].y);
+                }
+            }
         };
-        bload(0, c0);
+        load(0, c0, t0);
+        if (NG == 2) {                                                   // (no registers for a second set of fragments)
 #pragma unroll
-        for (int pair = 0; pair < 7; ++pair) {
+            for (int kt = 0; kt < 7; ++kt) {
+                tmem_wait_ld();
+                mmas(r0, c0, t0);
+                if (kt < 6) { r_load(half_f, kt + 1, r0); load(kt + 1, c0, t0); }
+            }
+            return;
+        }
+#pragma unroll
+        for (int kt = 0; kt < 7; ++kt) {
             tmem_wait_ld();
-            if (pair & 1) { if (pair < 6) { r_load(half_f, pair + 1, r0); bload(pair + 1, c0); } mmas(r1, c1); }
-            else { if (pair < 6) { r_load(half_f, pair + 1, r1); bload(pair + 1, c1); } mmas(r0, c0); }
+            if (kt & 1) { if (kt < 6) { r_load(half_f, kt + 1, r0); load(kt + 1, c0, t0); } mmas(r1, c1, t1); }
+            else { if (kt < 6) { r_load(half_f, kt + 1, r1); load(kt + 1, c1, t1); } mmas(r0, c0, t0); }
         }
     };
     // the parts of a value are adjacent columns
-    auto part_sum = [&](const float (&c)[4], float &lo, float &hi) {
-        lo = c[0] + c[1]; hi = c[2] + c[3];
-    };
+    auto part_sum = [&](const float (&c)[4], float &lo, float &hi) { lo = c[0] + c[1]; hi = c[2] + c[3]; };
     auto r_store = [&]() {
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp) {
-                float *d = partR + ((rq >> 1) * 4 * NG + 4 * grp + t4) * CPR + (4 * (rq & 1) + 2 * rj + n) * 16 + g4;
-                part_sum(accR[n][grp], d[0], d[8]);
-            }
-    };
-    // The 40 rows in shared memory, a quarter of K per lane quadrant: the first two tiles on warps 12..15, the third (eight rows)
-    // on warps 8..11
-    float acc2[2][NG][4];
-    auto r2_clear = [&]() {
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc2[n][grp][k] = 0.f;
-    };
-    auto r2_products = [&](int half_f) {
-        const uint32_t a0 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + (lane >> 4)) * CT2 + ((lane >> 3) & 1) * 8 + (lane & 7)) * 16);
-        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
-        auto run = [&](auto NT_C) {
-            constexpr int NT = decltype(NT_C)::value, n0 = NT == 1 ? 2 : 0;
-            uint32_t a[2][NT][4];
-            uint2 b[2][NG];
-            auto load = [&](int kt) {
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp) b[kt & 1][grp] = cl_lds8(b0 + kt * 4 * QSTR + grp * GSTR);
-                // (rows 8..15 of the third tile do not exist: its lanes read rows 0..7 again)
-#pragma unroll
-                for (int n = 0; n < NT; ++n) cl_ldmatrix4(a0 + (uint32_t)((2 * kt * CT2 + 16 * (n0 + n)) * 16) - (NT == 1 ? ((lane >> 3) & 1) * 128u : 0u), a[kt & 1][n]);
-            };
-            load(0);
-#pragma unroll
-            for (int kt = 0; kt < 7; ++kt) {
-                if (kt < 6) load(kt + 1);
-#pragma unroll
-                for (int n = 0; n < NT; ++n)
-#pragma unroll
-                    for (int grp = 0; grp < NG; ++grp)
-                        cl_mma(acc2[n][grp], make_uint4(a[kt & 1][n][0], a[kt & 1][n][1], a[kt & 1][n][2], a[kt & 1][n][3]), b[kt & 1][grp].x, b[kt & 1][grp].y);
-            }
-        };
-        if (rj) run(std::integral_constant<int, 2>{});
-        else run(std::integral_constant<int, 1>{});
-    };
-    auto r2_store = [&]() {
-#pragma unroll
         for (int grp = 0; grp < NG; ++grp) {
-            float *d = part2 + (rq * 4 * NG + 4 * grp + t4) * CP2 + g4 + (rj ? 0 : 32);
+            float *d = partR + (rq * 4 * NG + 4 * grp + t4) * CPR + g4;
 #pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                float lo, hi;
-                part_sum(acc2[n][grp], lo, hi);
-                if (rj || n == 0) d[16 * n] = lo;
-                if (rj) d[16 * n + 8] = hi;
-            }
+            for (int n = 0; n < 4; ++n) part_sum(acc[n][grp], d[(4 * rj + n) * 16], d[(4 * rj + n) * 16 + 8]);
+            part_sum(acc[4][grp], d[(rj ? 8 : 9) * 16], d[(rj ? 8 : 9) * 16 + 8]);
+            if (!rj) d[160] = acc[5][grp][0] + acc[5][grp][1];
         }
     };
 
@@ -422,14 +393,10 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 
     const float r_inv = p.inv_R * h_inv;
     struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
-    // a row of R h of this row of the batch: both halves (or all quarters) of K
+    // a row of R h of this row of the batch
     auto r_row = [&](int i) {
-        float v;
-        if (i < 128) v = partR[st_d * CPR + i] + partR[(4 * NG + st_d) * CPR + i];
-        else {
-            const float *q = part2 + st_d * CP2 + i - 128;
-            v = (q[0] + q[4 * NG * CP2]) + (q[8 * NG * CP2] + q[12 * NG * CP2]);
-        }
+        const float *q = partR + st_d * CPR + i;
+        const float v = (q[0] + q[4 * NG * CPR]) + (q[8 * NG * CPR] + q[12 * NG * CPR]);
         return v * r_inv;
     };
     // everything of the gates of one half that does not depend on the pending draw
@@ -506,15 +473,10 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 
     // ---- prologue: R h of the initial state, coarse gates of step 0
     if (warp >= 8) {
-        uint32_t r0[16];
         r_clear();
 #pragma unroll 1
-        for (int half_f = 0; half_f < 2; ++half_f) { r_load(half_f, 0, r0); r_products(half_f, r0); }
+        for (int half_f = 0; half_f < 2; ++half_f) r_products(half_f);
         r_store();
-        r2_clear();
-#pragma unroll 1
-        for (int half_f = 0; half_f < 2; ++half_f) r2_products(half_f);
-        r2_store();
     }
     if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
     __syncthreads();
@@ -539,182 +501,182 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const bool last = n == 2 * T;
         const unsigned yuse = (unsigned)((n - 1) >> 1), quse = (unsigned)(n - 1);
         const uint32_t xin = sbase + (uint32_t)(CB_SMEM + in * CS_IMG), qin = sbase + (uint32_t)(CB_SMEM + 2 * CS_IMG);
-        if (warp < 8) {
-            if (tid == 0 && !bad) {
-                mbar_arrive_expect(smem_u32(&xq), ybytes);
-                mbar_arrive_expect(smem_u32(&xl), lbytes);
-                if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
-            }
-            float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
-            int forced = -1;
-            if (drawer) {
-                u01 = s_u[half][st_d];
-                const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
-                if (!last)
+        if (tid == 0 && !bad) {
+            mbar_arrive_expect(smem_u32(&xq), ybytes);
+            mbar_arrive_expect(smem_u32(&xl), lbytes);
+            if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
+        }
+        float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
+        int forced = -1;
+        if (drawer) {
+            u01 = s_u[half][st_d];
+            const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
+            if (!last)
 #pragma unroll
-                    for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
-                if (DBG) {
-                    const uint8_t *fz = half ? p.c_forced : p.f_forced;
-                    if (fz) forced = fz[(size_t)gb * T + (half ? s : s - 1)];
+                for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
+            if (DBG) {
+                const uint8_t *fz = half ? p.c_forced : p.f_forced;
+                if (fz) forced = fz[(size_t)gb * T + (half ? s : s - 1)];
+            }
+        }
+        // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
+        {
+            uint4 av[7];
+            const int tile = warp & 1, split = warp >> 1;
+            const uint4 *A = wH[half] + (tile * 28 + 7 * split) * 32 + lane;
+#pragma unroll
+            for (int i = 0; i < 7; ++i) av[i] = A[i * 32];
+            STAMP0();
+            wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
+            STAMP(8 * half + 0);
+            const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp) {
+                uint2 b[7];
+                float acc[2][4];
+#pragma unroll
+                for (int i = 0; i < 7; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
+#pragma unroll
+                for (int i = 0; i < 7; ++i) cl_mma(acc[i & 1], av[i], b[i].x, b[i].y);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
+                float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
+                part_sum(acc[0], d[0], d[8]);
+            }
+        }
+        cl_bar_sync(1, 256);
+        STAMP(8 * half + 1);
+        // ---- K-split sums, bias, relu, parts; every sending warp adds up the same sums (cheaper than a hand-over) and serves
+        // four CTAs: warps 0..3 the first group of rows, 4..7 the second
+        if ((NG == 2 || warp < 4) && pc_on) {
+            const int grp = NG == 2 ? warp >> 2 : 0, st = 4 * grp + pc_a;
+            if (st < nrc && !bad) {
+                const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
+                float4 v = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int sp = 0; sp < 4; ++sp) {
+                    const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
+                    v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                 }
+                const float inv = half ? inv_h0 : inv_h1;
+                v.x = fmaxf(fmaf(v.x, inv, bias.x), 0.f) * (half ? q_s0 : q_s1); v.y = fmaxf(fmaf(v.y, inv, bias.y), 0.f) * (half ? q_s0 : q_s1);
+                v.z = fmaxf(fmaf(v.z, inv, bias.z), 0.f) * (half ? q_s0 : q_s1); v.w = fmaxf(fmaf(v.w, inv, bias.w), 0.f) * (half ? q_s0 : q_s1);
+                uint2 lo;
+                const uint2 hi = cl_split4(v.x, v.y, v.z, v.w, lo);
+                const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
             }
-            // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
-            {
-                uint4 av[7];
-                const int tile = warp & 1, split = warp >> 1;
-                const uint4 *A = wH[half] + (tile * 28 + 7 * split) * 32 + lane;
+        }
+        cl_bar_sync(2, 512);                 // the background warps are done with the last half-step and go on
+        STAMP(8 * half + 2);
+        // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
+        if (warp < 7) {
+            uint4 lv[4];
+            const uint4 *A = wL[half] + 4 * warp * 32 + lane;
 #pragma unroll
-                for (int i = 0; i < 7; ++i) av[i] = A[i * 32];
-                STAMP0();
-                wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
-                STAMP(8 * half + 0);
-                const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
+            for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
+            const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + 4 * (lane & 3));
+            wait_bar(&xq, quse, (int)s, 2 + 4 * half);
+            STAMP(8 * half + 3);
+            const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) {
-                    uint2 b[7];
-                    float acc[2][4];
+            for (int grp = 0; grp < NG; ++grp) {
+                uint2 b[4];
+                float acc[2][4];
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+                for (int i = 0; i < 4; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
+                for (int c = 0; c < 2; ++c)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
+                    for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
 #pragma unroll
-                    for (int i = 0; i < 7; ++i) cl_mma(acc[i & 1], av[i], b[i].x, b[i].y);
+                for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i].x, b[i].y);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
-                    float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
-                    part_sum(acc[0], d[0], d[8]);
-                }
+                for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
+                float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
+                part_sum(acc[0], d[0], d[8]);
             }
-            cl_bar_sync(1, 256);
-            STAMP(8 * half + 1);
-            // ---- K-split sums, bias, relu, parts; every sending warp adds up the same sums (cheaper than a hand-over) and serves
-            // four CTAs: warps 0..3 the first group of rows, 4..7 the second
-            if ((NG == 2 || warp < 4) && pc_on) {
-                const int grp = NG == 2 ? warp >> 2 : 0, st = 4 * grp + pc_a;
-                if (st < nrc && !bad) {
-                    const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
+            if (warp >= 4) cl_bar_arrive(3, 224);
+            else {
+                cl_bar_sync(3, 224);
+                STAMP(8 * half + 4);
+                if (lane < 4 * nrc && !bad) {
+                    const int st = lane >> 2;
                     float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                    for (int sp = 0; sp < 4; ++sp) {
-                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
+                    for (int sp = 0; sp < 7; ++sp) {
+                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + 4 * (lane & 3));
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
-                    const float inv = half ? inv_h0 : inv_h1;
-                    v.x = fmaxf(fmaf(v.x, inv, bias.x), 0.f) * (half ? q_s0 : q_s1); v.y = fmaxf(fmaf(v.y, inv, bias.y), 0.f) * (half ? q_s0 : q_s1);
-                    v.z = fmaxf(fmaf(v.z, inv, bias.z), 0.f) * (half ? q_s0 : q_s1); v.w = fmaxf(fmaf(v.w, inv, bias.w), 0.f) * (half ? q_s0 : q_s1);
-                    uint2 lo;
-                    const uint2 hi = cl_split4(v.x, v.y, v.z, v.w, lo);
-                    const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
+                    const float inv = half ? inv_l0 : inv_l1;
+                    const uint32_t a = smem_u32(lbuf + st * 256 + CL * rank + 4 * (lane & 3)), bar = smem_u32(&xl);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
+                    for (int k = 0; k < 4; ++k)
+                        st_async_v4(a + delta4[k], fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + delta4[k]);
                 }
+                STAMP(8 * half + 5);
             }
-            cl_bar_sync(2, 512);                 // the background warps are done with the last half-step (and go on, in the fine half)
-            STAMP(8 * half + 2);
-            // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
-            if (warp < 7) {
-                uint4 lv[4];
-                const uint4 *A = wL[half] + 4 * warp * 32 + lane;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
-                const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + 4 * (lane & 3));
-                wait_bar(&xq, quse, (int)s, 2 + 4 * half);
-                STAMP(8 * half + 3);
-                const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp) {
-                    uint2 b[4];
-                    float acc[2][4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i].x, b[i].y);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
-                    float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
-                    part_sum(acc[0], d[0], d[8]);
-                }
-                if (warp >= 4) cl_bar_arrive(3, 224);
-                else {
-                    cl_bar_sync(3, 224);
-                    STAMP(8 * half + 4);
-                    if (lane < 4 * nrc && !bad) {
-                        const int st = lane >> 2;
-                        float4 v = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                        for (int sp = 0; sp < 7; ++sp) {
-                            const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + 4 * (lane & 3));
-                            v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
-                        }
-                        const float inv = half ? inv_l0 : inv_l1;
-                        const uint32_t a = smem_u32(lbuf + st * 256 + CL * rank + 4 * (lane & 3)), bar = smem_u32(&xl);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            st_async_v4(a + delta4[k], fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + delta4[k]);
-                    }
-                    STAMP(8 * half + 5);
-                }
-            } else if (!last) prepare_rows(1 - half, half ? s + 1 : s);
-            if (half) cl_bar_arrive(5, 512);     // coarse half: the background warps go on
-            // ---- one row per warp: what does not depend on the draw, the draw, the gates
-            if (drawer) {
-                if (!half) cl_bar_sync(4, 256 + n_draw);                  // R h is complete
-                const GatePre gp = gates_prepare(half, gv);
-                wait_bar(&xl, quse, (int)s, 3 + 4 * half);
-                STAMP0();
-                float l[8];
-                {
-                    const float4 a = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane), b = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane + 4);
-                    l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
-                }
-                const int drawn = cl_draw(l, u01, lane);
-                const int fed = (DBG && forced >= 0) ? forced : drawn;
-                STAMP(8 * half + 6);
-                if (!last) gates_and_stage(half, s, fed, gp);
-                STAMP(8 * half + 7);
-                if (half) c_prev = fed; else f_prev = fed;
-                drawn_out = drawn;
-                if (DBG && p.dbg_logits && writer && !bad) {
-                    float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) d[k] = l[k];
-                }
+        } else if (!last) prepare_rows(1 - half, half ? s + 1 : s);
+        // ---- one row per warp: what does not depend on the draw, the draw, the gates
+        if (drawer) {
+            if (!half) cl_bar_sync(4, 256 + n_draw);                  // R h is complete
+            const GatePre gp = gates_prepare(half, gv);
+            wait_bar(&xl, quse, (int)s, 3 + 4 * half);
+            STAMP0();
+            float l[8];
+            {
+                const float4 a = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane), b = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane + 4);
+                l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
             }
-            if (!last) {
-                cl_bar_sync(1, 256);
-                send_y(half, s);
+            const int drawn = cl_draw(l, u01, lane);
+            const int fed = (DBG && forced >= 0) ? forced : drawn;
+            STAMP(8 * half + 6);
+            if (!last) gates_and_stage(half, s, fed, gp);
+            STAMP(8 * half + 7);
+            if (half) c_prev = fed; else f_prev = fed;
+            drawn_out = drawn;
+            if (DBG && p.dbg_logits && writer && !bad) {
+                float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) d[k] = l[k];
             }
-            // the samples leave when the state is on its way
-            if (writer && lane == 0 && !bad) {
-                if (DBG) {
-                    uint8_t *o = half ? p.c_out : p.f_out;
-                    if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
-                }
-                if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
+        }
+        if (!last) {
+            cl_bar_sync(1, 256);
+            send_y(half, s);
+        }
+        // the samples leave when the state is on its way
+        if (writer && lane == 0 && !bad) {
+            if (DBG) {
+                uint8_t *o = half ? p.c_out : p.f_out;
+                if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
             }
-        } else {
-            // ---- the rows of R: in the fine half right after the hidden layer is sent (its coarse rows are needed by the gates at
-            // the end), in the coarse half when the logits are
-            uint32_t r0[16];
-            r_load(in, 0, r0);
-            cl_bar_sync(2, 512);
-            if (half) { cl_bar_sync(5, 512); r_clear(); r2_clear(); }
-            r_products(in, r0);
-            if (!half) { r_store(); cl_bar_arrive(4, 256 + n_draw); }
-            r2_products(in);
-            if (!half) r2_store();
+            if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
         }
     };
+    if (warp < 8) {
 #pragma unroll 1
-    for (long long s2 = 0; s2 < T; ++s2) {
-        half_step(std::integral_constant<int, 1>{}, 2 * s2 + 1);
-        half_step(std::integral_constant<int, 0>{}, 2 * s2 + 2);
+        for (long long s2 = 0; s2 < T; ++s2) {
+            half_step(std::integral_constant<int, 1>{}, 2 * s2 + 1);
+            half_step(std::integral_constant<int, 0>{}, 2 * s2 + 2);
+        }
+    } else {
+        // ---- the rows of R, right after the hidden layer is sent (its sums and sends do not share the load / store pipe with them)
+#pragma unroll 1
+        for (long long s2 = 0; s2 < T; ++s2) {
+            r_clear();
+            cl_bar_sync(2, 512);
+            r_products(0);
+            cl_bar_sync(2, 512);
+            r_products(1);
+            r_store();
+            cl_bar_arrive(4, 256 + n_draw);
+        }
     }
 #undef STAMP
 #undef STAMP0
@@ -843,10 +805,10 @@ int rescl_prepare(wrnn_model *m)
             pack(dO[2 + h], CL * rank, CL, reinterpret_cast<uint16_t *>(base + 2 * CW_HID + h * CW_LOG));
         }
         uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
-        for (int i = 0; i < CT2; ++i)
+        for (int i = 0; i < CRS; ++i)
             for (int k8 = 0; k8 < 2 * CK8; ++k8) {
-                const uint16_t *src = r_row(rank, 128 + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
-                for (int e = 0; e < 8; ++e) r2[((size_t)k8 * CT2 + i) * 8 + e] = src[4 * (e >> 1) + (e & 1)];
+                const uint16_t *src = r_row(rank, 16 * CRT + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
+                for (int e = 0; e < 8; ++e) r2[((size_t)k8 * CRS + i) * 8 + e] = src[4 * (e >> 1) + (e & 1)];
             }
         float *sm = reinterpret_cast<float *>(base + 2 * CW_HID + 2 * CW_LOG + CW_R2);
         for (int i = 0; i < 6 * CU; ++i) {
@@ -856,19 +818,19 @@ int rescl_prepare(wrnn_model *m)
         float *b = sm + 6 * CU * 3;
         for (int r = 0; r < CU; ++r) { b[r] = m->hb1[CU * rank + r]; b[32 + r] = m->hb3[CU * rank + r]; }
         for (int r = 0; r < CL; ++r) { b[64 + r] = m->hb2[CL * rank + r]; b[64 + CL + r] = m->hb4[CL * rank + r]; }
-        // tensor memory: lane quadrant q holds tiles 4 (q & 1) .. + 3 and half q >> 1 of the k-tiles of both halves of the state;
-        // columns [half of the state][j][pair of k-tiles][tile 2 j + n][k-tile][4 registers of the A fragment]
+        // tensor memory: lane quadrant q holds quarter q of the k-tiles of both halves of the state; columns as the kernel states them
         uint16_t *tm = reinterpret_cast<uint16_t *>(base + CB_SMEM);
-        for (int q = 0; q < 4; ++q)
-            for (int c = 0; c < 448; ++c) {
-                const int reg = c & 3, kt1 = (c >> 2) & 1, n = (c >> 3) & 1, pair = (c >> 4) % 7, j = (c / 112) & 1, half_f = c / 224;
-                const int tile = 4 * (q & 1) + 2 * j + n, kt = 28 * half_f + 14 * (q >> 1) + 2 * pair + kt1;
-                for (int lane = 0; lane < 32; ++lane) {
-                    const uint16_t *src = r_row(rank, 16 * tile + (lane >> 2) + 8 * (reg & 1)) + 16 * kt + 4 * (lane & 3) + 2 * (reg >> 1);
-                    uint16_t *d = tm + ((size_t)c * 128 + 32 * q + lane) * 2;
-                    d[0] = src[0]; d[1] = src[1];
-                }
+        for (int i = 0; i < 16 * CRT; ++i) {
+            const int tile = i >> 4, reg0 = (i >> 3) & 1;
+            const uint16_t *src = r_row(rank, i);
+            for (int kt = 0; kt < 56; ++kt) {
+                const int half_f = kt / 28, q = kt % 28 / 7, k7 = kt % 7;
+                const int c0 = tile < 4 ? (half_f * 7 + k7) * 16 + 4 * tile : 2 * 7 * 16 + (half_f * 7 + k7) * 20 + 4 * (tile - 4);
+                for (int t = 0; t < 4; ++t)
+                    for (int h = 0; h < 2; ++h)
+                        std::memcpy(tm + ((size_t)(c0 + reg0 + 2 * h) * 128 + 32 * q + 4 * (i & 7) + t) * 2, src + 16 * kt + 4 * t + 2 * h, 4);
             }
+        }
     }
     ResClPack *pk = new ResClPack(k);
     if (cudaMalloc((void **)&pk->d_blob, blob.size()) != cudaSuccess || cudaMemcpy(pk->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
