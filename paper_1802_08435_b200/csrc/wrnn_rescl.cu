@@ -430,13 +430,16 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             }
         }
     };
+    // three rows of a group travel as four: 48-byte runs in the receivers' images are slower than 64-byte ones (21 rows: 4.74 us
+    // per step with three, 4.52 with four)
+    const int nsend = (nrc & 3) == 3 ? nrc + 1 : nrc;
     // warps 0..7: the staged state values of this CTA's units -> images in the cluster's CTAs, two each
     auto send_y = [&](int half_g, long long s) {
         if (bad || !pc_on || (DBG && (int)s == skip_at)) return;
         const uint32_t a = sbase + (uint32_t)(CB_SMEM + half_g * CS_IMG) + pc_off, bar = smem_u32(&xy[half_g]);
 #pragma unroll
         for (int grp = 0; grp < NG; ++grp)
-            if (4 * grp + pc_a < nrc) {
+            if (4 * grp + pc_a < nsend) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((4 * grp + pc_a) * 7 + pc_quad) * 16);
 #pragma unroll
                 for (int k = 0; k < 2; ++k) cl_st_async16(a + grp * GSTR + dy[k], v, bar + dy[k]);
@@ -445,7 +448,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const float inv_h0 = p.inv_O1[0] * h_inv, inv_h1 = p.inv_O1[1] * h_inv, inv_l0 = p.inv_O2[0] * h_inv, inv_l1 = p.inv_O2[1] * h_inv;
     const float q_s0 = p.q_scale[0] * ldexpf(1.f, -s_hexp), q_s1 = p.q_scale[1] * ldexpf(1.f, -s_hexp);
     const int n_draw = 32 * nrc;                                         // threads of the drawing warps
-    const unsigned ybytes = (unsigned)(nrc * CK * 4), lbytes = (unsigned)(nrc * 1024);
+    const unsigned ybytes = (unsigned)(nsend * CK * 4), lbytes = (unsigned)(nrc * 1024);
 
     // ---- warp 7 prepares, one row per lane, what the draws of a half-step need: the uniform and the conditioning frame (the
     // same for both halves of a step), tracked without a division per step
@@ -530,22 +533,26 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
             STAMP(8 * half + 0);
             const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
+            uint2 b[NG][7];
+            float acc[NG][2][4];
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) b[grp][i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc[grp][k >> 2][k & 3] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[grp][i & 1], av[i], b[grp][i].x, b[grp][i].y);
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp) {
-                uint2 b[7];
-                float acc[2][4];
 #pragma unroll
-                for (int i = 0; i < 7; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
-#pragma unroll
-                for (int i = 0; i < 7; ++i) cl_mma(acc[i & 1], av[i], b[i].x, b[i].y);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
+                for (int k = 0; k < 4; ++k) acc[grp][0][k] += acc[grp][1][k];
                 float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
-                part_sum(acc[0], d[0], d[8]);
+                part_sum(acc[grp][0], d[0], d[8]);
             }
         }
         cl_bar_sync(1, 256);
@@ -554,7 +561,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         // four CTAs: warps 0..3 the first group of rows, 4..7 the second
         if ((NG == 2 || warp < 4) && pc_on) {
             const int grp = NG == 2 ? warp >> 2 : 0, st = 4 * grp + pc_a;
-            if (st < nrc && !bad) {
+            if (st < nsend && !bad) {
                 const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
                 float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -584,22 +591,26 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             wait_bar(&xq, quse, (int)s, 2 + 4 * half);
             STAMP(8 * half + 3);
             const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
+            uint2 b[NG][4];
+            float acc[NG][2][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) b[grp][i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+#pragma unroll
+            for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) acc[grp][k >> 2][k & 3] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[grp][i & 1], lv[i], b[grp][i].x, b[grp][i].y);
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp) {
-                uint2 b[4];
-                float acc[2][4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) b[i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[c][k] = 0.f;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) cl_mma(acc[i & 1], lv[i], b[i].x, b[i].y);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[0][k] += acc[1][k];
+                for (int k = 0; k < 4; ++k) acc[grp][0][k] += acc[grp][1][k];
                 float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
-                part_sum(acc[0], d[0], d[8]);
+                part_sum(acc[grp][0], d[0], d[8]);
             }
             if (warp >= 4) cl_bar_arrive(3, 224);
             else {
