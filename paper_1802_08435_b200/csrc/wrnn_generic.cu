@@ -257,24 +257,52 @@ __global__ void __launch_bounds__(512, 1) generic_step_kernel(const GenericParam
 // Prologue: g[b][k][row] = W_cond[row][:] . frame[b][k][:] + b_gate[row]   (the per-step
 // conditioning vector; one frame is held for `hop` samples).
 
+// NP pairs per block and pass: a weight is read once for NP of them (the weights come from L2: one pair per block kept 2,048
+// pairs -- a chunk of 128 steps of 16 rows -- at 107 us).  The sum over D runs in the same order whatever NP.
+template <int NP>
 __global__ void cond_project_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT,
                                     const float *__restrict__ b_gate, float *__restrict__ g, int G, int D,
                                     long long n_pairs)
 {
     // blockIdx.y strides over the (row of the batch, frame) pairs, so no grid dimension limits their number
-    extern __shared__ float fr[];
+    extern __shared__ __align__(16) float fr[];              // [D][NP]
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
-    for (long long kb = blockIdx.y; kb < n_pairs; kb += gridDim.y) {
-        const float *f = cond + (size_t)kb * D;
+    for (long long k0 = (long long)blockIdx.y * NP; k0 < n_pairs; k0 += (long long)gridDim.y * NP) {
         __syncthreads();
-        for (int d = threadIdx.x; d < D; d += blockDim.x) fr[d] = f[d];
+        for (int i = threadIdx.x; i < D * NP; i += blockDim.x) {
+            const int q = i / D, d = i - q * D;
+            fr[d * NP + q] = k0 + q < n_pairs ? cond[(size_t)(k0 + q) * D + d] : 0.f;
+        }
         __syncthreads();
         if (row < G) {
-            float acc = 0.f;
-            for (int d = 0; d < D; ++d) acc = fmaf(W_condT[(size_t)d * G + row], fr[d], acc);
-            g[(size_t)kb * G + row] = acc + (b_gate ? b_gate[row] : 0.f);
+            float acc[NP];
+#pragma unroll
+            for (int q = 0; q < NP; ++q) acc[q] = 0.f;
+#pragma unroll 8
+            for (int d = 0; d < D; ++d) {
+                const float w = W_condT[(size_t)d * G + row];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) acc[q] = fmaf(w, fr[d * NP + q], acc[q]);
+            }
+            const float b = b_gate ? b_gate[row] : 0.f;
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+                if (k0 + q < n_pairs) g[(size_t)(k0 + q) * G + row] = acc[q] + b;
         }
     }
+}
+
+// As many pairs per block as leave the chip two blocks per SM (a block of 256 rows of the gates takes some 11 columns of the
+// grid at H = 896): short calls are bound by latency and keep one pair per block.
+static void cond_project_launch(const float *cond, const float *W_condT, const float *b_gate, float *g, int G, int D, long long n_pairs, cudaStream_t s)
+{
+    const int np = n_pairs >= 448 ? 16 : n_pairs >= 112 ? 4 : 1;
+    const dim3 grid((G + 255) / 256, (unsigned)std::min<long long>((n_pairs + np - 1) / np, 65535));
+    const size_t smem = (size_t)np * D * sizeof(float);
+    if (np == 16 && smem <= 48 * 1024) cond_project_kernel<16><<<grid, 256, smem, s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+    else if (np >= 4 && (size_t)4 * D * sizeof(float) <= 48 * 1024)
+        cond_project_kernel<4><<<dim3(grid.x, (unsigned)std::min<long long>((n_pairs + 3) / 4, 65535)), 256, (size_t)4 * D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+    else cond_project_kernel<1><<<dim3(grid.x, (unsigned)std::min<long long>(n_pairs, 65535)), 256, D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
 }
 
 __global__ void cond_bias_only_kernel(const float *__restrict__ b_gate, float *__restrict__ g, int G, int batch)
@@ -289,10 +317,7 @@ int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, cuda
     if (m->cond_dim == 0) {
         cond_bias_only_kernel<<<(G * batch + 255) / 256, 256, 0, s>>>(m->b_gate, m->g, G, batch);
     } else {
-        const long long n_pairs = (long long)batch * n_frames;
-        dim3 grid((G + 255) / 256, (unsigned)std::min<long long>(n_pairs, 65535));
-        cond_project_kernel<<<grid, 256, m->cond_dim * sizeof(float), s>>>(cond, m->W_condT, m->b_gate, m->g, G,
-                                                                           m->cond_dim, n_pairs);
+        cond_project_launch(cond, m->W_condT, m->b_gate, m->g, G, m->cond_dim, (long long)batch * n_frames, s);
     }
     ++g_launches;
     return cudaGetLastError() == cudaSuccess ? WRNN_OK : WRNN_ERR_CUDA;
@@ -529,8 +554,7 @@ extern "C" int wrnn_sample_noalloc(wrnn_model *m, const wrnn_cond *cond, int64_t
         cond_bias_only_kernel<<<(unsigned)((G * B + 255) / 256), 256, 0, s>>>(m->b_gate, g, (int)G, batch);
     } else {
         const long long n_pairs = (long long)(B * nf);
-        dim3 grid((unsigned)((G + 255) / 256), (unsigned)std::min<long long>(n_pairs, 65535));
-        cond_project_kernel<<<grid, 256, m->cond_dim * sizeof(float), s>>>(a.cond, m->W_condT, m->b_gate, g, (int)G, m->cond_dim, n_pairs);
+        cond_project_launch(a.cond, m->W_condT, m->b_gate, g, (int)G, m->cond_dim, n_pairs, s);
     }
     ++g_launches;
     if (cudaGetLastError() != cudaSuccess) { m->err = "conditioning projection launch failed"; return WRNN_ERR_CUDA; }

@@ -392,6 +392,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const float *g_row = p.g + (size_t)gb * p.n_frames * 3 * H + gj;
 
     const float r_inv = p.inv_R * h_inv;
+    float dbg_v[4] = {0.f, 0.f, 0.f, 0.f};                               // what the dumps want of this half-step's gates
+    auto dump_gates = [&](int half_g, long long s) {
+        const int jj = half_g * CK + gj;
+        if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[jj] = dbg_v[0]; o[H + jj] = dbg_v[1]; o[2 * H + jj] = dbg_v[2]; }
+        if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + jj] = dbg_v[3];
+    };
     struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
     // a row of R h of this row of the batch
     auto r_row = [&](int i) {
@@ -423,11 +429,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             const __half hi = __float2half_rn(x);
             d[0] = hi;
             d[4] = __float2half_rn(x - __half2float(hi));
-            if (DBG) {
-                const int jj = half_g * CK + gj;
-                if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[jj] = u; o[H + jj] = r; o[2 * H + jj] = e; }
-                if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + jj] = hn;
-            }
+            if (DBG) { dbg_v[0] = u; dbg_v[1] = r; dbg_v[2] = e; dbg_v[3] = hn; }
         }
     };
     // three rows of a group travel as four: 48-byte runs in the receivers' images are slower than 64-byte ones (21 rows: 4.74 us
@@ -492,6 +494,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     }
     __syncthreads();
     if (warp < 8) send_y(0, 0);
+    if (DBG && gater) dump_gates(0, 0);
 
     // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
     // n = 2 s the fine half (input y_f(s - 1): fine head -> f_{s-1}, R h_{s-1} completed, then the coarse gates of step s).
@@ -633,6 +636,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 STAMP(8 * half + 5);
             }
         } else if (!last) prepare_rows(1 - half, half ? s + 1 : s);
+        float dbg_l[8] = {};
         // ---- one row per warp: what does not depend on the draw, the draw, the gates
         if (drawer) {
             if (!half) cl_bar_sync(4, 256 + n_draw);                  // R h is complete
@@ -651,17 +655,21 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             STAMP(8 * half + 7);
             if (half) c_prev = fed; else f_prev = fed;
             drawn_out = drawn;
-            if (DBG && p.dbg_logits && writer && !bad) {
-                float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+            if (DBG)
 #pragma unroll
-                for (int k = 0; k < 8; ++k) d[k] = l[k];
-            }
+                for (int k = 0; k < 8; ++k) dbg_l[k] = l[k];
         }
         if (!last) {
             cl_bar_sync(1, 256);
             send_y(half, s);
         }
-        // the samples leave when the state is on its way
+        // the samples (and the dumps) leave when the state is on its way
+        if (DBG && gater && !last && !bad) dump_gates(half, s);
+        if (DBG && p.dbg_logits && writer && !bad) {
+            float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) d[k] = dbg_l[k];
+        }
         if (writer && lane == 0 && !bad) {
             if (DBG) {
                 uint8_t *o = half ? p.c_out : p.f_out;

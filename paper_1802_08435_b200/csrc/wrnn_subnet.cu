@@ -30,7 +30,7 @@ struct wrnn_subscale_net {
     __nv_bfloat16 *Wc = nullptr;      // [layers][taps][conv_ch][res_ch]
     __nv_bfloat16 *Wr = nullptr;      // [layers][res_ch][conv_ch]
     __nv_bfloat16 *Wo = nullptr;      // [64][res_ch] (rows >= cond_dim zero)
-    float *W_in = nullptr, *b_in = nullptr, *b_conv = nullptr, *b_res = nullptr, *b_out = nullptr;
+    float *W_in = nullptr /* [B][res_ch] */, *b_in = nullptr, *b_conv = nullptr, *b_res = nullptr, *b_out = nullptr;
     // activations of one call: n_seg row segments of n_alloc positions each
     int n_seg = 0, n_alloc = 0;
     float *xf = nullptr;                              // [n_seg * n_alloc][res_ch] fp32 residual stream
@@ -44,7 +44,7 @@ struct wrnn_subscale_net {
 namespace wrnn {
 
 constexpr int SN_BM = 128;           // positions per tile (the M side: one TMEM lane per position)
-constexpr int SN_THREADS = 192;      // warp 0: TMA producer, warp 1: MMA issuer, warps 2..5: epilogue
+constexpr int SN_THREADS = 256;      // warp 0: TMA of the high parts, warp 1: MMA issuer, warps 2..5: epilogue, warps 6, 7: TMA of the low parts, of the weights
 enum { SN_CONV = 0, SN_RES = 1, SN_OUT = 2 };
 
 struct SubnetGemmParams {
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     const uint32_t ring0 = smem_u32(ring);
 
     if (tid == 0) {
-        for (int i = 0; i < STAGES; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), 1); }
+        for (int i = 0; i < STAGES; ++i) { mbar_init(smem_u32(&full[i]), 3); mbar_init(smem_u32(&empty[i]), 1); }
         mbar_init(smem_u32(&done), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -101,16 +101,22 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     const int nkb = p.taps * p.n_kb_tap;
     const int arow0 = seg * p.n_alloc + mt * SN_BM;          // first activation row (position) of this tile
     bool ok = true;
-    if (warp == 0 && lane == 0) {
+    if ((warp == 0 || warp >= 6) && lane == 0) {
+        // one producer per operand: a tiled load occupies its issuing thread for some 230 cycles, and with all three in one
+        // thread a k-block took 1,200 cycles whatever the rows (a convolution launch 22 us from one row to sixteen)
+        const int op = warp == 0 ? 0 : warp - 5;                // high parts, low parts, weights
+        const CUtensorMap *tm = op == 0 ? &tmAh : op == 1 ? &tmAl : &tmW;
+        const uint32_t off = op * A_BYTES, bytes = op < 2 ? A_BYTES : W_BYTES;
+        const int y0 = op < 2 ? arow0 : p.w_row0 + nt * BN, ystep = op < 2 ? p.dil : p.w_tap_rows;
+        int st = 0, ph = 1, kc = 0, y = y0;
         for (int kb = 0; kb < nkb; ++kb) {
-            const int st = kb % STAGES, ph = (kb / STAGES) & 1;
-            if (!mbar_wait(smem_u32(&empty[st]), ph ^ 1, p.limit_ns)) { ok = false; break; }
-            const int tap = kb / p.n_kb_tap, kc = (kb - tap * p.n_kb_tap) * TC_BK;
-            const uint32_t fb = smem_u32(&full[st]), base = ring0 + st * STAGE_BYTES;
-            mbar_expect_tx(fb, STAGE_BYTES);
-            tma_load_2d(base, &tmAh, fb, kc, arow0 + tap * p.dil);
-            tma_load_2d(base + A_BYTES, &tmAl, fb, kc, arow0 + tap * p.dil);
-            tma_load_2d(base + 2 * A_BYTES, &tmW, fb, kc, p.w_row0 + tap * p.w_tap_rows + nt * BN);
+            if (!mbar_wait(smem_u32(&empty[st]), ph, p.limit_ns)) { ok = false; break; }
+            const uint32_t fb = smem_u32(&full[st]);
+            mbar_expect_tx(fb, bytes);
+            tma_load_2d(ring0 + st * STAGE_BYTES + off, tm, fb, kc, y);
+            kc += TC_BK;
+            if (kc == p.n_kb_tap * TC_BK) { kc = 0; y += ystep; }
+            if (++st == STAGES) { st = 0; ph ^= 1; }
         }
     } else if (warp == 1 && lane == 0) {
         const uint32_t idesc = umma_idesc_bf16(SN_BM, BN);
@@ -128,7 +134,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
             umma_commit(smem_u32(&empty[st]));
         }
         if (ok) umma_commit(smem_u32(&done));
-    } else if (warp >= 2) {
+    } else if (warp >= 2 && warp < 6) {
         if (mbar_wait(smem_u32(&done), 0, p.limit_ns)) {
             tc_fence_after();
             const int q = warp & 3;                             // TMEM lane quadrant this warp may read
@@ -203,28 +209,42 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     }
 }
 
-// x_0 = W_in X + b_in for the positions [0, n_pos) of every segment, fp32 and bf16 parts (N1, N2 of the reading above)
+// x_0 = W_in X + b_in for the positions [0, n_pos) of every segment, fp32 and bf16 parts (N1, N2 of the reading above).  A block
+// takes SN_IN_POS positions: a weight is read once for all of them.
+constexpr int SN_IN_POS = 8;
 __global__ void subnet_input_kernel(const int16_t *__restrict__ hist, const float *__restrict__ W_in, const float *__restrict__ b_in, int Bsub,
                                     long long L, int C, int r_lo, long long p_lo, int lag, int n_alloc, int n_pos, float *__restrict__ xf,
                                     __nv_bfloat16 *__restrict__ xh, __nv_bfloat16 *__restrict__ xl)
 {
-    const int seg = blockIdx.y, j = blockIdx.x, r = r_lo + seg;
-    const long long pos = p_lo - (long long)seg * lag + j;
-    if (j >= n_pos) return;
-    __shared__ float X[64];
-    if ((int)threadIdx.x < Bsub) X[threadIdx.x] = ((int)threadIdx.x < r && pos < L) ? (float)hist[(size_t)threadIdx.x * L + pos] * (1.0f / 32768.0f) : 0.f;
+    const int seg = blockIdx.y, j0 = blockIdx.x * SN_IN_POS, r = r_lo + seg;
+    const long long pos0 = p_lo - (long long)seg * lag + j0;
+    __shared__ __align__(16) float X[64][SN_IN_POS];
+    for (int i = threadIdx.x; i < Bsub * SN_IN_POS; i += blockDim.x) {
+        const int z = i / SN_IN_POS, q = i % SN_IN_POS;
+        X[z][q] = (z < r && pos0 + q < L) ? (float)hist[(size_t)z * L + pos0 + q] * (1.0f / 32768.0f) : 0.f;
+    }
     __syncthreads();
-    const size_t row = (size_t)seg * n_alloc + j;
+    const size_t row = (size_t)seg * n_alloc + j0;
     for (int c = threadIdx.x; c < C; c += blockDim.x) {
-        float v = 0.f;
-        if (pos < L) {
-            v = b_in[c];
-            for (int z = 0; z < r; ++z) v = fmaf(W_in[(size_t)c * Bsub + z], X[z], v);
+        float v[SN_IN_POS];
+        const float b = b_in[c];
+#pragma unroll
+        for (int q = 0; q < SN_IN_POS; ++q) v[q] = b;
+        for (int z = 0; z < r; ++z) {
+            const float w = W_in[(size_t)z * C + c];
+#pragma unroll
+            for (int q = 0; q < SN_IN_POS; ++q) v[q] = fmaf(w, X[z][q], v[q]);
         }
-        xf[row * C + c] = v;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        xh[row * C + c] = h;
-        xl[row * C + c] = __float2bfloat16_rn(v - __bfloat162float(h));
+#pragma unroll
+        for (int q = 0; q < SN_IN_POS; ++q) {
+            if (j0 + q >= n_pos) break;
+            const float x = pos0 + q < L ? v[q] : 0.f;
+            const size_t o = (row + q) * C + c;
+            xf[o] = x;
+            const __nv_bfloat16 h = __float2bfloat16_rn(x);
+            xh[o] = h;
+            xl[o] = __float2bfloat16_rn(x - __bfloat162float(h));
+        }
     }
 }
 
@@ -314,7 +334,7 @@ int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, i
     int rc = ensure_acts(n, n_rows, n0);
     if (rc != WRNN_OK) return rc;
     if (cudaMemsetAsync(n->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
-    subnet_input_kernel<<<dim3(n0, n_rows), 256, 0, s>>>(hist, n->W_in, n->b_in, n->B, L, n->res_ch, r_lo, p_lo, lag, n->n_alloc, n0, n->xf, n->xh, n->xl);
+    subnet_input_kernel<<<dim3((n0 + SN_IN_POS - 1) / SN_IN_POS, n_rows), 256, 0, s>>>(hist, n->W_in, n->b_in, n->B, L, n->res_ch, r_lo, p_lo, lag, n->n_alloc, n0, n->xf, n->xh, n->xl);
     ++g_launches;
     SubnetGemmParams p;
     std::memset(&p, 0, sizeof(p));
@@ -384,7 +404,8 @@ extern "C" int wrnn_subscale_net_create(const wrnn_subscale_net_params *q, wrnn_
     }
     const size_t nc = (size_t)q->n_layers * q->taps * q->conv_ch * q->res_ch, nr = (size_t)q->n_layers * q->res_ch * q->conv_ch;
     std::vector<float> win((size_t)q->res_ch * q->B);
-    for (size_t i = 0; i < win.size(); ++i) win[i] = round_bf16_host(q->W_in[i]);
+    for (int c = 0; c < q->res_ch; ++c)                      // transposed: [B][res_ch]
+        for (int z = 0; z < q->B; ++z) win[(size_t)z * q->res_ch + c] = round_bf16_host(q->W_in[(size_t)c * q->B + z]);
     bool ok = upload_bf16(&n->Wc, q->W_conv, nc, nc) && upload_bf16(&n->Wr, q->W_res, nr, nr) &&
               upload_bf16(&n->Wo, q->W_out, (size_t)q->cond_dim * q->res_ch, (size_t)64 * q->res_ch) &&
               upload_f32(&n->W_in, win.data(), win.size()) && upload_f32(&n->b_in, q->b_in, q->res_ch) &&
