@@ -139,7 +139,8 @@ static bool use_rescl(const wrnn_model *m, int batch)
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
     const char *off = getenv(batch == 1 ? "WRNN_RESIDENT_LEAN" : "WRNN_NO_MULTI");
     if (off && off[0] == (batch == 1 ? '0' : '1')) return false;
-    return batch <= 128 && rescl_supported(m, batch) == WRNN_OK;
+    // (fp32 weights: 28 rows at a time; the any-shape kernel, the other one for several rows, takes 55 us per step at four)
+    return (m->dtype == WRNN_F32 || batch <= 128) && rescl_supported(m, batch) == WRNN_OK;
 }
 
 static bool use_resf32(const wrnn_model *m, int batch)
@@ -447,7 +448,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
         if (m->dtype == WRNN_BF16 && m->variant == 0) reslean_prepare(m);                        // optional: the row-split resident kernel serves the stream without it
-        if (m->dtype == WRNN_BF16 && m->variant == 0 && !reslean_checked(m)) rescl_prepare(m);
+        if (m->variant == 0 && !reslean_checked(m)) rescl_prepare(m);
         if (m->dtype == WRNN_BF16 && m->variant == 0 && max_batch >= 2) resmulti_prepare(m);   // optional: other kernels serve the batch without it
     }
     m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call

@@ -55,21 +55,26 @@ constexpr size_t CW_HID = 2 * 28 * 512;                      // O1 (O3) rows of 
 constexpr size_t CW_LOG = 28 * 512;                          // O2 (O4) rows: one tile
 constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
 constexpr int C_SMALL = 2 * 3 * CU * 3 + 2 * 32 + 2 * CL;    // I of the CTA's units [half][gate][unit][3], b1, b3 (32 each), b2, b4
-constexpr size_t CB_SMEM = 2 * CW_HID + 2 * CW_LOG + CW_R2 + C_SMALL * 4;
+__host__ __device__ constexpr size_t cl_blob_smem(bool w2) { return (w2 ? 2 : 1) * (2 * CW_HID + 2 * CW_LOG) + (w2 ? 0 : CW_R2) + C_SMALL * 4; }
 constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: [2 halves][7 k-tiles][9 tiles][4 registers]
 constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
-static_assert(CB_SMEM % 16 == 0, "the blob is copied in 16-byte pieces");
-constexpr int CNG = 2;                                       // column groups (of four rows) the carve-up has room for
-constexpr size_t CS_IMG = (size_t)CQ * CNG * 64;            // operand image of one vector
-constexpr size_t CS_PART = (size_t)7 * 4 * CNG * CPL * 4;    // partial sums (>= 4 * 4 * CNG * CPH * 4)
-static_assert(CS_PART >= (size_t)4 * 4 * CNG * CPH * 4, "the partial sums of both products share a buffer");
-constexpr size_t CS_PARTR = (size_t)4 * 4 * CNG * CPR * 4;     // R h
-constexpr size_t CS_BYTES = CB_SMEM + 3 * CS_IMG /* two state halves, hidden layer */ + (size_t)CMAXR * 1024 /* logits */ + CS_PART + CS_PARTR +
-                            (size_t)CMAXR * 2 * CU * 2 /* staged state */;
+static_assert(cl_blob_smem(false) % 16 == 0 && cl_blob_smem(true) % 16 == 0, "the blob is copied in 16-byte pieces");
+// fp32 weights, second part and the rows without room: [warp][half][pass][k-tile][4 fragments][32 lanes][16 B] per CTA, read from L2
+constexpr size_t CB_STREAM = (size_t)8 * 2 * 2 * 7 * 4 * 512;
+__host__ __device__ constexpr size_t cl_img(int ng) { return (size_t)CQ * ng * 64; }                // operand image of one vector
+__host__ __device__ constexpr size_t cl_part(int ng) { return (size_t)7 * 4 * ng * CPL * 4; }       // partial sums (>= 4 * 4 * ng * CPH * 4)
+static_assert((size_t)7 * 4 * CPL * 4 >= (size_t)4 * 4 * CPH * 4, "the partial sums of both products share a buffer");
+__host__ __device__ constexpr size_t cl_part_r(int ng) { return (size_t)4 * 4 * ng * CPR * 4; }     // R h
+__host__ __device__ constexpr size_t cl_smem(int ng, bool w2)
+{
+    return cl_blob_smem(w2) + 3 * cl_img(ng) /* two state halves, hidden layer */ + (size_t)4 * ng * 1024 /* logits */ + cl_part(ng) + cl_part_r(ng) +
+           (size_t)4 * ng * 2 * CU * 2 /* staged state */;
+}
 }  // namespace
 
 struct ResClPack {
-    uint8_t *d_blob = nullptr;               // [16 ranks][CB_SMEM | CB_TMEM]
+    uint8_t *d_blob = nullptr;               // [16 ranks][shared memory | tensor memory | streamed (fp32 weights)]
+    bool w2 = false;                         // fp32 weights: two fp16 parts
     long long *d_prof = nullptr;             // [16]
     int max_clusters = 0;
     float inv_R = 0.f, inv_O1[2] = {0.f, 0.f}, inv_O2[2] = {0.f, 0.f}, q_scale[2] = {0.f, 0.f};
@@ -157,6 +162,12 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
     const int c = ((p0 <= thr) + (p1 <= thr)) + ((p2 <= thr) + (p3 <= thr)) + (((p4 <= thr) + (p5 <= thr)) + ((p6 <= thr) + (p7 <= thr)));
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
 }
+__device__ __forceinline__ uint4 cl_ldg_stream(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
 // x (scaled by a power of two into the range of fp16) as high and low fp16 parts: x - high - low is at most 2^-24 |x|, half a
 // unit in the last place of fp32
@@ -171,9 +182,15 @@ __device__ __forceinline__ uint2 cl_split4(float a, float b, float c, float d, u
 // NG: groups of four rows.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
 // multiply the rows of R in the background, while the chain waits for exchanges.
-template <int NG, int MODE>
+// W2: fp32 weights, as high and low fp16 parts (error 2^-24 of a weight).  They are twice as much: the heads and the high parts of
+// nine tiles of R stay resident, the rest of R (344 KB per CTA and step) comes from L2 every step, in fragment order, straight
+// into the registers of the background warps.
+template <int NG, int MODE, bool W2>
 __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
 {
+    constexpr int NP = W2 ? 2 : 1;                                       // parts of a weight
+    constexpr size_t CB_SMEM = cl_blob_smem(W2), CS_IMG = cl_img(NG), CS_PART = cl_part(NG), CS_PARTR = cl_part_r(NG);
+    constexpr int CMAXR = 4 * NG;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
     __shared__ uint32_t s_tmem;
@@ -192,11 +209,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_u));
     const int rank = (int)rank_u;
 
-    // ---- shared memory carve-up (must match CS_BYTES)
-    const uint4 *wH[2] = {reinterpret_cast<const uint4 *>(smem + CW_HID), reinterpret_cast<const uint4 *>(smem)};                    // [half]: O3, O1
-    const uint4 *wL[2] = {reinterpret_cast<const uint4 *>(smem + 2 * CW_HID + CW_LOG), reinterpret_cast<const uint4 *>(smem + 2 * CW_HID)};
-    const uint32_t r2_addr = smem_u32(smem + 2 * CW_HID + 2 * CW_LOG);
-    const float *sI = reinterpret_cast<const float *>(smem + 2 * CW_HID + 2 * CW_LOG + CW_R2);      // [half][gate][unit][3]
+    // ---- shared memory carve-up (must match cl_smem)
+    // [half]: O3, O1 ([part][tile]); O4, O2 ([part])
+    const uint4 *wH[2] = {reinterpret_cast<const uint4 *>(smem + NP * CW_HID), reinterpret_cast<const uint4 *>(smem)};
+    const uint4 *wL[2] = {reinterpret_cast<const uint4 *>(smem + NP * (2 * CW_HID + CW_LOG)), reinterpret_cast<const uint4 *>(smem + NP * 2 * CW_HID)};
+    const uint32_t r2_addr = smem_u32(smem + NP * (2 * CW_HID + 2 * CW_LOG));
+    const float *sI = reinterpret_cast<const float *>(smem + CB_SMEM - C_SMALL * 4);               // [half][gate][unit][3]
     const float *sb1 = sI + 2 * 3 * CU * 3, *sb3 = sb1 + 32, *sb2 = sb3 + 32, *sb4 = sb2 + CL;
     uint8_t *ximg = smem + CB_SMEM;                                      // [2: coarse, fine] state image
     uint8_t *qimg = ximg + 2 * CS_IMG;
@@ -214,7 +232,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     {
-        const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM);
+        const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM + (W2 ? CB_STREAM : 0));
         const uint4 *src = reinterpret_cast<const uint4 *>(blob);
         uint4 *dst = reinterpret_cast<uint4 *>(smem);
         for (int i = tid; i < (int)(CB_SMEM / 16); i += 512) dst[i] = __ldg(src + i);
@@ -363,6 +381,58 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         }
     };
 
+    // fp32 weights: two passes over the half of the state, first the tiles that hold the coarse rows (0..3 and 4, 5), then the others
+    // (9 and 10; 6..8).  High parts of tiles 0..8 from tensor memory, the other fragments from L2, requested three or four k-tiles
+    // ahead (48 KB in flight per SM).  Tile 10 has eight rows: its high and low parts share a fragment.
+    const uint4 *stream = reinterpret_cast<const uint4 *>(p.blob + (size_t)rank * (CB_SMEM + CB_TMEM + CB_STREAM) + CB_SMEM + CB_TMEM) + (size_t)(warp & 7) * (2 * 2 * 7 * 4 * 32) + lane;
+    auto w2_pass = [&](int half_f, auto RJ_C, auto PASS_C, auto wait_fn) {
+        constexpr int RJ = decltype(RJ_C)::value, PASS = decltype(PASS_C)::value;
+        constexpr int NTM = PASS == 0 ? (RJ ? 2 : 4) : (RJ ? 3 : 0);     // tiles in tensor memory, of which the low parts are streamed
+        constexpr int NF = PASS == 0 ? NTM : 3, DEPTH = NF == 4 ? 3 : 4; // streamed fragments of a k-tile
+        constexpr int A0 = PASS == 0 ? 0 : (RJ ? 2 : 4);                 // first accumulator
+        const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
+        const uint32_t c0 = r_col + (uint32_t)(half_f * 7 * (RJ ? 20 : 16)) + (PASS && RJ ? 8 : 0);
+        const uint4 *src = stream + (size_t)((half_f * 2 + PASS) * 7) * 4 * 32;
+        uint4 f[DEPTH][NF];
+        auto request = [&](int kt) {
+#pragma unroll
+            for (int i = 0; i < NF; ++i) f[kt % DEPTH][i] = cl_ldg_stream(src + (kt * 4 + i) * 32);
+        };
+#pragma unroll
+        for (int kt = 0; kt < DEPTH; ++kt) request(kt);
+        wait_fn();
+#pragma unroll
+        for (int kt = 0; kt < 7; ++kt) {
+            uint32_t r[16];
+            if (NTM == 4) tmem_ld16(c0 + kt * 16, r);
+            else if (NTM >= 2) {
+                asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                             "=r"(r[6]), "=r"(r[7]) : "r"(c0 + kt * 20));
+                if (NTM == 3) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]) : "r"(c0 + kt * 20 + 8));
+            }
+            const uint2 b = cl_lds8(b0 + kt * 4 * QSTR);
+            tmem_wait_ld();
+#pragma unroll
+            for (int n = 0; n < NTM; ++n) cl_mma(acc[A0 + n][0], make_uint4(r[4 * n], r[4 * n + 1], r[4 * n + 2], r[4 * n + 3]), b.x, b.y);
+#pragma unroll
+            for (int i = 0; i < NF; ++i) cl_mma(acc[NTM ? A0 + i : (i == 2 ? 5 : 4)][0], f[kt % DEPTH][i], b.x, b.y);
+            if (kt + DEPTH < 7) request(kt + DEPTH);
+        }
+    };
+    auto w2_products = [&](int half_f, auto PASS_C, auto wait_fn) {
+        if (rj) w2_pass(half_f, std::integral_constant<int, 1>{}, PASS_C, wait_fn);
+        else w2_pass(half_f, std::integral_constant<int, 0>{}, PASS_C, wait_fn);
+    };
+    auto w2_store = [&](int pass) {
+        float *d = partR + (rq * 4 * NG + t4) * CPR + g4;
+#pragma unroll
+        for (int n = 0; n < 5; ++n) {
+            const bool first = rj ? n < 2 : n < 4;
+            if (first == (pass == 0)) part_sum(acc[n][0], d[(rj ? 4 + n : (n == 4 ? 9 : n)) * 16], d[(rj ? 4 + n : (n == 4 ? 9 : n)) * 16 + 8]);
+        }
+        if (pass && !rj) d[160] = (acc[5][0][0] + acc[5][0][1]) + (acc[5][0][2] + acc[5][0][3]);
+    };
+
     // ---- fixed addresses
     const uint32_t sbase = smem_u32(smem);
     uint32_t dy[2];                                                      // CTA (warp & 7) + 8 k of the cluster: what to add to an address of mine
@@ -480,8 +550,14 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     if (warp >= 8) {
         r_clear();
 #pragma unroll 1
-        for (int half_f = 0; half_f < 2; ++half_f) r_products(half_f);
-        r_store();
+        for (int half_f = 0; half_f < 2; ++half_f) {
+            if (W2) {
+                w2_products(half_f, std::integral_constant<int, 0>{}, [] {});
+                w2_products(half_f, std::integral_constant<int, 1>{}, [] {});
+            } else r_products(half_f);
+        }
+        if (W2) { w2_store(0); w2_store(1); }
+        else r_store();
     }
     if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
     __syncthreads();
@@ -527,13 +603,16 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         }
         // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
         {
-            uint4 av[7];
+            uint4 av[NP][7];
             const int tile = warp & 1, split = warp >> 1;
             const uint4 *A = wH[half] + (tile * 28 + 7 * split) * 32 + lane;
 #pragma unroll
-            for (int i = 0; i < 7; ++i) av[i] = A[i * 32];
+            for (int w = 0; w < NP; ++w)
+#pragma unroll
+                for (int i = 0; i < 7; ++i) av[w][i] = A[w * (CW_HID / 16) + i * 32];
             STAMP0();
             wait_bar(&xy[in], yuse, (int)s, 1 + 4 * half);
+            if (W2) cl_bar_arrive(half ? 5 : 7, 512);
             STAMP(8 * half + 0);
             const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
             uint2 b[NG][7];
@@ -549,7 +628,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll
             for (int i = 0; i < 7; ++i)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[grp][i & 1], av[i], b[grp][i].x, b[grp][i].y);
+                for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                    for (int w = 0; w < NP; ++w) cl_mma(acc[grp][(i + w) & 1], av[w][i], b[grp][i].x, b[grp][i].y);
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp) {
 #pragma unroll
@@ -582,14 +663,16 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 for (int k = 0; k < 4; ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
             }
         }
-        cl_bar_sync(2, 512);                 // the background warps are done with the last half-step and go on
+        cl_bar_sync(W2 && !half ? 6 : 2, 512);   // the background warps are done with the last half-step (and, bf16, go on)
         STAMP(8 * half + 2);
         // ---- the cluster's hidden layer -> this CTA's 16 logits rows, K over seven warps
         if (warp < 7) {
-            uint4 lv[4];
+            uint4 lv[NP][4];
             const uint4 *A = wL[half] + 4 * warp * 32 + lane;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) lv[i] = A[i * 32];
+            for (int w = 0; w < NP; ++w)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) lv[w][i] = A[w * (CW_LOG / 16) + i * 32];
             const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + 4 * (lane & 3));
             wait_bar(&xq, quse, (int)s, 2 + 4 * half);
             STAMP(8 * half + 3);
@@ -607,7 +690,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[grp][i & 1], lv[i], b[grp][i].x, b[grp][i].y);
+                for (int grp = 0; grp < NG; ++grp)
+#pragma unroll
+                    for (int w = 0; w < NP; ++w) cl_mma(acc[grp][(i + w) & 1], lv[w][i], b[grp][i].x, b[grp][i].y);
 #pragma unroll
             for (int grp = 0; grp < NG; ++grp) {
 #pragma unroll
@@ -689,12 +774,27 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll 1
         for (long long s2 = 0; s2 < T; ++s2) {
             r_clear();
-            cl_bar_sync(2, 512);
-            r_products(0);
-            cl_bar_sync(2, 512);
-            r_products(1);
-            r_store();
-            cl_bar_arrive(4, 256 + n_draw);
+            if (W2) {
+                // More to do: it starts as soon as the half of the state is there (barriers 5 and 7, at which the chain only arrives), and
+                // the coarse rows come first, the others when the gates have theirs.  Barriers 2 and 6, at which these warps only
+                // arrive, tell the chain that the products of the last half-step are done.  Both alternate: whoever only arrives may
+                // be one half-step ahead of the others, and cannot be two, because the other pair of barriers lies between.
+                auto go = [](int done, int start) { return [done, start] { cl_bar_arrive(done, 512); cl_bar_sync(start, 512); }; };
+                w2_products(0, std::integral_constant<int, 0>{}, go(2, 5));
+                w2_products(0, std::integral_constant<int, 1>{}, [] {});
+                w2_products(1, std::integral_constant<int, 0>{}, go(6, 7));
+                w2_store(0);
+                cl_bar_arrive(4, 256 + n_draw);
+                w2_products(1, std::integral_constant<int, 1>{}, [] {});
+                w2_store(1);
+            } else {
+                cl_bar_sync(2, 512);
+                r_products(0);
+                cl_bar_sync(2, 512);
+                r_products(1);
+                r_store();
+                cl_bar_arrive(4, 256 + n_draw);
+            }
         }
     }
 #undef STAMP
@@ -718,18 +818,19 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 }
 
 // ---------------------------------------------------------------------------------------------
-static const void *cl_kernel_of(int nr, bool dbg)
+static const void *cl_kernel_of(int nr, bool dbg, bool w2)
 {
-    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1> : (const void *)resident_cluster_kernel<1, 0>;
-    return dbg ? (const void *)resident_cluster_kernel<2, 1> : (const void *)resident_cluster_kernel<2, 0>;
+    if (w2) return dbg ? (const void *)resident_cluster_kernel<1, 1, true> : (const void *)resident_cluster_kernel<1, 0, true>;
+    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1, false> : (const void *)resident_cluster_kernel<1, 0, false>;
+    return dbg ? (const void *)resident_cluster_kernel<2, 1, false> : (const void *)resident_cluster_kernel<2, 0, false>;
 }
 
-static void cl_fill_launch(int n_clusters, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
+static void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
 {
     std::memset(cfg, 0, sizeof(*cfg));
     cfg->gridDim = dim3(n_clusters * CCS);
     cfg->blockDim = dim3(512);
-    cfg->dynamicSmemBytes = CS_BYTES;
+    cfg->dynamicSmemBytes = smem;
     cfg->stream = s;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CCS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -741,23 +842,71 @@ static void cl_fill_launch(int n_clusters, cudaLaunchConfig_t *cfg, cudaLaunchAt
 // clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
 static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
 {
-    const int most = k.max_clusters * CMAXR, waves = (batch + most - 1) / most;
+    const int most = k.max_clusters * (k.w2 ? 4 : 8), waves = (batch + most - 1) / most;
     *nr = (batch + waves * k.max_clusters - 1) / (waves * k.max_clusters);
     const int need = (batch + *nr - 1) / *nr;
     *n_clusters = need < CNC ? CNC : need;       // (a cluster without rows returns at once)
 }
 
+// fp32 -> fp16 bits, to nearest even (finite values below 2^15 keep their range here; infinities and NaNs stay what they are)
+static uint16_t half_bits(float v)
+{
+    uint32_t u;
+    std::memcpy(&u, &v, 4);
+    const uint32_t sign = (u >> 16) & 0x8000u, a = u & 0x7fffffffu;
+    if (a >= 0x7f800000u) return (uint16_t)(sign | (a > 0x7f800000u ? 0x7e00u : 0x7c00u));
+    if (a >= 0x38800000u) return (uint16_t)(sign | std::min(((a + 0xfffu + ((a >> 13) & 1u)) >> 13) - (112u << 10), 0x7c00u));
+    float f;
+    std::memcpy(&f, &a, 4);
+    f += 0.5f;                                   // the last bit of 0.5 is the subnormal step of fp16
+    std::memcpy(&u, &f, 4);
+    return (uint16_t)(sign | (u - 0x3f000000u));
+}
+static float half_value(uint16_t h)
+{
+    const uint32_t e = (h >> 10) & 31u, mant = h & 0x3ffu;
+    const float v = e == 31u ? (mant ? NAN : INFINITY) : e ? std::ldexp((float)(mant | 0x400u), (int)e - 25) : std::ldexp((float)mant, -24);
+    return h & 0x8000u ? -v : v;
+}
+// A dense matrix as one or two fp16 parts, scaled by 2^(14 - exp)
+struct HalfMatrix {
+    int exp = 0;
+    std::vector<uint16_t> part[2];
+    HalfMatrix(const BsrHost &M, int np)
+    {
+        float top = 0.f;
+        for (float v : M.vals) top = std::max(top, std::fabs(v));
+        exp = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+        const float scale = std::ldexp(1.f, 14 - exp);
+        const size_t cols = (size_t)M.cols4 * 4;
+        for (int w = 0; w < np; ++w) part[w].assign((size_t)M.rows4 * 4 * cols, 0);
+        for (int br = 0; br < M.rows4; ++br)
+            for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
+                for (int r = 0; r < 4; ++r) {
+                    const float *src = &M.vals[(size_t)b * 16 + 4 * r];
+                    const size_t o = (size_t)(4 * br + r) * cols + 4 * M.col[b];
+                    for (int c = 0; c < 4; ++c) {
+                        const float x = src[c] * scale;
+                        part[0][o + c] = half_bits(x);
+                        if (np == 2) part[1][o + c] = half_bits(x - half_value(part[0][o + c]));
+                    }
+                }
+    }
+};
+
 int rescl_prepare(wrnn_model *m)
 {
     const int H = m->H;
-    if (m->dtype != WRNN_BF16 || m->sparse || m->variant != 0 || H != 2 * CK) { m->err = "cluster-resident kernel: dense bf16 H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
+    if (m->sparse || m->variant != 0 || H != 2 * CK) { m->err = "cluster-resident kernel: dense H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
     cudaDeviceProp prop;
     cudaGetDeviceProperties(&prop, m->device);
     ResClPack k;
+    k.w2 = m->dtype == WRNN_F32;
     cudaFuncAttributes fa;
     for (int nr : {1, 5})
         for (int dbg = 0; dbg < 2; ++dbg) {
-            const void *f = cl_kernel_of(nr, dbg != 0);
+            const void *f = cl_kernel_of(nr, dbg != 0, k.w2);
+            const size_t CS_BYTES = cl_smem(nr > 4 && !k.w2 ? 2 : 1, k.w2);
             if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || CS_BYTES + fa.sharedSizeBytes > prop.sharedMemPerBlockOptin ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS_BYTES) != cudaSuccess) {
@@ -766,38 +915,28 @@ int rescl_prepare(wrnn_model *m)
         }
     {
         cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-        cl_fill_launch(CNC, &cfg, at, 0);
-        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(1, false), &cfg) != cudaSuccess || k.max_clusters < 1) {
+        cl_fill_launch(CNC, cl_smem(k.w2 ? 1 : 2, k.w2), &cfg, at, 0);
+        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.w2 ? 1 : 5, false, k.w2), &cfg) != cudaSuccess || k.max_clusters < 1) {
             cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
         }
     }
     // fp16 weights, every matrix scaled by a power of two to at most 2^14: the eight bits of a bf16 weight are kept unless it is
-    // below 2^-28 of the largest one, where at most 2^-39 of that is lost
-    auto to_half = [](const BsrHost &M, int *exp) {
-        const std::vector<uint16_t> b = dense_bf16_bits(M);
-        auto value = [](uint16_t v) { const uint32_t u = (uint32_t)v << 16; float f; std::memcpy(&f, &u, 4); return f; };
-        float top = 0.f;
-        for (uint16_t v : b) top = std::max(top, std::fabs(value(v)));
-        *exp = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
-        const float scale = std::ldexp(1.f, 14 - *exp);
-        std::vector<uint16_t> h(b.size());
-        for (size_t i = 0; i < b.size(); ++i) { const __half x = __float2half_rn(value(b[i]) * scale); std::memcpy(&h[i], &x, 2); }
-        return h;
-    };
-    int e[5];
-    const std::vector<uint16_t> dR = to_half(m->hR, &e[0]), dO[4] = {to_half(m->hO1, &e[1]), to_half(m->hO3, &e[2]), to_half(m->hO2, &e[3]), to_half(m->hO4, &e[4])};
+    // below 2^-28 of the largest one, where at most 2^-39 of that is lost; fp32 weights as two parts (2^-24 of a weight)
+    const int NP = k.w2 ? 2 : 1;
+    HalfMatrix R(m->hR, NP), O[4] = {{m->hO1, NP}, {m->hO3, NP}, {m->hO2, NP}, {m->hO4, NP}};
+    const int e[5] = {R.exp, O[0].exp, O[1].exp, O[2].exp, O[3].exp};
     // products of operands scaled by 2^(14 - exponent) each
     k.inv_R = std::ldexp(1.f, e[0] - 28);
     for (int h = 0; h < 2; ++h) {
         // |hidden value| <= sum |O1 row| + |b1| for a state below one (the kernel takes a larger initial state into account)
-        const BsrHost &O = h ? m->hO3 : m->hO1;
+        const BsrHost &M = h ? m->hO3 : m->hO1;
         const std::vector<float> &bias = h ? m->hb3 : m->hb1;
         float top = 0.f;
-        for (int br = 0; br < O.rows4; ++br)
+        for (int br = 0; br < M.rows4; ++br)
             for (int r = 0; r < 4; ++r) {
                 float sum = std::fabs(bias[4 * br + r]);
-                for (int b = O.row_ptr[br]; b < O.row_ptr[br + 1]; ++b)
-                    for (int c = 0; c < 4; ++c) sum += std::fabs(O.vals[(size_t)b * 16 + 4 * r + c]);
+                for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
+                    for (int c = 0; c < 4; ++c) sum += std::fabs(M.vals[(size_t)b * 16 + 4 * r + c]);
                 top = std::max(top, sum);
             }
         const int eq = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
@@ -805,31 +944,39 @@ int rescl_prepare(wrnn_model *m)
         k.q_scale[h] = std::ldexp(1.f, 14 - eq);
         k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);
     }
-    std::vector<uint8_t> blob(CCS * (CB_SMEM + CB_TMEM), 0);
-    // row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
-    auto r_row = [&](int rank, int i) { return &dR[((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
-    // A fragments of 16 rows (row r < n_rows, zero otherwise): lane (g, t) holds rows g, g + 8 at k 4t, 4t + 1, then at 4t + 2, 4t + 3 (the permuted k order)
+    const size_t smem_bytes = cl_blob_smem(k.w2), cta_bytes = smem_bytes + CB_TMEM + (k.w2 ? CB_STREAM : 0);
+    std::vector<uint8_t> blob(CCS * cta_bytes, 0);
+    // part w of row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
+    auto r_row = [&](int rank, int w, int i) { return &R.part[w][((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
+    // one row (g of a fragment's upper or lower eight) of the A fragment of a k-tile: lane (g, t) holds it at k 4t, 4t + 1 and at
+    // 4t + 2, 4t + 3 (the permuted k order), registers `lower` and 2 + `lower`
+    auto frag_row = [](uint16_t *frag, int g, int lower, const uint16_t *src) {
+        for (int t = 0; t < 4; ++t) {
+            uint16_t *d = frag + (4 * g + t) * 8 + 2 * lower;
+            d[0] = src[4 * t]; d[1] = src[4 * t + 1]; d[4] = src[4 * t + 2]; d[5] = src[4 * t + 3];
+        }
+    };
     auto pack = [&](const std::vector<uint16_t> &M, int first, int n_rows, uint16_t *dst) {
-        for (int kt = 0; kt < 28; ++kt)
-            for (int lane = 0; lane < 32; ++lane)
-                for (int q = 0; q < 4; ++q) {
-                    const int r = (lane >> 2) + 8 * (q & 1), c = 4 * (lane & 3) + 2 * (q >> 1);
-                    for (int j = 0; j < 2; ++j) dst[((size_t)kt * 32 + lane) * 8 + 2 * q + j] = r < n_rows ? M[(size_t)(first + r) * CK + 16 * kt + c + j] : 0;
-                }
+        for (int r = 0; r < n_rows; ++r)
+            for (int kt = 0; kt < 28; ++kt) frag_row(dst + (size_t)kt * 256, r & 7, r >> 3, &M[(size_t)(first + r) * CK + 16 * kt]);
     };
     for (int rank = 0; rank < CCS; ++rank) {
-        uint8_t *base = blob.data() + (size_t)rank * (CB_SMEM + CB_TMEM);
-        for (int h = 0; h < 2; ++h) {
-            for (int t = 0; t < 2; ++t) pack(dO[h], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + h * CW_HID + (size_t)t * 28 * 512));
-            pack(dO[2 + h], CL * rank, CL, reinterpret_cast<uint16_t *>(base + 2 * CW_HID + h * CW_LOG));
-        }
-        uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
-        for (int i = 0; i < CRS; ++i)
-            for (int k8 = 0; k8 < 2 * CK8; ++k8) {
-                const uint16_t *src = r_row(rank, 16 * CRT + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
-                for (int e = 0; e < 8; ++e) r2[((size_t)k8 * CRS + i) * 8 + e] = src[4 * (e >> 1) + (e & 1)];
+        uint8_t *base = blob.data() + (size_t)rank * cta_bytes;
+        for (int h = 0; h < 2; ++h)
+            for (int w = 0; w < NP; ++w) {
+                for (int t = 0; t < 2; ++t)
+                    pack(O[h].part[w], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + (h * NP + w) * CW_HID + (size_t)t * 28 * 512));
+                pack(O[2 + h].part[w], CL * rank, CL, reinterpret_cast<uint16_t *>(base + NP * 2 * CW_HID + (h * NP + w) * CW_LOG));
             }
-        float *sm = reinterpret_cast<float *>(base + 2 * CW_HID + 2 * CW_LOG + CW_R2);
+        if (!k.w2) {
+            uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
+            for (int i = 0; i < CRS; ++i)
+                for (int k8 = 0; k8 < 2 * CK8; ++k8) {
+                    const uint16_t *src = r_row(rank, 0, 16 * CRT + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
+                    for (int c = 0; c < 8; ++c) r2[((size_t)k8 * CRS + i) * 8 + c] = src[4 * (c >> 1) + (c & 1)];
+                }
+        }
+        float *sm = reinterpret_cast<float *>(base + smem_bytes - C_SMALL * 4);
         for (int i = 0; i < 6 * CU; ++i) {
             const size_t row = (size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU;
             for (int c = 0; c < 3; ++c) sm[i * 3 + c] = m->hI[row * 3 + c];
@@ -838,10 +985,10 @@ int rescl_prepare(wrnn_model *m)
         for (int r = 0; r < CU; ++r) { b[r] = m->hb1[CU * rank + r]; b[32 + r] = m->hb3[CU * rank + r]; }
         for (int r = 0; r < CL; ++r) { b[64 + r] = m->hb2[CL * rank + r]; b[64 + CL + r] = m->hb4[CL * rank + r]; }
         // tensor memory: lane quadrant q holds quarter q of the k-tiles of both halves of the state; columns as the kernel states them
-        uint16_t *tm = reinterpret_cast<uint16_t *>(base + CB_SMEM);
+        uint16_t *tm = reinterpret_cast<uint16_t *>(base + smem_bytes);
         for (int i = 0; i < 16 * CRT; ++i) {
             const int tile = i >> 4, reg0 = (i >> 3) & 1;
-            const uint16_t *src = r_row(rank, i);
+            const uint16_t *src = r_row(rank, 0, i);
             for (int kt = 0; kt < 56; ++kt) {
                 const int half_f = kt / 28, q = kt % 28 / 7, k7 = kt % 7;
                 const int c0 = tile < 4 ? (half_f * 7 + k7) * 16 + 4 * tile : 2 * 7 * 16 + (half_f * 7 + k7) * 20 + 4 * (tile - 4);
@@ -850,6 +997,27 @@ int rescl_prepare(wrnn_model *m)
                         std::memcpy(tm + ((size_t)(c0 + reg0 + 2 * h) * 128 + 32 * q + 4 * (i & 7) + t) * 2, src + 16 * kt + 4 * t + 2 * h, 4);
             }
         }
+        if (!k.w2) continue;
+        // streamed fragments of warp w8 = 4 j + q: pass 0 the low parts of tiles 0..3 (j = 0) or 4, 5; pass 1 tile 9 (both parts) and
+        // tile 10 (high parts over low parts), or the low parts of tiles 6..8
+        uint16_t *st = reinterpret_cast<uint16_t *>(base + smem_bytes + CB_TMEM);
+        for (int w8 = 0; w8 < 8; ++w8)
+            for (int half_f = 0; half_f < 2; ++half_f)
+                for (int pass = 0; pass < 2; ++pass)
+                    for (int k7 = 0; k7 < 7; ++k7)
+                        for (int f = 0; f < 4; ++f) {
+                            const int j = w8 >> 2, kt = 28 * half_f + 7 * (w8 & 3) + k7;
+                            if (f >= (pass ? 3 : j ? 2 : 4)) continue;
+                            uint16_t *frag = st + ((((size_t)(w8 * 2 + half_f) * 2 + pass) * 7 + k7) * 4 + f) * 256;
+                            for (int r = 0; r < 16; ++r) {
+                                int row, w = 1;
+                                if (!pass) row = 16 * (j ? 4 + f : f) + r;
+                                else if (j) row = 16 * (6 + f) + r;
+                                else if (f < 2) { row = 144 + r; w = f; }
+                                else { row = 160 + (r & 7); w = r >> 3; }
+                                frag_row(frag, r & 7, r >> 3, r_row(rank, w, row) + 16 * kt);
+                            }
+                        }
     }
     ResClPack *pk = new ResClPack(k);
     if (cudaMalloc((void **)&pk->d_blob, blob.size()) != cudaSuccess || cudaMemcpy(pk->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -883,8 +1051,8 @@ int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thread
     cl_geometry(*m->rescl, batch, &nr, &n_clusters);
     if (n_ctas) *n_ctas = n_clusters * CCS;
     if (n_threads) *n_threads = 512;
-    if (smem) *smem = (int)CS_BYTES;
-    if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(2 * CW_HID + 2 * CW_LOG + CW_R2 + CB_TMEM);
+    if (smem) *smem = (int)cl_smem(nr > 4 ? 2 : 1, m->rescl->w2);
+    if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(cl_blob_smem(m->rescl->w2) + CB_TMEM + (m->rescl->w2 ? CB_STREAM : 0));
     return WRNN_OK;
 }
 
@@ -915,9 +1083,9 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.dbg_gates || p.dbg_h || p.dbg_logits;
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-    cl_fill_launch(n_clusters, &cfg, at, s);
+    cl_fill_launch(n_clusters, cl_smem(nr > 4 ? 2 : 1, k.w2), &cfg, at, s);
     void *args[] = {&p};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg, k.w2), args);
     if (e != cudaSuccess) {
         m->err = std::string("cluster-resident kernel launch failed: ") + cudaGetErrorString(e);
         cudaGetLastError();
