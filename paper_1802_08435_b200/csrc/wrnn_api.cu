@@ -132,15 +132,16 @@ static bool use_reslean(const wrnn_model *m, int batch)
 
 // Rows of a dense bf16 H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
 // clusters of eight) and more in waves; the cluster-partitioned kernel takes all at once and costs almost the same whatever
-// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 10.1 / 25.2, 112: 20.2 / 25.8, 128: 26.3 /
-// 27.7, 150: 28.4 / 28.3, 256: 47 / 32.3.
+// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 7.1 / 25.2, 57: 12.5 / 25.3, 112: 14.3 / 25.8,
+// 168: 21.3 / 28.7, 224: 28.4 / 31.0, 256 (a fifth wave): 35.5 / 32.3.
+constexpr int RESCL_BF16_ROWS = 224;
 static bool use_rescl(const wrnn_model *m, int batch)
 {
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
     const char *off = getenv(batch == 1 ? "WRNN_RESIDENT_LEAN" : "WRNN_NO_MULTI");
     if (off && off[0] == (batch == 1 ? '0' : '1')) return false;
     // (fp32 weights: 28 rows at a time; the any-shape kernel, the other one for several rows, takes 55 us per step at four)
-    return (m->dtype == WRNN_F32 || batch <= 128) && rescl_supported(m, batch) == WRNN_OK;
+    return (m->dtype == WRNN_F32 || batch <= RESCL_BF16_ROWS) && rescl_supported(m, batch) == WRNN_OK;
 }
 
 static bool use_resf32(const wrnn_model *m, int batch)
@@ -150,23 +151,13 @@ static bool use_resf32(const wrnn_model *m, int batch)
 }
 
 // two or four streams of a dense bf16 model: pairs on the two-stream form of the resident kernel, one pair after the other
-// (the fallback of the multi-stream resident kernel, which takes 2 to 16 rows where the model has one)
+// (WRNN_NO_MULTI=1: the cluster-resident kernel takes the rows otherwise)
 static bool use_pair(const wrnn_model *m, int batch)
 {
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
     const char *off = getenv("WRNN_NO_PAIR");
     if (off && off[0] == '1') return false;
     return m->variant == 0 && resident_pair_supported(m, batch) == WRNN_OK;
-}
-
-// 2 to 16 lock-step streams of a dense bf16 H = 896 model: all of them in one launch on the resident weights
-// (WRNN_NO_MULTI=1 falls back to the two-stream and cluster-partitioned kernels: diagnostic)
-static bool use_multi(const wrnn_model *m, int batch)
-{
-    if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
-    const char *off = getenv("WRNN_NO_MULTI");
-    if (off && off[0] == '1') return false;
-    return m->variant == 0 && resmulti_supported(m, batch) == WRNN_OK;
 }
 
 static bool use_sparse(const wrnn_model *m, int batch)
@@ -242,7 +233,6 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     if (use_rescl(m, a.batch)) return rescl_run(m, a, s);
     // staggered rows: the cluster-partitioned kernel, else the any-shape kernel
     if (a.row_lag > 0) {
-        if (a.batch >= 2 && use_multi(m, a.batch)) return resmulti_run(m, a, s);
         if (a.batch >= 2 && use_bcluster(m, a.batch)) return bcluster_run(m, a, s);
         if (a.batch == 1 && use_reslean(m, 1)) return reslean_run(m, a, s);           // a lone row (the ramps of the schedule)
         if (a.batch == 1 && use_resident(m, 1)) return resident_run(m, a, s);
@@ -250,9 +240,6 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     }
     if (use_reslean(m, a.batch)) return reslean_run(m, a, s);
     if (use_resident(m, a.batch)) return resident_run(m, a, s);
-    // 2 to 16 rows: the multi-stream kernel (two rows 6.5 us per lock-step against 7.7 on the two-stream kernel, which serves
-    // them where the multi-stream kernel does not apply or under WRNN_NO_MULTI=1)
-    if (use_multi(m, a.batch)) return resmulti_run(m, a, s);
     if (use_pair(m, a.batch)) {
         for (int pair = 0; pair < a.batch / 2; ++pair) {
             rc = resident_pair_run(m, a, pair, s);
@@ -424,7 +411,17 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "sparse cluster kernel unavailable: " + why);
         }
     }
-    if (p->kernel == WRNN_KERNEL_AUTO || p->kernel == WRNN_KERNEL_BCLUSTER) {
+    // Only kernels that some call can reach are packed.  The cluster-resident kernel takes every row count of an fp32 model and up
+    // to 224 rows of a bf16 one; the first forms serve models it does not take and the two diagnostic switches.
+    const char *no_lean = getenv("WRNN_RESIDENT_LEAN"), *no_multi = getenv("WRNN_NO_MULTI");
+    const bool first_forms = (no_lean && no_lean[0] == '0') || (no_multi && no_multi[0] == '1');
+    const bool any = p->kernel == WRNN_KERNEL_AUTO;
+    if (any || p->kernel == WRNN_KERNEL_RESIDENT) {
+        if (m->dtype == WRNN_BF16) reslean_prepare(m);                  // only the checked build (WRNN_DEBUG=1), which then takes the single stream
+        if (!reslean_checked(m)) rescl_prepare(m);
+    }
+    const bool all_rows = m->rescl && !first_forms && (m->dtype == WRNN_F32 || max_batch <= RESCL_BF16_ROWS);
+    if (p->kernel == WRNN_KERNEL_BCLUSTER || (any && !all_rows)) {
         const int rc = bcluster_prepare(m);
         if (rc != WRNN_OK && p->kernel == WRNN_KERNEL_BCLUSTER) {
             const std::string why = m->err;
@@ -432,7 +429,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "cluster-partitioned kernel unavailable: " + why);
         }
     }
-    if (p->kernel == WRNN_KERNEL_AUTO || p->kernel == WRNN_KERNEL_BATCHED) {
+    if (p->kernel == WRNN_KERNEL_BATCHED || (any && !all_rows && !m->bcluster)) {
         const int rc = batched_prepare(m);
         if (rc != WRNN_OK && p->kernel == WRNN_KERNEL_BATCHED) {
             const std::string why = m->err;
@@ -440,16 +437,13 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "batched kernel unavailable: " + why);
         }
     }
-    if (p->kernel == WRNN_KERNEL_AUTO || p->kernel == WRNN_KERNEL_RESIDENT) {
+    if ((any || p->kernel == WRNN_KERNEL_RESIDENT) && (!m->rescl || first_forms)) {
         const int rc = m->dtype == WRNN_F32 ? resf32_prepare(m) : resident_prepare(m);
         if (rc != WRNN_OK && p->kernel == WRNN_KERNEL_RESIDENT) {
             const std::string why = m->err;
             wrnn_destroy(m);
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
-        if (m->dtype == WRNN_BF16 && m->variant == 0) reslean_prepare(m);                        // optional: the row-split resident kernel serves the stream without it
-        if (m->variant == 0 && !reslean_checked(m)) rescl_prepare(m);
-        if (m->dtype == WRNN_BF16 && m->variant == 0 && max_batch >= 2) resmulti_prepare(m);   // optional: other kernels serve the batch without it
     }
     m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call
     noalloc_warm(dev);
@@ -465,7 +459,6 @@ void wrnn_destroy(wrnn_model *m)
     resident_destroy(m);
     reslean_destroy(m);
     resf32_destroy(m);
-    resmulti_destroy(m);
     rescl_destroy(m);
     batched_destroy(m);
     bcluster_destroy(m);
@@ -651,7 +644,7 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
         if (rc != WRNN_OK) return fail(m, rc, "conditioning launch failed");
         // rows advance together on the multi-stream resident kernel where the model has one; without it up to three rows go
         // one after the other through the single-stream kernel
-        const int group = (n_rows >= 2 && (use_rescl(m, n_rows) || use_multi(m, n_rows))) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
+        const int group = (n_rows >= 2 && use_rescl(m, n_rows)) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
         for (int b0 = 0; b0 < n_rows; b0 += group) {
             const int r0 = r_a + b0;
             const long long p0 = p_lo - (long long)b0 * lag;
@@ -736,7 +729,7 @@ int wrnn_subscale_net_rows(wrnn_model *m, wrnn_subscale_net *net, const float *f
     float *v = reinterpret_cast<float *>(m->sub_scratch);
     int rc = subnet_run(net, hist, frames, n_frames, hop, L, r_lo, n_rows, p_lo, lag, n_steps, v, m->wait_limit_ns(), s);
     if (rc != WRNN_OK) return fail(m, rc, "conditioning launch failed");
-    const int group = (n_rows >= 2 && (use_rescl(m, n_rows) || use_multi(m, n_rows))) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
+    const int group = (n_rows >= 2 && use_rescl(m, n_rows)) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
     for (int b0 = 0; b0 < n_rows; b0 += group) {
         const int r0 = r_lo + b0;
         const long long p0 = p_lo - (long long)b0 * lag;
@@ -862,10 +855,6 @@ int wrnn_launch_info(wrnn_model *m, int32_t batch, int32_t *kernel, int32_t *n_c
         if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
         return resident_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
     }
-    if (use_multi(m, batch)) {
-        if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
-        return resmulti_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
-    }
     if (use_pair(m, batch)) {
         if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
         return resident_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
@@ -915,15 +904,12 @@ int wrnn_phase_names(wrnn_model *m, char *buf, int32_t cap)
     const char *first = "F.wait_y,F.hid_finish_send,F.wait_q,F.log_finish_send,F.wait_logits,F.draw_gates,"
                         "C.wait_y,C.hid_finish_send,C.wait_q,C.log_finish_send,C.wait_logits,C.draw_gates,"
                         "F.hid_products,C.hid_products,F.log_products,C.log_products";
-    const char *multi = "F.wait_y,F.hid_finish_send,F.wait_q,F.log_finish_send,F.wait_logits,F.draw_wait_recurrent,"
-                        "C.wait_y,C.hid_finish_send,C.wait_q,C.log_finish_send,C.wait_logits,C.draw_wait_recurrent,"
-                        "F.hid_products,C.hid_products,F.log_products,C.log_products";
     const char *lean = "F.wait_y,F.hid_products,F.hid_sums_send,F.recurrent_products,F.rsums_gateprep,F.wait_logit_rows_send,F.wait_logits,F.draw_gates,"
                        "C.wait_y,C.hid_products,C.hid_sums_send,C.recurrent_products,C.rsums_gateprep,C.wait_logit_rows_send,C.wait_logits,C.draw_gates";
     // per half: warp 0 of CTA 0 (wait, products, sums and sends), then its first drawing warp
     const char *cl = "F.wait_y,F.hid_products,F.hid_sums_send,F.wait_q,F.log_products,F.log_sums_send,F.draw,F.gates,"
                      "C.wait_y,C.hid_products,C.hid_sums_send,C.wait_q,C.log_products,C.log_sums_send,C.draw,C.gates";
-    const char *src = m->prof_cl ? cl : (!m->resf32 && m->prof_multi) ? multi : (!m->resf32 && m->prof_lean) ? lean : first;
+    const char *src = m->prof_cl ? cl : (!m->resf32 && m->prof_lean) ? lean : first;
     std::snprintf(buf, (size_t)cap, "%s", src);
     return WRNN_OK;
 }
@@ -934,7 +920,6 @@ int wrnn_phase_cycles(wrnn_model *m, int64_t *out16)
     static_assert(sizeof(long long) == sizeof(int64_t), "");
     if (m->prof_cl) return rescl_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->resf32) return resf32_phase_cycles(m, reinterpret_cast<long long *>(out16));
-    if (m->prof_multi) return resmulti_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->prof_lean) return reslean_phase_cycles(m, reinterpret_cast<long long *>(out16));
     return resident_phase_cycles(m, reinterpret_cast<long long *>(out16));
 }

@@ -63,7 +63,6 @@ struct BatchedPack;    // fragment-packed weights and activation images of the b
 struct SparsePack;     // compressed block rows of the single-cluster block-sparse kernel (opaque here)
 struct ResF32Pack;     // per-CTA fp32 weight shards of the single-stream fp32 resident kernel (opaque here)
 struct ResLeanPack;      // per-CTA weights of the lean single-stream resident kernel (opaque here)
-struct ResMultiPack;  // per-CTA weights of the multi-stream resident kernel (opaque here)
 struct ResClPack;      // per-CTA weights of the cluster-resident kernel (opaque here)
 struct BcPack;         // per-CTA weight slices and stacked activation images of the cluster-partitioned multi-row kernel
 
@@ -104,7 +103,6 @@ struct wrnn_model {
     wrnn::ResLeanPack *reslean = nullptr;
     bool prof_lean = false;           // the last call with phase timing ran on the lean single-stream resident kernel
     wrnn::ResF32Pack *resf32 = nullptr;
-    wrnn::ResMultiPack *resmulti = nullptr;
     wrnn::ResClPack *rescl = nullptr;
     bool prof_cl = false;             // the last call with phase timing ran on the cluster-resident kernel
     // wrnn_selftest_lost_word: bound of every device-side wait (0 = the default of two seconds) and the CTA / step whose
@@ -114,7 +112,6 @@ struct wrnn_model {
     long long dbg_skip_step = -1;
     unsigned long long wait_limit_ns() const { return dbg_limit_ns ? dbg_limit_ns : 2000000000ull; }
     bool prof_enabled = false;      // wrnn_phase_profile: the resident kernels stamp their phases
-    bool prof_multi = false;        // the last call with phase timing ran on the multi-stream resident kernel
     wrnn::BatchedPack *batched = nullptr;
     wrnn::SparsePack *sparse_pack = nullptr;
     wrnn::BcPack *bcluster = nullptr;
@@ -186,15 +183,7 @@ int reslean_launch_info(const wrnn_model *m, int *n_ctas, int *n_threads, int *s
 int reslean_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int reslean_phase_cycles(const wrnn_model *m, long long *out16);
 
-// wrnn_resmulti.cu: 2 to 16 lock-step streams of a dense bf16 H = 896 model on resident weights
-int resmulti_supported(const wrnn_model *m, int batch);
-int resmulti_prepare(wrnn_model *m);
-void resmulti_destroy(wrnn_model *m);
-int resmulti_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
-int resmulti_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
-int resmulti_phase_cycles(const wrnn_model *m, long long *out16);
-
-// wrnn_rescl.cu: rows of a dense bf16 H = 896 model, the whole model in one cluster (R in tensor memory)
+// wrnn_rescl.cu: rows of a dense H = 896 model (bf16 or fp32), the whole model in one cluster (R in tensor memory)
 int rescl_supported(const wrnn_model *m, int batch);
 int rescl_prepare(wrnn_model *m);
 void rescl_destroy(wrnn_model *m);

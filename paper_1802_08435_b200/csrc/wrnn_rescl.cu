@@ -70,6 +70,8 @@ __host__ __device__ constexpr size_t cl_smem(int ng, bool w2)
     return cl_blob_smem(w2) + 3 * cl_img(ng) /* two state halves, hidden layer */ + (size_t)4 * ng * 1024 /* logits */ + cl_part(ng) + cl_part_r(ng) +
            (size_t)4 * ng * 2 * CU * 2 /* staged state */;
 }
+// what a launch asks for: the larger form of a weight type (one CTA per SM either way)
+size_t cl_launch_smem(bool w2) { return cl_smem(w2 ? 1 : 2, w2); }
 }  // namespace
 
 struct ResClPack {
@@ -906,7 +908,7 @@ int rescl_prepare(wrnn_model *m)
     for (int nr : {1, 5})
         for (int dbg = 0; dbg < 2; ++dbg) {
             const void *f = cl_kernel_of(nr, dbg != 0, k.w2);
-            const size_t CS_BYTES = cl_smem(nr > 4 && !k.w2 ? 2 : 1, k.w2);
+            const size_t CS_BYTES = cl_launch_smem(k.w2);
             if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || CS_BYTES + fa.sharedSizeBytes > prop.sharedMemPerBlockOptin ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS_BYTES) != cudaSuccess) {
@@ -915,7 +917,7 @@ int rescl_prepare(wrnn_model *m)
         }
     {
         cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-        cl_fill_launch(CNC, cl_smem(k.w2 ? 1 : 2, k.w2), &cfg, at, 0);
+        cl_fill_launch(CNC, cl_launch_smem(k.w2), &cfg, at, 0);
         if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.w2 ? 1 : 5, false, k.w2), &cfg) != cudaSuccess || k.max_clusters < 1) {
             cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
         }
@@ -1051,7 +1053,7 @@ int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thread
     cl_geometry(*m->rescl, batch, &nr, &n_clusters);
     if (n_ctas) *n_ctas = n_clusters * CCS;
     if (n_threads) *n_threads = 512;
-    if (smem) *smem = (int)cl_smem(nr > 4 ? 2 : 1, m->rescl->w2);
+    if (smem) *smem = (int)cl_launch_smem(m->rescl->w2);
     if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(cl_blob_smem(m->rescl->w2) + CB_TMEM + (m->rescl->w2 ? CB_STREAM : 0));
     return WRNN_OK;
 }
@@ -1083,7 +1085,7 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.dbg_gates || p.dbg_h || p.dbg_logits;
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-    cl_fill_launch(n_clusters, cl_smem(nr > 4 ? 2 : 1, k.w2), &cfg, at, s);
+    cl_fill_launch(n_clusters, cl_launch_smem(k.w2), &cfg, at, s);
     void *args[] = {&p};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg, k.w2), args);
     if (e != cudaSuccess) {

@@ -569,6 +569,7 @@ int resf32_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
+    m->prof_cl = false;
     return WRNN_OK;
 }
 

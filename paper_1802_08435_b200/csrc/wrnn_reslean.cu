@@ -575,6 +575,7 @@ int reslean_prepare(wrnn_model *m)
     cudaGetDeviceProperties(&prop, m->device);
     if (k.NCTA > m->n_sms || (size_t)k.smem_bytes > prop.sharedMemPerBlockOptin) { m->err = "lean resident kernel does not fit this device"; return WRNN_ERR_UNSUPPORTED; }
     { const char *d = getenv("WRNN_DEBUG"); k.checked = d && d[0] == '1'; }
+    if (!fused && !k.checked) { m->err = "lean resident kernel: a plain model runs on the cluster-resident kernel"; return WRNN_ERR_UNSUPPORTED; }
     const void *fn = kernel_of(k, 0);
     for (int mode = 0; mode < 4; ++mode) {
         const void *f = kernel_of(k, mode);
@@ -711,7 +712,6 @@ int reslean_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
-    m->prof_multi = false;
     m->prof_lean = true;
     m->prof_cl = false;
     return WRNN_OK;
