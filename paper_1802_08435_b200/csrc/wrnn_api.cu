@@ -130,7 +130,7 @@ static bool use_reslean(const wrnn_model *m, int batch)
     return reslean_supported(m, batch) == WRNN_OK;
 }
 
-// Rows of a dense bf16 H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
+// Rows of a dense H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
 // clusters of eight) and more in waves; the cluster-partitioned kernel takes all at once and costs almost the same whatever
 // the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 7.1 / 25.2, 57: 12.5 / 25.3, 112: 14.3 / 25.8,
 // 168: 21.3 / 28.7, 224: 28.4 / 31.0, 256 (a fifth wave): 35.5 / 32.3.
@@ -392,14 +392,17 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
                       (int64_t)G * 3 * 4;
 
     if (fused) {
-        // one kernel serves this variant; without it the model cannot be stepped
-        const int rc = resident_prepare(m);
+        // the cluster-resident kernel; the lean kernel as the checked build (WRNN_DEBUG=1), the first form under WRNN_RESIDENT_LEAN=0
+        const char *no_lean = getenv("WRNN_RESIDENT_LEAN");
+        reslean_prepare(m);
+        if (!reslean_checked(m)) rescl_prepare(m);
+        const int rc = m->rescl && !(no_lean && no_lean[0] == '0') ? WRNN_OK : resident_prepare(m);
         if (rc != WRNN_OK) {
             const std::string why = m->err;
             wrnn_destroy(m);
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
-        reslean_prepare(m);     // optional: the lean form of the same kernel (the first form serves the variant without it)
+        m->err.clear();
         *out = m;
         return WRNN_OK;
     }

@@ -54,29 +54,36 @@ constexpr int CPH = 40, CPL = 24, CPR = 6 * CU;              // floats per (K-sp
 constexpr size_t CW_HID = 2 * 28 * 512;                      // O1 (O3) rows of a CTA as A fragments: two tiles
 constexpr size_t CW_LOG = 28 * 512;                          // O2 (O4) rows: one tile
 constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
-constexpr int C_SMALL = 2 * 3 * CU * 3 + 2 * 32 + 2 * CL;    // I of the CTA's units [half][gate][unit][3], b1, b3 (32 each), b2, b4
-__host__ __device__ constexpr size_t cl_blob_smem(bool w2) { return (w2 ? 2 : 1) * (2 * CW_HID + 2 * CW_LOG) + (w2 ? 0 : CW_R2) + C_SMALL * 4; }
+enum { CL_BF16 = 0, CL_F32 = 1, CL_FUSED = 2 };                // kinds of model: bf16 weights, fp32 weights, the Fused Subscale WaveRNN 2x (bf16)
+__host__ __device__ constexpr int cl_nin(int kind) { return kind == CL_FUSED ? 12 : 3; }
+__host__ __device__ constexpr int cl_rows(int kind) { return kind == CL_FUSED ? 4 : CL; }       // logits rows per CTA in use
+// I of the CTA's units [half][gate][unit][3 or 12], b1, b3 (32 each), b2, b4
+__host__ __device__ constexpr int cl_small(int kind) { return 2 * 3 * CU * cl_nin(kind) + 2 * 32 + 2 * CL; }
+__host__ __device__ constexpr size_t cl_blob_smem(int kind)
+{
+    return (kind == CL_F32 ? 2 : 1) * (2 * CW_HID + 2 * CW_LOG) + (kind == CL_F32 ? 0 : CW_R2) + cl_small(kind) * 4;
+}
 constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: [2 halves][7 k-tiles][9 tiles][4 registers]
 constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
-static_assert(cl_blob_smem(false) % 16 == 0 && cl_blob_smem(true) % 16 == 0, "the blob is copied in 16-byte pieces");
+static_assert(cl_blob_smem(CL_BF16) % 16 == 0 && cl_blob_smem(CL_F32) % 16 == 0 && cl_blob_smem(CL_FUSED) % 16 == 0, "the blob is copied in 16-byte pieces");
 // fp32 weights, second part and the rows without room: [warp][half][pass][k-tile][4 fragments][32 lanes][16 B] per CTA, read from L2
 constexpr size_t CB_STREAM = (size_t)8 * 2 * 2 * 7 * 4 * 512;
 __host__ __device__ constexpr size_t cl_img(int ng) { return (size_t)CQ * ng * 64; }                // operand image of one vector
 __host__ __device__ constexpr size_t cl_part(int ng) { return (size_t)7 * 4 * ng * CPL * 4; }       // partial sums (>= 4 * 4 * ng * CPH * 4)
 static_assert((size_t)7 * 4 * CPL * 4 >= (size_t)4 * 4 * CPH * 4, "the partial sums of both products share a buffer");
 __host__ __device__ constexpr size_t cl_part_r(int ng) { return (size_t)4 * 4 * ng * CPR * 4; }     // R h
-__host__ __device__ constexpr size_t cl_smem(int ng, bool w2)
+__host__ __device__ constexpr size_t cl_smem(int ng, int kind)
 {
-    return cl_blob_smem(w2) + 3 * cl_img(ng) /* two state halves, hidden layer */ + (size_t)4 * ng * 1024 /* logits */ + cl_part(ng) + cl_part_r(ng) +
+    return cl_blob_smem(kind) + 3 * cl_img(ng) /* two state halves, hidden layer */ + (size_t)4 * ng * 1024 /* logits */ + cl_part(ng) + cl_part_r(ng) +
            (size_t)4 * ng * 2 * CU * 2 /* staged state */;
 }
-// what a launch asks for: the larger form of a weight type (one CTA per SM either way)
-size_t cl_launch_smem(bool w2) { return cl_smem(w2 ? 1 : 2, w2); }
+// what a launch asks for: the larger form of a kind (one CTA per SM either way)
+size_t cl_launch_smem(int kind) { return cl_smem(kind == CL_BF16 ? 2 : 1, kind); }
 }  // namespace
 
 struct ResClPack {
     uint8_t *d_blob = nullptr;               // [16 ranks][shared memory | tensor memory | streamed (fp32 weights)]
-    bool w2 = false;                         // fp32 weights: two fp16 parts
+    int kind = CL_BF16;
     long long *d_prof = nullptr;             // [16]
     int max_clusters = 0;
     float inv_R = 0.f, inv_O1[2] = {0.f, 0.f}, inv_O2[2] = {0.f, 0.f}, q_scale[2] = {0.f, 0.f};
@@ -96,6 +103,9 @@ struct ClParams {
     const uint8_t *c_in, *f_in; uint8_t *c_st_out, *f_st_out;
     const uint8_t *c_forced, *f_forced;
     uint8_t *c_out, *f_out;
+    // the fused variant's 16-bit counterparts of the byte arrays (part A = the coarse half, part B = the fine half)
+    const uint16_t *a_in, *b_in; uint16_t *a_st_out, *b_st_out;
+    const uint16_t *a_forced, *b_forced; uint16_t *a_out, *b_out;
     int16_t *out;
     float *dbg_gates, *dbg_h, *dbg_logits;
     DevStatus *status;
@@ -187,11 +197,14 @@ __device__ __forceinline__ uint2 cl_split4(float a, float b, float c, float d, u
 // W2: fp32 weights, as high and low fp16 parts (error 2^-24 of a weight).  They are twice as much: the heads and the high parts of
 // nine tiles of R stay resident, the rest of R (344 KB per CTA and step) comes from L2 every step, in fragment order, straight
 // into the registers of the background warps.
-template <int NG, int MODE, bool W2>
+// FUSED: two 16-bit samples per step, one per half of the state, each as four 4-bit softmaxes of 16 consecutive logits; one row.
+template <int NG, int MODE, int KIND>
 __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
 {
+    constexpr bool W2 = KIND == CL_F32, FUSED = KIND == CL_FUSED;
     constexpr int NP = W2 ? 2 : 1;                                       // parts of a weight
-    constexpr size_t CB_SMEM = cl_blob_smem(W2), CS_IMG = cl_img(NG), CS_PART = cl_part(NG), CS_PARTR = cl_part_r(NG);
+    constexpr int NIN = cl_nin(KIND), NX = NIN / 3;                      // scalars of I per row, per symbol
+    constexpr size_t CB_SMEM = cl_blob_smem(KIND), CS_IMG = cl_img(NG), CS_PART = cl_part(NG), CS_PARTR = cl_part_r(NG);
     constexpr int CMAXR = 4 * NG;
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
@@ -216,8 +229,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const uint4 *wH[2] = {reinterpret_cast<const uint4 *>(smem + NP * CW_HID), reinterpret_cast<const uint4 *>(smem)};
     const uint4 *wL[2] = {reinterpret_cast<const uint4 *>(smem + NP * (2 * CW_HID + CW_LOG)), reinterpret_cast<const uint4 *>(smem + NP * 2 * CW_HID)};
     const uint32_t r2_addr = smem_u32(smem + NP * (2 * CW_HID + 2 * CW_LOG));
-    const float *sI = reinterpret_cast<const float *>(smem + CB_SMEM - C_SMALL * 4);               // [half][gate][unit][3]
-    const float *sb1 = sI + 2 * 3 * CU * 3, *sb3 = sb1 + 32, *sb2 = sb3 + 32, *sb4 = sb2 + CL;
+    const float *sI = reinterpret_cast<const float *>(smem + CB_SMEM - cl_small(KIND) * 4);        // [half][gate][unit][NIN]
+    const float *sb1 = sI + 2 * 3 * CU * NIN, *sb3 = sb1 + 32, *sb2 = sb3 + 32, *sb4 = sb2 + CL;
     uint8_t *ximg = smem + CB_SMEM;                                      // [2: coarse, fine] state image
     uint8_t *qimg = ximg + 2 * CS_IMG;
     float *lbuf = reinterpret_cast<float *>(qimg + CS_IMG);              // [rows][256]
@@ -456,7 +469,11 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const int gu = lane < CU ? lane : 0, gj = CU * rank + gu;
     int c_prev = 128, f_prev = 0;
     float hC = 0.f, hF = 0.f;
-    if (drawer) { c_prev = p.c_in ? p.c_in[gb] : 128; f_prev = p.f_in ? p.f_in[gb] : 0; }
+    if (drawer) {
+        if (FUSED) { c_prev = p.a_in ? p.a_in[0] : 0x8000; f_prev = p.b_in ? p.b_in[0] : 0x8000; }
+        else { c_prev = p.c_in ? p.c_in[gb] : 128; f_prev = p.f_in ? p.f_in[gb] : 0; }
+    }
+    auto xin = [](int v, int k) { return FUSED ? scale4((v >> (12 - 4 * k)) & 15) : scale8(v); };    // scalar k of a symbol as the network sees it
     if (gater && p.h_in) { hC = p.h_in[(size_t)gb * H + gj]; hF = p.h_in[(size_t)gb * H + CK + gj]; }
     const bool writer = drawer && rank == 2 * st_d;                      // the CTA whose drawing warp writes this row's samples
     int drawn_out = 0;
@@ -470,7 +487,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[jj] = dbg_v[0]; o[H + jj] = dbg_v[1]; o[2 * H + jj] = dbg_v[2]; }
         if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + jj] = dbg_v[3];
     };
-    struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
+    struct GatePre { float pu, pr, pe, ae, ku[NX], kr[NX], ke[NX]; };
     // a row of R h of this row of the batch
     auto r_row = [&](int i) {
         const float *q = partR + st_d * CPR + i;
@@ -480,19 +497,34 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     // everything of the gates of one half that does not depend on the pending draw
     auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
         GatePre q;
-        const float x0 = scale8(c_prev), x1 = scale8(f_prev);
-        const float *Iu = sI + ((half_g * 3 + 0) * CU + gu) * 3, *Ir = Iu + CU * 3, *Ie = Ir + CU * 3;
-        q.pu = r_row(half_g * 3 * CU + gu) + fmaf(Iu[0], x0, half_g ? fmaf(Iu[1], x1, gv[0]) : gv[0]);
-        q.pr = r_row(half_g * 3 * CU + CU + gu) + fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
-        q.pe = fmaf(Ie[0], x0, half_g ? fmaf(Ie[1], x1, gv[2]) : gv[2]);
+        const float *Iu = sI + ((half_g * 3 + 0) * CU + gu) * NIN, *Ir = Iu + CU * NIN, *Ie = Ir + CU * NIN;
+        // fine units: the last symbols of both halves are known, the coarse one of this step is pending; coarse units: the coarse
+        // symbol is known, the fine one pending
+        float su = gv[0], sr = gv[1], se = gv[2];
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            if (half_g) { const float x = xin(f_prev, k); su = fmaf(Iu[NX + k], x, su); sr = fmaf(Ir[NX + k], x, sr); se = fmaf(Ie[NX + k], x, se); }
+            const float x = xin(c_prev, k);
+            su = fmaf(Iu[k], x, su); sr = fmaf(Ir[k], x, sr); se = fmaf(Ie[k], x, se);
+        }
+        q.pu = r_row(half_g * 3 * CU + gu) + su;
+        q.pr = r_row(half_g * 3 * CU + CU + gu) + sr;
+        q.pe = se;
         q.ae = r_row(half_g * 3 * CU + 2 * CU + gu);
-        q.ku = half_g ? Iu[2] : Iu[1]; q.kr = half_g ? Ir[2] : Ir[1]; q.ke = half_g ? Ie[2] : Ie[1];
+        const int pend = half_g ? 2 * NX : NX;
+#pragma unroll
+        for (int k = 0; k < NX; ++k) { q.ku[k] = Iu[pend + k]; q.kr[k] = Ir[pend + k]; q.ke[k] = Ie[pend + k]; }
         return q;
     };
     auto gates_and_stage = [&](int half_g, long long s, int drawn, const GatePre &q) {
-        const float xk = scale8(drawn);
-        const float u = cl_sigmoid(fmaf(q.ku, xk, q.pu)), r = cl_sigmoid(fmaf(q.kr, xk, q.pr));
-        const float e = cl_tanh(fmaf(r, q.ae, fmaf(q.ke, xk, q.pe)));
+        float pu = q.pu, pr = q.pr, pe = q.pe;
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            const float xk = xin(drawn, k);
+            pu = fmaf(q.ku[k], xk, pu); pr = fmaf(q.kr[k], xk, pr); pe = fmaf(q.ke[k], xk, pe);
+        }
+        const float u = cl_sigmoid(pu), r = cl_sigmoid(pr);
+        const float e = cl_tanh(fmaf(r, q.ae, pe));
         const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
         if (half_g) hF = hn; else hC = hn;
         if (gater) {
@@ -522,7 +554,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const float inv_h0 = p.inv_O1[0] * h_inv, inv_h1 = p.inv_O1[1] * h_inv, inv_l0 = p.inv_O2[0] * h_inv, inv_l1 = p.inv_O2[1] * h_inv;
     const float q_s0 = p.q_scale[0] * ldexpf(1.f, -s_hexp), q_s1 = p.q_scale[1] * ldexpf(1.f, -s_hexp);
     const int n_draw = 32 * nrc;                                         // threads of the drawing warps
-    const unsigned ybytes = (unsigned)(nsend * CK * 4), lbytes = (unsigned)(nrc * 1024);
+    const unsigned ybytes = (unsigned)(nsend * CK * 4), lbytes = FUSED ? 256u : (unsigned)(nrc * 1024);
 
     // ---- warp 7 prepares, one row per lane, what the draws of a half-step need: the uniform and the conditioning frame (the
     // same for both halves of a step), tracked without a division per step
@@ -530,9 +562,10 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     int w_frame = 0, w_rem = 0;
     const int w_q = p.row_stride / p.hop, w_r = p.row_stride - w_q * p.hop;
     auto prepare_rows = [&](int half, long long s) {                     // of half-step 2 s + half
-        if (lane < nrc) {
+        if (lane < (FUSED ? 4 : nrc)) {                                  // FUSED: one lane per nibble
             const long long t = half ? s : s - 1;
-            s_u[half][lane] = uniform24(p.seed, p.stream0 + (unsigned)(row0 + lane), (unsigned long long)(w_pos + t), half ? 0u : 1u);
+            s_u[half][lane] = uniform24(p.seed, p.stream0 + (unsigned)(row0 + (FUSED ? 0 : lane)), (unsigned long long)(w_pos + t),
+                                        FUSED ? (half ? 0u : 4u) + (unsigned)lane : (half ? 0u : 1u));
             if (!half) {                                                 // the fine half computes the coarse gates of step s
                 w_frame += w_q; w_rem += w_r;
                 if (w_rem >= p.hop) { w_rem -= p.hop; ++w_frame; }
@@ -541,8 +574,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             s_fr[half][lane] = w_frame;
         }
     };
-    if (warp == 7 && lane < nrc) {
-        const long long b = row0 + lane, pos = p.row_lag > 0 ? 0 : p.step0 * p.row_stride + ((long long)p.stream0 + b) * p.row_offset_mul;
+    if (warp == 7 && lane < (FUSED ? 4 : nrc)) {
+        const long long b = row0 + (FUSED ? 0 : lane), pos = p.row_lag > 0 ? 0 : p.step0 * p.row_stride + ((long long)p.stream0 + b) * p.row_offset_mul;
         w_pos = p.step0 - b * p.row_lag;
         w_frame = (int)(pos / p.hop); w_rem = (int)(pos - (long long)w_frame * p.hop);
         prepare_rows(1, 0);
@@ -593,14 +626,19 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         float gv[3] = {0.f, 0.f, 0.f}, u01 = 0.f;
         int forced = -1;
         if (drawer) {
-            u01 = s_u[half][st_d];
+            u01 = s_u[half][FUSED ? lane >> 3 : st_d];
             const float *g = g_row + (size_t)s_fr[half][st_d] * 3 * H + half * CK;
             if (!last)
 #pragma unroll
                 for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
             if (DBG) {
-                const uint8_t *fz = half ? p.c_forced : p.f_forced;
-                if (fz) forced = fz[(size_t)gb * T + (half ? s : s - 1)];
+                if (FUSED) {
+                    const uint16_t *fz = half ? p.a_forced : p.b_forced;
+                    if (fz) forced = fz[half ? s : s - 1];
+                } else {
+                    const uint8_t *fz = half ? p.c_forced : p.f_forced;
+                    if (fz) forced = fz[(size_t)gb * T + (half ? s : s - 1)];
+                }
             }
         }
         // ---- hidden layer: this CTA's 28 rows (two tiles), K in four quarters; weight fragments before the wait
@@ -706,7 +744,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             else {
                 cl_bar_sync(3, 224);
                 STAMP(8 * half + 4);
-                if (lane < 4 * nrc && !bad) {
+                if (lane < (FUSED ? 1 : 4 * nrc) && !bad) {
                     const int st = lane >> 2;
                     float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -715,7 +753,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
                     const float inv = half ? inv_l0 : inv_l1;
-                    const uint32_t a = smem_u32(lbuf + st * 256 + CL * rank + 4 * (lane & 3)), bar = smem_u32(&xl);
+                    const uint32_t a = smem_u32(lbuf + (FUSED ? 4 * rank : st * 256 + CL * rank + 4 * (lane & 3))), bar = smem_u32(&xl);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         st_async_v4(a + delta4[k], fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + delta4[k]);
@@ -731,11 +769,18 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             wait_bar(&xl, quse, (int)s, 3 + 4 * half);
             STAMP0();
             float l[8];
-            {
+            int drawn;
+            if (FUSED) {
+                // 64 logits: two per lane; lanes [8 k, 8 k + 8) are the softmax of nibble k (most significant first)
+                const float2 a = reinterpret_cast<const float2 *>(lbuf)[lane];
+                l[0] = a.x; l[1] = a.y;
+                const int nib = group16_softmax_draw(l[0], l[1], u01, lane);
+                drawn = (__shfl_sync(FULL, nib, 0) << 12) | (__shfl_sync(FULL, nib, 8) << 8) | (__shfl_sync(FULL, nib, 16) << 4) | __shfl_sync(FULL, nib, 24);
+            } else {
                 const float4 a = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane), b = *reinterpret_cast<const float4 *>(lbuf + st_d * 256 + 8 * lane + 4);
                 l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
+                drawn = cl_draw(l, u01, lane);
             }
-            const int drawn = cl_draw(l, u01, lane);
             const int fed = (DBG && forced >= 0) ? forced : drawn;
             STAMP(8 * half + 6);
             if (!last) gates_and_stage(half, s, fed, gp);
@@ -744,7 +789,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             drawn_out = drawn;
             if (DBG)
 #pragma unroll
-                for (int k = 0; k < 8; ++k) dbg_l[k] = l[k];
+                for (int k = 0; k < (FUSED ? 2 : 8); ++k) dbg_l[k] = l[k];
         }
         if (!last) {
             cl_bar_sync(1, 256);
@@ -753,16 +798,23 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         // the samples (and the dumps) leave when the state is on its way
         if (DBG && gater && !last && !bad) dump_gates(half, s);
         if (DBG && p.dbg_logits && writer && !bad) {
-            float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * 256 + 8 * lane;
+            float *d = p.dbg_logits + (((size_t)(half ? s : s - 1) * p.batch + gb) * 2 + (half ? 0 : 1)) * (FUSED ? 64 : 256) + (FUSED ? 2 : 8) * lane;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) d[k] = dbg_l[k];
+            for (int k = 0; k < (FUSED ? 2 : 8); ++k) d[k] = dbg_l[k];
         }
         if (writer && lane == 0 && !bad) {
             if (DBG) {
-                uint8_t *o = half ? p.c_out : p.f_out;
-                if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
+                if (FUSED) {
+                    uint16_t *o = half ? p.a_out : p.b_out;
+                    if (o) o[half ? s : s - 1] = (uint16_t)drawn_out;
+                } else {
+                    uint8_t *o = half ? p.c_out : p.f_out;
+                    if (o) o[(size_t)gb * T + (half ? s : s - 1)] = (uint8_t)drawn_out;
+                }
             }
-            if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
+            // (fused: the two streams side by side, a_s and the sample part B emits in step s)
+            if (FUSED) { if (p.out) p.out[half ? s : T + s - 1] = (int16_t)((half ? c_prev : f_prev) - 32768); }
+            else if (!half && out_row) out_row[s - 1] = (int16_t)(256 * c_prev + f_prev - 32768);
         }
     };
     if (warp < 8) {
@@ -807,8 +859,13 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     if (!any_bad) {
         if (gater && p.h_out) { p.h_out[(size_t)gb * H + gj] = hC; p.h_out[(size_t)gb * H + CK + gj] = hF; }
         if (writer && lane == 0) {
-            if (p.c_st_out) p.c_st_out[gb] = (uint8_t)c_prev;
-            if (p.f_st_out) p.f_st_out[gb] = (uint8_t)f_prev;
+            if (FUSED) {
+                if (p.a_st_out) p.a_st_out[0] = (uint16_t)c_prev;
+                if (p.b_st_out) p.b_st_out[0] = (uint16_t)f_prev;
+            } else {
+                if (p.c_st_out) p.c_st_out[gb] = (uint8_t)c_prev;
+                if (p.f_st_out) p.f_st_out[gb] = (uint8_t)f_prev;
+            }
         }
     }
     if (DBG && p.prof && blockIdx.x == 0 && tid < 16) p.prof[tid] = s_prof[tid];
@@ -820,11 +877,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 }
 
 // ---------------------------------------------------------------------------------------------
-static const void *cl_kernel_of(int nr, bool dbg, bool w2)
+static const void *cl_kernel_of(int nr, bool dbg, int kind)
 {
-    if (w2) return dbg ? (const void *)resident_cluster_kernel<1, 1, true> : (const void *)resident_cluster_kernel<1, 0, true>;
-    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1, false> : (const void *)resident_cluster_kernel<1, 0, false>;
-    return dbg ? (const void *)resident_cluster_kernel<2, 1, false> : (const void *)resident_cluster_kernel<2, 0, false>;
+    if (kind == CL_F32) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_F32> : (const void *)resident_cluster_kernel<1, 0, CL_F32>;
+    if (kind == CL_FUSED) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_FUSED> : (const void *)resident_cluster_kernel<1, 0, CL_FUSED>;
+    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_BF16> : (const void *)resident_cluster_kernel<1, 0, CL_BF16>;
+    return dbg ? (const void *)resident_cluster_kernel<2, 1, CL_BF16> : (const void *)resident_cluster_kernel<2, 0, CL_BF16>;
 }
 
 static void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
@@ -844,7 +902,7 @@ static void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg,
 // clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
 static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
 {
-    const int most = k.max_clusters * (k.w2 ? 4 : 8), waves = (batch + most - 1) / most;
+    const int most = k.max_clusters * (k.kind == CL_BF16 ? 8 : 4), waves = (batch + most - 1) / most;
     *nr = (batch + waves * k.max_clusters - 1) / (waves * k.max_clusters);
     const int need = (batch + *nr - 1) / *nr;
     *n_clusters = need < CNC ? CNC : need;       // (a cluster without rows returns at once)
@@ -899,16 +957,16 @@ struct HalfMatrix {
 int rescl_prepare(wrnn_model *m)
 {
     const int H = m->H;
-    if (m->sparse || m->variant != 0 || H != 2 * CK) { m->err = "cluster-resident kernel: dense H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
+    if (m->sparse || H != 2 * CK) { m->err = "cluster-resident kernel: dense H = 896 only"; return WRNN_ERR_UNSUPPORTED; }
     cudaDeviceProp prop;
     cudaGetDeviceProperties(&prop, m->device);
     ResClPack k;
-    k.w2 = m->dtype == WRNN_F32;
+    k.kind = m->variant == 1 ? CL_FUSED : m->dtype == WRNN_F32 ? CL_F32 : CL_BF16;
     cudaFuncAttributes fa;
     for (int nr : {1, 5})
         for (int dbg = 0; dbg < 2; ++dbg) {
-            const void *f = cl_kernel_of(nr, dbg != 0, k.w2);
-            const size_t CS_BYTES = cl_launch_smem(k.w2);
+            const void *f = cl_kernel_of(nr, dbg != 0, k.kind);
+            const size_t CS_BYTES = cl_launch_smem(k.kind);
             if (cudaFuncGetAttributes(&fa, f) != cudaSuccess || CS_BYTES + fa.sharedSizeBytes > prop.sharedMemPerBlockOptin ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                 cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS_BYTES) != cudaSuccess) {
@@ -917,14 +975,15 @@ int rescl_prepare(wrnn_model *m)
         }
     {
         cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-        cl_fill_launch(CNC, cl_launch_smem(k.w2), &cfg, at, 0);
-        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.w2 ? 1 : 5, false, k.w2), &cfg) != cudaSuccess || k.max_clusters < 1) {
+        cl_fill_launch(CNC, cl_launch_smem(k.kind), &cfg, at, 0);
+        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.kind == CL_BF16 ? 5 : 1, false, k.kind), &cfg) != cudaSuccess || k.max_clusters < 1) {
             cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
         }
     }
     // fp16 weights, every matrix scaled by a power of two to at most 2^14: the eight bits of a bf16 weight are kept unless it is
     // below 2^-28 of the largest one, where at most 2^-39 of that is lost; fp32 weights as two parts (2^-24 of a weight)
-    const int NP = k.w2 ? 2 : 1;
+    const bool w2 = k.kind == CL_F32;
+    const int NP = w2 ? 2 : 1, NIN = cl_nin(k.kind), LR = cl_rows(k.kind);
     HalfMatrix R(m->hR, NP), O[4] = {{m->hO1, NP}, {m->hO3, NP}, {m->hO2, NP}, {m->hO4, NP}};
     const int e[5] = {R.exp, O[0].exp, O[1].exp, O[2].exp, O[3].exp};
     // products of operands scaled by 2^(14 - exponent) each
@@ -946,7 +1005,7 @@ int rescl_prepare(wrnn_model *m)
         k.q_scale[h] = std::ldexp(1.f, 14 - eq);
         k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);
     }
-    const size_t smem_bytes = cl_blob_smem(k.w2), cta_bytes = smem_bytes + CB_TMEM + (k.w2 ? CB_STREAM : 0);
+    const size_t smem_bytes = cl_blob_smem(k.kind), cta_bytes = smem_bytes + CB_TMEM + (w2 ? CB_STREAM : 0);
     std::vector<uint8_t> blob(CCS * cta_bytes, 0);
     // part w of row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
     auto r_row = [&](int rank, int w, int i) { return &R.part[w][((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
@@ -968,9 +1027,9 @@ int rescl_prepare(wrnn_model *m)
             for (int w = 0; w < NP; ++w) {
                 for (int t = 0; t < 2; ++t)
                     pack(O[h].part[w], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + (h * NP + w) * CW_HID + (size_t)t * 28 * 512));
-                pack(O[2 + h].part[w], CL * rank, CL, reinterpret_cast<uint16_t *>(base + NP * 2 * CW_HID + (h * NP + w) * CW_LOG));
+                pack(O[2 + h].part[w], LR * rank, LR, reinterpret_cast<uint16_t *>(base + NP * 2 * CW_HID + (h * NP + w) * CW_LOG));
             }
-        if (!k.w2) {
+        if (!w2) {
             uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
             for (int i = 0; i < CRS; ++i)
                 for (int k8 = 0; k8 < 2 * CK8; ++k8) {
@@ -978,14 +1037,14 @@ int rescl_prepare(wrnn_model *m)
                     for (int c = 0; c < 8; ++c) r2[((size_t)k8 * CRS + i) * 8 + c] = src[4 * (c >> 1) + (c & 1)];
                 }
         }
-        float *sm = reinterpret_cast<float *>(base + smem_bytes - C_SMALL * 4);
+        float *sm = reinterpret_cast<float *>(base + smem_bytes - cl_small(k.kind) * 4);
         for (int i = 0; i < 6 * CU; ++i) {
             const size_t row = (size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU;
-            for (int c = 0; c < 3; ++c) sm[i * 3 + c] = m->hI[row * 3 + c];
+            for (int c = 0; c < NIN; ++c) sm[i * NIN + c] = m->hI[row * NIN + c];
         }
-        float *b = sm + 6 * CU * 3;
+        float *b = sm + 6 * CU * NIN;
         for (int r = 0; r < CU; ++r) { b[r] = m->hb1[CU * rank + r]; b[32 + r] = m->hb3[CU * rank + r]; }
-        for (int r = 0; r < CL; ++r) { b[64 + r] = m->hb2[CL * rank + r]; b[64 + CL + r] = m->hb4[CL * rank + r]; }
+        for (int r = 0; r < LR; ++r) { b[64 + r] = m->hb2[LR * rank + r]; b[64 + CL + r] = m->hb4[LR * rank + r]; }
         // tensor memory: lane quadrant q holds quarter q of the k-tiles of both halves of the state; columns as the kernel states them
         uint16_t *tm = reinterpret_cast<uint16_t *>(base + smem_bytes);
         for (int i = 0; i < 16 * CRT; ++i) {
@@ -999,7 +1058,7 @@ int rescl_prepare(wrnn_model *m)
                         std::memcpy(tm + ((size_t)(c0 + reg0 + 2 * h) * 128 + 32 * q + 4 * (i & 7) + t) * 2, src + 16 * kt + 4 * t + 2 * h, 4);
             }
         }
-        if (!k.w2) continue;
+        if (!w2) continue;
         // streamed fragments of warp w8 = 4 j + q: pass 0 the low parts of tiles 0..3 (j = 0) or 4, 5; pass 1 tile 9 (both parts) and
         // tile 10 (high parts over low parts), or the low parts of tiles 6..8
         uint16_t *st = reinterpret_cast<uint16_t *>(base + smem_bytes + CB_TMEM);
@@ -1053,8 +1112,8 @@ int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thread
     cl_geometry(*m->rescl, batch, &nr, &n_clusters);
     if (n_ctas) *n_ctas = n_clusters * CCS;
     if (n_threads) *n_threads = 512;
-    if (smem) *smem = (int)cl_launch_smem(m->rescl->w2);
-    if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(cl_blob_smem(m->rescl->w2) + CB_TMEM + (m->rescl->w2 ? CB_STREAM : 0));
+    if (smem) *smem = (int)cl_launch_smem(m->rescl->kind);
+    if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(cl_blob_smem(m->rescl->kind) + CB_TMEM + (m->rescl->kind == CL_F32 ? CB_STREAM : 0));
     return WRNN_OK;
 }
 
@@ -1077,17 +1136,19 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     for (int h = 0; h < 2; ++h) { p.inv_O1[h] = k.inv_O1[h]; p.inv_O2[h] = k.inv_O2[h]; p.q_scale[h] = k.q_scale[h]; }
     p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
     p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
+    p.a_in = a.a_in; p.b_in = a.b_in; p.a_st_out = a.a_st_out; p.b_st_out = a.b_st_out;
+    p.a_forced = a.a_forced; p.b_forced = a.b_forced; p.a_out = a.a_out; p.b_out = a.b_out;
     p.dbg_gates = a.dbg_gates; p.dbg_h = a.dbg_h; p.dbg_logits = a.dbg_logits;
     p.status = m->status;
     p.limit_ns = m->wait_limit_ns();
     p.skip_rank = m->dbg_skip_cta >= 0 ? m->dbg_skip_cta % CCS : -1; p.skip_step = m->dbg_skip_step;
     p.prof = m->prof_enabled ? k.d_prof : nullptr;
     if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
-    const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.dbg_gates || p.dbg_h || p.dbg_logits;
+    const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.c_out || p.f_out || p.a_forced || p.b_forced || p.a_out || p.b_out || p.dbg_gates || p.dbg_h || p.dbg_logits;
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-    cl_fill_launch(n_clusters, cl_launch_smem(k.w2), &cfg, at, s);
+    cl_fill_launch(n_clusters, cl_launch_smem(k.kind), &cfg, at, s);
     void *args[] = {&p};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg, k.w2), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, dbg, k.kind), args);
     if (e != cudaSuccess) {
         m->err = std::string("cluster-resident kernel launch failed: ") + cudaGetErrorString(e);
         cudaGetLastError();

@@ -575,7 +575,7 @@ int reslean_prepare(wrnn_model *m)
     cudaGetDeviceProperties(&prop, m->device);
     if (k.NCTA > m->n_sms || (size_t)k.smem_bytes > prop.sharedMemPerBlockOptin) { m->err = "lean resident kernel does not fit this device"; return WRNN_ERR_UNSUPPORTED; }
     { const char *d = getenv("WRNN_DEBUG"); k.checked = d && d[0] == '1'; }
-    if (!fused && !k.checked) { m->err = "lean resident kernel: a plain model runs on the cluster-resident kernel"; return WRNN_ERR_UNSUPPORTED; }
+    if (!k.checked) { m->err = "lean resident kernel: the checked build only (models run on the cluster-resident kernel otherwise)"; return WRNN_ERR_UNSUPPORTED; }
     const void *fn = kernel_of(k, 0);
     for (int mode = 0; mode < 4; ++mode) {
         const void *f = kernel_of(k, mode);
