@@ -66,8 +66,13 @@ __host__ __device__ constexpr size_t cl_blob_smem(int kind)
 constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: [2 halves][7 k-tiles][9 tiles][4 registers]
 constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
 static_assert(cl_blob_smem(CL_BF16) % 16 == 0 && cl_blob_smem(CL_F32) % 16 == 0 && cl_blob_smem(CL_FUSED) % 16 == 0, "the blob is copied in 16-byte pieces");
-// fp32 weights, second part and the rows without room: [warp][half][pass][k-tile][4 fragments][32 lanes][16 B] per CTA, read from L2
-constexpr size_t CB_STREAM = (size_t)8 * 2 * 2 * 7 * 4 * 512;
+// fp32 weights, second part and the rows without room: [CTA][half][warp][k-tile v of 14][fragments of v][32 lanes][16 B] in an array of
+// its own, read from L2
+__host__ __device__ constexpr int cl_nf(int rj, int v) { return v < 7 ? (rj ? 2 : 4) : 3; }                       // fragments of a k-tile
+__host__ __device__ constexpr int cl_fo(int rj, int v) { return v < 7 ? v * (rj ? 2 : 4) : 7 * (rj ? 2 : 4) + (v - 7) * 3; }   // before it
+__host__ __device__ constexpr int cl_fw(int w8) { return w8 < 4 ? w8 * cl_fo(0, 14) : 4 * cl_fo(0, 14) + (w8 - 4) * cl_fo(1, 14); }   // before warp w8
+constexpr int CF_HALF = cl_fw(8);                            // fragments of a half: 336
+constexpr size_t CB_STREAM = (size_t)2 * CF_HALF * 512;
 __host__ __device__ constexpr size_t cl_img(int ng) { return (size_t)CQ * ng * 64; }                // operand image of one vector
 __host__ __device__ constexpr size_t cl_part(int ng) { return (size_t)7 * 4 * ng * CPL * 4; }       // partial sums (>= 4 * 4 * ng * CPH * 4)
 static_assert((size_t)7 * 4 * CPL * 4 >= (size_t)4 * 4 * CPH * 4, "the partial sums of both products share a buffer");
@@ -82,7 +87,8 @@ size_t cl_launch_smem(int kind) { return cl_smem(kind == CL_BF16 ? 2 : 1, kind);
 }  // namespace
 
 struct ResClPack {
-    uint8_t *d_blob = nullptr;               // [16 ranks][shared memory | tensor memory | streamed (fp32 weights)]
+    uint8_t *d_blob = nullptr;               // [16 ranks][shared memory | tensor memory]
+    uint4 *d_stream = nullptr;               // fp32 weights: [16 ranks][CB_STREAM]
     int kind = CL_BF16;
     long long *d_prof = nullptr;             // [16]
     int max_clusters = 0;
@@ -97,6 +103,7 @@ struct ClParams {
     int n_frames, hop, row_stride, row_offset_mul, row_lag;
     long long out_pitch;
     const uint8_t *blob;
+    const uint4 *stream;
     const float *g;                          // [batch][n_frames][3H]
     float inv_R, inv_O1[2], inv_O2[2], q_scale[2];   // 2^-14 over the power of two in R, in the hidden layers and logits rows; the one of the hidden-layer values
     const float *h_in; float *h_out;
@@ -174,6 +181,12 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
     const int c = ((p0 <= thr) + (p1 <= thr)) + ((p2 <= thr) + (p3 <= thr)) + (((p4 <= thr) + (p5 <= thr)) + ((p6 <= thr) + (p7 <= thr)));
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
 }
+// f(0), .., f(N - 1) with compile-time arguments
+template <int N, int I = 0, typename F>
+__device__ __forceinline__ void cl_for(F &&f)
+{
+    if constexpr (I < N) { f(std::integral_constant<int, I>{}); cl_for<N, I + 1>(f); }
+}
 __device__ __forceinline__ uint4 cl_ldg_stream(const uint4 *p)
 {
     uint4 v;
@@ -247,7 +260,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     {
-        const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM + (W2 ? CB_STREAM : 0));
+        const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM);
         const uint4 *src = reinterpret_cast<const uint4 *>(blob);
         uint4 *dst = reinterpret_cast<uint4 *>(smem);
         for (int i = tid; i < (int)(CB_SMEM / 16); i += 512) dst[i] = __ldg(src + i);
@@ -396,47 +409,47 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         }
     };
 
-    // fp32 weights: two passes over the half of the state, first the tiles that hold the coarse rows (0..3 and 4, 5), then the others
-    // (9 and 10; 6..8).  High parts of tiles 0..8 from tensor memory, the other fragments from L2, requested three or four k-tiles
-    // ahead (48 KB in flight per SM).  Tile 10 has eight rows: its high and low parts share a fragment.
-    const uint4 *stream = reinterpret_cast<const uint4 *>(p.blob + (size_t)rank * (CB_SMEM + CB_TMEM + CB_STREAM) + CB_SMEM + CB_TMEM) + (size_t)(warp & 7) * (2 * 2 * 7 * 4 * 32) + lane;
-    auto w2_pass = [&](int half_f, auto RJ_C, auto PASS_C, auto wait_fn) {
-        constexpr int RJ = decltype(RJ_C)::value, PASS = decltype(PASS_C)::value;
-        constexpr int NTM = PASS == 0 ? (RJ ? 2 : 4) : (RJ ? 3 : 0);     // tiles in tensor memory, of which the low parts are streamed
-        constexpr int NF = PASS == 0 ? NTM : 3, DEPTH = NF == 4 ? 3 : 4; // streamed fragments of a k-tile
-        constexpr int A0 = PASS == 0 ? 0 : (RJ ? 2 : 4);                 // first accumulator
+    // fp32 weights: two passes over a half of the state, first the tiles that hold the coarse rows (0..3 and 4, 5), then the others
+    // (9 and 10; 6..8).  High parts of tiles 0..8 from tensor memory, the other fragments from L2, requested three k-tiles ahead
+    // (some 40 KB in flight per SM) across passes and halves, so that a half-step starts with its first fragments there.  Tile 10
+    // has eight rows: its high and low parts share a fragment.
+    const uint4 *stream = p.stream + ((size_t)rank * 2 * CF_HALF + cl_fw(warp & 7)) * 32 + lane;
+    uint4 sf[W2 ? 3 : 1][4];
+    auto w2_request = [&](auto RJ_C, int half_f, auto V_C) {              // k-tile v of the 14 of a half: slot v % 3 (15 are counted)
+        constexpr int RJ = decltype(RJ_C)::value, V = decltype(V_C)::value, NF = cl_nf(RJ, V);
+        if (!W2) return;
+        const uint4 *src = stream + (size_t)(half_f * CF_HALF + cl_fo(RJ, V)) * 32;
+#pragma unroll
+        for (int i = 0; i < NF; ++i) sf[W2 ? V % 3 : 0][i] = cl_ldg_stream(src + i * 32);
+    };
+    auto w2_half = [&](auto RJ_C, int half_f, auto start, auto mid) {
+        constexpr int RJ = decltype(RJ_C)::value;
         const uint32_t b0 = smem_u32(ximg + half_f * CS_IMG) + 7 * rq * 4 * QSTR + frag;
-        const uint32_t c0 = r_col + (uint32_t)(half_f * 7 * (RJ ? 20 : 16)) + (PASS && RJ ? 8 : 0);
-        const uint4 *src = stream + (size_t)((half_f * 2 + PASS) * 7) * 4 * 32;
-        uint4 f[DEPTH][NF];
-        auto request = [&](int kt) {
-#pragma unroll
-            for (int i = 0; i < NF; ++i) f[kt % DEPTH][i] = cl_ldg_stream(src + (kt * 4 + i) * 32);
-        };
-#pragma unroll
-        for (int kt = 0; kt < DEPTH; ++kt) request(kt);
-        wait_fn();
-#pragma unroll
-        for (int kt = 0; kt < 7; ++kt) {
+        const uint32_t c0 = r_col + (uint32_t)(half_f * 7 * (RJ ? 20 : 16));
+        start();
+        cl_for<14>([&](auto V_C) {
+            constexpr int V = decltype(V_C)::value, PASS = V / 7, KT = V % 7;
+            constexpr int NTM = PASS == 0 ? (RJ ? 2 : 4) : (RJ ? 3 : 0);  // tiles in tensor memory, of which the low parts are streamed
+            constexpr int NF = cl_nf(RJ, V), A0 = PASS == 0 ? 0 : (RJ ? 2 : 4);
+            if (V == 7) mid();
             uint32_t r[16];
-            if (NTM == 4) tmem_ld16(c0 + kt * 16, r);
+            if (NTM == 4) tmem_ld16(c0 + KT * 16, r);
             else if (NTM >= 2) {
+                const uint32_t c = c0 + KT * 20 + (PASS ? 8 : 0);
                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                             "=r"(r[6]), "=r"(r[7]) : "r"(c0 + kt * 20));
-                if (NTM == 3) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]) : "r"(c0 + kt * 20 + 8));
+                             "=r"(r[6]), "=r"(r[7]) : "r"(c));
+                if (NTM == 3) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]) : "r"(c + 8));
             }
-            const uint2 b = cl_lds8(b0 + kt * 4 * QSTR);
+            const uint2 b = cl_lds8(b0 + KT * 4 * QSTR);
             tmem_wait_ld();
 #pragma unroll
             for (int n = 0; n < NTM; ++n) cl_mma(acc[A0 + n][0], make_uint4(r[4 * n], r[4 * n + 1], r[4 * n + 2], r[4 * n + 3]), b.x, b.y);
 #pragma unroll
-            for (int i = 0; i < NF; ++i) cl_mma(acc[NTM ? A0 + i : (i == 2 ? 5 : 4)][0], f[kt % DEPTH][i], b.x, b.y);
-            if (kt + DEPTH < 7) request(kt + DEPTH);
-        }
-    };
-    auto w2_products = [&](int half_f, auto PASS_C, auto wait_fn) {
-        if (rj) w2_pass(half_f, std::integral_constant<int, 1>{}, PASS_C, wait_fn);
-        else w2_pass(half_f, std::integral_constant<int, 0>{}, PASS_C, wait_fn);
+            for (int i = 0; i < NF; ++i) cl_mma(acc[NTM ? A0 + i : (i == 2 ? 5 : 4)][0], sf[W2 ? V % 3 : 0][i], b.x, b.y);
+            if constexpr (V < 11) w2_request(RJ_C, half_f, std::integral_constant<int, V + 3>{});
+            if constexpr (V >= 12) w2_request(RJ_C, 1 - half_f, std::integral_constant<int, V - 12>{});
+            if constexpr (V == 13) w2_request(RJ_C, 1 - half_f, std::integral_constant<int, 2>{});
+        });
     };
     auto w2_store = [&](int pass) {
         float *d = partR + (rq * 4 * NG + t4) * CPR + g4;
@@ -584,15 +597,20 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     // ---- prologue: R h of the initial state, coarse gates of step 0
     if (warp >= 8) {
         r_clear();
+        if (W2) {
+            auto pro = [&](auto RJ_C) {
+                cl_for<3>([&](auto V_C) { w2_request(RJ_C, 0, V_C); });
 #pragma unroll 1
-        for (int half_f = 0; half_f < 2; ++half_f) {
-            if (W2) {
-                w2_products(half_f, std::integral_constant<int, 0>{}, [] {});
-                w2_products(half_f, std::integral_constant<int, 1>{}, [] {});
-            } else r_products(half_f);
+                for (int half_f = 0; half_f < 2; ++half_f) w2_half(RJ_C, half_f, [] {}, [] {});
+            };
+            if (rj) pro(std::integral_constant<int, 1>{});
+            else pro(std::integral_constant<int, 0>{});
+            w2_store(0); w2_store(1);
+        } else {
+#pragma unroll 1
+            for (int half_f = 0; half_f < 2; ++half_f) r_products(half_f);
+            r_store();
         }
-        if (W2) { w2_store(0); w2_store(1); }
-        else r_store();
     }
     if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), ybytes);
     __syncthreads();
@@ -825,23 +843,27 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         }
     } else {
         // ---- the rows of R, right after the hidden layer is sent (its sums and sends do not share the load / store pipe with them)
+        if (W2) {
+            // More to do: it starts as soon as the half of the state is there (barriers 5 and 7, at which the chain only arrives), and
+            // the coarse rows come first, the others when the gates have theirs.  Barriers 2 and 6, at which these warps only
+            // arrive, tell the chain that the products of the last half-step are done.  Both alternate: whoever only arrives may
+            // be one half-step ahead of the others, and cannot be two, because the other pair of barriers lies between.
+            auto loop = [&](auto RJ_C) {
 #pragma unroll 1
-        for (long long s2 = 0; s2 < T; ++s2) {
-            r_clear();
-            if (W2) {
-                // More to do: it starts as soon as the half of the state is there (barriers 5 and 7, at which the chain only arrives), and
-                // the coarse rows come first, the others when the gates have theirs.  Barriers 2 and 6, at which these warps only
-                // arrive, tell the chain that the products of the last half-step are done.  Both alternate: whoever only arrives may
-                // be one half-step ahead of the others, and cannot be two, because the other pair of barriers lies between.
-                auto go = [](int done, int start) { return [done, start] { cl_bar_arrive(done, 512); cl_bar_sync(start, 512); }; };
-                w2_products(0, std::integral_constant<int, 0>{}, go(2, 5));
-                w2_products(0, std::integral_constant<int, 1>{}, [] {});
-                w2_products(1, std::integral_constant<int, 0>{}, go(6, 7));
-                w2_store(0);
-                cl_bar_arrive(4, 256 + n_draw);
-                w2_products(1, std::integral_constant<int, 1>{}, [] {});
-                w2_store(1);
-            } else {
+                for (long long n = 0; n < 2 * T; ++n) {
+                    const int half_f = (int)(n & 1);
+                    if (!half_f) r_clear();
+                    w2_half(RJ_C, half_f, [&] { cl_bar_arrive(half_f ? 6 : 2, 512); cl_bar_sync(half_f ? 7 : 5, 512); },
+                            [&] { if (half_f) { w2_store(0); cl_bar_arrive(4, 256 + n_draw); } });
+                    if (half_f) w2_store(1);
+                }
+            };
+            if (rj) loop(std::integral_constant<int, 1>{});
+            else loop(std::integral_constant<int, 0>{});
+        } else {
+#pragma unroll 1
+            for (long long s2 = 0; s2 < T; ++s2) {
+                r_clear();
                 cl_bar_sync(2, 512);
                 r_products(0);
                 cl_bar_sync(2, 512);
@@ -924,8 +946,13 @@ static uint16_t half_bits(float v)
 }
 static float half_value(uint16_t h)
 {
-    const uint32_t e = (h >> 10) & 31u, mant = h & 0x3ffu;
-    const float v = e == 31u ? (mant ? NAN : INFINITY) : e ? std::ldexp((float)(mant | 0x400u), (int)e - 25) : std::ldexp((float)mant, -24);
+    uint32_t u = (uint32_t)(h & 0x7fffu) << 13;
+    float v;
+    if (u < (1u << 23)) v = (float)(h & 0x3ffu) * 5.9604644775390625e-8f;        // subnormal: steps of 2^-24
+    else {
+        u = u >= (31u << 23) ? u | 0x7f800000u : u + (112u << 23);
+        std::memcpy(&v, &u, 4);
+    }
     return h & 0x8000u ? -v : v;
 }
 // A dense matrix as one or two fp16 parts, scaled by 2^(14 - exp)
@@ -1005,7 +1032,8 @@ int rescl_prepare(wrnn_model *m)
         k.q_scale[h] = std::ldexp(1.f, 14 - eq);
         k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);
     }
-    const size_t smem_bytes = cl_blob_smem(k.kind), cta_bytes = smem_bytes + CB_TMEM + (w2 ? CB_STREAM : 0);
+    const size_t smem_bytes = cl_blob_smem(k.kind), cta_bytes = smem_bytes + CB_TMEM;
+    std::vector<uint8_t> stream(w2 ? CCS * CB_STREAM : 0, 0);
     std::vector<uint8_t> blob(CCS * cta_bytes, 0);
     // part w of row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
     auto r_row = [&](int rank, int w, int i) { return &R.part[w][((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
@@ -1061,30 +1089,29 @@ int rescl_prepare(wrnn_model *m)
         if (!w2) continue;
         // streamed fragments of warp w8 = 4 j + q: pass 0 the low parts of tiles 0..3 (j = 0) or 4, 5; pass 1 tile 9 (both parts) and
         // tile 10 (high parts over low parts), or the low parts of tiles 6..8
-        uint16_t *st = reinterpret_cast<uint16_t *>(base + smem_bytes + CB_TMEM);
-        for (int w8 = 0; w8 < 8; ++w8)
-            for (int half_f = 0; half_f < 2; ++half_f)
-                for (int pass = 0; pass < 2; ++pass)
-                    for (int k7 = 0; k7 < 7; ++k7)
-                        for (int f = 0; f < 4; ++f) {
-                            const int j = w8 >> 2, kt = 28 * half_f + 7 * (w8 & 3) + k7;
-                            if (f >= (pass ? 3 : j ? 2 : 4)) continue;
-                            uint16_t *frag = st + ((((size_t)(w8 * 2 + half_f) * 2 + pass) * 7 + k7) * 4 + f) * 256;
-                            for (int r = 0; r < 16; ++r) {
-                                int row, w = 1;
-                                if (!pass) row = 16 * (j ? 4 + f : f) + r;
-                                else if (j) row = 16 * (6 + f) + r;
-                                else if (f < 2) { row = 144 + r; w = f; }
-                                else { row = 160 + (r & 7); w = r >> 3; }
-                                frag_row(frag, r & 7, r >> 3, r_row(rank, w, row) + 16 * kt);
-                            }
+        uint16_t *st = reinterpret_cast<uint16_t *>(stream.data() + (size_t)rank * CB_STREAM);
+        for (int half_f = 0; half_f < 2; ++half_f)
+            for (int w8 = 0; w8 < 8; ++w8)
+                for (int v = 0; v < 14; ++v)
+                    for (int f = 0; f < cl_nf(w8 >> 2, v); ++f) {
+                        const int j = w8 >> 2, kt = 28 * half_f + 7 * (w8 & 3) + v % 7;
+                        uint16_t *frag = st + ((size_t)half_f * CF_HALF + cl_fw(w8) + cl_fo(j, v) + f) * 256;
+                        for (int r = 0; r < 16; ++r) {
+                            int row, w = 1;
+                            if (v < 7) row = 16 * (j ? 4 + f : f) + r;
+                            else if (j) row = 16 * (6 + f) + r;
+                            else if (f < 2) { row = 144 + r; w = f; }
+                            else { row = 160 + (r & 7); w = r >> 3; }
+                            frag_row(frag, r & 7, r >> 3, r_row(rank, w, row) + 16 * kt);
                         }
+                    }
     }
     ResClPack *pk = new ResClPack(k);
     if (cudaMalloc((void **)&pk->d_blob, blob.size()) != cudaSuccess || cudaMemcpy(pk->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        (w2 && (cudaMalloc((void **)&pk->d_stream, stream.size()) != cudaSuccess || cudaMemcpy(pk->d_stream, stream.data(), stream.size(), cudaMemcpyHostToDevice) != cudaSuccess)) ||
         cudaMalloc((void **)&pk->d_prof, 16 * sizeof(long long)) != cudaSuccess || cudaMemset(pk->d_prof, 0, 16 * sizeof(long long)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(pk->d_blob); cudaFree(pk->d_prof);
+        cudaFree(pk->d_blob); cudaFree(pk->d_stream); cudaFree(pk->d_prof);
         delete pk;
         m->err = "device allocation for the cluster-resident kernel failed";
         return WRNN_ERR_NOMEM;
@@ -1096,7 +1123,7 @@ int rescl_prepare(wrnn_model *m)
 void rescl_destroy(wrnn_model *m)
 {
     if (!m->rescl) return;
-    cudaFree(m->rescl->d_blob); cudaFree(m->rescl->d_prof);
+    cudaFree(m->rescl->d_blob); cudaFree(m->rescl->d_stream); cudaFree(m->rescl->d_prof);
     delete m->rescl;
     m->rescl = nullptr;
 }
@@ -1131,7 +1158,7 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     p.row_stride = m->cond_dim ? a.row_stride : 0;
     p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
     p.row_lag = a.row_lag; p.out_pitch = a.out_pitch ? a.out_pitch : a.n_steps;
-    p.blob = k.d_blob; p.g = m->g;
+    p.blob = k.d_blob; p.stream = k.d_stream; p.g = m->g;
     p.inv_R = k.inv_R;
     for (int h = 0; h < 2; ++h) { p.inv_O1[h] = k.inv_O1[h]; p.inv_O2[h] = k.inv_O2[h]; p.q_scale[h] = k.q_scale[h]; }
     p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
