@@ -163,7 +163,7 @@ static bool use_pair(const wrnn_model *m, int batch)
 static bool use_sparse(const wrnn_model *m, int batch)
 {
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_SPARSE) return false;
-    return m->sparse_pack != nullptr && sparse_supported(m, batch, nullptr) == WRNN_OK;
+    return (m->sparse_pack || m->sparse1) && sparse_supported(m, batch, nullptr) == WRNN_OK;
 }
 
 static bool use_bcluster(const wrnn_model *m, int batch)

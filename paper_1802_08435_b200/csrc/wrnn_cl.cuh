@@ -1,0 +1,48 @@
+// Device helpers of the kernels that keep a whole model in one thread-block cluster: named barriers, the cluster barrier, and
+// the draw and the gate functions as a single warp does them with nothing else to wait for.
+#pragma once
+#include "wrnn_device.cuh"
+
+namespace wrnn {
+
+__device__ __forceinline__ void cl_bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void cl_bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void cluster_sync_all() { asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory"); }
+// 2^x, 1 / x straight from the special-function unit (arguments and results that matter here are normal numbers)
+__device__ __forceinline__ float cl_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float cl_rcp(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+constexpr float CL_LOG2E = 1.4426950408889634f;
+__device__ __forceinline__ float cl_sigmoid(float x) { return cl_rcp(1.0f + cl_ex2(-CL_LOG2E * x)); }
+__device__ __forceinline__ float cl_tanh(float x) { return fmaf(-2.0f, cl_rcp(1.0f + cl_ex2(2.0f * CL_LOG2E * x)), 1.0f); }
+// One warp, 256 logits, lane l holds [8 l, 8 l + 8): the smallest k whose running sum of exp(l_k - max) exceeds u times the
+// total; 255 if none does.  461 -> 387 cycles against warp_softmax_draw_fast (one warp alone).
+__device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
+{
+    float m = fmaxf(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])), fmaxf(fmaxf(l[4], l[5]), fmaxf(l[6], l[7])));
+    asm("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(m));
+    m *= CL_LOG2E;
+    float w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = cl_ex2(fmaf(l[i], CL_LOG2E, -m));
+    const float p0 = w[0], p1 = w[0] + w[1], p2 = p1 + w[2], p3 = p1 + (w[2] + w[3]), p4 = p3 + w[4], p5 = p3 + (w[4] + w[5]), p6 = p5 + w[6], p7 = p5 + (w[6] + w[7]);
+    // butterfly over groups of 4, 16 and 32 lanes: the total of the block and, in `run`, the sum of its lanes below this one
+    float tot = p7, run = 0.f;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 2) {
+        const float x1 = __shfl_xor_sync(FULL, tot, o), x2 = __shfl_xor_sync(FULL, tot, 2 * o), x3 = __shfl_xor_sync(FULL, tot, 3 * o);
+        const bool odd = lane & o, up = lane & (2 * o);
+        run += (odd ? x1 : 0.f) + (up ? x2 + x3 : 0.f);
+        tot = (tot + x1) + (x2 + x3);
+    }
+    {
+        const float x = __shfl_xor_sync(FULL, tot, 16);
+        if (lane & 16) run += x;
+        tot += x;
+    }
+    const float thr = fmaf(u, tot, -run);
+    // the running sums do not decrease: the first one above the threshold comes after those that are not
+    const int c = ((p0 <= thr) + (p1 <= thr)) + ((p2 <= thr) + (p3 <= thr)) + (((p4 <= thr) + (p5 <= thr)) + ((p6 <= thr) + (p7 <= thr)));
+    return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
+}
+
+}  // namespace wrnn

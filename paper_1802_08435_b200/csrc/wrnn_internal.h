@@ -60,7 +60,8 @@ struct StepArgs {
 
 struct ResidentPack;   // packed weights of the shared-memory-resident kernels (opaque here)
 struct BatchedPack;    // fragment-packed weights and activation images of the batched kernel (opaque here)
-struct SparsePack;     // compressed block rows of the single-cluster block-sparse kernel (opaque here)
+struct SparsePack;
+struct Sparse1Pack;     // compressed block rows of the single-cluster block-sparse kernel (opaque here)
 struct ResF32Pack;     // per-CTA fp32 weight shards of the single-stream fp32 resident kernel (opaque here)
 struct ResLeanPack;      // per-CTA weights of the lean single-stream resident kernel (opaque here)
 struct ResClPack;      // per-CTA weights of the cluster-resident kernel (opaque here)
@@ -114,6 +115,7 @@ struct wrnn_model {
     bool prof_enabled = false;      // wrnn_phase_profile: the resident kernels stamp their phases
     wrnn::BatchedPack *batched = nullptr;
     wrnn::SparsePack *sparse_pack = nullptr;
+    wrnn::Sparse1Pack *sparse1 = nullptr;
     wrnn::BcPack *bcluster = nullptr;
 
     // host images for packers
@@ -200,6 +202,11 @@ int resf32_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int resf32_phase_cycles(const wrnn_model *m, long long *out16);
 
 // wrnn_sparse.cu
+// the form inside one cluster; the sparse_* functions choose
+int sparse1_prepare(wrnn_model *m);
+void sparse1_destroy(wrnn_model *m);
+void sparse1_launch_info(const wrnn_model *m, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
+int sparse1_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int sparse_supported(const wrnn_model *m, int batch, std::string *why);
 int sparse_prepare(wrnn_model *m);
 void sparse_destroy(wrnn_model *m);

@@ -553,7 +553,7 @@ static uint16_t bf16_bits_s(float rounded)
 int sparse_supported(const wrnn_model *m, int batch, std::string *why)
 {
     if (batch != 1) { if (why) *why = "single-stream kernel"; return WRNN_ERR_UNSUPPORTED; }
-    if (!m->sparse_pack) { if (why) *why = "model was not packed for the sparse cluster kernel"; return WRNN_ERR_UNSUPPORTED; }
+    if (!m->sparse_pack && !m->sparse1) { if (why) *why = "model was not packed for the sparse cluster kernel"; return WRNN_ERR_UNSUPPORTED; }
     return WRNN_OK;
 }
 
@@ -582,6 +582,9 @@ int sparse_prepare(wrnn_model *m)
     const bool tall = m->mask_br == 16 && m->mask_bc == 1;
     if (!tall && (m->mask_br != 4 || m->mask_bc != 4)) { m->err = "sparse cluster kernel takes 4 x 4 or 16 x 1 blocks"; return WRNN_ERR_UNSUPPORTED; }
     if (Hh != 1024) { m->err = "only H/2 = 1024 is instantiated (8 warps x 8 k-tiles for the logits tile)"; return WRNN_ERR_UNSUPPORTED; }
+    // One cluster with a kernel of its own where the kept blocks fit it (6.54 us per step on four clusters, SPARSE1_US in one); larger
+    // models here.
+    if (!getenv("WRNN_SPARSE_CLUSTERS") && sparse1_prepare(m) == WRNN_OK) return WRNN_OK;
     // The rows of R are dealt over NC clusters of 16 (the heads are held once per cluster); more clusters mean fewer block
     // rows per CTA in the phase that dominates the step, at the price of the state crossing the chip through L2 instead
     // of the cluster's shared memory.  The largest count that divides the units and can be co-resident is taken.
@@ -828,6 +831,7 @@ int sparse_prepare(wrnn_model *m)
 
 void sparse_destroy(wrnn_model *m)
 {
+    sparse1_destroy(m);
     if (!m->sparse_pack) return;
     cudaFree(m->sparse_pack->d_blob);
     cudaFree(m->sparse_pack->d_slots);
@@ -838,6 +842,7 @@ void sparse_destroy(wrnn_model *m)
 int sparse_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes)
 {
     (void)batch;
+    if (m->sparse1) { sparse1_launch_info(m, n_ctas, n_threads, smem, weight_bytes); return WRNN_OK; }
     const SparsePack &k = *m->sparse_pack;
     if (n_ctas) *n_ctas = SCS * k.NC;
     if (n_threads) *n_threads = SNW * 32;
@@ -848,6 +853,7 @@ int sparse_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threa
 
 int sparse_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
 {
+    if (m->sparse1) return sparse1_run(m, a, s);
     const SparsePack &k = *m->sparse_pack;
     SparseParams p;
     std::memset(&p, 0, sizeof(p));

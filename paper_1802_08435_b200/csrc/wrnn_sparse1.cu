@@ -1,0 +1,649 @@
+// Block-sparse single-stream sampling inside ONE 16-CTA cluster: bf16 weights, H = 2048, batch 1, 4 x 4 or 16 x 1 blocks, for
+// models whose kept blocks fit the shared memory of a cluster (3.6 MB: about 94 % of the blocks pruned).
+//
+// What bounds a step is the chain state -> hidden layer -> logits -> draw -> gates -> state, twice: three all-gathers per
+// half-step and what lies between them.  Inside one cluster every all-gather goes through distributed shared memory (some 700
+// cycles for 1,024 values here), where the form on four clusters (wrnn_sparse.cu) passes the state through L2 (1,250 and
+// more).  The price, four times as many rows of R per CTA, is paid off the chain:
+//   * Warps 0..7 are the chain, and each of them goes through it alone: no barrier of the CTA and no hand-over in shared memory
+//     between an arrival and the next send.  Per half-step a warp takes 8 rows of the hidden layer over all of K (kept blocks;
+//     weights and block columns are in registers before the state arrives), four rows of the logits over half of K (dense, also in
+//     registers before the hidden layer arrives; the receivers add the two halves), draws -- all eight warps the same sample --
+//     and computes the gates of 8 units.  Each of the three results is 32 bytes or less per receiver: one st.async instruction
+//     whose lanes are (piece, receiver).
+//   * Warps 8..19 multiply the rows of R (96 block rows of 4, or 24 of 16, per half) in the background, while the chain waits.
+// A result can be stored into a peer without asking: whoever sends the next one has received something that every warp of
+// every CTA sent after its last use of the present one.  That the background warps are done with the state is what warp 0 waits
+// for before it sends its logits.
+// 6.54 us per step on four clusters -> SPARSE1_US here (4 x 4 blocks, 96 %).
+//
+// Every wait is bounded; a thread that gives up skips its waits and sends from there on and keeps meeting its barriers, and
+// all CTAs leave through the final cluster barrier.
+#include <algorithm>
+#include <cstring>
+
+#include "wrnn_cl.cuh"
+#include "wrnn_cluster.cuh"
+#include "wrnn_internal.h"
+#include "wrnn_tc.cuh"
+
+namespace wrnn {
+
+namespace {
+constexpr int PK = 1024;                 // H / 2
+constexpr int PCS = 16;                  // CTAs
+constexpr int PU = PK / PCS;             // state units of one half, rows of O1 and O3 per CTA
+constexpr int PL = 16;                   // logits rows per CTA
+constexpr int PCW = 8, PBW = 12;         // chain warps, background warps
+constexpr int PTHREADS = 32 * (PCW + PBW);
+constexpr int PPRE = 2;                  // block iterations of a hidden-layer slice whose weights are loaded before the state arrives
+constexpr int PSMALL = 6 * PU * 3 + 2 * PU + 2 * PL;      // floats: I [half][gate][unit][3], b1, b3, b2, b4
+constexpr int PVEC = 3 * PK + 512 + 2 * 6 * PU;           // floats: two state halves, hidden layer, logits [half of K][256], R h (partial, complete)
+// a warp's run of block slots: `at` is its first slot, T its iterations; a slot is 32 bytes of weights (two planes of 16 bytes, for
+// the hidden rows of 16 x 1 blocks one) and a column
+struct PSlice { int at, T; int16_t row[8]; };
+}  // namespace
+
+struct Sparse1Pack {
+    uint8_t *d_blob = nullptr;
+    bool tall = false;
+    size_t blob_bytes = 0;
+    size_t off_col[4], off_val[4], off_w[2], off_small = 0;      // arrays 0, 1: hidden rows of O3, O1; 2, 3: rows of R times y_c, y_f
+    int smem_bytes = 0;
+    int64_t weight_bytes_per_step = 0;
+};
+
+struct Sparse1Params {
+    unsigned off_col[4], off_val[4], off_w[2], off_small, blob_bytes;
+    long long n_steps, step0;
+    unsigned stream0;
+    unsigned long long seed;
+    int hop, row_stride, row_offset_mul;
+    const uint8_t *blob;
+    const float *g;
+    const float *h_in; float *h_out;
+    const uint8_t *c_in, *f_in; uint8_t *c_st_out, *f_st_out;
+    const uint8_t *c_forced, *f_forced;
+    uint8_t *c_out, *f_out;
+    int16_t *out;
+    float *dbg_gates, *dbg_h, *dbg_logits;
+    DevStatus *status;
+    unsigned long long limit_ns;
+    int skip_rank; long long skip_step;      // self-test: this CTA withholds the state it publishes at this step (-1: none)
+};
+
+// acc += a block's 16 weights (row-major 4 x 4) times its four activations
+__device__ __forceinline__ void p_block(float (&acc)[4], const uint4 &w0, const uint4 &w1, const float4 &x)
+{
+    acc[0] = fmaf(bf16lo(w0.x), x.x, fmaf(bf16hi(w0.x), x.y, fmaf(bf16lo(w0.y), x.z, fmaf(bf16hi(w0.y), x.w, acc[0]))));
+    acc[1] = fmaf(bf16lo(w0.z), x.x, fmaf(bf16hi(w0.z), x.y, fmaf(bf16lo(w0.w), x.z, fmaf(bf16hi(w0.w), x.w, acc[1]))));
+    acc[2] = fmaf(bf16lo(w1.x), x.x, fmaf(bf16hi(w1.x), x.y, fmaf(bf16lo(w1.y), x.z, fmaf(bf16hi(w1.y), x.w, acc[2]))));
+    acc[3] = fmaf(bf16lo(w1.z), x.x, fmaf(bf16hi(w1.z), x.y, fmaf(bf16lo(w1.w), x.z, fmaf(bf16hi(w1.w), x.w, acc[3]))));
+}
+// acc += eight rows of one column
+__device__ __forceinline__ void p_column(float *acc, const uint4 &w, float x)
+{
+    acc[0] = fmaf(bf16lo(w.x), x, acc[0]); acc[1] = fmaf(bf16hi(w.x), x, acc[1]);
+    acc[2] = fmaf(bf16lo(w.y), x, acc[2]); acc[3] = fmaf(bf16hi(w.y), x, acc[3]);
+    acc[4] = fmaf(bf16lo(w.z), x, acc[4]); acc[5] = fmaf(bf16hi(w.z), x, acc[5]);
+    acc[6] = fmaf(bf16lo(w.w), x, acc[6]); acc[7] = fmaf(bf16hi(w.w), x, acc[7]);
+}
+// half the values of each lane change places with those of the lane `o` away: N values -> N / 2 sums; the lanes with that bit set
+// keep the upper half
+template <int N>
+__device__ __forceinline__ void p_fold(float *v, int o, int lane)
+{
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < N / 2; ++j) v[j] = (up ? v[N / 2 + j] : v[j]) + __shfl_xor_sync(FULL, up ? v[j] : v[N / 2 + j], o);
+}
+
+// MODE 0: plain sampling; MODE 1: forced symbols, dumps and the self-test predicate.  TALL: 16 x 1 blocks.
+template <int MODE, bool TALL>
+__global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1Params p)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) unsigned long long xy[2], xq, xl, xr[2];     // arrivals: state halves, hidden layer, logits; background products of a half done
+    constexpr bool DBG = MODE != 0;
+    constexpr int H = 2 * PK;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x;
+
+    const float *sI = reinterpret_cast<const float *>(smem + p.off_small);
+    const float *sb1 = sI + 6 * PU * 3, *sb3 = sb1 + PU, *sb2 = sb3 + PU, *sb4 = sb2 + PL;
+    float *vec = reinterpret_cast<float *>(smem + p.blob_bytes);         // [2: coarse, fine][PK]
+    float *qvec = vec + 2 * PK, *lbuf = qvec + PK, *r_part = lbuf + 512, *r_full = r_part + 6 * PU;
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(p.blob + (size_t)rank * p.blob_bytes);
+        uint4 *dst = reinterpret_cast<uint4 *>(smem);
+        for (unsigned i = tid; i < p.blob_bytes / 16; i += PTHREADS) dst[i] = __ldg(src + i);
+        for (int i = tid; i < H; i += PTHREADS) vec[i] = p.h_in ? p.h_in[i] : 0.f;
+        if (tid == 0) {
+            mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
+            mbar_init(smem_u32(&xr[0]), PBW); mbar_init(smem_u32(&xr[1]), PBW);
+            mbar_fence_init();
+        }
+        __syncthreads();
+    }
+    Waiter wt{p.status, p.limit_ns};
+    bool bad = false;                                                    // this thread gave up
+    auto wait_bar = [&](unsigned long long *b, unsigned parity, int step, int phase) {
+        if (bad) return;
+        const unsigned a = smem_u32(b);
+        unsigned long long t0 = 0; unsigned cnt = 0;
+        while (!mbar_try(a, parity & 1u))
+            if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { bad = true; break; }
+    };
+    const PSlice *slices = reinterpret_cast<const PSlice *>(smem);       // [2 heads][PCW], then [2 halves][PBW]
+    const long long T = p.n_steps;
+
+    // ---- rows of R (background): block rows of one half of the state, four (sixteen) lanes each
+    auto r_products = [&](int half_f) {
+        const PSlice &sl = slices[2 * PCW + half_f * PBW + warp - PCW];
+        const uint4 *wv = reinterpret_cast<const uint4 *>(smem + p.off_val[2 + half_f]) + 2 * sl.at + lane;
+        const uint16_t *wc = reinterpret_cast<const uint16_t *>(smem + p.off_col[2 + half_f]) + sl.at + lane;
+        const float *x = vec + half_f * PK;
+        const int nt = sl.T;
+        float acc[16];
+#pragma unroll
+        for (int j = 0; j < (TALL ? 16 : 4); ++j) acc[j] = 0.f;
+        uint4 w0 = wv[0], w1 = wv[32];
+        int c = wc[0];
+#pragma unroll 1
+        for (int t = 0; t < nt; ++t) {
+            const int tn = t + 1 < nt ? t + 1 : t;
+            float4 xv;
+            if (TALL) xv.x = x[c]; else xv = *reinterpret_cast<const float4 *>(x + 4 * c);
+            const uint4 w0n = wv[64 * tn], w1n = wv[64 * tn + 32];
+            c = wc[32 * tn];
+            if (TALL) { p_column(acc, w0, xv.x); p_column(acc + 8, w1, xv.x); }
+            else p_block(*reinterpret_cast<float (*)[4]>(acc), w0, w1, xv);
+            w0 = w0n; w1 = w1n;
+        }
+        if (TALL) { p_fold<16>(acc, 8, lane); p_fold<8>(acc, 4, lane); }
+        p_fold<4>(acc, 2, lane); p_fold<2>(acc, 1, lane);
+        const int row = TALL ? 16 * sl.row[lane >> 4] + (lane & 15) : 4 * sl.row[lane >> 2] + (lane & 3);
+        if (half_f) r_full[row] = r_part[row] + acc[0];
+        else r_part[row] = acc[0];
+    };
+
+    // ---- prologue: R h of the initial state
+    if (warp >= PCW) {
+        r_products(0);
+        cl_bar_sync(1, 32 * PBW);
+        r_products(1);
+    }
+    if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), 4 * PK);
+    __syncthreads();
+    cluster_sync_all();                                                  // every peer's barriers are initialised before anyone sends
+
+    if (warp >= PCW) {
+#pragma unroll 1
+        for (long long n = 0; n < 2 * T; ++n) {
+            const int half_f = (int)(n & 1);
+            wait_bar(&xy[half_f], (unsigned)(n >> 1), (int)(n >> 1), 4 + half_f);
+            cl_bar_sync(1, 32 * PBW);                                    // the other half's sums are stored
+            r_products(half_f);
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&xr[half_f])) : "memory");
+        }
+    } else {
+        const uint32_t sbase = smem_u32(smem);
+        const uint32_t dd = map_to_rank(sbase, (unsigned)(lane & 15)) - sbase;   // the CTA this lane sends to: what to add to an address of mine
+        const int piece = lane >> 4;
+        // this warp's four values of a piece: rows (units) 4 piece .. 4 piece + 3 of its eight, where row j of the eight is in lane st * j
+        auto gather4 = [&](float v, int st, float (&o)[4]) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[j] = __shfl_sync(FULL, v, st * (4 * piece + j));
+        };
+        const uint32_t a_own = sbase + p.blob_bytes + (uint32_t)((PU * rank + 8 * warp + 4 * piece) * 4) + dd;     // of this piece in vec
+        const uint32_t a_log = smem_u32(lbuf) + (uint32_t)(((warp >> 2) * 256 + PL * rank + 4 * (warp & 3)) * 4) + dd;
+        const uint32_t b_q = smem_u32(&xq) + dd, b_l = smem_u32(&xl) + dd;
+        const int skip_at = (DBG && rank == p.skip_rank) ? (int)p.skip_step : -1;
+        const bool writer = rank == 0 && warp == 0;
+
+        int c_prev = p.c_in ? p.c_in[0] : 128, f_prev = p.f_in ? p.f_in[0] : 0;
+        // gates: lane l < 8 has unit 8 warp + l of the CTA's units
+        const int gu = 8 * warp + (lane & 7), gj = PU * rank + gu;
+        float hC = vec[gj], hF = vec[PK + gj];
+        // the conditioning frame of the step, tracked without a division per step
+        const long long pos0 = p.step0 * p.row_stride + (long long)p.stream0 * p.row_offset_mul;
+        int frame = (int)(pos0 / p.hop), rem = (int)(pos0 - (long long)frame * p.hop);
+        const int dq = p.row_stride / p.hop, dr = p.row_stride - dq * p.hop;
+
+        struct GatePre { float pu, pr, pe, ae, ku, kr, ke; };
+        // what does not depend on the pending draw
+        auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
+            GatePre q;
+            const float *Iu = sI + ((half_g * 3 + 0) * PU + gu) * 3, *Ir = Iu + PU * 3, *Ie = Ir + PU * 3;
+            const float x0 = scale8(c_prev), x1 = scale8(f_prev);
+            q.pu = fmaf(Iu[0], x0, half_g ? fmaf(Iu[1], x1, gv[0]) : gv[0]);
+            q.pr = fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
+            q.pe = fmaf(Ie[0], x0, half_g ? fmaf(Ie[1], x1, gv[2]) : gv[2]);
+            q.ku = half_g ? Iu[2] : Iu[1]; q.kr = half_g ? Ir[2] : Ir[1]; q.ke = half_g ? Ie[2] : Ie[1];
+            q.pu += r_full[(half_g * 3 + 0) * PU + gu];
+            q.pr += r_full[(half_g * 3 + 1) * PU + gu];
+            q.ae = r_full[(half_g * 3 + 2) * PU + gu];
+            return q;
+        };
+        float dbg_v[4] = {0.f, 0.f, 0.f, 0.f};
+        // the gates, and the new state on its way to every CTA
+        auto gates_and_send = [&](int half_g, long long s, int drawn, const GatePre &q) {
+            const float xk = scale8(drawn);
+            const float u = cl_sigmoid(fmaf(q.ku, xk, q.pu)), r = cl_sigmoid(fmaf(q.kr, xk, q.pr));
+            const float e = cl_tanh(fmaf(r, q.ae, fmaf(q.ke, xk, q.pe)));
+            const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
+            if (half_g) hF = hn; else hC = hn;
+            float o[4];
+            gather4(hn, 1, o);
+            if (!bad && !(DBG && (int)s == skip_at))
+                st_async_v4(a_own + half_g * PK * 4, o[0], o[1], o[2], o[3], smem_u32(&xy[half_g]) + dd);
+            if (DBG) { dbg_v[0] = u; dbg_v[1] = r; dbg_v[2] = e; dbg_v[3] = hn; }
+        };
+        auto dump_gates = [&](int half_g, long long s) {
+            if (lane >= 8 || bad) return;
+            const int jj = half_g * PK + gj;
+            if (p.dbg_gates) { float *d = p.dbg_gates + (size_t)s * 3 * H; d[jj] = dbg_v[0]; d[H + jj] = dbg_v[1]; d[2 * H + jj] = dbg_v[2]; }
+            if (p.dbg_h) p.dbg_h[(size_t)s * H + jj] = dbg_v[3];
+        };
+        const float *g_unit = p.g + gj;
+        {
+            float gv[3];
+#pragma unroll
+            for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g_unit + (size_t)frame * 3 * H + gate * H);
+            gates_and_send(0, 0, f_prev, gates_prepare(0, gv));
+            if (DBG) dump_gates(0, 0);
+        }
+
+        // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
+        // n = 2 s + 2 the fine half (input y_f(s): fine head -> f_s, R h_s completed, then the coarse gates of step s + 1).
+        auto half_step = [&](auto HALF_C, const long long s) {
+            constexpr int half = decltype(HALF_C)::value;                // 1: coarse half
+            const unsigned use = (unsigned)(2 * s + (half ? 0 : 1));     // half-steps before this one
+            const bool last = !half && s == T - 1;
+            const int sn = (int)s;
+            if (tid == 0 && !bad) {
+                mbar_arrive_expect(smem_u32(&xq), 4 * PK);
+                mbar_arrive_expect(smem_u32(&xl), 2 * 256 * 4);
+                if (!last) mbar_arrive_expect(smem_u32(&xy[half]), 4 * PK);
+            }
+            if (!half) {                                                 // the coarse gates of the next step
+                frame += dq; rem += dr;
+                if (rem >= p.hop) { rem -= p.hop; ++frame; }
+            }
+            float gv[3] = {0.f, 0.f, 0.f};
+            if (!last)
+#pragma unroll
+                for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g_unit + (size_t)frame * 3 * H + half * PK + gate * H);
+            const float u01 = uniform24(p.seed, p.stream0, (unsigned long long)(p.step0 + s), half ? 0u : 1u);
+            int forced = -1;
+            if (DBG) {
+                const uint8_t *fz = half ? p.c_forced : p.f_forced;
+                if (fz) forced = fz[s];
+            }
+            // ---- 1. eight rows of the hidden layer
+            {
+                const PSlice &sl = slices[half * PCW + warp];
+                const int nt = sl.T;
+                constexpr int WS = TALL ? 32 : 64;                       // 16-byte pieces of weights per iteration
+                const uint4 *wv = reinterpret_cast<const uint4 *>(smem + p.off_val[half]) + (TALL ? 1 : 2) * sl.at + lane;
+                const uint16_t *wc = reinterpret_cast<const uint16_t *>(smem + p.off_col[half]) + sl.at + lane;
+                const float *x = vec + (half ? 0 : PK);
+                const float bias = (half ? sb1 : sb3)[8 * warp + (lane >> 2)];
+                uint4 w0[PPRE], w1[PPRE];
+                int c[PPRE];
+#pragma unroll
+                for (int t = 0; t < PPRE; ++t) { w0[t] = wv[t * WS]; if (!TALL) w1[t] = wv[t * WS + 32]; c[t] = wc[32 * t]; }
+                float acc[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+                wait_bar(&xy[half ? 0 : 1], (unsigned)s, sn, 1 + 4 * half);
+                float4 xv[PPRE];
+#pragma unroll
+                for (int t = 0; t < PPRE; ++t) { if (TALL) xv[t].x = x[c[t]]; else xv[t] = *reinterpret_cast<const float4 *>(x + 4 * c[t]); }
+#pragma unroll
+                for (int t = 0; t < PPRE; ++t) { if (TALL) p_column(acc, w0[t], xv[t].x); else p_block(*reinterpret_cast<float (*)[4]>(acc + 4 * (t & 1)), w0[t], w1[t], xv[t]); }
+#pragma unroll 1
+                for (int t = PPRE; t < nt; ++t) {
+                    const int ct = wc[32 * t];
+                    if (TALL) p_column(acc, wv[t * WS], x[ct]);
+                    else p_block(*reinterpret_cast<float (*)[4]>(acc), wv[t * WS], wv[t * WS + 32], *reinterpret_cast<const float4 *>(x + 4 * ct));
+                }
+                // row lane >> 2 of the warp's eight, in all four lanes
+                if (TALL) p_fold<8>(acc, 16, lane);
+                else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[j] += acc[4 + j];
+                }
+                p_fold<4>(acc, 8, lane); p_fold<2>(acc, 4, lane);
+                float v = acc[0];
+                v += __shfl_xor_sync(FULL, v, 2);
+                v += __shfl_xor_sync(FULL, v, 1);
+                v = fmaxf(v + bias, 0.f);
+                float o[4];
+                gather4(v, 4, o);
+                if (!bad) st_async_v4(a_own + 2 * PK * 4, o[0], o[1], o[2], o[3], b_q);
+            }
+            // ---- 2. four rows of the logits, half of K: lane takes runs of four values, 128 apart
+            {
+                const int kh = warp >> 2, r0 = 4 * (warp & 3);
+                const uint2 *w2 = reinterpret_cast<const uint2 *>(smem + p.off_w[half]) + (size_t)(r0 * 2 + kh) * (PK / 8) + lane;   // [row][K / 4]
+                uint2 w[4][4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) w[r][j] = w2[r * (PK / 4) + 32 * j];
+                const float bias = kh ? 0.f : (half ? sb2 : sb4)[r0 + (lane >> 3)];
+                if (!half && warp == 0) wait_bar(&xr[0], (unsigned)s, sn, 6);    // the background warps are done with y_c(s)
+                wait_bar(&xq, use, sn, 2 + 4 * half);
+                const float4 *q4 = reinterpret_cast<const float4 *>(qvec) + kh * (PK / 8) + lane;
+                float4 q[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) q[j] = q4[32 * j];
+                float v[4] = {0.f, 0.f, 0.f, 0.f}, v2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        v[r] = fmaf(bf16lo(w[r][j].x), q[j].x, v[r]); v2[r] = fmaf(bf16hi(w[r][j].x), q[j].y, v2[r]);
+                        v[r] = fmaf(bf16lo(w[r][j].y), q[j].z, v[r]); v2[r] = fmaf(bf16hi(w[r][j].y), q[j].w, v2[r]);
+                    }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) v[r] += v2[r];
+                p_fold<4>(v, 16, lane); p_fold<2>(v, 8, lane);
+                float x = v[0];
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+                x += bias;
+                float o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[j] = __shfl_sync(FULL, x, 8 * j);
+                if (lane < 16 && !bad) st_async_v4(a_log, o[0], o[1], o[2], o[3], b_l);
+            }
+            // ---- 3. draw and gates
+            if (!half) wait_bar(&xr[1], (unsigned)s, sn, 7);                        // R h is complete
+            const GatePre gp = gates_prepare(half, gv);
+            wait_bar(&xl, use, sn, 3 + 4 * half);
+            float l[8];
+            {
+                const float4 *L = reinterpret_cast<const float4 *>(lbuf) + 2 * lane;
+                const float4 a = L[0], b = L[1], a2 = L[64], b2 = L[65];
+                l[0] = a.x + a2.x; l[1] = a.y + a2.y; l[2] = a.z + a2.z; l[3] = a.w + a2.w;
+                l[4] = b.x + b2.x; l[5] = b.y + b2.y; l[6] = b.z + b2.z; l[7] = b.w + b2.w;
+            }
+            const int drawn = cl_draw(l, u01, lane);
+            const int fed = (DBG && forced >= 0) ? forced : drawn;
+            if (!last) gates_and_send(half, half ? s : s + 1, fed, gp);
+            if (half) c_prev = fed; else f_prev = fed;
+            // the samples (and the dumps) leave when the state is on its way
+            if (DBG && !last) dump_gates(half, half ? s : s + 1);
+            if (writer && !bad) {
+                if (DBG && p.dbg_logits) {
+                    float *d = p.dbg_logits + ((size_t)2 * s + (half ? 0 : 1)) * 256 + 8 * lane;
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) d[k] = l[k];
+                }
+                if (lane == 0) {
+                    if (DBG) { uint8_t *o = half ? p.c_out : p.f_out; if (o) o[s] = (uint8_t)drawn; }
+                    if (!half && p.out) p.out[s] = (int16_t)(256 * c_prev + drawn - 32768);
+                }
+            }
+        };
+#pragma unroll 1
+        for (long long s = 0; s < T; ++s) {
+            half_step(std::integral_constant<int, 1>{}, s);
+            half_step(std::integral_constant<int, 0>{}, s);
+        }
+        if (writer && lane == 0 && !bad) {
+            if (p.c_st_out) p.c_st_out[0] = (uint8_t)c_prev;
+            if (p.f_st_out) p.f_st_out[0] = (uint8_t)f_prev;
+        }
+    }
+    // ---- results; nobody leaves while a peer may still write into its shared memory
+    const int any_bad = __syncthreads_or(bad);
+    if (rank == 0 && !any_bad && p.h_out)
+        for (int i = tid; i < H; i += PTHREADS) p.h_out[i] = vec[i];
+    cluster_sync_all();
+}
+
+// ---------------------------------------------------------------------------------------------
+static const void *p_fn(bool dbg, bool tall)
+{
+    if (tall) return dbg ? (const void *)sparse_chain_kernel<1, true> : (const void *)sparse_chain_kernel<0, true>;
+    return dbg ? (const void *)sparse_chain_kernel<1, false> : (const void *)sparse_chain_kernel<0, false>;
+}
+
+static void p_fill_launch(int smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
+{
+    std::memset(cfg, 0, sizeof(*cfg));
+    cfg->gridDim = dim3(PCS);
+    cfg->blockDim = dim3(PTHREADS);
+    cfg->dynamicSmemBytes = smem;
+    cfg->stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = PCS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+
+static uint16_t p_bf16(float rounded)
+{
+    uint32_t b;
+    std::memcpy(&b, &rounded, 4);
+    return (uint16_t)(b >> 16);
+}
+
+// m: a block-sparse bf16 model with H = 2048 and 4 x 4 or 16 x 1 blocks (sparse_prepare has checked that)
+int sparse1_prepare(wrnn_model *m)
+{
+    const int H = 2 * PK, Kb = PK / 4;
+    const bool tall = m->mask_br == 16;
+    const int BRH = tall ? 16 : 4, lpr = tall ? 16 : 4, rpw = 32 / lpr;          // rows of a block; lanes per block row and block rows per background warp
+    const int nbr = 6 * PU / BRH;                                                // block rows of R per CTA and half: all the background warps can take
+    static_assert(6 * PU / 4 == PBW * 8 && 6 * PU / 16 == PBW * 2, "the background warps take the rows of R in one go");
+
+    struct Blk { uint16_t col; float v[16]; };                                   // 4 x 4 row-major, or the 16 rows of a column
+    // kept blocks of one block row of M, in the columns of one half
+    auto row_blocks = [&](const BsrHost &M, int br0, int bc_lo, std::vector<Blk> *out) {
+        out->clear();
+        std::vector<int> slot(tall ? PK : 0, -1);
+        for (int r4 = 0; r4 < BRH / 4; ++r4)
+            for (int i = M.row_ptr[br0 + r4]; i < M.row_ptr[br0 + r4 + 1]; ++i) {
+                const int bc = M.col[i] - bc_lo;
+                if (bc < 0 || bc >= Kb) continue;
+                const float *v = &M.vals[(size_t)i * 16];
+                if (!tall) {
+                    Blk b;
+                    b.col = (uint16_t)bc;
+                    std::memcpy(b.v, v, sizeof(b.v));
+                    out->push_back(b);
+                    continue;
+                }
+                for (int c = 0; c < 4; ++c) {
+                    if (v[c] == 0.f && v[4 + c] == 0.f && v[8 + c] == 0.f && v[12 + c] == 0.f) continue;
+                    const int col = 4 * bc + c;
+                    if (slot[col] < 0) { slot[col] = (int)out->size(); Blk b; b.col = (uint16_t)col; std::memset(b.v, 0, sizeof(b.v)); out->push_back(b); }
+                    for (int r = 0; r < 4; ++r) (*out)[slot[col]].v[4 * r4 + r] = v[4 * r + c];
+                }
+            }
+        std::sort(out->begin(), out->end(), [](const Blk &a, const Blk &b) { return a.col < b.col; });
+    };
+
+    // block rows of every CTA and array: 0, 1: O3, O1 (PU rows); 2, 3: R times the coarse, fine half
+    std::vector<std::vector<Blk>> rows[PCS][4];
+    int64_t kept = 0;
+    for (int cta = 0; cta < PCS; ++cta)
+        for (int a = 0; a < 4; ++a) {
+            auto &R = rows[cta][a];
+            R.resize(a < 2 ? PU / BRH : nbr);
+            for (int b = 0; b < (int)R.size(); ++b) {
+                if (a < 2) row_blocks(a ? m->hO1 : m->hO3, (cta * PU + b * BRH) / 4, 0, &R[b]);
+                else {
+                    const int per = PU / BRH, half = b / (3 * per), gate = (b / per) % 3, u = b % per;
+                    row_blocks(m->hR, (gate * H + half * PK + cta * PU + u * BRH) / 4, (a - 2) * Kb, &R[b]);
+                }
+                kept += (int64_t)R[b].size();
+            }
+        }
+
+    // slices: [array][warp]; slots of a warp are 32 lanes x T iterations
+    std::vector<PSlice> slices((size_t)PCS * 2 * (PCW + PBW));
+    std::vector<std::vector<int>> order((size_t)PCS * 4);
+    int slots[4] = {0, 0, 0, 0};
+    for (int cta = 0; cta < PCS; ++cta)
+        for (int a = 0; a < 4; ++a) {
+            const auto &R = rows[cta][a];
+            auto &ord = order[cta * 4 + a];
+            for (int i = 0; i < (int)R.size(); ++i) ord.push_back(i);
+            if (a >= 2) std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return R[x].size() > R[y].size(); });
+            int at = 0;
+            for (int w = 0; w < (a < 2 ? PCW : PBW); ++w) {
+                PSlice &sl = slices[(size_t)cta * 2 * (PCW + PBW) + (a < 2 ? a * PCW : 2 * PCW + (a - 2) * PBW) + w];
+                std::memset(&sl, 0, sizeof(sl));
+                size_t longest = 0;
+                if (a < 2) {
+                    if (tall) longest = (R[w >> 1].size() + 31) / 32;                              // half a block row over 32 lanes
+                    else for (int b = 0; b < 2; ++b) longest = std::max(longest, (R[2 * w + b].size() + 15) / 16);
+                    longest = std::max(longest, (size_t)PPRE);
+                } else {
+                    for (int b = 0; b < rpw; ++b) { sl.row[b] = (int16_t)ord[w * rpw + b]; longest = std::max(longest, (R[ord[w * rpw + b]].size() + lpr - 1) / lpr); }
+                    longest = std::max(longest, (size_t)1);                                        // the loop's first loads are unconditional
+                }
+                sl.at = at; sl.T = (int)longest;
+                at += 32 * sl.T;
+            }
+            slots[a] = std::max(slots[a], at);
+        }
+
+    Sparse1Pack k;
+    k.tall = tall;
+    auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    size_t off = a16(sizeof(PSlice) * 2 * (PCW + PBW));
+    for (int a = 0; a < 4; ++a) {
+        k.off_val[a] = off; off += (size_t)slots[a] * (a < 2 && tall ? 16 : 32);
+        k.off_col[a] = off; off = a16(off + (size_t)slots[a] * 2);
+    }
+    for (int h = 0; h < 2; ++h) { k.off_w[h] = off; off += (size_t)PL * PK * 2; }
+    k.off_small = off; off = a16(off + (size_t)PSMALL * 4);
+    k.blob_bytes = off;
+    const size_t smem = off + (size_t)PVEC * 4;
+    cudaDeviceProp prop;
+    if (cudaGetDeviceProperties(&prop, m->device) != cudaSuccess) { cudaGetLastError(); return WRNN_ERR_CUDA; }
+    if (smem > prop.sharedMemPerBlockOptin - 256) { m->err = "pruned model does not fit the shared memory of one cluster"; return WRNN_ERR_UNSUPPORTED; }
+    k.smem_bytes = (int)smem;
+    for (int dbg = 0; dbg < 2; ++dbg)
+        if (cudaFuncSetAttribute(p_fn(dbg, tall), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaFuncSetAttribute(p_fn(dbg, tall), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(prop.sharedMemPerBlockOptin - 256)) != cudaSuccess) {
+            cudaGetLastError(); m->err = "cannot configure the 16-CTA cluster kernel"; return WRNN_ERR_UNSUPPORTED;
+        }
+    cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
+    p_fill_launch(k.smem_bytes, &cfg, at, 0);
+    int max_clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&max_clusters, p_fn(false, tall), &cfg) != cudaSuccess || max_clusters < 1) {
+        cudaGetLastError(); m->err = "a 16-CTA cluster cannot be resident on this device"; return WRNN_ERR_UNSUPPORTED;
+    }
+
+    std::vector<uint8_t> blob((size_t)PCS * k.blob_bytes, 0);
+    for (int cta = 0; cta < PCS; ++cta) {
+        uint8_t *base = blob.data() + (size_t)cta * k.blob_bytes;
+        std::memcpy(base, &slices[(size_t)cta * 2 * (PCW + PBW)], sizeof(PSlice) * 2 * (PCW + PBW));
+        const PSlice *sls = reinterpret_cast<const PSlice *>(base);
+        for (int a = 0; a < 4; ++a) {
+            uint16_t *col = reinterpret_cast<uint16_t *>(base + k.off_col[a]), *val = reinterpret_cast<uint16_t *>(base + k.off_val[a]);
+            const bool thin = a < 2 && tall;                                     // a slot holds eight rows of a column
+            for (int w = 0; w < (a < 2 ? PCW : PBW); ++w) {
+                const PSlice &sl = sls[(a < 2 ? a * PCW : 2 * PCW + (a - 2) * PBW) + w];
+                const int nb = thin ? 1 : a < 2 ? 2 : rpw, nl = 32 / nb;         // block rows of the warp, lanes of each
+                for (int g = 0; g < nb; ++g) {
+                    const auto &blocks = rows[cta][a][thin ? w >> 1 : a < 2 ? 2 * w + g : sl.row[g]];
+                    for (int i = 0; i < (int)blocks.size(); ++i) {
+                        const int t = i / nl, lane = nl * g + i % nl;
+                        col[sl.at + 32 * t + lane] = blocks[i].col;
+                        for (int h = 0; h < (thin ? 1 : 2); ++h)
+                            for (int e = 0; e < 8; ++e)
+                                val[thin ? ((size_t)sl.at + 32 * t + lane) * 8 + e : ((size_t)2 * sl.at + 64 * t + 32 * h + lane) * 8 + e] =
+                                    p_bf16(blocks[i].v[thin ? 8 * (w & 1) + e : 8 * h + e]);
+                    }
+                }
+            }
+        }
+        for (int h = 0; h < 2; ++h) {                                            // dense rows, as bf16: O4, O2
+            const BsrHost &M = h ? m->hO2 : m->hO4;
+            uint16_t *d = reinterpret_cast<uint16_t *>(base + k.off_w[h]);
+            for (int r = 0; r < PL; ++r) {
+                const int br = (cta * PL + r) / 4, rr = r % 4;
+                for (int i = M.row_ptr[br]; i < M.row_ptr[br + 1]; ++i)
+                    for (int c = 0; c < 4; ++c) d[(size_t)r * PK + 4 * M.col[i] + c] = p_bf16(M.vals[(size_t)i * 16 + 4 * rr + c]);
+            }
+        }
+        float *sm = reinterpret_cast<float *>(base + k.off_small);
+        for (int r = 0; r < 6 * PU; ++r) {
+            const int half = r / (3 * PU), gate = (r / PU) % 3, u = r % PU;
+            for (int c = 0; c < 3; ++c) sm[3 * r + c] = m->hI[(size_t)(gate * H + half * PK + cta * PU + u) * 3 + c];
+        }
+        sm += 6 * PU * 3;
+        for (int r = 0; r < PU; ++r) { sm[r] = m->hb1[cta * PU + r]; sm[PU + r] = m->hb3[cta * PU + r]; }
+        sm += 2 * PU;
+        for (int r = 0; r < PL; ++r) { sm[r] = m->hb2[cta * PL + r]; sm[PL + r] = m->hb4[cta * PL + r]; }
+    }
+    if (cudaMalloc((void **)&k.d_blob, blob.size()) != cudaSuccess || cudaMemcpy(k.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaGetLastError(); cudaFree(k.d_blob);
+        m->err = "device allocation for the sparse cluster kernel failed";
+        return WRNN_ERR_NOMEM;
+    }
+    // kept blocks and their columns once, row pointers, the dense O2, O4 and I
+    k.weight_bytes_per_step = kept * 34 + (int64_t)PCS * 2 * (PU / BRH + nbr + 1) * 4 + (int64_t)2 * 256 * PK * 2 + (int64_t)3 * H * 3 * 4;
+    m->sparse1 = new Sparse1Pack(k);
+    return WRNN_OK;
+}
+
+void sparse1_destroy(wrnn_model *m)
+{
+    if (!m->sparse1) return;
+    cudaFree(m->sparse1->d_blob);
+    delete m->sparse1;
+    m->sparse1 = nullptr;
+}
+
+void sparse1_launch_info(const wrnn_model *m, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes)
+{
+    if (n_ctas) *n_ctas = PCS;
+    if (n_threads) *n_threads = PTHREADS;
+    if (smem) *smem = m->sparse1->smem_bytes;
+    if (weight_bytes) *weight_bytes = m->sparse1->weight_bytes_per_step;
+}
+
+int sparse1_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
+{
+    const Sparse1Pack &k = *m->sparse1;
+    Sparse1Params p;
+    std::memset(&p, 0, sizeof(p));
+    for (int i = 0; i < 4; ++i) { p.off_col[i] = (unsigned)k.off_col[i]; p.off_val[i] = (unsigned)k.off_val[i]; }
+    p.off_w[0] = (unsigned)k.off_w[0]; p.off_w[1] = (unsigned)k.off_w[1]; p.off_small = (unsigned)k.off_small; p.blob_bytes = (unsigned)k.blob_bytes;
+    p.n_steps = a.n_steps; p.step0 = a.step0; p.stream0 = a.stream0; p.seed = a.seed;
+    p.hop = m->cond_dim ? a.hop : 1;
+    p.row_stride = m->cond_dim ? a.row_stride : 0;
+    p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
+    p.blob = k.d_blob; p.g = m->g;
+    p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
+    p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
+    p.dbg_gates = a.dbg_gates; p.dbg_h = a.dbg_h; p.dbg_logits = a.dbg_logits;
+    p.status = m->status;
+    p.limit_ns = m->wait_limit_ns();
+    p.skip_rank = m->dbg_skip_cta; p.skip_step = m->dbg_skip_step;
+    if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
+    const bool dbg = m->dbg_skip_cta >= 0 || p.c_forced || p.f_forced || p.c_out || p.f_out || p.dbg_gates || p.dbg_h || p.dbg_logits;
+    cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
+    p_fill_launch(k.smem_bytes, &cfg, at, s);
+    void *args[] = {&p};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, p_fn(dbg, k.tall), args);
+    if (e != cudaSuccess) {
+        m->err = std::string("sparse cluster kernel launch failed: ") + cudaGetErrorString(e);
+        cudaGetLastError();
+        return WRNN_ERR_CUDA;
+    }
+    ++g_launches;
+    return WRNN_OK;
+}
+
+}  // namespace wrnn
