@@ -36,9 +36,10 @@ constexpr int PU = PK / PCS;             // state units of one half, rows of O1 
 constexpr int PL = 16;                   // logits rows per CTA
 constexpr int PCW = 8, PBW = 12;         // chain warps, background warps
 constexpr int PTHREADS = 32 * (PCW + PBW);
-constexpr int PPRE = 2;                  // block iterations of a hidden-layer slice whose weights are loaded before the state arrives
+constexpr int PPRE = 2, BPRE = 3;        // iterations of a hidden-layer slice, of a slice of R, whose weights are loaded before the state arrives
 constexpr int PSMALL = 6 * PU * 3 + 2 * PU + 2 * PL;      // floats: I [half][gate][unit][3], b1, b3, b2, b4
-constexpr int PVEC = 3 * PK + 512 + 2 * 6 * PU;           // floats: two state halves, hidden layer, logits [half of K][256], R h (partial, complete)
+constexpr int PDW = PU / 32;             // drawing warps: one unit per lane
+constexpr int PVEC = 3 * PK + 256 + 2 * 6 * PU + 2 * PU + 2 * PL;       // floats: two state halves, hidden layer, logits, R h (partial, complete), staged y, q, logits
 // a warp's run of block slots: `at` is its first slot, T its iterations; a slot is 32 bytes of weights (two planes of 16 bytes, for
 // the hidden rows of 16 x 1 blocks one) and a column
 struct PSlice { int at, T; int16_t row[8]; };
@@ -103,7 +104,7 @@ template <int MODE, bool TALL>
 __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1Params p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ __align__(8) unsigned long long xy[2], xq, xl, xr[2];     // arrivals: state halves, hidden layer, logits; background products of a half done
+    __shared__ __align__(8) unsigned long long xy[2], xq, xl, xg[2], xr[2];   // arrivals: state halves, hidden layer, logits; background products of a half: may start, done
     constexpr bool DBG = MODE != 0;
     constexpr int H = 2 * PK;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -112,7 +113,8 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     const float *sI = reinterpret_cast<const float *>(smem + p.off_small);
     const float *sb1 = sI + 6 * PU * 3, *sb3 = sb1 + PU, *sb2 = sb3 + PU, *sb4 = sb2 + PL;
     float *vec = reinterpret_cast<float *>(smem + p.blob_bytes);         // [2: coarse, fine][PK]
-    float *qvec = vec + 2 * PK, *lbuf = qvec + PK, *r_part = lbuf + 512, *r_full = r_part + 6 * PU;
+    float *qvec = vec + 2 * PK, *lbuf = qvec + PK, *r_part = lbuf + 256, *r_full = r_part + 6 * PU;
+    float *ystage = r_full + 6 * PU, *qstage = ystage + PU, *lstage = qstage + PU;
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(p.blob + (size_t)rank * p.blob_bytes);
         uint4 *dst = reinterpret_cast<uint4 *>(smem);
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
         for (int i = tid; i < H; i += PTHREADS) vec[i] = p.h_in ? p.h_in[i] : 0.f;
         if (tid == 0) {
             mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
+            mbar_init(smem_u32(&xg[0]), PCW); mbar_init(smem_u32(&xg[1]), PCW);
             mbar_init(smem_u32(&xr[0]), PBW); mbar_init(smem_u32(&xr[1]), PBW);
             mbar_fence_init();
         }
@@ -137,41 +140,48 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     const PSlice *slices = reinterpret_cast<const PSlice *>(smem);       // [2 heads][PCW], then [2 halves][PBW]
     const long long T = p.n_steps;
 
-    // ---- rows of R (background): block rows of one half of the state, four (sixteen) lanes each
-    auto r_products = [&](int half_f) {
+    // ---- rows of R (background): block rows of one half of the state, four (sixteen) lanes each; `start` is called when the weights of
+    // the first BPRE iterations (as a rule all of them) are in registers
+    auto r_products = [&](int half_f, auto start) {
         const PSlice &sl = slices[2 * PCW + half_f * PBW + warp - PCW];
         const uint4 *wv = reinterpret_cast<const uint4 *>(smem + p.off_val[2 + half_f]) + 2 * sl.at + lane;
         const uint16_t *wc = reinterpret_cast<const uint16_t *>(smem + p.off_col[2 + half_f]) + sl.at + lane;
         const float *x = vec + half_f * PK;
         const int nt = sl.T;
+        const int row = TALL ? 16 * sl.row[lane >> 4] + (lane & 15) : 4 * sl.row[lane >> 2] + (lane & 3);
+        uint4 w0[BPRE], w1[BPRE];
+        int c[BPRE];
+#pragma unroll
+        for (int t = 0; t < BPRE; ++t) { w0[t] = wv[64 * t]; w1[t] = wv[64 * t + 32]; c[t] = wc[32 * t]; }
         float acc[16];
 #pragma unroll
         for (int j = 0; j < (TALL ? 16 : 4); ++j) acc[j] = 0.f;
-        uint4 w0 = wv[0], w1 = wv[32];
-        int c = wc[0];
+        start();
+        float4 xv[BPRE];
+#pragma unroll
+        for (int t = 0; t < BPRE; ++t) { if (TALL) xv[t].x = x[c[t]]; else xv[t] = *reinterpret_cast<const float4 *>(x + 4 * c[t]); }
+#pragma unroll
+        for (int t = 0; t < BPRE; ++t) {
+            if (TALL) { p_column(acc, w0[t], xv[t].x); p_column(acc + 8, w1[t], xv[t].x); }
+            else p_block(*reinterpret_cast<float (*)[4]>(acc), w0[t], w1[t], xv[t]);
+        }
 #pragma unroll 1
-        for (int t = 0; t < nt; ++t) {
-            const int tn = t + 1 < nt ? t + 1 : t;
-            float4 xv;
-            if (TALL) xv.x = x[c]; else xv = *reinterpret_cast<const float4 *>(x + 4 * c);
-            const uint4 w0n = wv[64 * tn], w1n = wv[64 * tn + 32];
-            c = wc[32 * tn];
-            if (TALL) { p_column(acc, w0, xv.x); p_column(acc + 8, w1, xv.x); }
-            else p_block(*reinterpret_cast<float (*)[4]>(acc), w0, w1, xv);
-            w0 = w0n; w1 = w1n;
+        for (int t = BPRE; t < nt; ++t) {
+            const int ct = wc[32 * t];
+            if (TALL) { const float xs = x[ct]; p_column(acc, wv[64 * t], xs); p_column(acc + 8, wv[64 * t + 32], xs); }
+            else p_block(*reinterpret_cast<float (*)[4]>(acc), wv[64 * t], wv[64 * t + 32], *reinterpret_cast<const float4 *>(x + 4 * ct));
         }
         if (TALL) { p_fold<16>(acc, 8, lane); p_fold<8>(acc, 4, lane); }
         p_fold<4>(acc, 2, lane); p_fold<2>(acc, 1, lane);
-        const int row = TALL ? 16 * sl.row[lane >> 4] + (lane & 15) : 4 * sl.row[lane >> 2] + (lane & 3);
         if (half_f) r_full[row] = r_part[row] + acc[0];
         else r_part[row] = acc[0];
     };
 
     // ---- prologue: R h of the initial state
     if (warp >= PCW) {
-        r_products(0);
+        r_products(0, [] {});
         cl_bar_sync(1, 32 * PBW);
-        r_products(1);
+        r_products(1, [] {});
     }
     if (tid == 0) mbar_arrive_expect(smem_u32(&xy[0]), 4 * PK);
     __syncthreads();
@@ -181,30 +191,27 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
 #pragma unroll 1
         for (long long n = 0; n < 2 * T; ++n) {
             const int half_f = (int)(n & 1);
-            wait_bar(&xy[half_f], (unsigned)(n >> 1), (int)(n >> 1), 4 + half_f);
-            cl_bar_sync(1, 32 * PBW);                                    // the other half's sums are stored
-            r_products(half_f);
+            r_products(half_f, [&] {
+                cl_bar_sync(1, 32 * PBW);                                // the other half's sums are stored
+                wait_bar(&xg[half_f], (unsigned)(n >> 1), (int)(n >> 1), 4 + half_f);
+            });
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&xr[half_f])) : "memory");
         }
     } else {
         const uint32_t sbase = smem_u32(smem);
-        const uint32_t dd = map_to_rank(sbase, (unsigned)(lane & 15)) - sbase;   // the CTA this lane sends to: what to add to an address of mine
-        const int piece = lane >> 4;
-        // this warp's four values of a piece: rows (units) 4 piece .. 4 piece + 3 of its eight, where row j of the eight is in lane st * j
-        auto gather4 = [&](float v, int st, float (&o)[4]) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) o[j] = __shfl_sync(FULL, v, st * (4 * piece + j));
-        };
-        const uint32_t a_own = sbase + p.blob_bytes + (uint32_t)((PU * rank + 8 * warp + 4 * piece) * 4) + dd;     // of this piece in vec
-        const uint32_t a_log = smem_u32(lbuf) + (uint32_t)(((warp >> 2) * 256 + PL * rank + 4 * (warp & 3)) * 4) + dd;
+        // what this warp sends goes to CTAs 2 warp and 2 warp + 1, in runs of 256 bytes (64 of the logits): lane = (CTA, 16-byte piece)
+        const uint32_t dd = map_to_rank(sbase, (unsigned)(2 * warp + (lane >> 4))) - sbase;    // what to add to an address of mine
+        const int piece = lane & 15;
+        const uint32_t a_own = sbase + p.blob_bytes + (uint32_t)((PU * rank + 4 * piece) * 4) + dd;                // of this piece in vec
+        const uint32_t a_log = smem_u32(lbuf) + (uint32_t)((PL * rank + 4 * piece) * 4) + dd;
         const uint32_t b_q = smem_u32(&xq) + dd, b_l = smem_u32(&xl) + dd;
         const int skip_at = (DBG && rank == p.skip_rank) ? (int)p.skip_step : -1;
         const bool writer = rank == 0 && warp == 0;
 
         int c_prev = p.c_in ? p.c_in[0] : 128, f_prev = p.f_in ? p.f_in[0] : 0;
-        // gates: lane l < 8 has unit 8 warp + l of the CTA's units
-        const int gu = 8 * warp + (lane & 7), gj = PU * rank + gu;
+        const bool drawer = warp < PDW;                                  // gates: lane l has unit 32 warp + l of the CTA's units
+        const int gu = drawer ? 32 * warp + lane : 0, gj = PU * rank + gu;
         float hC = vec[gj], hF = vec[PK + gj];
         // the conditioning frame of the step, tracked without a division per step
         const long long pos0 = p.step0 * p.row_stride + (long long)p.stream0 * p.row_offset_mul;
@@ -221,39 +228,43 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
             q.pr = fmaf(Ir[0], x0, half_g ? fmaf(Ir[1], x1, gv[1]) : gv[1]);
             q.pe = fmaf(Ie[0], x0, half_g ? fmaf(Ie[1], x1, gv[2]) : gv[2]);
             q.ku = half_g ? Iu[2] : Iu[1]; q.kr = half_g ? Ir[2] : Ir[1]; q.ke = half_g ? Ie[2] : Ie[1];
-            q.pu += r_full[(half_g * 3 + 0) * PU + gu];
-            q.pr += r_full[(half_g * 3 + 1) * PU + gu];
-            q.ae = r_full[(half_g * 3 + 2) * PU + gu];
+            q.ae = 0.f;
             return q;
         };
         float dbg_v[4] = {0.f, 0.f, 0.f, 0.f};
-        // the gates, and the new state on its way to every CTA
-        auto gates_and_send = [&](int half_g, long long s, int drawn, const GatePre &q) {
+        auto send_y = [&](int half_g, long long s) {
+            const float4 v = reinterpret_cast<const float4 *>(ystage)[piece];
+            if (!bad && !(DBG && (int)s == skip_at)) st_async_v4(a_own + half_g * PK * 4, v.x, v.y, v.z, v.w, smem_u32(&xy[half_g]) + dd);
+        };
+        auto gates = [&](int half_g, long long s, int drawn, GatePre &q) {
+            q.pu += r_full[(half_g * 3 + 0) * PU + gu];
+            q.pr += r_full[(half_g * 3 + 1) * PU + gu];
+            q.ae = r_full[(half_g * 3 + 2) * PU + gu];
             const float xk = scale8(drawn);
             const float u = cl_sigmoid(fmaf(q.ku, xk, q.pu)), r = cl_sigmoid(fmaf(q.kr, xk, q.pr));
             const float e = cl_tanh(fmaf(r, q.ae, fmaf(q.ke, xk, q.pe)));
             const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
             if (half_g) hF = hn; else hC = hn;
-            float o[4];
-            gather4(hn, 1, o);
-            if (!bad && !(DBG && (int)s == skip_at))
-                st_async_v4(a_own + half_g * PK * 4, o[0], o[1], o[2], o[3], smem_u32(&xy[half_g]) + dd);
+            ystage[gu] = hn;
             if (DBG) { dbg_v[0] = u; dbg_v[1] = r; dbg_v[2] = e; dbg_v[3] = hn; }
         };
         auto dump_gates = [&](int half_g, long long s) {
-            if (lane >= 8 || bad) return;
+            if (!drawer || bad) return;
             const int jj = half_g * PK + gj;
             if (p.dbg_gates) { float *d = p.dbg_gates + (size_t)s * 3 * H; d[jj] = dbg_v[0]; d[H + jj] = dbg_v[1]; d[2 * H + jj] = dbg_v[2]; }
             if (p.dbg_h) p.dbg_h[(size_t)s * H + jj] = dbg_v[3];
         };
         const float *g_unit = p.g + gj;
-        {
+        if (drawer) {
             float gv[3];
 #pragma unroll
             for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g_unit + (size_t)frame * 3 * H + gate * H);
-            gates_and_send(0, 0, f_prev, gates_prepare(0, gv));
-            if (DBG) dump_gates(0, 0);
+            GatePre gp = gates_prepare(0, gv);
+            gates(0, 0, f_prev, gp);
         }
+        cl_bar_sync(2, 32 * PCW);
+        send_y(0, 0);
+        if (DBG) dump_gates(0, 0);
 
         // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),
         // n = 2 s + 2 the fine half (input y_f(s): fine head -> f_s, R h_s completed, then the coarse gates of step s + 1).
@@ -264,7 +275,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
             const int sn = (int)s;
             if (tid == 0 && !bad) {
                 mbar_arrive_expect(smem_u32(&xq), 4 * PK);
-                mbar_arrive_expect(smem_u32(&xl), 2 * 256 * 4);
+                mbar_arrive_expect(smem_u32(&xl), 256 * 4);
                 if (!last) mbar_arrive_expect(smem_u32(&xy[half]), 4 * PK);
             }
             if (!half) {                                                 // the coarse gates of the next step
@@ -272,11 +283,14 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
                 if (rem >= p.hop) { rem -= p.hop; ++frame; }
             }
             float gv[3] = {0.f, 0.f, 0.f};
-            if (!last)
-#pragma unroll
-                for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g_unit + (size_t)frame * 3 * H + half * PK + gate * H);
-            const float u01 = uniform24(p.seed, p.stream0, (unsigned long long)(p.step0 + s), half ? 0u : 1u);
+            float u01 = 0.f;
             int forced = -1;
+            if (drawer) {
+                if (!last)
+#pragma unroll
+                    for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g_unit + (size_t)frame * 3 * H + half * PK + gate * H);
+                u01 = uniform24(p.seed, p.stream0, (unsigned long long)(p.step0 + s), half ? 0u : 1u);
+            }
             if (DBG) {
                 const uint8_t *fz = half ? p.c_forced : p.f_forced;
                 if (fz) forced = fz[s];
@@ -320,9 +334,11 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
                 v += __shfl_xor_sync(FULL, v, 2);
                 v += __shfl_xor_sync(FULL, v, 1);
                 v = fmaxf(v + bias, 0.f);
-                float o[4];
-                gather4(v, 4, o);
-                if (!bad) st_async_v4(a_own + 2 * PK * 4, o[0], o[1], o[2], o[3], b_q);
+                if ((lane & 3) == 0) qstage[8 * warp + (lane >> 2)] = v;
+                cl_bar_sync(2, 32 * PCW);
+                const float4 o = reinterpret_cast<const float4 *>(qstage)[piece];
+                if (!bad) st_async_v4(a_own + 2 * PK * 4, o.x, o.y, o.z, o.w, b_q);
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&xg[half ? 0 : 1])) : "memory");
             }
             // ---- 2. four rows of the logits, half of K: lane takes runs of four values, 128 apart
             {
@@ -355,26 +371,31 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
                 x += bias;
-                float o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) o[j] = __shfl_sync(FULL, x, 8 * j);
-                if (lane < 16 && !bad) st_async_v4(a_log, o[0], o[1], o[2], o[3], b_l);
+                if ((lane & 7) == 0) lstage[kh * PL + r0 + (lane >> 3)] = x;
+                cl_bar_sync(2, 32 * PCW);
+                if (piece < PL / 4 && !bad) {
+                    const float4 o = reinterpret_cast<const float4 *>(lstage)[piece], o2 = reinterpret_cast<const float4 *>(lstage)[PL / 4 + piece];
+                    st_async_v4(a_log, o.x + o2.x, o.y + o2.y, o.z + o2.z, o.w + o2.w, b_l);
+                }
             }
             // ---- 3. draw and gates
-            if (!half) wait_bar(&xr[1], (unsigned)s, sn, 7);                        // R h is complete
-            const GatePre gp = gates_prepare(half, gv);
-            wait_bar(&xl, use, sn, 3 + 4 * half);
             float l[8];
-            {
-                const float4 *L = reinterpret_cast<const float4 *>(lbuf) + 2 * lane;
-                const float4 a = L[0], b = L[1], a2 = L[64], b2 = L[65];
-                l[0] = a.x + a2.x; l[1] = a.y + a2.y; l[2] = a.z + a2.z; l[3] = a.w + a2.w;
-                l[4] = b.x + b2.x; l[5] = b.y + b2.y; l[6] = b.z + b2.z; l[7] = b.w + b2.w;
+            int drawn = 0;
+            if (drawer) {
+                GatePre gp = gates_prepare(half, gv);
+                wait_bar(&xl, use, sn, 3 + 4 * half);
+                const float4 a = reinterpret_cast<const float4 *>(lbuf)[2 * lane], b = reinterpret_cast<const float4 *>(lbuf)[2 * lane + 1];
+                l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
+                drawn = cl_draw(l, u01, lane);
+                const int fed = (DBG && forced >= 0) ? forced : drawn;
+                if (!half) wait_bar(&xr[1], (unsigned)s, sn, 7);         // R h is complete
+                if (!last) gates(half, half ? s : s + 1, fed, gp);
+                if (half) c_prev = fed; else f_prev = fed;
             }
-            const int drawn = cl_draw(l, u01, lane);
-            const int fed = (DBG && forced >= 0) ? forced : drawn;
-            if (!last) gates_and_send(half, half ? s : s + 1, fed, gp);
-            if (half) c_prev = fed; else f_prev = fed;
+            if (!last) {
+                cl_bar_sync(2, 32 * PCW);
+                send_y(half, half ? s : s + 1);
+            }
             // the samples (and the dumps) leave when the state is on its way
             if (DBG && !last) dump_gates(half, half ? s : s + 1);
             if (writer && !bad) {
@@ -507,7 +528,7 @@ int sparse1_prepare(wrnn_model *m)
                     longest = std::max(longest, (size_t)PPRE);
                 } else {
                     for (int b = 0; b < rpw; ++b) { sl.row[b] = (int16_t)ord[w * rpw + b]; longest = std::max(longest, (R[ord[w * rpw + b]].size() + lpr - 1) / lpr); }
-                    longest = std::max(longest, (size_t)1);                                        // the loop's first loads are unconditional
+                    longest = std::max(longest, (size_t)BPRE);
                 }
                 sl.at = at; sl.T = (int)longest;
                 at += 32 * sl.T;
@@ -554,17 +575,38 @@ int sparse1_prepare(wrnn_model *m)
             for (int w = 0; w < (a < 2 ? PCW : PBW); ++w) {
                 const PSlice &sl = sls[(a < 2 ? a * PCW : 2 * PCW + (a - 2) * PBW) + w];
                 const int nb = thin ? 1 : a < 2 ? 2 : rpw, nl = 32 / nb;         // block rows of the warp, lanes of each
+                // Which of its row's lanes and iterations takes a block is free.  The lanes whose activations are loaded together (8 at
+                // 16 bytes each, 32 at 4) should find them in different banks: a block goes where the fewest share its bank.
+                const int bl = tall ? 32 : 8, per_t = 32 / bl;                   // lanes that load together (and bank classes), groups of them per iteration
+                std::vector<std::vector<int>> share((size_t)sl.T * per_t, std::vector<int>(bl, 0));
+                std::vector<int> any_col((size_t)sl.T * per_t, 0);
+                std::vector<char> used((size_t)32 * sl.T, 0);
                 for (int g = 0; g < nb; ++g) {
                     const auto &blocks = rows[cta][a][thin ? w >> 1 : a < 2 ? 2 * w + g : sl.row[g]];
-                    for (int i = 0; i < (int)blocks.size(); ++i) {
-                        const int t = i / nl, lane = nl * g + i % nl;
-                        col[sl.at + 32 * t + lane] = blocks[i].col;
+                    const int lanes = std::min(nl, bl), b0 = nl * g / bl, b1 = (nl * g + nl - 1) / bl;
+                    std::vector<int> fill((size_t)sl.T * per_t, 0);              // of this row
+                    for (const Blk &blk : blocks) {
+                        const int cls = blk.col % bl;
+                        int best = -1;
+                        for (int t = 0; t < sl.T; ++t)
+                            for (int b = b0; b <= b1; ++b) {
+                                const int i = t * per_t + b;
+                                if (fill[i] == lanes) continue;
+                                if (best < 0 || share[i][cls] < share[best][cls] || (share[i][cls] == share[best][cls] && fill[i] < fill[best])) best = i;
+                            }
+                        const int t = best / per_t, lane = std::max(nl * g, (best % per_t) * bl) + fill[best];
+                        ++fill[best]; ++share[best][cls];
+                        any_col[best] = blk.col;
+                        used[32 * t + lane] = 1;
+                        col[sl.at + 32 * t + lane] = blk.col;
                         for (int h = 0; h < (thin ? 1 : 2); ++h)
                             for (int e = 0; e < 8; ++e)
                                 val[thin ? ((size_t)sl.at + 32 * t + lane) * 8 + e : ((size_t)2 * sl.at + 64 * t + 32 * h + lane) * 8 + e] =
-                                    p_bf16(blocks[i].v[thin ? 8 * (w & 1) + e : 8 * h + e]);
+                                    p_bf16(blk.v[thin ? 8 * (w & 1) + e : 8 * h + e]);
                     }
                 }
+                for (int i = 0; i < 32 * sl.T; ++i)                              // empty slots (zero weights) read what a neighbour reads
+                    if (!used[i]) col[sl.at + i] = (uint16_t)any_col[(i / 32) * per_t + (i % 32) / bl];
             }
         }
         for (int h = 0; h < 2; ++h) {                                            // dense rows, as bf16: O4, O2
