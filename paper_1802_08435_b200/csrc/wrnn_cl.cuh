@@ -1,6 +1,9 @@
-// Device helpers of the kernels that keep a whole model in one thread-block cluster: named barriers, the cluster barrier, and
-// the draw and the gate functions as a single warp does them with nothing else to wait for.
+// Device helpers of the kernels that keep a whole model in one thread-block cluster: named barriers, the cluster barrier,
+// products of fp16 weights with the high and low fp16 parts of fp32 values, and the draw and the gate functions as a single warp
+// does them with nothing else to wait for.
 #pragma once
+#include <cuda_fp16.h>
+
 #include "wrnn_device.cuh"
 
 namespace wrnn {
@@ -43,6 +46,22 @@ __device__ __forceinline__ int cl_draw(const float (&l)[8], float u, int lane)
     // the running sums do not decrease: the first one above the threshold comes after those that are not
     const int c = ((p0 <= thr) + (p1 <= thr)) + ((p2 <= thr) + (p3 <= thr)) + (((p4 <= thr) + (p5 <= thr)) + ((p6 <= thr) + (p7 <= thr)));
     return __reduce_min_sync(FULL, c == 8 ? 255 : 8 * lane + c);
+}
+__device__ __forceinline__ void cl_mma(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
+// x (scaled by a power of two into the range of fp16) as high and low fp16 parts: x - high - low is at most 2^-24 |x|, half a
+// unit in the last place of fp32
+__device__ __forceinline__ uint2 cl_split4(float a, float b, float c, float d, uint2 &low)
+{
+    const __half2 h0 = __floats2half2_rn(a, b), h1 = __floats2half2_rn(c, d);
+    const __half2 l0 = __floats2half2_rn(a - __low2float(h0), b - __high2float(h0)), l1 = __floats2half2_rn(c - __low2float(h1), d - __high2float(h1));
+    low = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
+    return make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
 }
 
 }  // namespace wrnn

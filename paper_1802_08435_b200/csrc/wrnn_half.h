@@ -1,0 +1,77 @@
+// Host-side preparation of fp16 operands: conversions, and matrices scaled by a power of two into the range of fp16.
+#pragma once
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "wrnn_internal.h"
+
+namespace wrnn {
+
+// fp32 -> fp16 bits, to nearest even (finite values below 2^15 keep their range here; infinities and NaNs stay what they are)
+inline uint16_t half_bits(float v)
+{
+    uint32_t u;
+    std::memcpy(&u, &v, 4);
+    const uint32_t sign = (u >> 16) & 0x8000u, a = u & 0x7fffffffu;
+    if (a >= 0x7f800000u) return (uint16_t)(sign | (a > 0x7f800000u ? 0x7e00u : 0x7c00u));
+    if (a >= 0x38800000u) return (uint16_t)(sign | std::min(((a + 0xfffu + ((a >> 13) & 1u)) >> 13) - (112u << 10), 0x7c00u));
+    float f;
+    std::memcpy(&f, &a, 4);
+    f += 0.5f;                                   // the last bit of 0.5 is the subnormal step of fp16
+    std::memcpy(&u, &f, 4);
+    return (uint16_t)(sign | (u - 0x3f000000u));
+}
+inline float half_value(uint16_t h)
+{
+    uint32_t u = (uint32_t)(h & 0x7fffu) << 13;
+    float v;
+    if (u < (1u << 23)) v = (float)(h & 0x3ffu) * 5.9604644775390625e-8f;        // subnormal: steps of 2^-24
+    else {
+        u = u >= (31u << 23) ? u | 0x7f800000u : u + (112u << 23);
+        std::memcpy(&v, &u, 4);
+    }
+    return h & 0x8000u ? -v : v;
+}
+// A dense matrix as one or two fp16 parts, scaled by 2^(14 - exp)
+struct HalfMatrix {
+    int exp = 0;
+    std::vector<uint16_t> part[2];
+    HalfMatrix(const BsrHost &M, int np)
+    {
+        float top = 0.f;
+        for (float v : M.vals) top = std::max(top, std::fabs(v));
+        exp = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+        const float scale = std::ldexp(1.f, 14 - exp);
+        const size_t cols = (size_t)M.cols4 * 4;
+        for (int w = 0; w < np; ++w) part[w].assign((size_t)M.rows4 * 4 * cols, 0);
+        for (int br = 0; br < M.rows4; ++br)
+            for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
+                for (int r = 0; r < 4; ++r) {
+                    const float *src = &M.vals[(size_t)b * 16 + 4 * r];
+                    const size_t o = (size_t)(4 * br + r) * cols + 4 * M.col[b];
+                    for (int c = 0; c < 4; ++c) {
+                        const float x = src[c] * scale;
+                        part[0][o + c] = half_bits(x);
+                        if (np == 2) part[1][o + c] = half_bits(x - half_value(part[0][o + c]));
+                    }
+                }
+    }
+};
+// Exponent of a bound on the hidden layer relu(M y + bias) for a state y below one: sum |row| + |bias| < 2^result
+inline int hidden_exp(const BsrHost &M, const std::vector<float> &bias)
+{
+    float top = 0.f;
+    for (int br = 0; br < M.rows4; ++br)
+        for (int r = 0; r < 4; ++r) {
+            float sum = std::fabs(bias[4 * br + r]);
+            for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
+                for (int c = 0; c < 4; ++c) sum += std::fabs(M.vals[(size_t)b * 16 + 4 * r + c]);
+            top = std::max(top, sum);
+        }
+    return top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+}
+
+}  // namespace wrnn

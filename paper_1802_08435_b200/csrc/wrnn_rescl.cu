@@ -37,6 +37,7 @@
 
 #include "wrnn_cl.cuh"
 #include "wrnn_cluster.cuh"
+#include "wrnn_half.h"
 #include "wrnn_internal.h"
 #include "wrnn_tc.cuh"
 
@@ -126,12 +127,6 @@ __device__ __forceinline__ void cl_ldmatrix4(uint32_t addr, uint32_t (&r)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
-__device__ __forceinline__ void cl_mma(float (&c)[4], const uint4 &a, uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
 // shared-memory address of another CTA of the cluster (as map_to_rank, free to be moved)
 __device__ __forceinline__ uint32_t cl_map(uint32_t addr, int rank) { uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r; }
 __device__ __forceinline__ void cl_st_async16(unsigned addr, uint4 v, unsigned mbar)
@@ -155,17 +150,6 @@ __device__ __forceinline__ uint4 cl_ldg_stream(const uint4 *p)
     asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint2 cl_lds8(uint32_t addr) { uint2 v; asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory"); return v; }
-// x (scaled by a power of two into the range of fp16) as high and low fp16 parts: x - high - low is at most 2^-24 |x|, half a
-// unit in the last place of fp32
-__device__ __forceinline__ uint2 cl_split4(float a, float b, float c, float d, uint2 &low)
-{
-    const __half2 h0 = __floats2half2_rn(a, b), h1 = __floats2half2_rn(c, d);
-    const __half2 l0 = __floats2half2_rn(a - __low2float(h0), b - __high2float(h0)), l1 = __floats2half2_rn(c - __low2float(h1), d - __high2float(h1));
-    low = make_uint2(*reinterpret_cast<const uint32_t *>(&l0), *reinterpret_cast<const uint32_t *>(&l1));
-    return make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
-}
-
 // NG: groups of four rows.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
 // multiply the rows of R in the background, while the chain waits for exchanges.
@@ -892,57 +876,6 @@ static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
     *n_clusters = need < CNC ? CNC : need;       // (a cluster without rows returns at once)
 }
 
-// fp32 -> fp16 bits, to nearest even (finite values below 2^15 keep their range here; infinities and NaNs stay what they are)
-static uint16_t half_bits(float v)
-{
-    uint32_t u;
-    std::memcpy(&u, &v, 4);
-    const uint32_t sign = (u >> 16) & 0x8000u, a = u & 0x7fffffffu;
-    if (a >= 0x7f800000u) return (uint16_t)(sign | (a > 0x7f800000u ? 0x7e00u : 0x7c00u));
-    if (a >= 0x38800000u) return (uint16_t)(sign | std::min(((a + 0xfffu + ((a >> 13) & 1u)) >> 13) - (112u << 10), 0x7c00u));
-    float f;
-    std::memcpy(&f, &a, 4);
-    f += 0.5f;                                   // the last bit of 0.5 is the subnormal step of fp16
-    std::memcpy(&u, &f, 4);
-    return (uint16_t)(sign | (u - 0x3f000000u));
-}
-static float half_value(uint16_t h)
-{
-    uint32_t u = (uint32_t)(h & 0x7fffu) << 13;
-    float v;
-    if (u < (1u << 23)) v = (float)(h & 0x3ffu) * 5.9604644775390625e-8f;        // subnormal: steps of 2^-24
-    else {
-        u = u >= (31u << 23) ? u | 0x7f800000u : u + (112u << 23);
-        std::memcpy(&v, &u, 4);
-    }
-    return h & 0x8000u ? -v : v;
-}
-// A dense matrix as one or two fp16 parts, scaled by 2^(14 - exp)
-struct HalfMatrix {
-    int exp = 0;
-    std::vector<uint16_t> part[2];
-    HalfMatrix(const BsrHost &M, int np)
-    {
-        float top = 0.f;
-        for (float v : M.vals) top = std::max(top, std::fabs(v));
-        exp = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
-        const float scale = std::ldexp(1.f, 14 - exp);
-        const size_t cols = (size_t)M.cols4 * 4;
-        for (int w = 0; w < np; ++w) part[w].assign((size_t)M.rows4 * 4 * cols, 0);
-        for (int br = 0; br < M.rows4; ++br)
-            for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
-                for (int r = 0; r < 4; ++r) {
-                    const float *src = &M.vals[(size_t)b * 16 + 4 * r];
-                    const size_t o = (size_t)(4 * br + r) * cols + 4 * M.col[b];
-                    for (int c = 0; c < 4; ++c) {
-                        const float x = src[c] * scale;
-                        part[0][o + c] = half_bits(x);
-                        if (np == 2) part[1][o + c] = half_bits(x - half_value(part[0][o + c]));
-                    }
-                }
-    }
-};
-
 int rescl_prepare(wrnn_model *m)
 {
     const int H = m->H;
@@ -978,18 +911,7 @@ int rescl_prepare(wrnn_model *m)
     // products of operands scaled by 2^(14 - exponent) each
     k.inv_R = std::ldexp(1.f, e[0] - 28);
     for (int h = 0; h < 2; ++h) {
-        // |hidden value| <= sum |O1 row| + |b1| for a state below one (the kernel takes a larger initial state into account)
-        const BsrHost &M = h ? m->hO3 : m->hO1;
-        const std::vector<float> &bias = h ? m->hb3 : m->hb1;
-        float top = 0.f;
-        for (int br = 0; br < M.rows4; ++br)
-            for (int r = 0; r < 4; ++r) {
-                float sum = std::fabs(bias[4 * br + r]);
-                for (int b = M.row_ptr[br]; b < M.row_ptr[br + 1]; ++b)
-                    for (int c = 0; c < 4; ++c) sum += std::fabs(M.vals[(size_t)b * 16 + 4 * r + c]);
-                top = std::max(top, sum);
-            }
-        const int eq = top > 0.f && std::isfinite(top) ? std::ilogb(top) + 1 : 0;
+        const int eq = hidden_exp(h ? m->hO3 : m->hO1, h ? m->hb3 : m->hb1);
         k.inv_O1[h] = std::ldexp(1.f, e[1 + h] - 28);
         k.q_scale[h] = std::ldexp(1.f, 14 - eq);
         k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);

@@ -24,6 +24,7 @@
 
 #include "wrnn_cl.cuh"
 #include "wrnn_cluster.cuh"
+#include "wrnn_half.h"
 #include "wrnn_internal.h"
 #include "wrnn_tc.cuh"
 
@@ -37,25 +38,27 @@ constexpr int PL = 16;                   // logits rows per CTA
 constexpr int PCW = 8, PBW = 12;         // chain warps, background warps
 constexpr int PTHREADS = 32 * (PCW + PBW);
 constexpr int PPRE = 2, BPRE = 3;        // iterations of a hidden-layer slice, of a slice of R, whose weights are loaded before the state arrives
-constexpr int PSMALL = 6 * PU * 3 + 2 * PU + 2 * PL;      // floats: I [half][gate][unit][3], b1, b3, b2, b4
+constexpr int PSMALL = 6 * PU * 3 + 2 * PU + PCW * PL;      // floats: I [half][gate][unit][3], b1, b3, b2, b4
 constexpr int PDW = PU / 32;             // drawing warps: one unit per lane
-constexpr int PVEC = 3 * PK + 256 + 2 * 6 * PU + 2 * PU + 2 * PL;       // floats: two state halves, hidden layer, logits, R h (partial, complete), staged y, q, logits
-// a warp's run of block slots: `at` is its first slot, T its iterations; a slot is 32 bytes of weights (two planes of 16 bytes, for
-// the hidden rows of 16 x 1 blocks one) and a column
-struct PSlice { int at, T; int16_t row[8]; };
+constexpr int PVEC = 3 * PK + 256 + 2 * 6 * PU + 2 * PU + PCW * PL;       // floats: two state halves, hidden layer, logits, R h (partial, complete), staged y, q, K-split logits
+// a warp's run of block slots: `at` is its first slot, T its iterations; a slot is 32 bytes of weights and a column.  Hidden rows: weights in
+// shared memory as two planes of 16 bytes (16 x 1 blocks: 16 bytes).  Rows of R: in tensor memory, eight columns an iteration from `tcol`
+struct PSlice { int at, T, tcol; int16_t row[8]; };
 }  // namespace
 
 struct Sparse1Pack {
     uint8_t *d_blob = nullptr;
     bool tall = false;
     size_t blob_bytes = 0;
-    size_t off_col[4], off_val[4], off_w[2], off_small = 0;      // arrays 0, 1: hidden rows of O3, O1; 2, 3: rows of R times y_c, y_f
+    size_t off_col[4], off_val[2], off_small = 0, tmem_cols = 0;
+    float inv_w[2], q_scale[2];      // arrays 0, 1: hidden rows of O3, O1; 2, 3: rows of R times y_c, y_f
     int smem_bytes = 0;
     int64_t weight_bytes_per_step = 0;
 };
 
 struct Sparse1Params {
-    unsigned off_col[4], off_val[4], off_w[2], off_small, blob_bytes;
+    unsigned off_col[4], off_val[2], off_small, blob_bytes, tmem_cols;
+    float inv_w[2], q_scale[2];              // logits rows, hidden layer of the fine, coarse half: what undoes, does the scaling for fp16
     long long n_steps, step0;
     unsigned stream0;
     unsigned long long seed;
@@ -89,6 +92,11 @@ __device__ __forceinline__ void p_column(float *acc, const uint4 &w, float x)
     acc[4] = fmaf(bf16lo(w.z), x, acc[4]); acc[5] = fmaf(bf16hi(w.z), x, acc[5]);
     acc[6] = fmaf(bf16lo(w.w), x, acc[6]); acc[7] = fmaf(bf16hi(w.w), x, acc[7]);
 }
+// eight columns of tensor memory: a block's 32 bytes, one block per lane
+__device__ __forceinline__ void p_tmem_ld8(uint32_t col, uint4 &a, uint4 &b)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "r"(col));
+}
 // half the values of each lane change places with those of the lane `o` away: N values -> N / 2 sums; the lanes with that bit set
 // keep the upper half
 template <int N>
@@ -105,6 +113,8 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
 {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl, xg[2], xr[2];   // arrivals: state halves, hidden layer, logits; background products of a half: may start, done
+    __shared__ int s_hexp;
+    __shared__ uint32_t s_tmem;
     constexpr bool DBG = MODE != 0;
     constexpr int H = 2 * PK;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -116,18 +126,41 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     float *qvec = vec + 2 * PK, *lbuf = qvec + PK, *r_part = lbuf + 256, *r_full = r_part + 6 * PU;
     float *ystage = r_full + 6 * PU, *qstage = ystage + PU, *lstage = qstage + PU;
     {
-        const uint4 *src = reinterpret_cast<const uint4 *>(p.blob + (size_t)rank * p.blob_bytes);
+        const uint8_t *blob = p.blob + (size_t)rank * (p.blob_bytes + p.tmem_cols * 512);
+        const uint4 *src = reinterpret_cast<const uint4 *>(blob);
         uint4 *dst = reinterpret_cast<uint4 *>(smem);
         for (unsigned i = tid; i < p.blob_bytes / 16; i += PTHREADS) dst[i] = __ldg(src + i);
         for (int i = tid; i < H; i += PTHREADS) vec[i] = p.h_in ? p.h_in[i] : 0.f;
         if (tid == 0) {
+            s_hexp = 0;
             mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
             mbar_init(smem_u32(&xg[0]), PCW); mbar_init(smem_u32(&xg[1]), PCW);
             mbar_init(smem_u32(&xr[0]), PBW); mbar_init(smem_u32(&xr[1]), PBW);
             mbar_fence_init();
         }
+        if (warp == 1) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        tc_fence_before();
         __syncthreads();
+        tc_fence_after();
+        const uint32_t *tsrc = reinterpret_cast<const uint32_t *>(blob + p.blob_bytes) + 32 * (warp & 3) + lane;
+        const uint32_t tdst = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+#pragma unroll 1
+        for (unsigned c = 8 * (warp >> 2); c < p.tmem_cols; c += 8 * (PTHREADS / 128)) {
+            uint32_t r[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) r[k] = __ldg(tsrc + (size_t)(c + k) * 128);
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(tdst + c), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]),
+                         "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
     }
+    const uint32_t tmem = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     Waiter wt{p.status, p.limit_ns};
     bool bad = false;                                                    // this thread gave up
     auto wait_bar = [&](unsigned long long *b, unsigned parity, int step, int phase) {
@@ -137,6 +170,12 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
         while (!mbar_try(a, parity & 1u))
             if ((++cnt & 1023u) == 0 && wt.expired(t0, step, phase)) { bad = true; break; }
     };
+    // the power of two that covers the state: one but for what the caller passes in
+    if (p.h_in) {
+        float m = 1.f;
+        for (int i = tid; i < H; i += PTHREADS) m = fmaxf(m, fabsf(vec[i]));
+        if (!(m <= 1.f)) atomicMax(&s_hexp, min(127, ilogbf(m) + 1));
+    }
     const PSlice *slices = reinterpret_cast<const PSlice *>(smem);       // [2 heads][PCW], then [2 halves][PBW]
     const long long T = p.n_steps;
 
@@ -144,7 +183,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     // the first BPRE iterations (as a rule all of them) are in registers
     auto r_products = [&](int half_f, auto start) {
         const PSlice &sl = slices[2 * PCW + half_f * PBW + warp - PCW];
-        const uint4 *wv = reinterpret_cast<const uint4 *>(smem + p.off_val[2 + half_f]) + 2 * sl.at + lane;
+        const uint32_t wt_col = tmem + sl.tcol;
         const uint16_t *wc = reinterpret_cast<const uint16_t *>(smem + p.off_col[2 + half_f]) + sl.at + lane;
         const float *x = vec + half_f * PK;
         const int nt = sl.T;
@@ -152,7 +191,8 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
         uint4 w0[BPRE], w1[BPRE];
         int c[BPRE];
 #pragma unroll
-        for (int t = 0; t < BPRE; ++t) { w0[t] = wv[64 * t]; w1[t] = wv[64 * t + 32]; c[t] = wc[32 * t]; }
+        for (int t = 0; t < BPRE; ++t) { p_tmem_ld8(wt_col + 8 * t, w0[t], w1[t]); c[t] = wc[32 * t]; }
+        tmem_wait_ld();
         float acc[16];
 #pragma unroll
         for (int j = 0; j < (TALL ? 16 : 4); ++j) acc[j] = 0.f;
@@ -168,8 +208,10 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
 #pragma unroll 1
         for (int t = BPRE; t < nt; ++t) {
             const int ct = wc[32 * t];
-            if (TALL) { const float xs = x[ct]; p_column(acc, wv[64 * t], xs); p_column(acc + 8, wv[64 * t + 32], xs); }
-            else p_block(*reinterpret_cast<float (*)[4]>(acc), wv[64 * t], wv[64 * t + 32], *reinterpret_cast<const float4 *>(x + 4 * ct));
+            p_tmem_ld8(wt_col + 8 * t, w0[0], w1[0]);
+            tmem_wait_ld();
+            if (TALL) { const float xs = x[ct]; p_column(acc, w0[0], xs); p_column(acc + 8, w1[0], xs); }
+            else p_block(*reinterpret_cast<float (*)[4]>(acc), w0[0], w1[0], *reinterpret_cast<const float4 *>(x + 4 * ct));
         }
         if (TALL) { p_fold<16>(acc, 8, lane); p_fold<8>(acc, 4, lane); }
         p_fold<4>(acc, 2, lane); p_fold<2>(acc, 1, lane);
@@ -255,6 +297,9 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
             if (p.dbg_h) p.dbg_h[(size_t)s * H + jj] = dbg_v[3];
         };
         const float *g_unit = p.g + gj;
+        float q_s[2], inv_l[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { q_s[h] = p.q_scale[h] * ldexpf(1.f, -s_hexp); inv_l[h] = p.inv_w[h] * ldexpf(1.f, s_hexp); }
         if (drawer) {
             float gv[3];
 #pragma unroll
@@ -333,49 +378,46 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
                 float v = acc[0];
                 v += __shfl_xor_sync(FULL, v, 2);
                 v += __shfl_xor_sync(FULL, v, 1);
-                v = fmaxf(v + bias, 0.f);
+                v = fmaxf(v + bias, 0.f) * q_s[half];
                 if ((lane & 3) == 0) qstage[8 * warp + (lane >> 2)] = v;
                 cl_bar_sync(2, 32 * PCW);
                 const float4 o = reinterpret_cast<const float4 *>(qstage)[piece];
-                if (!bad) st_async_v4(a_own + 2 * PK * 4, o.x, o.y, o.z, o.w, b_q);
+                uint2 lo;
+                const uint2 hi = cl_split4(o.x, o.y, o.z, o.w, lo);
+                if (!bad) st_async_v4(a_own + 2 * PK * 4, __uint_as_float(hi.x), __uint_as_float(hi.y), __uint_as_float(lo.x), __uint_as_float(lo.y), b_q);
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&xg[half ? 0 : 1])) : "memory");
             }
-            // ---- 2. four rows of the logits, half of K: lane takes runs of four values, 128 apart
+            // ---- 2. the 16 rows of the logits, an eighth of K: tensor cores, fp16 weights times the high and low parts of the hidden layer
             {
-                const int kh = warp >> 2, r0 = 4 * (warp & 3);
-                const uint2 *w2 = reinterpret_cast<const uint2 *>(smem + p.off_w[half]) + (size_t)(r0 * 2 + kh) * (PK / 8) + lane;   // [row][K / 4]
-                uint2 w[4][4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) w[r][j] = w2[r * (PK / 4) + 32 * j];
-                const float bias = kh ? 0.f : (half ? sb2 : sb4)[r0 + (lane >> 3)];
+                uint32_t w[2][16];
+                tmem_ld16(tmem + 64 * (warp >> 2) + 32 * half, w[0]);
+                tmem_ld16(tmem + 64 * (warp >> 2) + 32 * half + 16, w[1]);
+                const float4 bias = reinterpret_cast<const float4 *>(half ? sb2 : sb4)[lane & 3];
                 if (!half && warp == 0) wait_bar(&xr[0], (unsigned)s, sn, 6);    // the background warps are done with y_c(s)
+                tmem_wait_ld();
                 wait_bar(&xq, use, sn, 2 + 4 * half);
-                const float4 *q4 = reinterpret_cast<const float4 *>(qvec) + kh * (PK / 8) + lane;
-                float4 q[4];
+                // column n of B: the high (even n) or low parts; only columns 0 and 1 are read
+                const uint32_t b0 = smem_u32(qvec) + (uint32_t)((8 * warp * 4 + (lane & 3)) * 16 + ((lane >> 2) & 1) * 8);
+                uint2 b[8];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) q[j] = q4[32 * j];
-                float v[4] = {0.f, 0.f, 0.f, 0.f}, v2[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int i = 0; i < 8; ++i) b[i] = cl_lds8(b0 + i * 64);
+                float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        v[r] = fmaf(bf16lo(w[r][j].x), q[j].x, v[r]); v2[r] = fmaf(bf16hi(w[r][j].x), q[j].y, v2[r]);
-                        v[r] = fmaf(bf16lo(w[r][j].y), q[j].z, v[r]); v2[r] = fmaf(bf16hi(w[r][j].y), q[j].w, v2[r]);
-                    }
-#pragma unroll
-                for (int r = 0; r < 4; ++r) v[r] += v2[r];
-                p_fold<4>(v, 16, lane); p_fold<2>(v, 8, lane);
-                float x = v[0];
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-                x += bias;
-                if ((lane & 7) == 0) lstage[kh * PL + r0 + (lane >> 3)] = x;
+                for (int i = 0; i < 8; ++i) cl_mma(acc[i & 1], make_uint4(w[i >> 2][4 * (i & 3)], w[i >> 2][4 * (i & 3) + 1], w[i >> 2][4 * (i & 3) + 2], w[i >> 2][4 * (i & 3) + 3]), b[i].x, b[i].y);
+                if ((lane & 3) == 0) {
+                    float *d = lstage + warp * PL + (lane >> 2);
+                    d[0] = (acc[0][0] + acc[1][0]) + (acc[0][1] + acc[1][1]);
+                    d[8] = (acc[0][2] + acc[1][2]) + (acc[0][3] + acc[1][3]);
+                }
                 cl_bar_sync(2, 32 * PCW);
                 if (piece < PL / 4 && !bad) {
-                    const float4 o = reinterpret_cast<const float4 *>(lstage)[piece], o2 = reinterpret_cast<const float4 *>(lstage)[PL / 4 + piece];
-                    st_async_v4(a_log, o.x + o2.x, o.y + o2.y, o.z + o2.z, o.w + o2.w, b_l);
+                    float4 v = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int k = 0; k < PCW; ++k) {
+                        const float4 a = reinterpret_cast<const float4 *>(lstage + k * PL)[piece];
+                        v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
+                    }
+                    st_async_v4(a_log, fmaf(v.x, inv_l[half], bias.x), fmaf(v.y, inv_l[half], bias.y), fmaf(v.z, inv_l[half], bias.z), fmaf(v.w, inv_l[half], bias.w), b_l);
                 }
             }
             // ---- 3. draw and gates
@@ -424,6 +466,10 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     const int any_bad = __syncthreads_or(bad);
     if (rank == 0 && !any_bad && p.h_out)
         for (int i = tid; i < H; i += PTHREADS) p.h_out[i] = vec[i];
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(512) : "memory");
     cluster_sync_all();
 }
 
@@ -541,15 +587,27 @@ int sparse1_prepare(wrnn_model *m)
     auto a16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
     size_t off = a16(sizeof(PSlice) * 2 * (PCW + PBW));
     for (int a = 0; a < 4; ++a) {
-        k.off_val[a] = off; off += (size_t)slots[a] * (a < 2 && tall ? 16 : 32);
+        if (a < 2) { k.off_val[a] = off; off += (size_t)slots[a] * (tall ? 16 : 32); }
         k.off_col[a] = off; off = a16(off + (size_t)slots[a] * 2);
     }
-    for (int h = 0; h < 2; ++h) { k.off_w[h] = off; off += (size_t)PL * PK * 2; }
     k.off_small = off; off = a16(off + (size_t)PSMALL * 4);
     k.blob_bytes = off;
     const size_t smem = off + (size_t)PVEC * 4;
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, m->device) != cudaSuccess) { cudaGetLastError(); return WRNN_ERR_CUDA; }
+    // tensor memory: the logits rows of the chain warps, then the rows of R.  Warp w reaches the lanes 32 (w mod 4) .. + 31
+    k.tmem_cols = 2 * 64;
+    for (int cta = 0; cta < PCS; ++cta) {
+        int next[4] = {128, 128, 128, 128};
+        for (int i = 2 * PCW; i < 2 * (PCW + PBW); ++i) {
+            PSlice &sl = slices[(size_t)cta * 2 * (PCW + PBW) + i];
+            int &n = next[(i - 2 * PCW) % PBW & 3];
+            sl.tcol = n;
+            n += 8 * sl.T;
+            k.tmem_cols = std::max(k.tmem_cols, (size_t)n);
+        }
+    }
+    if (k.tmem_cols > 512) { m->err = "pruned model does not fit the tensor memory of one cluster"; return WRNN_ERR_UNSUPPORTED; }
     if (smem > prop.sharedMemPerBlockOptin - 256) { m->err = "pruned model does not fit the shared memory of one cluster"; return WRNN_ERR_UNSUPPORTED; }
     k.smem_bytes = (int)smem;
     for (int dbg = 0; dbg < 2; ++dbg)
@@ -564,13 +622,22 @@ int sparse1_prepare(wrnn_model *m)
         cudaGetLastError(); m->err = "a 16-CTA cluster cannot be resident on this device"; return WRNN_ERR_UNSUPPORTED;
     }
 
-    std::vector<uint8_t> blob((size_t)PCS * k.blob_bytes, 0);
+    // fp16 logits rows, scaled by a power of two to at most 2^14 (the eight bits of a bf16 weight are kept unless it is below 2^-28 of
+    // the largest one), times hidden values scaled to at most 2^14
+    const HalfMatrix O[2] = {{m->hO4, 1}, {m->hO2, 1}};
+    for (int h = 0; h < 2; ++h) {
+        const int eq = hidden_exp(h ? m->hO1 : m->hO3, h ? m->hb1 : m->hb3);
+        k.q_scale[h] = std::ldexp(1.f, 14 - eq);
+        k.inv_w[h] = std::ldexp(1.f, O[h].exp - 14 + eq - 14);
+    }
+    const size_t cta_bytes = k.blob_bytes + k.tmem_cols * 512;
+    std::vector<uint8_t> blob(PCS * cta_bytes, 0);
     for (int cta = 0; cta < PCS; ++cta) {
-        uint8_t *base = blob.data() + (size_t)cta * k.blob_bytes;
+        uint8_t *base = blob.data() + (size_t)cta * cta_bytes, *tm = base + k.blob_bytes;          // tensor memory: [column][128 lanes][4]
         std::memcpy(base, &slices[(size_t)cta * 2 * (PCW + PBW)], sizeof(PSlice) * 2 * (PCW + PBW));
         const PSlice *sls = reinterpret_cast<const PSlice *>(base);
         for (int a = 0; a < 4; ++a) {
-            uint16_t *col = reinterpret_cast<uint16_t *>(base + k.off_col[a]), *val = reinterpret_cast<uint16_t *>(base + k.off_val[a]);
+            uint16_t *col = reinterpret_cast<uint16_t *>(base + k.off_col[a]), *val = a < 2 ? reinterpret_cast<uint16_t *>(base + k.off_val[a]) : nullptr;
             const bool thin = a < 2 && tall;                                     // a slot holds eight rows of a column
             for (int w = 0; w < (a < 2 ? PCW : PBW); ++w) {
                 const PSlice &sl = sls[(a < 2 ? a * PCW : 2 * PCW + (a - 2) * PBW) + w];
@@ -599,6 +666,13 @@ int sparse1_prepare(wrnn_model *m)
                         any_col[best] = blk.col;
                         used[32 * t + lane] = 1;
                         col[sl.at + 32 * t + lane] = blk.col;
+                        if (a >= 2) {
+                            for (int e = 0; e < 16; ++e) {
+                                const uint16_t v = p_bf16(blk.v[e]);
+                                std::memcpy(tm + ((size_t)(sl.tcol + 8 * t + e / 2) * 128 + 32 * (w & 3) + lane) * 4 + 2 * (e & 1), &v, 2);
+                            }
+                            continue;
+                        }
                         for (int h = 0; h < (thin ? 1 : 2); ++h)
                             for (int e = 0; e < 8; ++e)
                                 val[thin ? ((size_t)sl.at + 32 * t + lane) * 8 + e : ((size_t)2 * sl.at + 64 * t + 32 * h + lane) * 8 + e] =
@@ -609,15 +683,14 @@ int sparse1_prepare(wrnn_model *m)
                     if (!used[i]) col[sl.at + i] = (uint16_t)any_col[(i / 32) * per_t + (i % 32) / bl];
             }
         }
-        for (int h = 0; h < 2; ++h) {                                            // dense rows, as bf16: O4, O2
-            const BsrHost &M = h ? m->hO2 : m->hO4;
-            uint16_t *d = reinterpret_cast<uint16_t *>(base + k.off_w[h]);
-            for (int r = 0; r < PL; ++r) {
-                const int br = (cta * PL + r) / 4, rr = r % 4;
-                for (int i = M.row_ptr[br]; i < M.row_ptr[br + 1]; ++i)
-                    for (int c = 0; c < 4; ++c) d[(size_t)r * PK + 4 * M.col[i] + c] = p_bf16(M.vals[(size_t)i * 16 + 4 * rr + c]);
-            }
-        }
+        // A fragments of the 16 rows: lane (g, t) of k-tile kt holds rows g, g + 8 at k 16 kt + 4 t .. + 3 (the k order is permuted so that
+        // its part of B is four neighbouring values)
+        for (int h = 0; h < 2; ++h)
+            for (int kt = 0; kt < PK / 16; ++kt)
+                for (int lane = 0; lane < 32; ++lane)
+                    for (int reg = 0; reg < 4; ++reg)
+                        std::memcpy(tm + ((size_t)(64 * (kt >> 5) + 32 * h + 4 * (kt & 7) + reg) * 128 + 32 * ((kt >> 3) & 3) + lane) * 4,
+                                    &O[h].part[0][(size_t)(cta * PL + (lane >> 2) + 8 * (reg & 1)) * PK + 16 * kt + 4 * (lane & 3) + 2 * (reg >> 1)], 4);
         float *sm = reinterpret_cast<float *>(base + k.off_small);
         for (int r = 0; r < 6 * PU; ++r) {
             const int half = r / (3 * PU), gate = (r / PU) % 3, u = r % PU;
@@ -660,8 +733,10 @@ int sparse1_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     const Sparse1Pack &k = *m->sparse1;
     Sparse1Params p;
     std::memset(&p, 0, sizeof(p));
-    for (int i = 0; i < 4; ++i) { p.off_col[i] = (unsigned)k.off_col[i]; p.off_val[i] = (unsigned)k.off_val[i]; }
-    p.off_w[0] = (unsigned)k.off_w[0]; p.off_w[1] = (unsigned)k.off_w[1]; p.off_small = (unsigned)k.off_small; p.blob_bytes = (unsigned)k.blob_bytes;
+    for (int i = 0; i < 4; ++i) { p.off_col[i] = (unsigned)k.off_col[i]; if (i < 2) p.off_val[i] = (unsigned)k.off_val[i]; }
+    p.tmem_cols = (unsigned)k.tmem_cols;
+    for (int h = 0; h < 2; ++h) { p.inv_w[h] = k.inv_w[h]; p.q_scale[h] = k.q_scale[h]; }
+    p.off_small = (unsigned)k.off_small; p.blob_bytes = (unsigned)k.blob_bytes;
     p.n_steps = a.n_steps; p.step0 = a.step0; p.stream0 = a.stream0; p.seed = a.seed;
     p.hop = m->cond_dim ? a.hop : 1;
     p.row_stride = m->cond_dim ? a.row_stride : 0;
