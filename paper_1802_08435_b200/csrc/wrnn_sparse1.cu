@@ -1,21 +1,25 @@
 // Block-sparse single-stream sampling inside ONE 16-CTA cluster: bf16 weights, H = 2048, batch 1, 4 x 4 or 16 x 1 blocks, for
-// models whose kept blocks fit the shared memory of a cluster (3.6 MB: about 94 % of the blocks pruned).
+// models whose kept blocks fit the shared and tensor memory of a cluster (up to about 8 % of the blocks kept).
 //
 // What bounds a step is the chain state -> hidden layer -> logits -> draw -> gates -> state, twice: three all-gathers per
 // half-step and what lies between them.  Inside one cluster every all-gather goes through distributed shared memory (some 700
 // cycles for 1,024 values here), where the form on four clusters (wrnn_sparse.cu) passes the state through L2 (1,250 and
-// more).  The price, four times as many rows of R per CTA, is paid off the chain:
-//   * Warps 0..7 are the chain, and each of them goes through it alone: no barrier of the CTA and no hand-over in shared memory
-//     between an arrival and the next send.  Per half-step a warp takes 8 rows of the hidden layer over all of K (kept blocks;
-//     weights and block columns are in registers before the state arrives), four rows of the logits over half of K (dense, also in
-//     registers before the hidden layer arrives; the receivers add the two halves), draws -- all eight warps the same sample --
-//     and computes the gates of 8 units.  Each of the three results is 32 bytes or less per receiver: one st.async instruction
-//     whose lanes are (piece, receiver).
-//   * Warps 8..19 multiply the rows of R (96 block rows of 4, or 24 of 16, per half) in the background, while the chain waits.
-// A result can be stored into a peer without asking: whoever sends the next one has received something that every warp of
-// every CTA sent after its last use of the present one.  That the background warps are done with the state is what warp 0 waits
-// for before it sends its logits.
-// 6.54 us per step on four clusters -> SPARSE1_US here (4 x 4 blocks, 96 %).
+// more).  The price, four times as many rows of R per CTA, is paid off the chain: 6.54 us per step on four clusters, 3.97 here
+// (4 x 4 blocks, 4 % kept; 16 x 1: 6.7 -> 3.98).
+//   * Warps 0..7 are the chain.  Hidden layer: a warp has 8 rows over all of K, their kept blocks and block columns in registers
+//     before the state arrives.  Logits: 16 dense rows, K over the eight warps, tensor cores (fp16 weights from tensor memory
+//     times the high and low fp16 parts of the hidden layer, which is how it is sent).  Draw and gates: warps 0 and 1, the same
+//     sample, 32 units each.
+//   * Whatever is sent is first put together in shared memory: each of the eight warps then serves two CTAs with one st.async
+//     whose lanes write 256 contiguous bytes to each.  (Without that hand-over -- 32 bytes from every warp to every CTA, no barrier
+//     in the half-step -- a step takes 4.94 us: it is the number of separate runs that an exchange pays for.)
+//   * Warps 8..19 multiply the rows of R in the background once the hidden layer is on its way (earlier: 4.15 us).  Their weights are
+//     in tensor memory, because shared-memory loads queue behind one another with the chain's: 4.27 us with all weights in shared
+//     memory.  Which lane and iteration takes a block of a row is free, and is chosen so that the activations that are loaded
+//     together lie in different banks.
+// A result can be stored into a peer without asking: whoever sends the next one has received something that every CTA sent
+// after its last use of the present one.  That the background warps are done with the coarse half of the state is what warp 0
+// waits for before the logits of the fine half leave.
 //
 // Every wait is bounded; a thread that gives up skips its waits and sends from there on and keeps meeting its barriers, and
 // all CTAs leave through the final cluster barrier.

@@ -794,6 +794,29 @@ def test_sparse_cluster_kernel_on_fewer_clusters(env, monkeypatch, n_clusters):
         B.wrnn_destroy(m)
 
 
+@pytest.mark.parametrize("sparsity,block,n_ctas", [(0.96, (4, 4), 16), (0.96, (16, 1), 16), (0.995, (4, 4), 16), (0.93, (4, 4), 16), (0.88, (4, 4), 64)])
+def test_sparse_kernel_densities(env, sparsity, block, n_ctas):
+    """The block-sparse kernel inside one cluster at its own edges -- hardly any block kept (block rows of R without any, slices of
+    the shortest length), as many as a cluster holds (slices longer than what is kept in registers) -- and a model that goes to four
+    clusters: teacher-forced with dumps, then a free run against the oracle's stream."""
+    torch, B = env
+    w = synth.make_weights(2048)
+    masks = synth.make_block_masks(2048, sparsity, block=block)
+    w = synth.rescale_kept(w, masks)
+    cond = synth.make_cond(1, 2)
+    om = orc.OracleModel(w, "bf16", masks, block)
+    res = om.run(cond, 100, 1, SEED, dump=True)
+    m = B.wrnn_create(w, "bf16", masks, kernel=B.WRNN_KERNEL_SPARSE, block=block)
+    try:
+        assert B.wrnn_launch_info(m, 1)["n_ctas"] == n_ctas
+        r = pu.teacher_forced_parity(torch, B, m, om, cond, 100, 1, SEED, oracle_free=res)
+        _report("sparse kernel, %g %% pruned, %d x %d" % (100 * sparsity, *block), r)
+        _tol_check(r, "bf16")
+        _check_free_run_against_oracle(_free_run(torch, B, m, cond, 100, 1, SEED), res)
+    finally:
+        B.wrnn_destroy(m)
+
+
 def test_sparse_16x1_blocks_cluster_kernel(env):
     """The H = 2048 model pruned to 96 % with 16 x 1 blocks (Section 3.2's m x 1 shape, one activation per block) on
     the single-cluster kernel and on the generic kernel, both against the dense-with-zeros oracle."""
