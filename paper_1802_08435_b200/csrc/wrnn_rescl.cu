@@ -150,21 +150,24 @@ __device__ __forceinline__ uint4 cl_ldg_stream(const uint4 *p)
     asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-// NG: groups of four rows.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
+// ROWS: most rows of a cluster, 1, 4 or 8.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
 // multiply the rows of R in the background, while the chain waits for exchanges.
 // W2: fp32 weights, as high and low fp16 parts (error 2^-24 of a weight).  They are twice as much: the heads and the high parts of
 // nine tiles of R stay resident, the rest of R (344 KB per CTA and step) comes from L2 every step, in fragment order, straight
 // into the registers of the background warps.
 // FUSED: two 16-bit samples per step, one per half of the state, each as four 4-bit softmaxes of 16 consecutive logits; one row.
-template <int NG, int MODE, int KIND>
+template <int ROWS, int MODE, int KIND>
 __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams p)
 {
     constexpr bool W2 = KIND == CL_F32, FUSED = KIND == CL_FUSED;
     constexpr int NP = W2 ? 2 : 1;                                       // parts of a weight
     constexpr int NIN = cl_nin(KIND), NX = NIN / 3;                      // scalars of I per row, per symbol
+    constexpr bool ONE = ROWS == 1;
+    constexpr int NG = ROWS > 4 ? 2 : 1;                                 // groups of four rows
     constexpr size_t CB_SMEM = cl_blob_smem(KIND), CS_IMG = cl_img(NG), CS_PART = cl_part(NG), CS_PARTR = cl_part_r(NG);
     constexpr int CMAXR = 4 * NG;
+    constexpr int IR = ONE ? 1 : 4;                                      // rows that share a quad of an operand image
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
     __shared__ uint32_t s_tmem;
@@ -197,12 +200,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     float *partR = part + CS_PART / 4;                                   // [4 quarters of K][rows][168]: R h
     uint8_t *ystage = reinterpret_cast<uint8_t *>(partR + CS_PARTR / 4); // [row][quad][16 or 24 bytes]: new state values of this CTA's units
 
-    // Operand image of a vector: [group][quad][4 rows][high x 4, low x 4] -- a producer's four values of a row travel in one 16-byte
+    // Operand image of a vector: [group][quad][IR rows][high x 4, low x 4] -- a producer's four values of a row travel in one 16-byte
     // store, and the B fragment of lane (column g = row, part; t = quad of the k-tile) is one 8-byte load.  The k order of a tile
     // is permuted accordingly in all weights: slot c holds k = 4 ((c & 7) / 2) + 2 (c / 8) + (c & 1).
-    constexpr uint32_t QSTR = 64, GSTR = CQ * 64;
-    auto img_off = [](int st, int quad) { return (uint32_t)((st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16); };
-    const uint32_t frag = t4 * QSTR + g4 * 8;                            // of k-tile 0, group 0
+    constexpr uint32_t QSTR = 16 * IR, GSTR = CQ * 64;
+    auto img_off = [](int st, int quad) { return ONE ? (uint32_t)quad * 16 : (uint32_t)((st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16); };
+    const uint32_t frag = t4 * QSTR + (ONE ? g4 & 1 : g4) * 8;                            // of k-tile 0, group 0
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     {
@@ -345,6 +348,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     // the parts of a value are adjacent columns
     auto part_sum = [&](const float (&c)[4], float &lo, float &hi) { lo = c[0] + c[1]; hi = c[2] + c[3]; };
     auto r_store = [&]() {
+        if (ONE && t4 != 0) return;                                      // (the other columns of B repeat the row)
 #pragma unroll
         for (int grp = 0; grp < NG; ++grp) {
             float *d = partR + (rq * 4 * NG + 4 * grp + t4) * CPR + g4;
@@ -398,6 +402,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         });
     };
     auto w2_store = [&](int pass) {
+        if (ONE && t4 != 0) return;
         float *d = partR + (rq * 4 * NG + t4) * CPR + g4;
 #pragma unroll
         for (int n = 0; n < 5; ++n) {
@@ -409,12 +414,14 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 
     // ---- fixed addresses
     const uint32_t sbase = smem_u32(smem);
-    uint32_t dy[2];                                                      // CTA (warp & 7) + 8 k of the cluster: what to add to an address of mine
+    // Receivers of what this warp sends, as what to add to an address of mine.  Several rows: a lane stores its piece into each of
+    // them in turn.  One row: a lane has a receiver and a piece, so that a warp sends with one instruction.
+    uint32_t dy[2], delta4[4];                                           // state: CTAs (warp & 7) + 8 k; hidden layer, logits: (warp & 3) + 4 k
 #pragma unroll
-    for (int k = 0; k < 2; ++k) dy[k] = map_to_rank(sbase, (unsigned)((warp & 7) + 8 * k)) - sbase;
-    uint32_t delta4[4];                                                  // CTA (warp & 3) + 4 k
+    for (int k = 0; k < 2; ++k) dy[k] = map_to_rank(sbase, (unsigned)((warp & 7) + 8 * (ONE ? lane / 7 & 1 : k))) - sbase;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) delta4[k] = map_to_rank(sbase, (unsigned)((warp & 3) + 4 * k)) - sbase;
+    for (int k = 0; k < 4; ++k) delta4[k] = map_to_rank(sbase, (unsigned)((warp & 3) + 4 * (ONE ? lane / 7 & 3 : k))) - sbase;
+    const uint32_t delta_l = map_to_rank(sbase, (unsigned)((warp & 3) + 4 * (FUSED ? lane & 3 : lane >> 2 & 3))) - sbase;
     // A lane's piece of this CTA's 28 values: four values of a row, lane = (row of a group of four, quad)
     const int pc_a = lane / 7, pc_quad = lane - 7 * pc_a;
     const bool pc_on = lane < 28;
@@ -500,14 +507,14 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
     const int nsend = (nrc & 3) == 3 ? nrc + 1 : nrc;
     // warps 0..7: the staged state values of this CTA's units -> images in the cluster's CTAs, two each
     auto send_y = [&](int half_g, long long s) {
-        if (bad || !pc_on || (DBG && (int)s == skip_at)) return;
+        if (bad || (ONE ? lane >= 14 : !pc_on) || (DBG && (int)s == skip_at)) return;
         const uint32_t a = sbase + (uint32_t)(CB_SMEM + half_g * CS_IMG) + pc_off, bar = smem_u32(&xy[half_g]);
 #pragma unroll
         for (int grp = 0; grp < NG; ++grp)
-            if (4 * grp + pc_a < nsend) {
-                const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((4 * grp + pc_a) * 7 + pc_quad) * 16);
+            if (ONE || 4 * grp + pc_a < nsend) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((ONE ? 0 : 4 * grp + pc_a) * 7 + pc_quad) * 16);
 #pragma unroll
-                for (int k = 0; k < 2; ++k) cl_st_async16(a + grp * GSTR + dy[k], v, bar + dy[k]);
+                for (int k = 0; k < (ONE ? 1 : 2); ++k) cl_st_async16(a + grp * GSTR + dy[k], v, bar + dy[k]);
             }
     };
     const float inv_h0 = p.inv_O1[0] * h_inv, inv_h1 = p.inv_O1[1] * h_inv, inv_l0 = p.inv_O2[0] * h_inv, inv_l1 = p.inv_O2[1] * h_inv;
@@ -640,7 +647,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc[grp][0][k] += acc[grp][1][k];
                 float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
-                part_sum(acc[grp][0], d[0], d[8]);
+                if (!ONE || t4 == 0) part_sum(acc[grp][0], d[0], d[8]);
             }
         }
         cl_bar_sync(1, 256);
@@ -648,7 +655,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         // ---- K-split sums, bias, relu, parts; every sending warp adds up the same sums (cheaper than a hand-over) and serves
         // four CTAs: warps 0..3 the first group of rows, 4..7 the second
         if ((NG == 2 || warp < 4) && pc_on) {
-            const int grp = NG == 2 ? warp >> 2 : 0, st = 4 * grp + pc_a;
+            const int grp = NG == 2 ? warp >> 2 : 0, st = ONE ? 0 : 4 * grp + pc_a;
             if (st < nsend && !bad) {
                 const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
                 float4 v = {0.f, 0.f, 0.f, 0.f};
@@ -664,7 +671,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
                 const uint2 hi = cl_split4(v.x, v.y, v.z, v.w, lo);
                 const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
+                for (int k = 0; k < (ONE ? 1 : 4); ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
             }
         }
         cl_bar_sync(W2 && !half ? 6 : 2, 512);   // the background warps are done with the last half-step (and, bf16, go on)
@@ -677,7 +684,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             for (int w = 0; w < NP; ++w)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) lv[w][i] = A[w * (CW_LOG / 16) + i * 32];
-            const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + 4 * (lane & 3));
+            const float4 lbias = *reinterpret_cast<const float4 *>((half ? sb2 : sb4) + (FUSED ? 0 : 4 * (lane & 3)));
             wait_bar(&xq, quse, (int)s, 2 + 4 * half);
             STAMP(8 * half + 3);
             const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
@@ -702,25 +709,27 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc[grp][0][k] += acc[grp][1][k];
                 float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
-                part_sum(acc[grp][0], d[0], d[8]);
+                if (!ONE || t4 == 0) part_sum(acc[grp][0], d[0], d[8]);
             }
             if (warp >= 4) cl_bar_arrive(3, 224);
             else {
                 cl_bar_sync(3, 224);
                 STAMP(8 * half + 4);
-                if (lane < (FUSED ? 1 : 4 * nrc) && !bad) {
-                    const int st = lane >> 2;
+                if (lane < (FUSED ? 4 : ONE ? 16 : 4 * nrc) && !bad) {
+                    const int st = ONE ? 0 : lane >> 2;
                     float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int sp = 0; sp < 7; ++sp) {
-                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + 4 * (lane & 3));
+                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + (FUSED ? 0 : 4 * (lane & 3)));
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
                     const float inv = half ? inv_l0 : inv_l1;
                     const uint32_t a = smem_u32(lbuf + (FUSED ? 4 * rank : st * 256 + CL * rank + 4 * (lane & 3))), bar = smem_u32(&xl);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        st_async_v4(a + delta4[k], fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + delta4[k]);
+                    for (int k = 0; k < (ONE ? 1 : 4); ++k) {
+                        const uint32_t d = ONE ? delta_l : delta4[k];
+                        st_async_v4(a + d, fmaf(v.x, inv, lbias.x), fmaf(v.y, inv, lbias.y), fmaf(v.z, inv, lbias.z), fmaf(v.w, inv, lbias.w), bar + d);
+                    }
                 }
                 STAMP(8 * half + 5);
             }
@@ -847,10 +856,11 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
 // ---------------------------------------------------------------------------------------------
 static const void *cl_kernel_of(int nr, bool dbg, int kind)
 {
-    if (kind == CL_F32) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_F32> : (const void *)resident_cluster_kernel<1, 0, CL_F32>;
-    if (kind == CL_FUSED) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_FUSED> : (const void *)resident_cluster_kernel<1, 0, CL_FUSED>;
-    if (nr <= 4) return dbg ? (const void *)resident_cluster_kernel<1, 1, CL_BF16> : (const void *)resident_cluster_kernel<1, 0, CL_BF16>;
-    return dbg ? (const void *)resident_cluster_kernel<2, 1, CL_BF16> : (const void *)resident_cluster_kernel<2, 0, CL_BF16>;
+#define CL_K(R, K) (dbg ? (const void *)resident_cluster_kernel<R, 1, K> : (const void *)resident_cluster_kernel<R, 0, K>)
+    if (kind == CL_FUSED) return CL_K(1, CL_FUSED);
+    if (kind == CL_F32) return nr == 1 ? CL_K(1, CL_F32) : CL_K(4, CL_F32);
+    return nr == 1 ? CL_K(1, CL_BF16) : nr <= 4 ? CL_K(4, CL_BF16) : CL_K(8, CL_BF16);
+#undef CL_K
 }
 
 static void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
@@ -885,7 +895,7 @@ int rescl_prepare(wrnn_model *m)
     ResClPack k;
     k.kind = m->variant == 1 ? CL_FUSED : m->dtype == WRNN_F32 ? CL_F32 : CL_BF16;
     cudaFuncAttributes fa;
-    for (int nr : {1, 5})
+    for (int nr : {1, 2, 5})
         for (int dbg = 0; dbg < 2; ++dbg) {
             const void *f = cl_kernel_of(nr, dbg != 0, k.kind);
             const size_t CS_BYTES = cl_launch_smem(k.kind);
