@@ -473,14 +473,16 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             const float x = xin(c_prev, k);
             su = fmaf(Iu[k], x, su); sr = fmaf(Ir[k], x, sr); se = fmaf(Ie[k], x, se);
         }
-        q.pu = r_row(half_g * 3 * CU + gu) + su;
-        q.pr = r_row(half_g * 3 * CU + CU + gu) + sr;
-        q.pe = se;
-        q.ae = r_row(half_g * 3 * CU + 2 * CU + gu);
+        q.pu = su; q.pr = sr; q.pe = se; q.ae = 0.f;
         const int pend = half_g ? 2 * NX : NX;
 #pragma unroll
         for (int k = 0; k < NX; ++k) { q.ku[k] = Iu[pend + k]; q.kr[k] = Ir[pend + k]; q.ke[k] = Ie[pend + k]; }
         return q;
+    };
+    auto gates_add_r = [&](int half_g, GatePre &q) {
+        q.pu += r_row(half_g * 3 * CU + gu);
+        q.pr += r_row(half_g * 3 * CU + CU + gu);
+        q.ae = r_row(half_g * 3 * CU + 2 * CU + gu);
     };
     auto gates_and_stage = [&](int half_g, long long s, int drawn, const GatePre &q) {
         float pu = q.pu, pr = q.pr, pe = q.pe;
@@ -572,7 +574,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         const float *g = g_row + (size_t)s_fr[1][st_d] * 3 * H;
 #pragma unroll
         for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
-        gates_and_stage(0, 0, f_prev, gates_prepare(0, gv));
+        GatePre gp = gates_prepare(0, gv);
+        gates_add_r(0, gp);
+        gates_and_stage(0, 0, f_prev, gp);
     }
     __syncthreads();
     if (warp < 8) send_y(0, 0);
@@ -737,8 +741,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
         float dbg_l[8] = {};
         // ---- one row per warp: what does not depend on the draw, the draw, the gates
         if (drawer) {
-            if (!half) cl_bar_sync(4, 256 + n_draw);                  // R h is complete
-            const GatePre gp = gates_prepare(half, gv);
+            GatePre gp = gates_prepare(half, gv);
+            if (half) gates_add_r(half, gp);
             wait_bar(&xl, quse, (int)s, 3 + 4 * half);
             STAMP0();
             float l[8];
@@ -756,6 +760,10 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const ClParams
             }
             const int fed = (DBG && forced >= 0) ? forced : drawn;
             STAMP(8 * half + 6);
+            if (!half) {
+                cl_bar_sync(4, 256 + n_draw);                            // R h is complete: as a rule not before the draw (3.63 us per step with the wait there)
+                gates_add_r(half, gp);
+            }
             if (!last) gates_and_stage(half, s, fed, gp);
             STAMP(8 * half + 7);
             if (half) c_prev = fed; else f_prev = fed;
