@@ -235,7 +235,7 @@ def roofline(ctx, wl, info, model, n_steps, ms_per_step, cond_bytes, out_bytes):
         roof = {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                 "frac": ach / peaks["bf16_tflops_sustained"], "traffic": traffic, "traffic_note": traffic_note,
                 "peak_source": peaks["source"] + " sustained", "algorithmic_flops_per_step": flops}
-        if info["kernel"] == 2:      # the multi-stream resident kernel stamps the phases of its first CTA's first warp
+        if info["kernel"] == 2:      # the cluster-resident kernel stamps the phases of its first CTA's first warp
             pc = B.wrnn_phase_cycles(model)
             names = B.wrnn_phase_names(model)
             roof["phase_cycles_per_step"] = {k: round(v / n_steps, 1) for k, v in zip(names, pc)}

@@ -223,8 +223,7 @@ int wrnn_sample_subscale(wrnn_model *m, const float *cond, int32_t n_frames, int
  * stream id r, step = position, conditioning vector v_r[i] at step i.  The result does not depend on chunk or lag.
  * frames: DEVICE [B][n_frames][cond_dim]; V: DEVICE [B-1][F+1][cond_dim]; bias: DEVICE [cond_dim]; out: DEVICE int16
  * [n_total] in the original order.  B <= max_batch given at create.  Asynchronous on cuda_stream.  Dense bf16 H = 896
- * models of up to 16 rows advance all active rows in one launch of the multi-stream resident kernel (a lone row on the
- * single-stream resident kernel); other dense bf16 models use the cluster-partitioned kernel for two or more active rows;
+ * models advance all active rows in one launch of the cluster-resident kernel; other dense bf16 models use the cluster-partitioned kernel for two or more active rows;
  * everything else runs on the any-shape kernel.
  * wrnn_subscale_conditioning computes v_row[0..L) alone from a given history (DEVICE int16 [B][L]) into
  * v (DEVICE [L][cond_dim]).

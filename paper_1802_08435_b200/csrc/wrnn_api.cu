@@ -120,7 +120,7 @@ static bool use_resident(const wrnn_model *m, int batch)
     return m->resident != nullptr && resident_supported(m, batch, nullptr) == WRNN_OK;
 }
 
-// one stream of a dense bf16 H = 896 model: the lean form of the resident kernel (wrnn_reslean.cu)
+// one stream of a dense bf16 H = 896 model: the checked build of the lean resident kernel (wrnn_reslean.cu)
 // (WRNN_RESIDENT_LEAN=0 keeps the first form: diagnostic, for A/B measurements on one device)
 static bool use_reslean(const wrnn_model *m, int batch)
 {
@@ -645,7 +645,7 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
     auto run_rows = [&](int r_a, int n_rows, long long p_lo, int n) -> int {
         int rc = cond_rows(hist, v, L, r_a, n_rows, p_lo, n);
         if (rc != WRNN_OK) return fail(m, rc, "conditioning launch failed");
-        // rows advance together on the multi-stream resident kernel where the model has one; without it up to three rows go
+        // rows advance together on the cluster-resident kernel where the model has one; without it up to three rows go
         // one after the other through the single-stream kernel
         const int group = (n_rows >= 2 && use_rescl(m, n_rows)) ? n_rows : (n_rows <= 3 && (use_reslean(m, 1) || use_resident(m, 1))) ? 1 : n_rows;
         for (int b0 = 0; b0 < n_rows; b0 += group) {

@@ -1,4 +1,5 @@
-// Shared-memory-resident persistent sampling kernel for one stream, dense bf16 weights: the lean form.
+// Shared-memory-resident persistent sampling kernel for one stream, dense bf16 weights: the lean form.  Models run on the
+// cluster-resident kernel (wrnn_rescl.cu); this one is the checked build (WRNN_DEBUG=1 at create).
 //
 // Same machine as wrnn_resident.cu (Section 2.1 of the paper: one persistent launch per utterance, every weight on chip;
 // two chip-wide exchanges per step in the order of Fig. 1; both heads replicated once per 16-CTA cluster and row-sharded
@@ -11,8 +12,7 @@
 //     before it): two rows per warp on eight warps, a lane the element pairs lane, lane + 32, ... of both, six shuffles add up;
 //   * both cluster exchanges are asynchronous stores that count their bytes on the receiver's mbarrier;
 //   * the uniform, the forced symbol and the gate offsets of a half-step are pinned before its first wait;
-//   * the body of a half-step exists once per half, and plain sampling, teacher forcing (forced symbols, dumps), the phase
-//     stamps and the self-test predicate each run an instantiation of their own (template parameter MODE).
+//   * the body of a half-step exists once per half.
 // Hidden-layer and recurrent products are m16n8k16 bf16 MMAs on A-fragment-packed weights with the fp32 input as an
 // exact three-way bf16 split.  Every wait is bounded; a CTA that gives up records where and all CTAs leave through the
 // final cluster barrier.
@@ -109,12 +109,10 @@ __host__ __device__ constexpr size_t rl_smem_bytes(bool f)
 // would leave its array is skipped, and the kernel runs to its normal exit.
 constexpr int RL_N_GUARDS = 13;
 constexpr unsigned RL_GUARD_WORD = 0x5afec0deu;
-// MODE 0: plain sampling (no forced symbols, no dumps, no stamps, no self-test predicate: what wrnn_sample runs);
-// MODE 1: the instantiation that wrnn_selftest_lost_word runs (one CTA withholds one publication); MODE 2: the one with the
-// phase stamps of wrnn_phase_profile; MODE 3: teacher forcing and dumps.  Modes 1 to 3 all take forced symbols and dumps.
-template <bool CHK, bool FUSED, int MODE>
+template <bool FUSED>
 __global__ void __launch_bounds__(512, 1) resident_lean_kernel(const ResLeanParams p)
 {
+    constexpr bool CHK = true, HOOK = false, PROF = true, DBG = true;
     constexpr int RL_NLOG = rl_nlog(FUSED), RL_LR = rl_lr(FUSED), NIN = rl_nin(FUSED), NP = NIN / 3;
     constexpr size_t RL_W_BYTES = rl_w_bytes(FUSED), RL_BLOB_BYTES = rl_blob_bytes(FUSED);
     extern __shared__ __align__(16) uint8_t smem[];
@@ -185,7 +183,6 @@ __global__ void __launch_bounds__(512, 1) resident_lean_kernel(const ResLeanPara
 
     Waiter wt{p.status, p.limit_ns};
     bool my_bad = false;
-    constexpr bool HOOK = MODE == 1, PROF = MODE == 2 || CHK, DBG = MODE != 0 || CHK;
     const bool prof_on = PROF && p.prof != nullptr && (cta == 0 || p.prof_all) && warp == 0;
     __shared__ long long s_prof[16];
     __shared__ __align__(8) unsigned long long pub_bar;      // one arrival per half-step: this CTA's gate threads have published
@@ -531,21 +528,14 @@ __global__ void __launch_bounds__(512, 1) resident_lean_kernel(const ResLeanPara
 }
 
 // ---------------------------------------------------------------------------------------------
-static const void *kernel_of(const ResLeanPack &k, int mode)
-{
-    if (k.checked) return k.fused ? (const void *)resident_lean_kernel<true, true, 0> : (const void *)resident_lean_kernel<true, false, 0>;
-    if (mode == 1) return k.fused ? (const void *)resident_lean_kernel<false, true, 1> : (const void *)resident_lean_kernel<false, false, 1>;
-    if (mode == 2) return k.fused ? (const void *)resident_lean_kernel<false, true, 2> : (const void *)resident_lean_kernel<false, false, 2>;
-    if (mode == 3) return k.fused ? (const void *)resident_lean_kernel<false, true, 3> : (const void *)resident_lean_kernel<false, false, 3>;
-    return k.fused ? (const void *)resident_lean_kernel<false, true, 0> : (const void *)resident_lean_kernel<false, false, 0>;
-}
+static const void *kernel_of(const ResLeanPack &k) { return k.fused ? (const void *)resident_lean_kernel<true> : (const void *)resident_lean_kernel<false>; }
 
 static void fill_launch(const ResLeanPack &k, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s, bool coop)
 {
     std::memset(cfg, 0, sizeof(*cfg));
     cfg->gridDim = dim3(k.NCTA);
     cfg->blockDim = dim3(512);
-    cfg->dynamicSmemBytes = k.smem_bytes + (k.checked ? RL_N_GUARDS * 16 : 0);
+    cfg->dynamicSmemBytes = k.smem_bytes + RL_N_GUARDS * 16;
     cfg->stream = s;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = RL_CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -576,13 +566,10 @@ int reslean_prepare(wrnn_model *m)
     if (k.NCTA > m->n_sms || (size_t)k.smem_bytes > prop.sharedMemPerBlockOptin) { m->err = "lean resident kernel does not fit this device"; return WRNN_ERR_UNSUPPORTED; }
     { const char *d = getenv("WRNN_DEBUG"); k.checked = d && d[0] == '1'; }
     if (!k.checked) { m->err = "lean resident kernel: the checked build only (models run on the cluster-resident kernel otherwise)"; return WRNN_ERR_UNSUPPORTED; }
-    const void *fn = kernel_of(k, 0);
-    for (int mode = 0; mode < 4; ++mode) {
-        const void *f = kernel_of(k, mode);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem_bytes + (k.checked ? RL_N_GUARDS * 16 : 0)) != cudaSuccess) {
-            cudaGetLastError(); m->err = "lean resident kernel: cannot set the launch attributes"; return WRNN_ERR_UNSUPPORTED;
-        }
+    const void *fn = kernel_of(k);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem_bytes + RL_N_GUARDS * 16) != cudaSuccess) {
+        cudaGetLastError(); m->err = "lean resident kernel: cannot set the launch attributes"; return WRNN_ERR_UNSUPPORTED;
     }
     {
         cudaLaunchConfig_t cfg; cudaLaunchAttribute at[2];
@@ -668,7 +655,7 @@ int reslean_launch_info(const wrnn_model *m, int *n_ctas, int *n_threads, int *s
     const ResLeanPack &k = *m->reslean;
     if (n_ctas) *n_ctas = k.NCTA;
     if (n_threads) *n_threads = 512;
-    if (smem) *smem = k.smem_bytes + (k.checked ? RL_N_GUARDS * 16 : 0);
+    if (smem) *smem = k.smem_bytes + RL_N_GUARDS * 16;
     if (weight_bytes) *weight_bytes = k.weight_bytes_per_step;
     return WRNN_OK;
 }
@@ -705,7 +692,7 @@ int reslean_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     { const char *d = getenv("WRNN_DEBUG_POKE"); p.chk_poke = (k.checked && d && d[0] == '1') ? 1 : 0; }
     void *args[] = {&p};
     const bool teacher = p.c_forced || p.f_forced || p.a_forced || p.b_forced || p.dbg_gates || p.dbg_h || p.dbg_logits;
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel_of(k, m->dbg_skip_cta >= 0 ? 1 : (p.prof ? 2 : (teacher ? 3 : 0))), args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, kernel_of(k), args);
     if (e != cudaSuccess) {
         m->err = std::string("lean resident kernel launch failed: ") + cudaGetErrorString(e);
         cudaGetLastError();

@@ -794,6 +794,30 @@ def test_sparse_cluster_kernel_on_fewer_clusters(env, monkeypatch, n_clusters):
         B.wrnn_destroy(m)
 
 
+@pytest.mark.parametrize("batch", [2, 7, 8, 28, 29])
+def test_cluster_resident_kernel_fp32_row_counts(env, batch):
+    """fp32 weights on the cluster-resident kernel at the edges of its dispatch: one row per cluster (up to seven), several, the most
+    that the clusters take at once and a second wave.  Teacher-forced with dumps, then a run that is resumed against one in one piece."""
+    torch, B = env
+    w = synth.make_weights(896)
+    cond = synth.make_cond(batch, 2)
+    om = orc.OracleModel(w, "f32")
+    m = B.wrnn_create(w, "f32", max_batch=batch)
+    try:
+        assert B.wrnn_launch_info(m, batch)["n_ctas"] % 16 == 0
+        r = pu.teacher_forced_parity(torch, B, m, om, cond, 60, batch, SEED, row_stride=1, row_offset_mul=3, threads=pu.NCPU)
+        _report("cluster-resident kernel, fp32, %d rows" % batch, r)
+        _tol_check(r, "f32")
+        h = torch.zeros((batch, 896), dtype=torch.float32, device="cuda:0")
+        cp, fp = torch.full((batch,), 128, dtype=torch.uint8, device="cuda:0"), torch.zeros((batch,), dtype=torch.uint8, device="cuda:0")
+        full = _free_run(torch, B, m, cond, 60, batch, SEED, row_offset_mul=3)
+        a = _free_run(torch, B, m, cond, 23, batch, SEED, h=h, c_prev=cp, f_prev=fp, row_offset_mul=3)
+        b = _free_run(torch, B, m, cond, 37, batch, SEED, h=h, c_prev=cp, f_prev=fp, step0=23, row_offset_mul=3)
+        assert np.array_equal(np.concatenate([a, b], axis=1), full)
+    finally:
+        B.wrnn_destroy(m)
+
+
 @pytest.mark.parametrize("sparsity,block,n_ctas", [(0.96, (4, 4), 16), (0.96, (16, 1), 16), (0.995, (4, 4), 16), (0.93, (4, 4), 16), (0.88, (4, 4), 64)])
 def test_sparse_kernel_densities(env, sparsity, block, n_ctas):
     """The block-sparse kernel inside one cluster at its own edges -- hardly any block kept (block rows of R without any, slices of
