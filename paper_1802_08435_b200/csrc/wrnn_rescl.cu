@@ -1,29 +1,36 @@
-// Cluster-resident persistent sampling kernel: the whole dense bf16 H = 896 model lives in ONE 16-CTA cluster -- the
-// recurrent matrix in tensor memory, everything else in shared memory -- and a cluster advances its own rows alone.
+// Cluster-resident persistent sampling kernel: a whole dense H = 896 model lives in ONE 16-CTA cluster, most of the recurrent
+// matrix in tensor memory and everything else in shared memory, and a cluster advances its own rows alone.  Three kinds of
+// model: bf16 weights, fp32 weights, the Fused Subscale WaveRNN 2x.
 //
 // A step of the sampler (Fig. 1 of the paper) is a chain of exchanges, not of arithmetic: what bounds it is how long it
-// takes to hand the state, the hidden layer and the logits from the SM that computed them to the SMs that need them.  The
-// model is 6.1 MB; the shared memory of a 16-CTA cluster is 3.6 MB, but its tensor memory is another 4.2 MB, and
-// tcgen05.mma takes its A operand from there.  With the model inside one cluster every exchange is an all-gather through
-// distributed shared memory (measured here: 420 cycles + bytes / 17.5 per SM, against 1,000 - 1,500 cycles for the same
-// through L2 and across the chip), clusters never meet, and seven of them advance seven times as many rows in the same time.
+// takes to hand the state, the hidden layer and the logits from the SM that computed them to the SMs that need them, twice per
+// step.  A bf16 model is 6.1 MB; the shared memory of a 16-CTA cluster is 3.6 MB, but its tensor memory is another 4.2 MB.  With
+// the model inside one cluster every exchange is an all-gather through distributed shared memory (measured here: 420 cycles +
+// 0.87 per byte and receiver, against 1,000 - 1,500 cycles for the same through L2 and across the chip), clusters never meet, and
+// seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.39, 8 rows 3.73, 28 rows 4.38, 56 rows
+// 6.96 (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 37); fp32 4.9 (8.9); fused 3.7 (4.54).
 //
 // Per CTA (rank r of its cluster): state units 28 r .. 28 r + 27 of both halves with their 168 rows of R, rows 28 r .. of O1
 // and O3, rows 16 r .. of O2 and O4.
-//   * R: 128 rows (all 84 coarse rows and 44 fine ones) in tensor memory, the other 40 fine rows in shared memory.  Both feed
-//     mma.sync: a TMEM column is one register of an A fragment for the warps of its lane quadrant, so tcgen05.ld brings four
-//     fragments per instruction and no shared-memory load is spent on them.  (tcgen05.mma takes 46 cycles per K = 16 whatever
-//     N is up to 64; at eight operand columns mma.sync at 8 cycles per sub-partition does three times as much per cycle, and
-//     needs no proxy fence and no read-back of accumulators: 6.4 us per step with tcgen05.mma.)  The products are needed by
-//     the gates at the end of the half-step (coarse rows x fine columns) or later, and run beside the head.
-//   * The heads are on the critical path: K split over 4 (hidden layer) and 7 (logits) groups of warps, whose weight
-//     fragments are loaded from shared memory before the wait for the input (the loads, 4 cycles of the load / store unit per
-//     fragment, are what took the time in the shared-memory-resident kernels, not the MMAs).
-//   * State halves and hidden layers cross the cluster as bf16 parts of their fp32 values -- three exact parts when a
-//     cluster has one row, high and low parts (residual 2^-18) when it has several, as in the other multi-row kernels --
-//     stored by their producers straight into every receiver's operand image of 8 x 16-byte matrices, as ldmatrix reads them.
-//   * Every CTA draws every row of its cluster (one warp per row) and computes the gates of its own 28 units in the same
-//     warp, so the drawn symbol never leaves the warp.
+//   * Warps 0..7 are the chain: hidden layer (K split over four warps per tile), logits (K over seven), draw and gates (one row of
+//     the batch per warp: every CTA draws every row of its cluster, so that the drawn symbol never leaves the warp), sends.
+//   * Warps 8..15 multiply the rows of R in the background, from when the hidden layer is on its way; the chain waits for them
+//     after the draw of the fine half (before it: 3.63 us per step at one row).
+//   * R: 144 of the 168 rows in tensor memory, the other 24 in shared memory.  Both feed mma.sync: a column is one register of an A
+//     fragment for the warps of its lane quadrant, so tcgen05.ld brings four fragments per instruction and no shared-memory
+//     load is spent on them.  (tcgen05.mma takes 46 cycles per K = 16 whatever N is up to 64; at eight operand columns mma.sync at 8
+//     cycles per sub-partition does three times as much per cycle, and needs no read-back of accumulators: 6.4 us per step
+//     with tcgen05.mma.)
+//   * fp32 values cross the cluster as high and low fp16 parts of the value scaled by a power of two (error 2^-24 of the value, half
+//     a unit in the last place of fp32), bf16 weights are fp16 exactly after such a scaling; stored by their producers straight
+//     into every receiver's operand image.
+//   * What is sent to one receiver should be one run of bytes, and one instruction of a warp: a single row has an image of its
+//     own (112 contiguous bytes per CTA; as one row of four, 16-byte pieces 64 bytes apart: 3.84 us per step, 3.63).
+//   * fp32 weights: see W2 below.  Fused: 12 inputs per gate row, 64 logits as four softmaxes of 16.
+// What bounds it now, at one row: 3 x 2 all-gathers of 430 - 570 cycles, 2 x 390 for a draw, 2 x 200 for the gates, and products and sums of
+// 2 x 500, in 6,500 cycles; counters at one row: 0.22 instructions per cycle and sub-partition, stalls on barriers first.  Without the shared-
+// memory loads of the hidden layer's weights it would be 3.12 us; holding them in registers (setmaxnreg) starves the background
+// warps (3.51 - 4.4), loading them half a step ahead delays the logits (3.53).
 // Every wait is bounded; a warp that gives up records where, skips its remaining waits and sends and keeps meeting its
 // barriers, and all CTAs leave through the final cluster barrier.
 #include <cuda_fp16.h>
