@@ -132,8 +132,8 @@ static bool use_reslean(const wrnn_model *m, int batch)
 
 // Rows of a dense H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
 // clusters of eight) and more in waves; the cluster-partitioned kernel takes all at once and costs almost the same whatever
-// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 7.1 / 25.2, 57: 12.5 / 25.3, 112: 14.3 / 25.8,
-// 168: 21.3 / 28.7, 224: 28.4 / 31.0, 256 (a fifth wave): 35.5 / 32.3.
+// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 7.0 / 25.2, 57: 11.9 / 25.3, 112: 13.9 / 25.8,
+// 168: 20.9 / 28.7, 224: 27.9 / 31.0, 256 (a fifth wave): 34.8 / 32.2.
 constexpr int RESCL_BF16_ROWS = 224;
 static bool use_rescl(const wrnn_model *m, int batch)
 {

@@ -8,7 +8,7 @@
 // the model inside one cluster every exchange is an all-gather through distributed shared memory (measured here: 420 cycles +
 // 0.87 per byte and receiver, against 1,000 - 1,500 cycles for the same through L2 and across the chip), clusters never meet, and
 // seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.39, 8 rows 3.73, 28 rows 4.38, 56 rows
-// 6.96 (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 37); fp32 4.9 (8.9); fused 3.7 (4.54).
+// 6.96 (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 37); fp32 4.9 (7.4); fused 3.45 (4.54).
 //
 // Per CTA (rank r of its cluster): state units 28 r .. 28 r + 27 of both halves with their 168 rows of R, rows 28 r .. of O1
 // and O3, rows 16 r .. of O2 and O4.
