@@ -582,7 +582,7 @@ int sparse_prepare(wrnn_model *m)
     const bool tall = m->mask_br == 16 && m->mask_bc == 1;
     if (!tall && (m->mask_br != 4 || m->mask_bc != 4)) { m->err = "sparse cluster kernel takes 4 x 4 or 16 x 1 blocks"; return WRNN_ERR_UNSUPPORTED; }
     if (Hh != 1024) { m->err = "only H/2 = 1024 is instantiated (8 warps x 8 k-tiles for the logits tile)"; return WRNN_ERR_UNSUPPORTED; }
-    // One cluster with a kernel of its own where the kept blocks fit it (H = 2048, 4 % kept: 3.97 us per step, 6.54 on four clusters);
+    // One cluster with a kernel of its own where the kept blocks fit it (H = 2048, 4 % kept: 3.92 us per step, 6.54 on four clusters);
     // models with more blocks here.
     if (!getenv("WRNN_SPARSE_CLUSTERS") && sparse1_prepare(m) == WRNN_OK) return WRNN_OK;
     // The rows of R are dealt over NC clusters of 16 (the heads are held once per cluster); more clusters mean fewer block

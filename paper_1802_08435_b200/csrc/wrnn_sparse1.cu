@@ -4,8 +4,8 @@
 // What bounds a step is the chain state -> hidden layer -> logits -> draw -> gates -> state, twice: three all-gathers per
 // half-step and what lies between them.  Inside one cluster every all-gather goes through distributed shared memory (some 700
 // cycles for 1,024 values here), where the form on four clusters (wrnn_sparse.cu) passes the state through L2 (1,250 and
-// more).  The price, four times as many rows of R per CTA, is paid off the chain: 6.54 us per step on four clusters, 3.97 here
-// (4 x 4 blocks, 4 % kept; 16 x 1: 6.7 -> 3.98).
+// more).  The price, four times as many rows of R per CTA, is paid off the chain: 6.54 us per step on four clusters, 3.92 here
+// (4 x 4 blocks, 4 % kept; 16 x 1: 6.7 -> 3.97).
 //   * Warps 0..7 are the chain.  Hidden layer: a warp has 8 rows over all of K, their kept blocks and block columns in registers
 //     before the state arrives.  Logits: 16 dense rows, K over the eight warps, tensor cores (fp16 weights from tensor memory
 //     times the high and low fp16 parts of the hidden layer, which is how it is sent).  Draw and gates: warps 0 and 1, the same
@@ -41,7 +41,11 @@ constexpr int PU = PK / PCS;             // state units of one half, rows of O1 
 constexpr int PL = 16;                   // logits rows per CTA
 constexpr int PCW = 8, PBW = 12;         // chain warps, background warps
 constexpr int PTHREADS = 32 * (PCW + PBW);
-constexpr int PPRE = 2, BPRE = 3;        // iterations of a hidden-layer slice, of a slice of R, whose weights are loaded before the state arrives
+constexpr int PPRE = 2;                  // iterations of a hidden-layer slice whose weights are loaded before the state arrives
+// the same of a slice of R, of which every slice has the first p_min; a 16 x 1 block has sixteen sums and less room for weights
+// (4 x 4: 3.97 us per step with three, 3.93 with up to four; 16 x 1: 3.98, 4.05)
+__host__ __device__ constexpr int p_pre(bool tall) { return tall ? 3 : 4; }
+__host__ __device__ constexpr int p_min(bool tall) { return tall ? 3 : 2; }
 constexpr int PSMALL = 6 * PU * 3 + 2 * PU + PCW * PL;      // floats: I [half][gate][unit][3], b1, b3, b2, b4
 constexpr int PDW = PU / 32;             // drawing warps: one unit per lane
 constexpr int PVEC = 3 * PK + 256 + 2 * 6 * PU + 2 * PU + PCW * PL;       // floats: two state halves, hidden layer, logits, R h (partial, complete), staged y, q, K-split logits
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
     const long long T = p.n_steps;
 
     // ---- rows of R (background): block rows of one half of the state, four (sixteen) lanes each; `start` is called when the weights of
-    // the first BPRE iterations (as a rule all of them) are in registers
+    // the first p_pre iterations (as a rule all of them) are in registers
     auto r_products = [&](int half_f, auto start) {
         const PSlice &sl = slices[2 * PCW + half_f * PBW + warp - PCW];
         const uint32_t wt_col = tmem + sl.tcol;
@@ -192,10 +196,12 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
         const float *x = vec + half_f * PK;
         const int nt = sl.T;
         const int row = TALL ? 16 * sl.row[lane >> 4] + (lane & 15) : 4 * sl.row[lane >> 2] + (lane & 3);
+        constexpr int BPRE = p_pre(TALL), BMIN = p_min(TALL);
         uint4 w0[BPRE], w1[BPRE];
         int c[BPRE];
 #pragma unroll
-        for (int t = 0; t < BPRE; ++t) { p_tmem_ld8(wt_col + 8 * t, w0[t], w1[t]); c[t] = wc[32 * t]; }
+        for (int t = 0; t < BPRE; ++t)
+            if (t < BMIN || t < nt) { p_tmem_ld8(wt_col + 8 * t, w0[t], w1[t]); c[t] = wc[32 * t]; }
         tmem_wait_ld();
         float acc[16];
 #pragma unroll
@@ -203,9 +209,11 @@ __global__ void __launch_bounds__(PTHREADS, 1) sparse_chain_kernel(const Sparse1
         start();
         float4 xv[BPRE];
 #pragma unroll
-        for (int t = 0; t < BPRE; ++t) { if (TALL) xv[t].x = x[c[t]]; else xv[t] = *reinterpret_cast<const float4 *>(x + 4 * c[t]); }
+        for (int t = 0; t < BPRE; ++t)
+            if (t < BMIN || t < nt) { if (TALL) xv[t].x = x[c[t]]; else xv[t] = *reinterpret_cast<const float4 *>(x + 4 * c[t]); }
 #pragma unroll
         for (int t = 0; t < BPRE; ++t) {
+            if (t >= BMIN && t >= nt) break;
             if (TALL) { p_column(acc, w0[t], xv[t].x); p_column(acc + 8, w1[t], xv[t].x); }
             else p_block(*reinterpret_cast<float (*)[4]>(acc), w0[t], w1[t], xv[t]);
         }
@@ -578,7 +586,7 @@ int sparse1_prepare(wrnn_model *m)
                     longest = std::max(longest, (size_t)PPRE);
                 } else {
                     for (int b = 0; b < rpw; ++b) { sl.row[b] = (int16_t)ord[w * rpw + b]; longest = std::max(longest, (R[ord[w * rpw + b]].size() + lpr - 1) / lpr); }
-                    longest = std::max(longest, (size_t)BPRE);
+                    longest = std::max(longest, (size_t)p_min(tall));
                 }
                 sl.at = at; sl.T = (int)longest;
                 at += 32 * sl.T;
