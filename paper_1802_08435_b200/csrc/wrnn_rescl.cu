@@ -40,45 +40,23 @@
 // warps (3.51 - 4.4), loading them half a step ahead delays the logits (3.53).
 // Every wait is bounded; a warp that gives up records where, skips its remaining waits and sends and keeps meeting its
 // barriers, and all CTAs leave through the final cluster barrier.
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
 
-#include <cstdlib>
-#include <cstring>
-
-#include "wrnn_cl.cuh"
-#include "wrnn_cluster.cuh"
-#include "wrnn_half.h"
-#include "wrnn_internal.h"
-#include "wrnn_tc.cuh"
+#include "wrnn_rescl.cuh"
 
 namespace wrnn {
 
 namespace {
-constexpr int CK = 448;                  // H / 2
-constexpr int CU = 28;                   // state units of one half, hidden-layer rows per CTA
-constexpr int CL = 16;                   // logits rows per CTA
-constexpr int CCS = 16;                  // CTAs per cluster
-constexpr int CK8 = CK / 8, CQ = CK / 4; // groups of eight and of four values of a half
-constexpr int CRT = 9, CRS = 6 * CU - 16 * CRT;             // of the 168 rows of R: tiles of 16 in tensor memory, the 24 rows left in shared memory
-constexpr int CPH = 40, CPL = 24, CPR = 6 * CU;              // floats per (K-split, row) of the partial sums: conflict-free for the fragment owners
+constexpr int CPH = 40, CPL = 24;              // floats per (K-split, row) of the partial sums: conflict-free for the fragment owners
 constexpr size_t CW_HID = 2 * 28 * 512;                      // O1 (O3) rows of a CTA as A fragments: two tiles
 constexpr size_t CW_LOG = 28 * 512;                          // O2 (O4) rows: one tile
-constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
-enum { CL_BF16 = 0, CL_F32 = 1, CL_FUSED = 2 };                // kinds of model: bf16 weights, fp32 weights, the Fused Subscale WaveRNN 2x (bf16)
-__host__ __device__ constexpr int cl_nin(int kind) { return kind == CL_FUSED ? 12 : 3; }
-__host__ __device__ constexpr int cl_rows(int kind) { return kind == CL_FUSED ? 4 : CL; }       // logits rows per CTA in use
 // I of the CTA's units [half][gate][unit][3 or 12], b1, b3 (32 each), b2, b4
 __host__ __device__ constexpr int cl_small(int kind) { return 2 * 3 * CU * cl_nin(kind) + 2 * 32 + 2 * CL; }
 __host__ __device__ constexpr size_t cl_blob_smem(int kind)
 {
     return (kind == CL_F32 ? 2 : 1) * (2 * CW_HID + 2 * CW_LOG) + (kind == CL_F32 ? 0 : CW_R2) + cl_small(kind) * 4;
 }
-constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: [2 halves][7 k-tiles][9 tiles][4 registers]
-constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
 static_assert(cl_blob_smem(CL_BF16) % 16 == 0 && cl_blob_smem(CL_F32) % 16 == 0 && cl_blob_smem(CL_FUSED) % 16 == 0, "the blob is copied in 16-byte pieces");
 // fp32 weights, second part and the rows without room: [CTA][half][warp][k-tile v of 14][fragments of v][32 lanes][16 B] in an array of
 // its own, read from L2
@@ -110,185 +88,9 @@ struct ResClPack {
     long long *d_prof = nullptr;             // [16]
     int max_clusters = 0;
     bool checked = false;                    // every call runs the checked form
-    float inv_R = 0.f, inv_O1[2] = {0.f, 0.f}, inv_O2[2] = {0.f, 0.f}, q_scale[2] = {0.f, 0.f};
+    ClScales sc;
 };
 
-struct ClParams {
-    int batch, nr;              // rows of the call, rows per cluster
-    long long n_steps, step0;
-    unsigned stream0;
-    unsigned long long seed;
-    int n_frames, hop, row_stride, row_offset_mul, row_lag;
-    long long out_pitch;
-    const uint8_t *blob;
-    const uint4 *stream;
-    const float *g;                          // [batch][n_frames][3H]
-    float inv_R, inv_O1[2], inv_O2[2], q_scale[2];   // 2^-14 over the power of two in R, in the hidden layers and logits rows; the one of the hidden-layer values
-    const float *h_in; float *h_out;
-    const uint8_t *c_in, *f_in; uint8_t *c_st_out, *f_st_out;
-    const uint8_t *c_forced, *f_forced;
-    uint8_t *c_out, *f_out;
-    // the fused variant's 16-bit counterparts of the byte arrays (part A = the coarse half, part B = the fine half)
-    const uint16_t *a_in, *b_in; uint16_t *a_st_out, *b_st_out;
-    const uint16_t *a_forced, *b_forced; uint16_t *a_out, *b_out;
-    int16_t *out;
-    float *dbg_gates, *dbg_h, *dbg_logits;
-    DevStatus *status;
-    unsigned long long limit_ns;
-    int skip_rank; long long skip_step;      // self-test: CTAs of this rank withhold the state they publish at this step (-1: none)
-    long long *prof;
-    int poke; unsigned smem_bytes;           // checked form: one deliberate write past the end of region 6, by CTA 3; shared memory of the launch
-    // for cl_wide_steps: the model as the any-shape kernel has it, and its scratch rows
-    const void *wR, *wO[4];                  // R; O1, O3, O2, O4: 4 x 4 blocks, row by row
-    const float *wI, *wb[4];                 // I; b1, b3, b2, b4
-    float *q, *logits;                       // [batch][H / 2], [batch][256]
-};
-
-__device__ __forceinline__ void cl_ldmatrix4(uint32_t addr, uint32_t (&r)[4])
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void cl_st_async16(unsigned addr, uint4 v, unsigned mbar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(mbar) : "memory");
-}
-// f(0), .., f(N - 1) with compile-time arguments
-template <int N, int I = 0, typename F>
-__device__ __forceinline__ void cl_for(F &&f)
-{
-    if constexpr (I < N) { f(std::integral_constant<int, I>{}); cl_for<N, I + 1>(f); }
-}
-__device__ __forceinline__ uint4 cl_ldg_stream(const uint4 *p)
-{
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
-}
-// Steps of a cluster whose rows were given a state beyond what the operand images hold (CL_WIDE): plain fp32, one row of a matrix per
-// warp, everything exchanged through global memory, until no state is that large any more (a unit that changes is below one from then
-// on; what is not finite stays here).  Rare, so nothing of it is fast.  Returns the number of steps taken; sym [2][8] carries the
-// last symbols of the rows.  The state is in p.h_out throughout.
-constexpr float CL_WIDE = 2.f, CL_STATE = 16384.f;            // CL_STATE: what the state is multiplied by in the images (fp16 ends at 65504)
-template <int KIND>
-__device__ __noinline__ long long cl_wide_steps(const ClParams &p, int row0, int nrc, int rank, float *A, int (*sym)[8])
-{
-    constexpr bool FUSED = KIND == CL_FUSED;
-    constexpr int H = 2 * CK, NIN = cl_nin(KIND), NX = NIN / 3, LR = cl_rows(KIND), NL = CCS * LR;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // row `row` of a matrix of `cols` columns times x, on every lane
-    auto dot = [&](const void *M, int row, int cols, const float *x) {
-        float acc = 0.f;
-        for (int c = lane; c < cols / 4; c += 32) {
-            const size_t at = ((size_t)(row >> 2) * (cols / 4) + c) * 16 + 4 * (row & 3);
-            const float4 v = __ldcg(reinterpret_cast<const float4 *>(x) + c);
-            float4 w;
-            if (KIND == CL_F32) w = __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(M) + at));
-            else {
-                const uint2 b = __ldg(reinterpret_cast<const uint2 *>(static_cast<const uint16_t *>(M) + at));
-                w = make_float4(bf16lo(b.x), bf16hi(b.x), bf16lo(b.y), bf16hi(b.y));
-            }
-            acc = fmaf(w.x, v.x, fmaf(w.y, v.y, fmaf(w.z, v.z, fmaf(w.w, v.w, acc))));
-        }
-        return warp_sum(acc);
-    };
-    auto x_of = [](int v, int k) { return FUSED ? scale4((v >> (12 - 4 * k)) & 15) : scale8(v); };
-    // gates of one half: half 1 with the symbol of this step in sym[0], the last ones in `last`
-    auto gates = [&](int half_g, long long s, const int (*last)[8]) {
-        for (int i = tid; i < nrc * CU; i += 512) {
-            const int st = i / CU, u = i - st * CU, j = half_g * CK + CU * rank + u, gb = row0 + st;
-            const long long pos = (p.step0 + s) * p.row_stride + ((long long)p.stream0 + gb) * p.row_offset_mul;
-            const float *g = p.g + ((size_t)gb * p.n_frames + (size_t)(p.row_lag > 0 ? s : pos / p.hop)) * 3 * H + j;
-            float pre[3];
-            for (int gate = 0; gate < 3; ++gate) {
-                const float *I = p.wI + ((size_t)gate * H + j) * NIN;
-                float v = g[gate * H];
-                for (int k = 0; k < NX; ++k) {
-                    v = fmaf(I[k], x_of(last[0][st], k), fmaf(I[NX + k], x_of(last[1][st], k), v));
-                    if (half_g) v = fmaf(I[2 * NX + k], x_of(sym[0][st], k), v);
-                }
-                pre[gate] = v;
-            }
-            const float *a = A + st * CPR + half_g * 3 * CU + u;
-            const float uu = sigmoidf_acc(pre[0] + a[0]), r = sigmoidf_acc(pre[1] + a[CU]), e = tanhf(fmaf(r, a[2 * CU], pre[2]));
-            float *h = p.h_out + (size_t)gb * H + j;
-            const float hn = fmaf(uu, __ldcg(h), (1.0f - uu) * e);
-            __stcg(h, hn);
-            if (p.dbg_gates) { float *o = p.dbg_gates + ((size_t)s * p.batch + gb) * 3 * H; o[j] = uu; o[H + j] = r; o[2 * H + j] = e; }
-            if (p.dbg_h) p.dbg_h[((size_t)s * p.batch + gb) * H + j] = hn;
-        }
-        cluster_sync_all();
-    };
-    // head of one half (0: coarse): hidden layer, logits, the draw of row `warp`, the same in every CTA; the symbol fed back
-    auto head = [&](int hd, long long s) {
-        for (int i = warp; i < nrc * CU; i += 16) {
-            const int gb = row0 + i / CU, row = CU * rank + i % CU;
-            const float v = dot(p.wO[hd], row, CK, p.h_out + (size_t)gb * H + hd * CK);
-            if (lane == 0) __stcg(p.q + (size_t)gb * CK + row, fmaxf(v + p.wb[hd][row], 0.f));
-        }
-        cluster_sync_all();
-        for (int i = warp; i < nrc * LR; i += 16) {
-            const int gb = row0 + i / LR, row = LR * rank + i % LR;
-            const float v = dot(p.wO[2 + hd], row, CK, p.q + (size_t)gb * CK);
-            if (lane == 0) __stcg(p.logits + (size_t)gb * 256 + row, v + p.wb[2 + hd][row]);
-        }
-        cluster_sync_all();
-        if (warp < nrc) {
-            const int gb = row0 + warp;
-            const unsigned long long t = (unsigned long long)(p.step0 - (long long)gb * p.row_lag + s);
-            const float *L = p.logits + (size_t)gb * 256;
-            constexpr int PER = NL / 32;
-            float l[8];
-            for (int k = 0; k < PER; ++k) l[k] = __ldcg(L + PER * lane + k);
-            int drawn;
-            if (FUSED) {
-                const int nib = group16_softmax_draw(l[0], l[1], uniform24(p.seed, p.stream0 + (unsigned)gb, t, 4 * hd + (lane >> 3)), lane);
-                drawn = (__shfl_sync(FULL, nib, 0) << 12) | (__shfl_sync(FULL, nib, 8) << 8) | (__shfl_sync(FULL, nib, 16) << 4) | __shfl_sync(FULL, nib, 24);
-            } else drawn = warp_softmax_draw(l, uniform24(p.seed, p.stream0 + (unsigned)gb, t, hd), lane);
-            int fed = drawn;
-            if (FUSED) { const uint16_t *fz = hd ? p.b_forced : p.a_forced; if (fz) fed = fz[s]; }
-            else { const uint8_t *fz = hd ? p.f_forced : p.c_forced; if (fz) fed = fz[(size_t)gb * p.n_steps + s]; }
-            if (rank == 2 * warp) {
-                if (p.dbg_logits)
-                    for (int k = 0; k < PER; ++k) p.dbg_logits[(((size_t)s * p.batch + gb) * 2 + hd) * NL + PER * lane + k] = l[k];
-                if (lane == 0) {
-                    if (FUSED) {
-                        uint16_t *o = hd ? p.b_out : p.a_out;
-                        if (o) o[s] = (uint16_t)drawn;
-                        if (p.out) p.out[hd ? p.n_steps + s : s] = (int16_t)(fed - 32768);
-                    } else {
-                        uint8_t *o = hd ? p.f_out : p.c_out;
-                        if (o) o[(size_t)gb * p.n_steps + s] = (uint8_t)drawn;
-                        if (hd && p.out) p.out[(long long)gb * p.out_pitch + s] = (int16_t)(256 * sym[0][warp] + fed - 32768);
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) sym[hd][warp] = fed;
-        }
-        __syncthreads();
-    };
-    long long s = 0;
-    for (bool wide = true; wide && s < p.n_steps; ++s) {
-        for (int i = warp; i < nrc * CPR; i += 16) {
-            const int st = i / CPR, r = i - st * CPR;                        // as in the blob: half * 84 + gate * 28 + unit
-            const float v = dot(p.wR, (r / CU) % 3 * H + r / (3 * CU) * CK + CU * rank + r % CU, H, p.h_out + (size_t)(row0 + st) * H);
-            if (lane == 0) A[st * CPR + r] = v;
-        }
-        __shared__ int last[2][8];
-        if (tid < 16) last[tid >> 3][tid & 7] = sym[tid >> 3][tid & 7];
-        __syncthreads();
-        cluster_sync_all();                                                  // everybody has read the old state
-        gates(0, s, last);
-        head(0, s);
-        gates(1, s, last);
-        head(1, s);
-        int any = 0;
-        for (int i = tid; i < nrc * H; i += 512) any |= fabsf(__ldcg(p.h_out + (size_t)row0 * H + i)) > CL_WIDE;
-        wide = __syncthreads_or(any);
-        cluster_sync_all();
-    }
-    return s;
-}
 // ROWS: most rows of a cluster: 1, 4 or 8; fp32 weights 1 or 2.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate; MODE 2:
 // these and the checks.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
@@ -311,9 +113,9 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     constexpr int IR = ONE ? 1 : 4;                                      // rows that share a quad of an operand image
     constexpr bool DBG = MODE != 0, CHK = MODE == 2;
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ __align__(8) unsigned long long xy[2], xq, xl;            // arrivals: state halves, hidden layer, logits
+    __shared__ __align__(8) unsigned long long xw, xy[2], xq, xl;        // arrivals: weights, state halves, hidden layer, logits
     __shared__ uint32_t s_tmem;
-    __shared__ int s_sym[2][8];                                          // cl_wide_steps
+    __shared__ int s_sym[2][16];                                         // cl_wide_steps
     __shared__ float s_u[2][CMAXR];                                      // [coarse half?][row]: uniform, conditioning frame
     __shared__ int s_fr[2][CMAXR];
     __shared__ long long s_prof[MODE != 0 ? 16 : 1];
@@ -358,18 +160,17 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         if (p.h_in)
             for (int i = tid; i < nrc * H; i += 512) wide |= fabsf(__ldcg(p.h_in + (size_t)row0 * H + i)) > CL_WIDE;
         const uint8_t *blob = p.blob + (size_t)rank * (CB_SMEM + CB_TMEM);
-        const uint4 *src = reinterpret_cast<const uint4 *>(blob);
-        uint4 *dst = reinterpret_cast<uint4 *>(smem);
-        for (int i = tid; i < (int)(CB_SMEM / 16); i += 512) dst[i] = __ldg(src + i);
+        if (tid == 0) {
+            mbar_init(smem_u32(&xw), 1); mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
+            mbar_fence_init();
+            fence_proxy_async();
+            cl_load_bulk(smem_u32(smem), blob, (uint32_t)CB_SMEM, smem_u32(&xw));
+        }
         uint4 *z = reinterpret_cast<uint4 *>(ximg);
         for (int i = tid; i < (int)(3 * XSTR / 16); i += 512) z[i] = make_uint4(0, 0, 0, 0);
         if (warp == 1) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
-        if (tid == 0) {
-            mbar_init(smem_u32(&xy[0]), 1); mbar_init(smem_u32(&xy[1]), 1); mbar_init(smem_u32(&xq), 1); mbar_init(smem_u32(&xl), 1);
-            mbar_fence_init();
         }
         if (DBG && tid < 16) s_prof[tid] = 0;
         tc_fence_before();
@@ -387,21 +188,12 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                 else { if (p.c_st_out) p.c_st_out[row0 + tid] = (uint8_t)s_sym[0][tid]; if (p.f_st_out) p.f_st_out[row0 + tid] = (uint8_t)s_sym[1][tid]; }
             }
             if (s0 == p.n_steps) {
+                mbar_wait(smem_u32(&xw), 0, p.limit_ns);                  // no copy in flight when the CTA leaves
                 if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_tmem), "r"(512) : "memory");
                 return;
             }
         }
-        const uint32_t *tsrc = reinterpret_cast<const uint32_t *>(blob + CB_SMEM) + 32 * (warp & 3) + lane;
-        const uint32_t tdst = s_tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-#pragma unroll 1
-        for (int c = 8 * (warp >> 2); c < CTC; c += 32) {
-            uint32_t r[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) r[k] = __ldg(tsrc + (size_t)(c + k) * 128);
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(tdst + c), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]),
-                         "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        cl_load_tmem(s_tmem, blob + CB_SMEM, warp, lane);
         // images of the initial state
         if (p.h_in)
             for (int i = tid; i < nrc * H; i += 512) {
@@ -412,6 +204,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                 im[4] = __float2half_rn(x - __half2float(im[0]));
             }
     }
+    bool bad = !mbar_wait(smem_u32(&xw), 0, p.limit_ns);                 // this thread gave up: it skips waits and sends from here on
+    if (bad && atomicCAS(&p.status->code, DEV_OK, DEV_TIMEOUT) == DEV_OK) { p.status->cta = blockIdx.x; p.status->step = 0; p.status->phase = 9; }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -431,7 +225,6 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     const uint32_t tmem = s_tmem;
 
     Waiter wt{p.status, p.limit_ns};
-    bool bad = false;                                                    // this thread gave up: it skips waits and sends from here on
     const bool prof_on = DBG && p.prof != nullptr && blockIdx.x == 0 && warp == 0;
     long long prof_t = clock64();
 #define STAMP(i) do { if (DBG && prof_on) { const long long now_ = clock64(); if (lane == 0) s_prof[i] += now_ - prof_t; prof_t = now_; } } while (0)
@@ -679,7 +472,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     auto r_row = [&](int i) {
         const float *q = partR + st_d * CPR + i;
         const float v = (q[0] + q[4 * NG * CPR]) + (q[8 * NG * CPR] + q[12 * NG * CPR]);
-        return v * p.inv_R;
+        return v * p.sc.inv_R;
     };
     // everything of the gates of one half that does not depend on the pending draw
     auto gates_prepare = [&](int half_g, const float (&gv)[3]) {
@@ -889,8 +682,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                     const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
                     v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                 }
-                const float inv = p.inv_O1[1 - half];
-                const float qs = p.q_scale[1 - half];
+                const float inv = p.sc.inv_O1[1 - half];
+                const float qs = p.sc.q_scale[1 - half];
                 v.x = fmaxf(fmaf(v.x, inv, bias.x), 0.f) * qs; v.y = fmaxf(fmaf(v.y, inv, bias.y), 0.f) * qs;
                 v.z = fmaxf(fmaf(v.z, inv, bias.z), 0.f) * qs; v.w = fmaxf(fmaf(v.w, inv, bias.w), 0.f) * qs;
                 uint2 lo;
@@ -949,7 +742,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                         const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + (FUSED ? 0 : 4 * (lane & 3)));
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
-                    const float inv = p.inv_O2[1 - half];
+                    const float inv = p.sc.inv_O2[1 - half];
                     const uint32_t a = smem_u32(lbuf + (FUSED ? 4 * rank : st * 256 + CL * rank + 4 * (lane & 3))), bar = smem_u32(&xl);
 #pragma unroll
                     for (int k = 0; k < (ONE ? 1 : 4); ++k) {
@@ -1093,18 +886,6 @@ static const void *cl_kernel_of(int nr, int mode, int kind)
 #undef CL_K
 }
 
-static void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
-{
-    std::memset(cfg, 0, sizeof(*cfg));
-    cfg->gridDim = dim3(n_clusters * CCS);
-    cfg->blockDim = dim3(512);
-    cfg->dynamicSmemBytes = smem;
-    cfg->stream = s;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CCS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg->attrs = at;
-    cfg->numAttrs = 1;
-}
 
 // Rows per cluster and clusters of a batch.  Clusters never wait for one another, so a batch of more rows than the resident
 // clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
@@ -1141,48 +922,21 @@ int rescl_prepare(wrnn_model *m)
     const bool w2 = k.kind == CL_F32;
     const int NP = w2 ? 2 : 1, NIN = cl_nin(k.kind), LR = cl_rows(k.kind);
     HalfMatrix R(m->hR, NP), O[4] = {{m->hO1, NP}, {m->hO3, NP}, {m->hO2, NP}, {m->hO4, NP}};
-    const int e[5] = {R.exp, O[0].exp, O[1].exp, O[2].exp, O[3].exp};
-    // products of operands scaled by 2^(14 - exponent) each
-    k.inv_R = std::ldexp(1.f, e[0] - 28);
-    for (int h = 0; h < 2; ++h) {
-        const int eq = hidden_exp(h ? m->hO3 : m->hO1, h ? m->hb3 : m->hb1);
-        k.inv_O1[h] = std::ldexp(1.f, e[1 + h] - 28);
-        k.q_scale[h] = std::ldexp(1.f, 14 - eq);
-        k.inv_O2[h] = std::ldexp(1.f, e[3 + h] - 14 + eq - 14);
-    }
+    k.sc = ClScales(m, R, O);
     const size_t smem_bytes = cl_blob_smem(k.kind), cta_bytes = smem_bytes + CB_TMEM;
     std::vector<uint8_t> stream(w2 ? CCS * CB_STREAM : 0, 0);
     std::vector<uint8_t> blob(CCS * cta_bytes, 0);
     // part w of row i of a CTA's 168 rows of R: half * 84 + gate * 28 + unit
-    auto r_row = [&](int rank, int w, int i) { return &R.part[w][((size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU) * H]; };
-    // one row (g of a fragment's upper or lower eight) of the A fragment of a k-tile: lane (g, t) holds it at k 4t, 4t + 1 and at
-    // 4t + 2, 4t + 3 (the permuted k order), registers `lower` and 2 + `lower`
-    auto frag_row = [](uint16_t *frag, int g, int lower, const uint16_t *src) {
-        for (int t = 0; t < 4; ++t) {
-            uint16_t *d = frag + (4 * g + t) * 8 + 2 * lower;
-            d[0] = src[4 * t]; d[1] = src[4 * t + 1]; d[4] = src[4 * t + 2]; d[5] = src[4 * t + 3];
-        }
-    };
-    auto pack = [&](const std::vector<uint16_t> &M, int first, int n_rows, uint16_t *dst) {
-        for (int r = 0; r < n_rows; ++r)
-            for (int kt = 0; kt < 28; ++kt) frag_row(dst + (size_t)kt * 256, r & 7, r >> 3, &M[(size_t)(first + r) * CK + 16 * kt]);
-    };
+    auto r_row = [&](int rank, int w, int i) { return &R.part[w][r_row_at(rank, i)]; };
     parallel_for(CCS, [&](int rank) {
         uint8_t *base = blob.data() + (size_t)rank * cta_bytes;
         for (int h = 0; h < 2; ++h)
             for (int w = 0; w < NP; ++w) {
                 for (int t = 0; t < 2; ++t)
-                    pack(O[h].part[w], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + (h * NP + w) * CW_HID + (size_t)t * 28 * 512));
-                pack(O[2 + h].part[w], LR * rank, LR, reinterpret_cast<uint16_t *>(base + NP * 2 * CW_HID + (h * NP + w) * CW_LOG));
+                    pack_448(O[h].part[w], CU * rank + 16 * t, std::min(16, CU - 16 * t), reinterpret_cast<uint16_t *>(base + (h * NP + w) * CW_HID + (size_t)t * 28 * 512));
+                pack_448(O[2 + h].part[w], LR * rank, LR, reinterpret_cast<uint16_t *>(base + NP * 2 * CW_HID + (h * NP + w) * CW_LOG));
             }
-        if (!w2) {
-            uint16_t *r2 = reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG);
-            for (int i = 0; i < CRS; ++i)
-                for (int k8 = 0; k8 < 2 * CK8; ++k8) {
-                    const uint16_t *src = r_row(rank, 0, 16 * CRT + i) + 16 * (k8 >> 1) + 2 * (k8 & 1);
-                    for (int c = 0; c < 8; ++c) r2[((size_t)k8 * CRS + i) * 8 + c] = src[4 * (c >> 1) + (c & 1)];
-                }
-        }
+        if (!w2) pack_r2(R.part[0], rank, reinterpret_cast<uint16_t *>(base + 2 * CW_HID + 2 * CW_LOG));
         float *sm = reinterpret_cast<float *>(base + smem_bytes - cl_small(k.kind) * 4);
         for (int i = 0; i < 6 * CU; ++i) {
             const size_t row = (size_t)((i / CU) % 3) * H + (size_t)(i / (3 * CU)) * CK + CU * rank + i % CU;
@@ -1192,16 +946,13 @@ int rescl_prepare(wrnn_model *m)
         for (int r = 0; r < CU; ++r) { b[r] = m->hb1[CU * rank + r]; b[32 + r] = m->hb3[CU * rank + r]; }
         for (int r = 0; r < LR; ++r) { b[64 + r] = m->hb2[LR * rank + r]; b[64 + CL + r] = m->hb4[LR * rank + r]; }
         // tensor memory: lane quadrant q holds quarter q of the k-tiles of both halves of the state; columns as the kernel states them
-        uint16_t *tm = reinterpret_cast<uint16_t *>(base + smem_bytes);
         for (int i = 0; i < 16 * CRT; ++i) {
             const int tile = i >> 4, reg0 = (i >> 3) & 1;
             const uint16_t *src = r_row(rank, 0, i);
             for (int kt = 0; kt < 56; ++kt) {
                 const int half_f = kt / 28, q = kt % 28 / 7, k7 = kt % 7;
                 const int c0 = tile < 4 ? (half_f * 7 + k7) * 16 + 4 * tile : 2 * 7 * 16 + (half_f * 7 + k7) * 20 + 4 * (tile - 4);
-                for (int t = 0; t < 4; ++t)
-                    for (int h = 0; h < 2; ++h)
-                        std::memcpy(tm + ((size_t)(c0 + reg0 + 2 * h) * 128 + 32 * q + 4 * (i & 7) + t) * 2, src + 16 * kt + 4 * t + 2 * h, 4);
+                cl_pack_tmem_row(base + smem_bytes, q, c0, i & 7, reg0, src + 16 * kt);
             }
         }
         if (!w2) return;
@@ -1266,34 +1017,14 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
 {
     const ResClPack &k = *m->rescl;
     ClParams p;
-    std::memset(&p, 0, sizeof(p));
     int nr, n_clusters;
     cl_geometry(k, a.batch, &nr, &n_clusters);
-    p.batch = a.batch; p.nr = nr;
-    p.n_steps = a.n_steps; p.step0 = a.step0; p.stream0 = a.stream0; p.seed = a.seed;
-    p.n_frames = m->cond_dim ? a.n_frames : 1;
-    p.hop = m->cond_dim ? a.hop : 1;
-    p.row_stride = m->cond_dim ? a.row_stride : 0;
-    p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
-    p.row_lag = a.row_lag; p.out_pitch = a.out_pitch ? a.out_pitch : a.n_steps;
-    p.blob = k.d_blob; p.stream = k.d_stream; p.g = m->g;
-    p.inv_R = k.inv_R;
-    for (int h = 0; h < 2; ++h) { p.inv_O1[h] = k.inv_O1[h]; p.inv_O2[h] = k.inv_O2[h]; p.q_scale[h] = k.q_scale[h]; }
-    p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
-    p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
-    p.a_in = a.a_in; p.b_in = a.b_in; p.a_st_out = a.a_st_out; p.b_st_out = a.b_st_out;
-    p.a_forced = a.a_forced; p.b_forced = a.b_forced; p.a_out = a.a_out; p.b_out = a.b_out;
-    p.dbg_gates = a.dbg_gates; p.dbg_h = a.dbg_h; p.dbg_logits = a.dbg_logits;
-    p.status = m->status;
-    p.limit_ns = m->wait_limit_ns();
-    p.skip_rank = m->dbg_skip_cta >= 0 ? m->dbg_skip_cta % CCS : -1; p.skip_step = m->dbg_skip_step;
+    cl_fill_params(m, a, k.sc, &p);
+    p.nr = nr; p.blob = k.d_blob; p.stream = k.d_stream;
     p.prof = m->prof_enabled ? k.d_prof : nullptr;
-    p.wR = m->R.vals; p.wI = m->I; p.q = m->q; p.logits = m->logits;
-    p.wO[0] = m->O1.vals; p.wO[1] = m->O3.vals; p.wO[2] = m->O2.vals; p.wO[3] = m->O4.vals;
-    p.wb[0] = m->b1; p.wb[1] = m->b3; p.wb[2] = m->b2; p.wb[3] = m->b4;
     if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     if (k.checked) { const char *poke = getenv("WRNN_DEBUG_POKE"); p.poke = poke && poke[0] == '1'; }
-    const bool dbg = m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.c_out || p.f_out || p.a_forced || p.b_forced || p.a_out || p.b_out || p.dbg_gates || p.dbg_h || p.dbg_logits;
+    const bool dbg = cl_wants_dumps(m, p);
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
     p.smem_bytes = (unsigned)(k.checked ? cl_checked_smem(nr, k.kind) : cl_launch_smem(k.kind));
     cl_fill_launch(n_clusters, p.smem_bytes, &cfg, at, s);
