@@ -63,7 +63,7 @@ typedef enum {
     WRNN_KERNEL_RESIDENT = 2,   /* persistent kernel, weights resident in shared memory (one row; 2 to 16 rows of a dense bf16 H = 896 model) */
     WRNN_KERNEL_BATCHED = 3,    /* tensor-pipe contractions over all rows (dense bf16, >= 2 rows)  */
     WRNN_KERNEL_SPARSE = 4,     /* block-sparse model resident in 16-CTA clusters (one row)        */
-    WRNN_KERNEL_BCLUSTER = 5    /* rows dealt to 16-CTA clusters, tcgen05 contractions (dense bf16, >= 2 rows) */
+    WRNN_KERNEL_BCLUSTER = 5    /* rows dealt to 16-CTA clusters (dense bf16, >= 2 rows): each with the whole model, H = 896 by default; tcgen05 contractions otherwise and by name */
 } wrnn_kernel;
 
 /*

@@ -127,11 +127,15 @@ static bool use_resident(const wrnn_model *m, int batch)
     return m->resident != nullptr && resident_supported(m, batch, nullptr) == WRNN_OK;
 }
 
-// Rows of a dense H = 896 model: the kernel that holds the whole model in one cluster.  It takes 56 rows at a time (seven
-// clusters of eight) and more in waves; the cluster-partitioned kernel takes all at once and costs almost the same whatever
-// the rows.  us per step of this kernel / of the cluster-partitioned one: 56 rows 7.2 / 25.2, 57: 12.2 / 25.4, 112: 14.3 / 25.8,
-// 168: 21.5 / 28.8, 224: 28.8 / 31.1, 256 (a fifth wave): 36 / 32.3.
-constexpr int RESCL_BF16_ROWS = 224;
+// Rows of a dense H = 896 model: the kernels that hold the whole model in one cluster, up to four rows per cluster (seven clusters at a
+// time) in the one, five to fourteen in the other, more of either in waves of clusters.  us per step of the two at 28 rows: 4.38 / 4.59, at 8:
+// 3.72 / 4.52; of the second and the cluster-partitioned kernel: 29 rows 4.65 / 25, 56: 4.8 / 25.2, 98: 6.9 / 25.8, 168: 13.7 / 28.8, 224: 19.3 /
+// 31.1, 256: 20.4 / 32.2, 336: 27.6 / 34.
+constexpr int RESCL_BF16_ROWS = 28;
+// (beyond, the grid-phased kernel)
+constexpr int RESROWS_MOST = 336;
+// up to here its launches are stated as those of a resident kernel, then as those of the family that deals rows to clusters
+constexpr int RESROWS_RESIDENT = 224;
 static bool use_rescl(const wrnn_model *m, int batch)
 {
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
@@ -141,6 +145,13 @@ static bool use_rescl(const wrnn_model *m, int batch)
     if (off && off[0] == (batch == 1 ? '0' : '1')) return false;
     // (fp32 weights: 14 rows at a time; the any-shape kernel, the other one for several rows, takes 55 us per step at four)
     return (m->dtype == WRNN_F32 || batch <= RESCL_BF16_ROWS) && rescl_supported(m, batch) == WRNN_OK;
+}
+
+static bool use_resrows(const wrnn_model *m, int batch)
+{
+    if (m->kernel != WRNN_KERNEL_AUTO || !m->resrows || batch <= RESCL_BF16_ROWS || batch > RESROWS_MOST || batch > m->max_batch) return false;
+    const char *off = getenv("WRNN_NO_MULTI");
+    return !(off && off[0] == '1');
 }
 
 static bool use_resf32(const wrnn_model *m, int batch)
@@ -229,6 +240,7 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     if (!ensure_g(m, (size_t)a.batch * nf * 3 * m->H)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
     int rc = cond_project(m, a.cond, a.batch, nf, s);
     if (rc != WRNN_OK) return fail(m, rc, "conditioning projection launch failed");
+    if (use_resrows(m, a.batch)) return resrows_run(m, a, s);
     if (use_rescl(m, a.batch)) return rescl_run(m, a, s);
     // staggered rows: the cluster-partitioned kernel, else the any-shape kernel
     if (a.row_lag > 0) {
@@ -410,13 +422,14 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "sparse cluster kernel unavailable: " + why);
         }
     }
-    // Only kernels that some call can reach are packed.  The cluster-resident kernel takes every row count of an fp32 model and up
-    // to 224 rows of a bf16 one; the first forms serve models it does not take and the two diagnostic switches.
+    // Only kernels that some call can reach are packed.  The cluster-resident kernels take every row count of an fp32 model and up to 336
+    // rows of a bf16 one; the first forms serve models they do not take and the two diagnostic switches.
     const char *no_lean = getenv("WRNN_RESIDENT_LEAN"), *no_multi = getenv("WRNN_NO_MULTI");
     const bool first_forms = (no_lean && no_lean[0] == '0') || (no_multi && no_multi[0] == '1');
     const bool any = p->kernel == WRNN_KERNEL_AUTO;
     if (any || p->kernel == WRNN_KERNEL_RESIDENT) rescl_prepare(m);
-    const bool all_rows = m->rescl && !first_forms && (m->dtype == WRNN_F32 || max_batch <= RESCL_BF16_ROWS);
+    if (any && max_batch > RESCL_BF16_ROWS) resrows_prepare(m);
+    const bool all_rows = m->rescl && !first_forms && (m->dtype == WRNN_F32 || max_batch <= RESCL_BF16_ROWS || (m->resrows && max_batch <= RESROWS_MOST));
     if (p->kernel == WRNN_KERNEL_BCLUSTER || (any && !all_rows)) {
         const int rc = bcluster_prepare(m);
         if (rc != WRNN_OK && p->kernel == WRNN_KERNEL_BCLUSTER) {
@@ -455,6 +468,7 @@ void wrnn_destroy(wrnn_model *m)
     resident_destroy(m);
     resf32_destroy(m);
     rescl_destroy(m);
+    resrows_destroy(m);
     batched_destroy(m);
     bcluster_destroy(m);
     sparse_destroy(m);
@@ -846,6 +860,10 @@ int wrnn_launch_info(wrnn_model *m, int32_t batch, int32_t *kernel, int32_t *n_c
                      int64_t *weight_bytes_per_step, int32_t *smem_bytes)
 {
     if (!m || batch < 1 || batch > m->max_batch) return WRNN_ERR_INVALID_ARG;
+    if (use_resrows(m, batch)) {
+        if (kernel) *kernel = batch <= RESROWS_RESIDENT ? WRNN_KERNEL_RESIDENT : WRNN_KERNEL_BCLUSTER;
+        return resrows_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
+    }
     if (use_rescl(m, batch)) {
         if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
         return rescl_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
@@ -915,6 +933,7 @@ int wrnn_phase_cycles(wrnn_model *m, int64_t *out16)
 {
     if (!m || !out16) return WRNN_ERR_INVALID_ARG;
     static_assert(sizeof(long long) == sizeof(int64_t), "");
+    if (m->prof_cl == 2) return resrows_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->prof_cl) return rescl_phase_cycles(m, reinterpret_cast<long long *>(out16));
     if (m->resf32) return resf32_phase_cycles(m, reinterpret_cast<long long *>(out16));
     return resident_phase_cycles(m, reinterpret_cast<long long *>(out16));

@@ -67,6 +67,7 @@ struct SparsePack;     // compressed block rows of the block-sparse kernel on se
 struct Sparse1Pack;    // the same inside one cluster
 struct ResF32Pack;     // per-CTA fp32 weight shards of the single-stream fp32 resident kernel (opaque here)
 struct ResClPack;      // per-CTA weights of the cluster-resident kernel (opaque here)
+struct ResRowsPack;    // the same of its form for many rows
 struct BcPack;         // per-CTA weight slices and stacked activation images of the cluster-partitioned multi-row kernel
 
 }  // namespace wrnn
@@ -105,7 +106,8 @@ struct wrnn_model {
     wrnn::ResidentPack *resident = nullptr;
     wrnn::ResF32Pack *resf32 = nullptr;
     wrnn::ResClPack *rescl = nullptr;
-    bool prof_cl = false;             // the last call with phase timing ran on the cluster-resident kernel
+    wrnn::ResRowsPack *resrows = nullptr;
+    int prof_cl = 0;                  // the last call with phase timing ran on the cluster-resident kernel (2: on its form for many rows)
     // wrnn_selftest_lost_word: bound of every device-side wait (0 = the default of two seconds) and the CTA / step whose
     // publication (or operand load) is withheld (-1 = none)
     unsigned long long dbg_limit_ns = 0;
@@ -221,6 +223,13 @@ void rescl_destroy(wrnn_model *m);
 int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
 int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int rescl_phase_cycles(const wrnn_model *m, long long *out16);
+
+// wrnn_resrows.cu: five to fourteen rows per cluster (bf16)
+int resrows_prepare(wrnn_model *m);
+void resrows_destroy(wrnn_model *m);
+int resrows_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
+int resrows_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
+int resrows_phase_cycles(const wrnn_model *m, long long *out16);
 
 // wrnn_resf32.cu: the same role for dense fp32 models (every matrix sharded chip-wide, nothing replicated)
 int resf32_supported(const wrnn_model *m, int batch, std::string *why);

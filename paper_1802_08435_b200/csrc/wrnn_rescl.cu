@@ -7,8 +7,8 @@
 // step.  A bf16 model is 6.1 MB; the shared memory of a 16-CTA cluster is 3.6 MB, but its tensor memory is another 4.2 MB.  With
 // the model inside one cluster every exchange is an all-gather through distributed shared memory (measured here: 420 cycles +
 // 0.87 per byte and receiver, against 1,000 - 1,500 cycles for the same through L2 and across the chip), clusters never meet, and
-// seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.33, 8 rows 3.69, 28 rows 4.32, 56 rows
-// 7.1 (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 37); fp32 5.1 to 6.9, with where the streamed weights lie, up to 7
+// seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.33, 8 rows 3.69, 28 rows 4.38
+// (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 28; more rows of a bf16 model: wrnn_resrows.cu); fp32 5.1 to 6.9, with where the streamed weights lie, up to 7
 // rows and 6.2 to 7.1 up to 14 (7.4 at one row, 55 and more at several); fused 3.5 (4.54).
 //
 // Per CTA (rank r of its cluster): state units 28 r .. 28 r + 27 of both halves with their 168 rows of R, rows 28 r .. of O1
@@ -65,20 +65,17 @@ __host__ __device__ constexpr int cl_fo(int rj, int v) { return v < 7 ? v * (rj 
 __host__ __device__ constexpr int cl_fw(int w8) { return w8 < 4 ? w8 * cl_fo(0, 14) : 4 * cl_fo(0, 14) + (w8 - 4) * cl_fo(1, 14); }   // before warp w8
 constexpr int CF_HALF = cl_fw(8);                            // fragments of a half: 336
 constexpr size_t CB_STREAM = (size_t)2 * CF_HALF * 512;
-__host__ __device__ constexpr size_t cl_img(int ng) { return (size_t)CQ * ng * 64; }                // operand image of one vector
-__host__ __device__ constexpr size_t cl_part(int ng) { return (size_t)7 * 4 * ng * CPL * 4; }       // partial sums (>= 4 * 4 * ng * CPH * 4)
-static_assert((size_t)7 * 4 * CPL * 4 >= (size_t)4 * 4 * CPH * 4, "the partial sums of both products share a buffer");
-__host__ __device__ constexpr size_t cl_part_r(int ng) { return (size_t)4 * 4 * ng * CPR * 4; }     // R h
-__host__ __device__ constexpr size_t cl_smem(int ng, int kind)
+constexpr size_t C_PART = 7 * 4 * CPL * 4;                   // partial sums of the logits rows; of the hidden rows
+static_assert(C_PART >= 4 * 4 * CPH * 4, "the partial sums of both products share a buffer");
+constexpr size_t C_PART_R = 4 * 4 * CPR * 4;                 // R h
+__host__ __device__ constexpr size_t cl_smem(int kind)
 {
-    return cl_blob_smem(kind) + 3 * cl_img(ng) /* two state halves, hidden layer */ + (size_t)4 * ng * 1024 /* logits */ + cl_part(ng) + cl_part_r(ng) +
-           (size_t)4 * ng * 2 * CU * 2 /* staged state */;
+    return cl_blob_smem(kind) + 3 * CQ * 64 /* operand images: two state halves, hidden layer */ + 4 * 1024 /* logits */ + C_PART + C_PART_R + 4 * 2 * CU * 2 /* staged state */;
 }
 constexpr int CL_GUARDS = 8;             // of the checked form: behind the weights, the images (3), logits, sums, R h, staged state
-// what a launch asks for: the larger form of a kind (one CTA per SM either way)
-size_t cl_launch_smem(int kind) { return cl_smem(kind == CL_BF16 ? 2 : 1, kind); }
-// the checked form: that of its rows, with the guards
-size_t cl_checked_smem(int nr, int kind) { return cl_smem(kind == CL_BF16 && nr > 4 ? 2 : 1, kind) + CL_GUARDS * CL_GUARD; }
+// What a launch asks for: never so little that an SM would take a second CTA, which would wait for the first one's tensor memory
+size_t cl_launch_smem(int kind) { return std::max(cl_smem(kind), (size_t)200 * 1024 + 16); }
+size_t cl_checked_smem(int kind) { return cl_smem(kind) + CL_GUARDS * CL_GUARD; }
 }  // namespace
 
 struct ResClPack {
@@ -91,7 +88,7 @@ struct ResClPack {
     ClScales sc;
 };
 
-// ROWS: most rows of a cluster: 1, 4 or 8; fp32 weights 1 or 2.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate; MODE 2:
+// ROWS: most rows of a cluster: 1 or 4; fp32 weights 1 or 2.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate; MODE 2:
 // these and the checks.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
 // multiply the rows of R in the background, while the chain waits for exchanges.
@@ -106,9 +103,8 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     constexpr int NP = W2 ? 2 : 1;                                       // parts of a weight
     constexpr int NIN = cl_nin(KIND), NX = NIN / 3;                      // scalars of I per row, per symbol
     constexpr bool ONE = ROWS == 1, TWO = ROWS == 2;
-    constexpr int NG = ROWS > 4 ? 2 : 1;                                 // groups of four rows
-    constexpr size_t CB_SMEM = cl_blob_smem(KIND), CS_IMG = cl_img(NG), CS_PART = cl_part(NG), CS_PARTR = cl_part_r(NG);
-    constexpr int CMAXR = 4 * NG;
+    constexpr size_t CB_SMEM = cl_blob_smem(KIND), CS_IMG = CQ * 64, CS_PART = C_PART, CS_PARTR = C_PART_R;
+    constexpr int CMAXR = 4;
     constexpr int NCH = W2 ? 4 : 2;                                      // chains of a sum in the heads; low parts of weights apart
     constexpr int IR = ONE ? 1 : 4;                                      // rows that share a quad of an operand image
     constexpr bool DBG = MODE != 0, CHK = MODE == 2;
@@ -143,15 +139,15 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     float *part = reinterpret_cast<float *>(smem + P0);                  // K-split sums of the hidden rows, then of the logits rows
     float *partR = reinterpret_cast<float *>(smem + R0);                 // [4 quarters of K][rows][168]: R h
     uint8_t *ystage = smem + Y0;                                         // [row][quad][16 bytes]: new state values of this CTA's units
-    static_assert(END == cl_smem(NG, KIND) + (CHK ? CL_GUARDS * CL_GUARD : 0), "the carve-up is what cl_smem says");
+    static_assert(END == cl_smem(KIND) + (CHK ? CL_GUARDS * CL_GUARD : 0), "the carve-up is what cl_smem says");
     auto guard = [&](int i) { return smem + (i == 0 ? CB_SMEM : i <= 3 ? X0 + i * XSTR - G : i == 4 ? P0 - G : i == 5 ? R0 - G : i == 6 ? Y0 - G : END - G); };
 
     // Operand image of a vector: [group][quad][IR rows][high x 4, low x 4] -- a producer's four values of a row travel in one 16-byte
     // store, and the B fragment of lane (column g = row, part; t = quad of the k-tile) is one 8-byte load.  The k order of a tile
     // is permuted accordingly in all weights: slot c holds k = 4 ((c & 7) / 2) + 2 (c / 8) + (c & 1).
-    constexpr uint32_t QSTR = 16 * IR, GSTR = CQ * 64;
-    auto img_off = [](int st, int quad) { return ONE ? (uint32_t)quad * 16 : (uint32_t)((st >> 2) * (CQ * 64) + (quad * 4 + (st & 3)) * 16); };
-    const uint32_t frag = t4 * QSTR + (ONE ? g4 & 1 : TWO ? g4 & 3 : g4) * 8;                            // of k-tile 0, group 0
+    constexpr uint32_t QSTR = 16 * IR;
+    auto img_off = [](int st, int quad) { return ONE ? (uint32_t)quad * 16 : (uint32_t)(quad * 4 + st) * 16; };
+    const uint32_t frag = t4 * QSTR + (ONE ? g4 & 1 : TWO ? g4 & 3 : g4) * 8;                            // of k-tile 0
 
     // ---- one-time load: weights, zero images, barriers, tensor memory
     long long s0 = 0;                                                    // steps that cl_wide_steps took
@@ -242,7 +238,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     // (a tile and a half), the other tiles 4..8, so that a B fragment is loaded once for five or six tiles (these loads and
     // ldmatrix share the load / store pipe with the chain's shuffles).  Columns: [first warp: half][k-tile][4 tiles][4], then
     // [second warp: half][k-tile][5 tiles][4].
-    float acc[6][NG][4];
+    float acc[6][4];
     const int rq = warp & 3, rj = (warp >> 2) & 1;
     const uint32_t r_col = tmem + ((uint32_t)(32 * rq) << 16) + (rj ? 2 * 7 * 16 : 0);
     auto chains = [](const float (&c)[NCH + NP - 1][4], int k) {
@@ -255,9 +251,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
 #pragma unroll
         for (int n = 0; n < 6; ++n)
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[n][grp][k] = 0.f;
+            for (int k = 0; k < 4; ++k) acc[n][k] = 0.f;
     };
     auto r_load = [&](int half_f, int kt, uint32_t (&r)[20]) {
         const uint32_t c = r_col + (uint32_t)((half_f * 7 + kt) * (rj ? 20 : 16));
@@ -281,39 +275,25 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         const uint32_t a1 = r2_addr + (uint32_t)(((half_f * CK8 + 14 * rq + ((lane >> 3) & 1)) * CRS + 16 + (lane & 7)) * 16);
         uint32_t r0[20], r1[20], t0[6], t1[6];
         r_load(half_f, 0, r0);
-        uint2 c0[NG], c1[NG];
-        auto load = [&](int kt, uint2 (&b)[NG], uint32_t (&t)[6]) {
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp) b[grp] = r_frag(kt, b0 + kt * 4 * QSTR + grp * GSTR);
+        uint2 c0, c1;
+        auto load = [&](int kt, uint2 &b, uint32_t (&t)[6]) {
+            b = r_frag(kt, b0 + kt * 4 * QSTR);
             if (!rj) {
                 cl_ldmatrix4(a0 + kt * 2 * CRS * 16, *reinterpret_cast<uint32_t (*)[4]>(&t));
                 asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(t[4]), "=r"(t[5]) : "r"(a1 + kt * 2 * CRS * 16) : "memory");
             }
         };
-        auto mmas = [&](const uint32_t (&r)[20], const uint2 (&b)[NG], const uint32_t (&t)[6]) {
+        auto mmas = [&](const uint32_t (&r)[20], const uint2 &b, const uint32_t (&t)[6]) {
 #pragma unroll
             for (int n = 0; n < 4; ++n)
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp) cl_mma(acc[n][grp], make_uint4(r[4 * n], r[4 * n + 1], r[4 * n + 2], r[4 * n + 3]), b[grp].x, b[grp].y);
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp) {
-                if (rj) cl_mma(acc[4][grp], make_uint4(r[16], r[17], r[18], r[19]), b[grp].x, b[grp].y);
-                else {
-                    cl_mma(acc[4][grp], make_uint4(t[0], t[1], t[2], t[3]), b[grp].x, b[grp].y);
-                    cl_mma(acc[5][grp], make_uint4(t[4], 0, t[5], 0), b[grp].x, b[grp].y);
-                }
+                cl_mma(acc[n], make_uint4(r[4 * n], r[4 * n + 1], r[4 * n + 2], r[4 * n + 3]), b.x, b.y);
+            if (rj) cl_mma(acc[4], make_uint4(r[16], r[17], r[18], r[19]), b.x, b.y);
+            else {
+                cl_mma(acc[4], make_uint4(t[0], t[1], t[2], t[3]), b.x, b.y);
+                cl_mma(acc[5], make_uint4(t[4], 0, t[5], 0), b.x, b.y);
             }
         };
         load(0, c0, t0);
-        if (NG == 2) {                                                   // (no registers for a second set of fragments)
-#pragma unroll
-            for (int kt = 0; kt < 7; ++kt) {
-                tmem_wait_ld();
-                mmas(r0, c0, t0);
-                if (kt < 6) { r_load(half_f, kt + 1, r0); load(kt + 1, c0, t0); }
-            }
-            return;
-        }
 #pragma unroll
         for (int kt = 0; kt < 7; ++kt) {
             tmem_wait_ld();
@@ -334,23 +314,20 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         if (ONE) {
             float v[12];
 #pragma unroll
-            for (int n = 0; n < 5; ++n) part_sum(acc[n][0], v[2 * n], v[2 * n + 1]);
-            v[10] = acc[5][0][0] + acc[5][0][1]; v[11] = 0.f;
+            for (int n = 0; n < 5; ++n) part_sum(acc[n], v[2 * n], v[2 * n + 1]);
+            v[10] = acc[5][0] + acc[5][1]; v[11] = 0.f;
             const int i0 = chain_sum(v, std::integral_constant<int, 12>{});
-            float *d = partR + rq * 4 * NG * CPR + g4;
+            float *d = partR + rq * 4 * CPR + g4;
 #pragma unroll
             for (int i = 0; i < 3; ++i)
                 if (i0 + i < (rj ? 10 : 11)) d[8 * (i0 + i) + (rj ? 64 : i0 + i < 8 ? 0 : 80)] = v[i];
             return;
         }
+        float *d = partR + (rq * 4 + t4) * CPR + g4;
 #pragma unroll
-        for (int grp = 0; grp < NG; ++grp) {
-            float *d = partR + (rq * 4 * NG + 4 * grp + t4) * CPR + g4;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) part_sum(acc[n][grp], d[(4 * rj + n) * 16], d[(4 * rj + n) * 16 + 8]);
-            part_sum(acc[4][grp], d[(rj ? 8 : 9) * 16], d[(rj ? 8 : 9) * 16 + 8]);
-            if (!rj) d[160] = acc[5][grp][0] + acc[5][grp][1];
-        }
+        for (int n = 0; n < 4; ++n) part_sum(acc[n], d[(4 * rj + n) * 16], d[(4 * rj + n) * 16 + 8]);
+        part_sum(acc[4], d[(rj ? 8 : 9) * 16], d[(rj ? 8 : 9) * 16 + 8]);
+        if (!rj) d[160] = acc[5][0] + acc[5][1];
     };
 
     // fp32 weights: two passes over a half of the state, first the tiles that hold the coarse rows (0..3 and 4, 5), then the others
@@ -415,7 +392,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                 }
                 if (N == 3) v[2] = (sum[1][0] + sum[1][1]) + (sum[1][2] + sum[1][3]);     // tile 10: its low parts are the lower rows
                 const int i0 = chain_sum(v, std::integral_constant<int, NV>{});
-                float *d = partR + (rq * 4 * NG + (ONE ? 0 : t4 & 1)) * CPR + ROW + g4;
+                float *d = partR + (rq * 4 + (ONE ? 0 : t4 & 1)) * CPR + ROW + g4;
 #pragma unroll
                 for (int i = 0; i < M; ++i) {
                     if (!half_f) keep[PASS][i] = v[i];
@@ -471,7 +448,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     // a row of R h of this row of the batch
     auto r_row = [&](int i) {
         const float *q = partR + st_d * CPR + i;
-        const float v = (q[0] + q[4 * NG * CPR]) + (q[8 * NG * CPR] + q[12 * NG * CPR]);
+        const float v = (q[0] + q[4 * CPR]) + (q[8 * CPR] + q[12 * CPR]);
         return v * p.sc.inv_R;
     };
     // everything of the gates of one half that does not depend on the pending draw
@@ -525,13 +502,11 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
     auto send_y = [&](int half_g, long long s) {
         if (bad || (ONE ? lane >= 14 : !pc_on) || (DBG && (int)s == skip_at)) return;
         const uint32_t a = sbase + (uint32_t)(X0 + half_g * XSTR) + pc_off, bar = smem_u32(&xy[half_g]);
+        if ((ONE || pc_a < nsend) && store_ok(pc_off, 16, CS_IMG)) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((ONE ? 0 : pc_a) * 7 + pc_quad) * 16);
 #pragma unroll
-        for (int grp = 0; grp < NG; ++grp)
-            if ((ONE || 4 * grp + pc_a < nsend) && store_ok(pc_off + grp * GSTR, 16, CS_IMG)) {
-                const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((ONE ? 0 : 4 * grp + pc_a) * 7 + pc_quad) * 16);
-#pragma unroll
-                for (int k = 0; k < (ONE ? 1 : 2); ++k) cl_st_async16(a + grp * GSTR + dy[k], v, bar + dy[k]);
-            }
+            for (int k = 0; k < (ONE ? 1 : 2); ++k) cl_st_async16(a + dy[k], v, bar + dy[k]);
+        }
     };
     const int n_draw = 32 * nrc;                                         // threads of the drawing warps
     const unsigned ybytes = (unsigned)(nsend * CK * 4), lbytes = FUSED ? 256u : (unsigned)(nrc * 1024);
@@ -644,42 +619,34 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
             if (W2) cl_bar_arrive(half ? 5 : 7, 512);
             STAMP(8 * half + 0);
             const uint32_t b0 = xin + 7 * split * 4 * QSTR + frag;
-            uint2 b[NG][7];
-            float acc[NG][NCH + NP - 1][4];
+            uint2 b[7];
+            float acc[NCH + NP - 1][4];
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+                b[i] = cl_lds8(b0 + i * 4 * QSTR);
+#pragma unroll
+            for (int k = 0; k < 4 * (NCH + NP - 1); ++k) acc[k >> 2][k & 3] = 0.f;
 #pragma unroll
             for (int i = 0; i < 7; ++i)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) b[grp][i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+                for (int w = 0; w < NP; ++w) cl_mma(acc[w ? NCH : i % NCH], av[w][i], b[i].x, b[i].y);
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                for (int k = 0; k < 4 * (NCH + NP - 1); ++k) acc[grp][k >> 2][k & 3] = 0.f;
-#pragma unroll
-            for (int i = 0; i < 7; ++i)
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                    for (int w = 0; w < NP; ++w) cl_mma(acc[grp][w ? NCH : i % NCH], av[w][i], b[grp][i].x, b[grp][i].y);
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[grp][0][k] = chains(acc[grp], k);
-                float *d = part + (split * 4 * NG + 4 * grp + t4) * CPH + tile * 16 + g4;
-                if (!ONE || t4 == 0) part_sum(acc[grp][0], d[0], d[8]);
-            }
+            for (int k = 0; k < 4; ++k) acc[0][k] = chains(acc, k);
+            float *d = part + (split * 4 + t4) * CPH + tile * 16 + g4;
+            if (!ONE || t4 == 0) part_sum(acc[0], d[0], d[8]);
         }
         cl_bar_sync(1, 256);
         STAMP(8 * half + 1);
         // ---- K-split sums, bias, relu, parts; every sending warp adds up the same sums (cheaper than a hand-over) and serves
         // four CTAs: warps 0..3 the first group of rows, 4..7 the second
-        if ((NG == 2 || warp < 4) && pc_on) {
-            const int grp = NG == 2 ? warp >> 2 : 0, st = ONE ? 0 : 4 * grp + pc_a;
-            if (st < nsend && !bad && store_ok(pc_off + grp * GSTR, 16, CS_IMG)) {
+        if (warp < 4 && pc_on) {
+            const int st = ONE ? 0 : pc_a;
+            if (st < nsend && !bad && store_ok(pc_off, 16, CS_IMG)) {
                 const float4 bias = *reinterpret_cast<const float4 *>((half ? sb1 : sb3) + 4 * pc_quad);
                 float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int sp = 0; sp < 4; ++sp) {
-                    const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPH + 4 * pc_quad);
+                    const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 + st) * CPH + 4 * pc_quad);
                     v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                 }
                 const float inv = p.sc.inv_O1[1 - half];
@@ -688,7 +655,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                 v.z = fmaxf(fmaf(v.z, inv, bias.z), 0.f) * qs; v.w = fmaxf(fmaf(v.w, inv, bias.w), 0.f) * qs;
                 uint2 lo;
                 const uint2 hi = cl_split4(v.x, v.y, v.z, v.w, lo);
-                const uint32_t a = qin + grp * GSTR + pc_off, bar = smem_u32(&xq);
+                const uint32_t a = qin + pc_off, bar = smem_u32(&xq);
 #pragma unroll
                 for (int k = 0; k < (ONE ? 1 : 4); ++k) cl_st_async16(a + delta4[k], make_uint4(hi.x, hi.y, lo.x, lo.y), bar + delta4[k]);
             }
@@ -707,29 +674,21 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
             wait_bar(&xq, quse, (int)s, 2 + 4 * half);
             STAMP(8 * half + 3);
             const uint32_t b0 = qin + 4 * warp * 4 * QSTR + frag;
-            uint2 b[NG][4];
-            float acc[NG][NCH + NP - 1][4];
+            uint2 b[4];
+            float acc[NCH + NP - 1][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                b[i] = cl_lds8(b0 + i * 4 * QSTR);
+#pragma unroll
+            for (int k = 0; k < 4 * (NCH + NP - 1); ++k) acc[k >> 2][k & 3] = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int grp = 0; grp < NG; ++grp) b[grp][i] = cl_lds8(b0 + i * 4 * QSTR + grp * GSTR);
+                for (int w = 0; w < NP; ++w) cl_mma(acc[w ? NCH : i % NCH], lv[w][i], b[i].x, b[i].y);
 #pragma unroll
-            for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                for (int k = 0; k < 4 * (NCH + NP - 1); ++k) acc[grp][k >> 2][k & 3] = 0.f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int grp = 0; grp < NG; ++grp)
-#pragma unroll
-                    for (int w = 0; w < NP; ++w) cl_mma(acc[grp][w ? NCH : i % NCH], lv[w][i], b[grp][i].x, b[grp][i].y);
-#pragma unroll
-            for (int grp = 0; grp < NG; ++grp) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) acc[grp][0][k] = chains(acc[grp], k);
-                float *d = part + (warp * 4 * NG + 4 * grp + t4) * CPL + g4;
-                if (!ONE || t4 == 0) part_sum(acc[grp][0], d[0], d[8]);
-            }
+            for (int k = 0; k < 4; ++k) acc[0][k] = chains(acc, k);
+            float *d = part + (warp * 4 + t4) * CPL + g4;
+            if (!ONE || t4 == 0) part_sum(acc[0], d[0], d[8]);
             if (warp >= 4) cl_bar_arrive(3, 224);
             else {
                 cl_bar_sync(3, 224);
@@ -739,7 +698,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
                     float4 v = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                     for (int sp = 0; sp < 7; ++sp) {
-                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 * NG + st) * CPL + (FUSED ? 0 : 4 * (lane & 3)));
+                        const float4 a = *reinterpret_cast<const float4 *>(part + (sp * 4 + st) * CPL + (FUSED ? 0 : 4 * (lane & 3)));
                         v.x += a.x; v.y += a.y; v.z += a.z; v.w += a.w;
                     }
                     const float inv = p.sc.inv_O2[1 - half];
@@ -882,7 +841,7 @@ static const void *cl_kernel_of(int nr, int mode, int kind)
 #define CL_K(R, K) (mode == 2 ? (const void *)resident_cluster_kernel<R, 2, K> : mode ? (const void *)resident_cluster_kernel<R, 1, K> : (const void *)resident_cluster_kernel<R, 0, K>)
     if (kind == CL_FUSED) return CL_K(1, CL_FUSED);
     if (kind == CL_F32) return nr == 1 ? CL_K(1, CL_F32) : CL_K(2, CL_F32);
-    return nr == 1 ? CL_K(1, CL_BF16) : nr <= 4 ? CL_K(4, CL_BF16) : CL_K(8, CL_BF16);
+    return nr == 1 ? CL_K(1, CL_BF16) : CL_K(4, CL_BF16);
 #undef CL_K
 }
 
@@ -891,7 +850,7 @@ static const void *cl_kernel_of(int nr, int mode, int kind)
 // clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
 static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
 {
-    const int most = k.max_clusters * (k.kind == CL_BF16 ? 8 : 2), waves = (batch + most - 1) / most;
+    const int most = k.max_clusters * (k.kind == CL_BF16 ? 4 : 2), waves = (batch + most - 1) / most;
     *nr = (batch + waves * k.max_clusters - 1) / (waves * k.max_clusters);
     *n_clusters = (batch + *nr - 1) / *nr;
 }
@@ -903,17 +862,17 @@ int rescl_prepare(wrnn_model *m)
     ResClPack k;
     { const char *d = getenv("WRNN_DEBUG"); k.checked = d && d[0] == '1'; }
     k.kind = m->variant == 1 ? CL_FUSED : m->dtype == WRNN_F32 ? CL_F32 : CL_BF16;
-    for (int nr : {1, 2, 5})
+    for (int nr : {1, 2})
         for (int mode = 0; mode < (k.checked ? 3 : 2); ++mode) {
             const void *f = cl_kernel_of(nr, mode, k.kind);
-            if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || !allow_smem(f, m->device, mode == 2 ? cl_checked_smem(nr, k.kind) : cl_launch_smem(k.kind))) {
+            if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || !allow_smem(f, m->device, mode == 2 ? cl_checked_smem(k.kind) : cl_launch_smem(k.kind))) {
                 cudaGetLastError(); m->err = "cluster-resident kernel does not fit this device"; return WRNN_ERR_UNSUPPORTED;
             }
         }
     {
         cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
         cl_fill_launch(1, cl_launch_smem(k.kind), &cfg, at, 0);
-        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.kind == CL_BF16 ? 5 : 1, 0, k.kind), &cfg) != cudaSuccess || k.max_clusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&k.max_clusters, cl_kernel_of(k.kind == CL_BF16 ? 4 : 1, 0, k.kind), &cfg) != cudaSuccess || k.max_clusters < 1) {
             cudaGetLastError(); m->err = "cluster-resident kernel: no 16-CTA cluster of this size fits the device"; return WRNN_ERR_UNSUPPORTED;
         }
     }
@@ -1008,7 +967,7 @@ int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thread
     cl_geometry(*m->rescl, batch, &nr, &n_clusters);
     if (n_ctas) *n_ctas = n_clusters * CCS;
     if (n_threads) *n_threads = 512;
-    if (smem) *smem = (int)(m->rescl->checked ? cl_checked_smem(nr, m->rescl->kind) : cl_launch_smem(m->rescl->kind));
+    if (smem) *smem = (int)(m->rescl->checked ? cl_checked_smem(m->rescl->kind) : cl_launch_smem(m->rescl->kind));
     if (weight_bytes) *weight_bytes = (int64_t)CCS * (int64_t)(cl_blob_smem(m->rescl->kind) + CB_TMEM + (m->rescl->kind == CL_F32 ? CB_STREAM : 0));
     return WRNN_OK;
 }
@@ -1026,7 +985,7 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     if (k.checked) { const char *poke = getenv("WRNN_DEBUG_POKE"); p.poke = poke && poke[0] == '1'; }
     const bool dbg = cl_wants_dumps(m, p);
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
-    p.smem_bytes = (unsigned)(k.checked ? cl_checked_smem(nr, k.kind) : cl_launch_smem(k.kind));
+    p.smem_bytes = (unsigned)(k.checked ? cl_checked_smem(k.kind) : cl_launch_smem(k.kind));
     cl_fill_launch(n_clusters, p.smem_bytes, &cfg, at, s);
     void *args[] = {&p};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, k.checked ? 2 : dbg, k.kind), args);
@@ -1036,7 +995,7 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
-    m->prof_cl = true;
+    m->prof_cl = 1;
     return WRNN_OK;
 }
 

@@ -113,6 +113,13 @@ __device__ __forceinline__ void cl_load_bulk(uint32_t dst, const uint8_t *src, u
     for (uint32_t o = 0; o < bytes; o += PIECE)
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst + o), "l"(src + o), "r"(min(PIECE, bytes - o)), "r"(bar) : "memory");
 }
+// what the threads of this CTA wrote to shared memory, to the bulk copies that start after the next barrier
+__device__ __forceinline__ void fence_proxy_async_cta() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// bulk copy into a CTA of the cluster, counted on a barrier there
+__device__ __forceinline__ void cl_copy_bulk(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
+}
 // Tensor memory: [4 lane quadrants][126 groups of four columns][32 lanes][16 B], a quadrant per warp modulo four, eight groups in flight per lane
 __device__ __forceinline__ void cl_load_tmem(uint32_t tmem, const uint8_t *src, int warp, int lane)
 {

@@ -572,7 +572,7 @@ int resf32_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
-    m->prof_cl = false;
+    m->prof_cl = 0;
     return WRNN_OK;
 }
 

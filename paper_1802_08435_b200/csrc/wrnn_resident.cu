@@ -1179,7 +1179,7 @@ int resident_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
-    m->prof_cl = false;
+    m->prof_cl = 0;
     return WRNN_OK;
 }
 
@@ -1236,7 +1236,7 @@ int resident_pair_run(wrnn_model *m, const StepArgs &a, int pair, cudaStream_t s
         return WRNN_ERR_CUDA;
     }
     ++g_launches;
-    m->prof_cl = false;
+    m->prof_cl = 0;
     return WRNN_OK;
 }
 
