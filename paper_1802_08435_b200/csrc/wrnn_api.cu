@@ -237,9 +237,12 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     if (a.n_steps == 0) return WRNN_OK;
     if (cudaSetDevice(m->device) != cudaSuccess) return fail(m, WRNN_ERR_CUDA, "cudaSetDevice failed");
     const int nf = m->cond_dim ? a.n_frames : 1;
-    if (!ensure_g(m, (size_t)a.batch * nf * 3 * m->H)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
-    int rc = cond_project(m, a.cond, a.batch, nf, s);
-    if (rc != WRNN_OK) return fail(m, rc, "conditioning projection launch failed");
+    int rc = WRNN_OK;
+    if (!a.g) {
+        if (!ensure_g(m, (size_t)a.batch * nf * 3 * m->H)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
+        rc = cond_project(m, a.cond, a.batch, nf, m->g, s);
+        if (rc != WRNN_OK) return fail(m, rc, "conditioning projection launch failed");
+    }
     if (use_resrows(m, a.batch)) return resrows_run(m, a, s);
     if (use_rescl(m, a.batch)) return rescl_run(m, a, s);
     // staggered rows: the cluster-partitioned kernel, else the any-shape kernel
@@ -615,9 +618,10 @@ namespace wrnn {
 // Subscale generation with dependent rows on the staggered schedule, whatever the conditioning network: `cond_rows`
 // computes the conditioning vectors v[n_rows][n][D] of one stepping call (rows r_a .. r_a + n_rows - 1, row b of the call
 // from position p_lo - b * lag on) from the sample history hist [B][L]; `reserve` makes room for calls of that many rows and steps.
-template <typename CondFn, typename ReserveFn>
+// `whole`, where it takes the call, steps all rows itself (it returns -1 where it does not): hst, hist, cp, fp are the zeroed carry state and history.
+template <typename CondFn, typename ReserveFn, typename WholeFn>
 static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop, int32_t F, int32_t chunk, int32_t lag, int64_t n_total, int32_t B,
-                                   uint64_t seed, int16_t *out, cudaStream_t s, CondFn cond_rows, ReserveFn reserve)
+                                   uint64_t seed, int16_t *out, cudaStream_t s, CondFn cond_rows, ReserveFn reserve, WholeFn whole)
 {
     if (m->variant != 0) return fail(m, WRNN_ERR_UNSUPPORTED, "subscale generation takes a WaveRNN model (variant 0)");
     if (m->cond_dim <= 0) return fail(m, WRNN_ERR_INVALID_ARG, "the model must be conditioned");
@@ -647,6 +651,11 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
     if (cudaMemsetAsync(hst, 0, (size_t)B * H * sizeof(float), s) != cudaSuccess || cudaMemsetAsync(cp, 128, B, s) != cudaSuccess ||
         cudaMemsetAsync(fp, 0, B, s) != cudaSuccess || cudaMemsetAsync(hist, 0, (size_t)B * L * sizeof(int16_t), s) != cudaSuccess)
         return fail(m, WRNN_ERR_CUDA, "scratch initialisation failed");
+
+    if (const int rc = whole(L, v, hst, hist, cp, fp); rc >= 0) {
+        if (rc != WRNN_OK) return rc;
+        return fold_launch(hist, n_total, B, out, true, s);
+    }
 
     auto run_rows = [&](int r_a, int n_rows, long long p_lo, int n) -> int {
         int rc = cond_rows(hist, v, L, r_a, n_rows, p_lo, n);
@@ -684,6 +693,72 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
     }
     return fold_launch(hist, n_total, B, out, true, s);
 }
+
+// A whole staggered generation in blocks of 64 positions, of which the network's conditioning of one is computed while the block before it is
+// stepped: what a row looks at in earlier rows lies lag - reach >= 128 steps back (the network 46 %, its 124 recomputed positions
+// of every 128 included, and the stepping half of 84 ms for sixteen rows of 6,000 positions, one after the other).  Network and projection run on one
+// stream, the stepping on another, of higher priority; both are joined to the caller's.  -1: not such a call.
+static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float *frames, int n_frames, int hop, int lag, long long L, int B, uint64_t seed, float *v,
+                              float *hst, int16_t *hist, uint8_t *cp, uint8_t *fp, cudaStream_t s)
+{
+    constexpr int N = 64;
+    if (!subnet_ring_fits(net, lag)) return -1;
+    const int D = m->cond_dim, H = m->H, most = (int)std::min<long long>(B, (L + lag - 1) / lag + 1);
+    for (int n = 1; n <= most; ++n)
+        if (!use_rescl(m, n) && !use_resrows(m, n)) return -1;
+    const size_t gn = (size_t)B * N * 3 * H;
+    if (!ensure_g(m, 2 * gn)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
+    if (const int rc = subnet_ring_reserve(net); rc != WRNN_OK) return fail(m, rc, "conditioning scratch allocation failed");
+    const cudaStream_t sn = subnet_side(net, 0), st = subnet_side(net, 1);
+    const auto follow = [](cudaStream_t to, int e, cudaStream_t from, wrnn_subscale_net *q) {
+        return cudaEventRecord(subnet_event(q, e), from) == cudaSuccess && cudaStreamWaitEvent(to, subnet_event(q, e), 0) == cudaSuccess;
+    };
+    if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess || subnet_clear_status(net, s) != WRNN_OK || !follow(sn, 4, s, net) ||
+        cudaStreamWaitEvent(st, subnet_event(net, 4), 0) != cudaSuccess)
+        return fail(m, WRNN_ERR_CUDA, "streams of the conditioning network");
+    const int warm = (subnet_reach(net) + N - 1) / N;                       // blocks that a row's network starts early
+    const long long end = (long long)(B - 1) * lag + L;
+    long long stepped[2] = {-1, -1};                                        // the block that each of the two events of the stepping stands for
+    int rc = WRNN_OK;
+    for (long long k = -warm; k * N < end && rc == WRNN_OK; ++k) {
+        const long long t = k * N;
+        // the network: every row whose next block is not before its first by more than `warm` nor beyond its end
+        const int n_hi = (int)std::min<long long>(B - 1, (t + (long long)warm * N) / lag), n_lo = t >= L ? (int)((t - L) / lag) + 1 : 0;
+        if (n_lo > n_hi) continue;                                          // (a gap between rows: lag > L)
+        for (int e = 0; e < 2; ++e)                                         // every stepping call of two blocks ago and before
+            if (stepped[e] >= 0 && stepped[e] <= k - 2 && cudaStreamWaitEvent(sn, subnet_event(net, 2 + e), 0) != cudaSuccess) rc = WRNN_ERR_CUDA;
+        if (rc == WRNN_OK) rc = subnet_ring_run(net, hist, frames, n_frames, hop, L, n_lo, n_hi - n_lo + 1, t, lag, v, m->wait_limit_ns(), sn);
+        if (t < 0 || rc != WRNN_OK) continue;
+        const int r_lo = n_lo, r_hi = (int)std::min<long long>(B - 1, t / lag), rows = r_hi - r_lo + 1;
+        if (rows < 1) continue;
+        float *g = m->g + (k & 1) * gn;
+        rc = cond_project(m, v + (size_t)r_lo * N * D, rows, N, g, sn);
+        if (rc == WRNN_OK && !follow(st, (int)(k & 1), sn, net)) rc = WRNN_ERR_CUDA;
+        // the oldest row may end inside the block: all rows up to there, then the others
+        const long long left = L - (t - (long long)r_lo * lag);
+        for (int from = 0, n = (int)std::min<long long>(N, left); from < N && rc == WRNN_OK; from += n, n = N - from) {
+            const int first = from > 0 ? 1 : 0, nr = rows - first, r0 = r_lo + first;
+            if (nr < 1) break;
+            const long long p0 = t + from - (long long)r0 * lag;
+            StepArgs a;
+            std::memset(&a, 0, sizeof(a));
+            a.g = g + ((size_t)first * N + from) * 3 * H; a.n_frames = N; a.hop = 1; a.row_stride = 1;
+            a.n_steps = n; a.batch = nr; a.seed = seed; a.step0 = p0; a.stream0 = (unsigned)r0;
+            a.h_in = a.h_out = hst + (size_t)r0 * H;
+            a.c_in = a.c_st_out = cp + r0; a.f_in = a.f_st_out = fp + r0;
+            a.out = hist + (size_t)r0 * L + p0;
+            a.row_lag = lag; a.out_pitch = L - lag;
+            // leave the SMs that the network's widest product takes, twelve per pair of rows, free where four rows per cluster allow that
+            a.clusters = std::max(1, (m->n_sms - 12 * ((rows + 1) / 2)) / 16);
+            rc = run_steps(m, a, st);
+        }
+        if (cudaEventRecord(subnet_event(net, 2 + (k & 1)), st) != cudaSuccess) rc = WRNN_ERR_CUDA;
+        stepped[k & 1] = k;
+    }
+    // whatever happened, the caller's stream waits for what was launched
+    if (!follow(s, 4, sn, net) || !follow(s, 4, st, net)) rc = WRNN_ERR_CUDA;
+    return rc == WRNN_OK ? rc : fail(m, rc, "staggered generation");
+}
 }  // namespace wrnn
 
 extern "C" {
@@ -700,7 +775,7 @@ int wrnn_sample_subscale_dependent(wrnn_model *m, const float *frames, int32_t n
                                    [&](const int16_t *hist, float *v, long long L, int r_a, int n_rows, long long p_lo, int n) {
                                        return subscale_cond_launch(hist, frames, V, bias, v, B, L, F, D, n_frames, hop, r_a, n_rows, p_lo, lag, n, s);
                                    },
-                                   [](int, int) { return (int)WRNN_OK; });
+                                   [](int, int) { return (int)WRNN_OK; }, [](long long, float *, float *, int16_t *, uint8_t *, uint8_t *) { return -1; });
 }
 
 int wrnn_sample_subscale_net(wrnn_model *m, wrnn_subscale_net *net, const float *frames, int32_t n_frames, int32_t hop, int32_t F, int32_t chunk,
@@ -716,7 +791,12 @@ int wrnn_sample_subscale_net(wrnn_model *m, wrnn_subscale_net *net, const float 
                                    [&](const int16_t *hist, float *v, long long L, int r_a, int n_rows, long long p_lo, int n) {
                                        return subnet_run(net, hist, frames, n_frames, hop, L, r_a, n_rows, p_lo, lag, n, v, m->wait_limit_ns(), s);
                                    },
-                                   [&](int n_rows, int n_steps) { return subnet_reserve(net, n_rows, n_steps); });
+                                   [&](int n_rows, int n_steps) { return subnet_reserve(net, n_rows, n_steps); },
+                                   [&](long long L, float *v, float *hst, int16_t *hist, uint8_t *cp, uint8_t *fp) {
+                                       // (v holds B x chunk vectors: two chunks of 64 positions and more, a chunk of 64 and more)
+                                       if (chunk < 64) return -1;
+                                       return subscale_net_whole(m, net, frames, n_frames, hop, lag, L, B, seed, v, hst, hist, cp, fp, s);
+                                   });
 }
 
 int wrnn_subscale_net_rows(wrnn_model *m, wrnn_subscale_net *net, const float *frames, int32_t n_frames, int32_t hop, int32_t lag, int16_t *hist,

@@ -11,6 +11,8 @@
 #include <algorithm>
 #include <cstdio>
 
+#include <type_traits>
+
 #include "wrnn_internal.h"
 
 namespace wrnn {
@@ -259,60 +261,138 @@ __global__ void __launch_bounds__(512, 1) generic_step_kernel(const GenericParam
 
 // NP pairs per block and pass: a weight is read once for NP of them (the weights come from L2: one pair per block kept 2,048
 // pairs -- a chunk of 128 steps of 16 rows -- at 107 us).  The sum over D runs in the same order whatever NP.
+// Few pairs: NP per block, four rows of the gates per thread (their weights of an input are one load), the weights of the next eight inputs
+// on their way while these are multiplied: bound by the latency of the loads.
+constexpr int COND_THREADS = 128;
 template <int NP>
-__global__ void cond_project_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT,
-                                    const float *__restrict__ b_gate, float *__restrict__ g, int G, int D,
-                                    long long n_pairs)
+__global__ void __launch_bounds__(COND_THREADS) cond_project_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT,
+                                                                    const float *__restrict__ b_gate, float *__restrict__ g, int G, int D,
+                                                                    long long n_pairs)
 {
     // blockIdx.y strides over the (row of the batch, frame) pairs, so no grid dimension limits their number
     extern __shared__ __align__(16) float fr[];              // [D][NP]
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = 4 * (blockIdx.x * COND_THREADS + threadIdx.x);           // (G = 3 H, H a multiple of eight)
     for (long long k0 = (long long)blockIdx.y * NP; k0 < n_pairs; k0 += (long long)gridDim.y * NP) {
         __syncthreads();
-        for (int i = threadIdx.x; i < D * NP; i += blockDim.x) {
+        for (int i = threadIdx.x; i < D * NP; i += COND_THREADS) {
             const int q = i / D, d = i - q * D;
             fr[d * NP + q] = k0 + q < n_pairs ? cond[(size_t)(k0 + q) * D + d] : 0.f;
         }
+        float4 w[8];
+        auto weights = [&](int d0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (d0 + i < D) w[i] = __ldg(reinterpret_cast<const float4 *>(W_condT + (size_t)(d0 + i) * G + row));
+        };
+        if (row < G) weights(0);
         __syncthreads();
         if (row < G) {
-            float acc[NP];
+            float4 acc[NP];
 #pragma unroll
-            for (int q = 0; q < NP; ++q) acc[q] = 0.f;
+            for (int q = 0; q < NP; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             // runs of eight are added up on their own: the sum is the same for a whole frame, and so is its rounding error, which the state
             // then follows (state over 300 steps, 2-norm of the error against 64 bits: 1.66e-7 with one chain of 64, 1.20e-7)
             for (int d0 = 0; d0 < D; d0 += 8) {
-                float run[NP];
+                float4 run[NP], v[8];
 #pragma unroll
-                for (int q = 0; q < NP; ++q) run[q] = 0.f;
+                for (int i = 0; i < 8; ++i) v[i] = w[i];
+                weights(d0 + 8);
+#pragma unroll
+                for (int q = 0; q < NP; ++q) run[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     if (d0 + i < D) {
-                        const float w = W_condT[(size_t)(d0 + i) * G + row];
 #pragma unroll
-                        for (int q = 0; q < NP; ++q) run[q] = fmaf(w, fr[(d0 + i) * NP + q], run[q]);
+                        for (int q = 0; q < NP; ++q) {
+                            const float x = fr[(d0 + i) * NP + q];
+                            run[q].x = fmaf(v[i].x, x, run[q].x); run[q].y = fmaf(v[i].y, x, run[q].y);
+                            run[q].z = fmaf(v[i].z, x, run[q].z); run[q].w = fmaf(v[i].w, x, run[q].w);
+                        }
                     }
 #pragma unroll
-                for (int q = 0; q < NP; ++q) acc[q] += run[q];
+                for (int q = 0; q < NP; ++q) { acc[q].x += run[q].x; acc[q].y += run[q].y; acc[q].z += run[q].z; acc[q].w += run[q].w; }
             }
-            const float b = b_gate ? b_gate[row] : 0.f;
+            const float4 b = b_gate ? __ldg(reinterpret_cast<const float4 *>(b_gate + row)) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < NP; ++q)
-                if (k0 + q < n_pairs) g[(size_t)(k0 + q) * G + row] = acc[q] + b;
+                if (k0 + q < n_pairs)
+                    *reinterpret_cast<float4 *>(g + (size_t)(k0 + q) * G + row) = make_float4(acc[q].x + b.x, acc[q].y + b.y, acc[q].z + b.z, acc[q].w + b.w);
         }
     }
 }
 
-// As many pairs per block as leave the chip two blocks per SM (a block of 256 rows of the gates takes some 11 columns of the
-// grid at H = 896): short calls are bound by latency and keep one pair per block.
+// Many pairs: a tile of 64 pairs x 128 rows per block, weights and frames of 32 inputs at a time in shared memory, eight pairs x four rows per thread --
+// three 16-byte loads for 32 products (a value of a frame is the same for a whole warp).  With every weight read from L2 by every block of 16
+// pairs, 1,024 pairs took 31 us at H = 896; @@FIG@@ now.
+constexpr int COND_TP = 64, COND_TR = 128, COND_TD = 32;
+__global__ void __launch_bounds__(256) cond_project_tile_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT, const float *__restrict__ b_gate,
+                                                                float *__restrict__ g, int G, int D, long long n_pairs)
+{
+    __shared__ __align__(16) float sw[COND_TD][COND_TR], sx[COND_TD][COND_TP + 4];
+    const int tid = threadIdx.x, lane = tid & 31, pg = tid >> 5;                 // rows row0 + 4 lane .., pairs k0 + 8 pg ..
+    const int row0 = blockIdx.x * COND_TR, row = row0 + 4 * lane;
+    for (long long k0 = (long long)blockIdx.y * COND_TP; k0 < n_pairs; k0 += (long long)gridDim.y * COND_TP) {
+        float4 acc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int dc = 0; dc < D; dc += COND_TD) {
+            const int n = min(COND_TD, D - dc);
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < COND_TD * COND_TR / 4 / 256; ++k) {
+                const int i = tid + 256 * k, d = i >> 5, r = row0 + 4 * (i & 31);
+                *reinterpret_cast<float4 *>(&sw[d][4 * (i & 31)]) =
+                    d < n && r < G ? __ldg(reinterpret_cast<const float4 *>(W_condT + (size_t)(dc + d) * G + r)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < COND_TD * COND_TP / 256; ++k) {
+                const int i = tid + 256 * k, d = i & (COND_TD - 1), q = i / COND_TD;
+                sx[d][q] = d < n && k0 + q < n_pairs ? __ldg(cond + (size_t)(k0 + q) * D + dc + d) : 0.f;
+            }
+            __syncthreads();
+            // runs of eight as above
+            for (int d0 = 0; d0 < n; d0 += 8) {
+                float4 run[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) run[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 w = *reinterpret_cast<const float4 *>(&sw[d0 + i][4 * lane]);
+                    const float4 xa = *reinterpret_cast<const float4 *>(&sx[d0 + i][8 * pg]), xb = *reinterpret_cast<const float4 *>(&sx[d0 + i][8 * pg + 4]);
+                    const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        run[q].x = fmaf(w.x, x[q], run[q].x); run[q].y = fmaf(w.y, x[q], run[q].y);
+                        run[q].z = fmaf(w.z, x[q], run[q].z); run[q].w = fmaf(w.w, x[q], run[q].w);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) { acc[q].x += run[q].x; acc[q].y += run[q].y; acc[q].z += run[q].z; acc[q].w += run[q].w; }
+            }
+        }
+        if (row < G) {
+            const float4 b = b_gate ? __ldg(reinterpret_cast<const float4 *>(b_gate + row)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (k0 + 8 * pg + q < n_pairs)
+                    *reinterpret_cast<float4 *>(g + (size_t)(k0 + 8 * pg + q) * G + row) = make_float4(acc[q].x + b.x, acc[q].y + b.y, acc[q].z + b.z, acc[q].w + b.w);
+        }
+    }
+}
+
+// Tiles from 256 pairs on (84 blocks at H = 896 and more); below, as many pairs per block as leave the chip two blocks per SM, one in short calls.
+// The sums are the same in all of them.
 static void cond_project_launch(const float *cond, const float *W_condT, const float *b_gate, float *g, int G, int D, long long n_pairs, cudaStream_t s)
 {
-    const int np = n_pairs >= 448 ? 16 : n_pairs >= 112 ? 4 : 1;
-    const dim3 grid((G + 255) / 256, (unsigned)std::min<long long>((n_pairs + np - 1) / np, 65535));
-    const size_t smem = (size_t)np * D * sizeof(float);
-    if (np == 16 && smem <= 48 * 1024) cond_project_kernel<16><<<grid, 256, smem, s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
-    else if (np >= 4 && (size_t)4 * D * sizeof(float) <= 48 * 1024)
-        cond_project_kernel<4><<<dim3(grid.x, (unsigned)std::min<long long>((n_pairs + 3) / 4, 65535)), 256, (size_t)4 * D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
-    else cond_project_kernel<1><<<dim3(grid.x, (unsigned)std::min<long long>(n_pairs, 65535)), 256, D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+    auto few = [&](auto NP_C) {
+        constexpr int NP = decltype(NP_C)::value;
+        const dim3 grid((G + 4 * COND_THREADS - 1) / (4 * COND_THREADS), (unsigned)std::min<long long>((n_pairs + NP - 1) / NP, 65535));
+        cond_project_kernel<NP><<<grid, COND_THREADS, (size_t)NP * D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+    };
+    if (n_pairs >= 256)
+        cond_project_tile_kernel<<<dim3((G + COND_TR - 1) / COND_TR, (unsigned)std::min<long long>((n_pairs + COND_TP - 1) / COND_TP, 65535)), 256, 0, s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+    else if (n_pairs >= 100 && (size_t)4 * D * sizeof(float) <= 48 * 1024) few(std::integral_constant<int, 4>{});
+    else few(std::integral_constant<int, 1>{});
 }
 
 __global__ void cond_bias_only_kernel(const float *__restrict__ b_gate, float *__restrict__ g, int G, int batch)
@@ -321,13 +401,13 @@ __global__ void cond_bias_only_kernel(const float *__restrict__ b_gate, float *_
     if (i < G * batch) g[i] = b_gate ? b_gate[i % G] : 0.f;
 }
 
-int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, cudaStream_t s)
+int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, float *g, cudaStream_t s)
 {
     const int G = 3 * m->H;
     if (m->cond_dim == 0) {
-        cond_bias_only_kernel<<<(G * batch + 255) / 256, 256, 0, s>>>(m->b_gate, m->g, G, batch);
+        cond_bias_only_kernel<<<(G * batch + 255) / 256, 256, 0, s>>>(m->b_gate, g, G, batch);
     } else {
-        cond_project_launch(cond, m->W_condT, m->b_gate, m->g, G, m->cond_dim, (long long)batch * n_frames, s);
+        cond_project_launch(cond, m->W_condT, m->b_gate, g, G, m->cond_dim, (long long)batch * n_frames, s);
     }
     ++g_launches;
     return cudaGetLastError() == cudaSuccess ? WRNN_OK : WRNN_ERR_CUDA;

@@ -55,6 +55,9 @@ struct StepArgs {
     // step of the call (0 = rows in lock step); out_pitch = samples between the rows of `out` (0 = n_steps)
     int row_lag;
     long long out_pitch;
+    // projected conditioning [batch][n_frames][3H] that is there already (null: projected from cond by this call), with a status word that is cleared
+    const float *g;
+    int clusters;            // at most so many 16-CTA clusters at a time, where that is possible (0: as many as there are)
     // fused subscale variant: 16-bit samples of parts A and B in place of the bytes above (batch 1)
     const uint16_t *a_in, *b_in; uint16_t *a_st_out, *b_st_out;
     const uint16_t *a_forced, *b_forced;         // [n_steps] or null
@@ -149,7 +152,7 @@ int check_step(wrnn_model *m, const wrnn_cond *cond, int64_t n_steps, int32_t ba
 // wrnn_generic.cu
 int generic_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem);
 int generic_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);   // returns wrnn_status
-int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, cudaStream_t s);
+int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, float *g, cudaStream_t s);
 void noalloc_warm(int device);   // resolves the device address of the fixed scratch array of wrnn_sample_noalloc (once per device)
 int fold_launch(const int16_t *x, long long n_total, int B, int16_t *sub, bool unfold, cudaStream_t s);
 int fs2_unfold_launch(const int16_t *ab, long long n, int16_t *u, cudaStream_t s);
@@ -160,6 +163,14 @@ int subscale_cond_launch(const int16_t *hist, const float *frames, const float *
 int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows,
                long long p_lo, int lag, int n_steps, float *v, unsigned long long limit_ns, cudaStream_t s);
 int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps);        // activations for calls of up to that many rows and steps
+// the same in blocks of 64 positions for a whole staggered generation, on rings (see wrnn_subnet.cu)
+bool subnet_ring_fits(const wrnn_subscale_net *n, int lag);
+int subnet_ring_reserve(wrnn_subscale_net *n);
+int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows, long long t0, int lag,
+                    float *v, unsigned long long limit_ns, cudaStream_t s);
+int subnet_clear_status(wrnn_subscale_net *n, cudaStream_t s);
+cudaStream_t subnet_side(const wrnn_subscale_net *n, int i);              // 0: the network's, 1: the stepping calls'
+cudaEvent_t subnet_event(const wrnn_subscale_net *n, int i);
 int subnet_reach(const wrnn_subscale_net *n);
 int subnet_B(const wrnn_subscale_net *n);
 int subnet_cond_dim(const wrnn_subscale_net *n);

@@ -848,10 +848,11 @@ static const void *cl_kernel_of(int nr, int mode, int kind)
 
 // Rows per cluster and clusters of a batch.  Clusters never wait for one another, so a batch of more rows than the resident
 // clusters take at CMAXR rows each runs as several waves of clusters, evenly filled.
-static void cl_geometry(const ResClPack &k, int batch, int *nr, int *n_clusters)
+static void cl_geometry(const ResClPack &k, int batch, int clusters, int *nr, int *n_clusters)
 {
-    const int most = k.max_clusters * (k.kind == CL_BF16 ? 4 : 2), waves = (batch + most - 1) / most;
-    *nr = (batch + waves * k.max_clusters - 1) / (waves * k.max_clusters);
+    const int per = k.kind == CL_BF16 ? 4 : 2, most = k.max_clusters * per, waves = (batch + most - 1) / most;
+    const int c = clusters > 0 && waves == 1 ? std::min(k.max_clusters, std::max(clusters, (batch + per - 1) / per)) : k.max_clusters;
+    *nr = (batch + waves * c - 1) / (waves * c);
     *n_clusters = (batch + *nr - 1) / *nr;
 }
 
@@ -964,7 +965,7 @@ int rescl_supported(const wrnn_model *m, int batch)
 int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes)
 {
     int nr, n_clusters;
-    cl_geometry(*m->rescl, batch, &nr, &n_clusters);
+    cl_geometry(*m->rescl, batch, 0, &nr, &n_clusters);
     if (n_ctas) *n_ctas = n_clusters * CCS;
     if (n_threads) *n_threads = 512;
     if (smem) *smem = (int)(m->rescl->checked ? cl_checked_smem(m->rescl->kind) : cl_launch_smem(m->rescl->kind));
@@ -977,11 +978,11 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     const ResClPack &k = *m->rescl;
     ClParams p;
     int nr, n_clusters;
-    cl_geometry(k, a.batch, &nr, &n_clusters);
+    cl_geometry(k, a.batch, a.clusters, &nr, &n_clusters);
     cl_fill_params(m, a, k.sc, &p);
     p.nr = nr; p.blob = k.d_blob; p.stream = k.d_stream;
     p.prof = m->prof_enabled ? k.d_prof : nullptr;
-    if (cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
+    if (!a.g && cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     if (k.checked) { const char *poke = getenv("WRNN_DEBUG_POKE"); p.poke = poke && poke[0] == '1'; }
     const bool dbg = cl_wants_dumps(m, p);
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];

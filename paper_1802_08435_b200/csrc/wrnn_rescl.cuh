@@ -315,7 +315,7 @@ void cl_fill_params(wrnn_model *m, const StepArgs &a, const ClScales &sc, ClPara
     p.row_stride = m->cond_dim ? a.row_stride : 0;
     p.row_offset_mul = m->cond_dim ? a.row_offset_mul : 0;
     p.row_lag = a.row_lag; p.out_pitch = a.out_pitch ? a.out_pitch : a.n_steps;
-    p.g = m->g; p.sc = sc;
+    p.g = a.g ? a.g : m->g; p.sc = sc;
     p.h_in = a.h_in; p.h_out = a.h_out; p.c_in = a.c_in; p.f_in = a.f_in; p.c_st_out = a.c_st_out; p.f_st_out = a.f_st_out;
     p.c_forced = a.c_forced; p.f_forced = a.f_forced; p.c_out = a.c_out; p.f_out = a.f_out; p.out = a.out;
     p.a_in = a.a_in; p.b_in = a.b_in; p.a_st_out = a.a_st_out; p.b_st_out = a.b_st_out;

@@ -46,6 +46,7 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *tm,
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
                  ::"r"(dst), "l"(tm), "r"(bar), "r"(x), "r"(y), "r"(z) : "memory");
 }
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap *tm) { asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory"); }
 // shared-memory matrix descriptor of a K-major tile with 128-byte swizzle (rows of 128 bytes, 8-row atoms of 1 KB)
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
 {
@@ -80,6 +81,23 @@ __device__ __forceinline__ void umma_bf16_kblock(uint32_t tmem_d, uint32_t a_lo,
                  "mov.b64 da, {a3, %5};\nmov.b64 db, {b3, %5};\n"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, t;\n}"
                  ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate_first), "r"(UMMA_DESC_HI) : "memory");
+}
+// The same for an A operand in two parts (high, low) against one B: per K = 16 first the high, then the low one.
+__device__ __forceinline__ void umma_bf16_kblock_parts(uint32_t tmem_d, uint32_t h_lo, uint32_t l_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate_first)
+{
+    asm volatile("{\n.reg .pred p, t;\n.reg .b32 h1, h2, h3, l1, l2, l3, b1, b2, b3;\n.reg .b64 da, dl, db;\n"
+                 "setp.ne.b32 p, %5, 0;\nsetp.eq.u32 t, %4, %4;\n"
+                 "add.u32 h1, %1, 2;\nadd.u32 l1, %2, 2;\nadd.u32 b1, %3, 2;\nadd.u32 h2, %1, 4;\nadd.u32 l2, %2, 4;\nadd.u32 b2, %3, 4;\n"
+                 "add.u32 h3, %1, 6;\nadd.u32 l3, %2, 6;\nadd.u32 b3, %3, 6;\n"
+                 "mov.b64 da, {%1, %6};\nmov.b64 dl, {%2, %6};\nmov.b64 db, {%3, %6};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\ntcgen05.mma.cta_group::1.kind::f16 [%0], dl, db, %4, t;\n"
+                 "mov.b64 da, {h1, %6};\nmov.b64 dl, {l1, %6};\nmov.b64 db, {b1, %6};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\ntcgen05.mma.cta_group::1.kind::f16 [%0], dl, db, %4, t;\n"
+                 "mov.b64 da, {h2, %6};\nmov.b64 dl, {l2, %6};\nmov.b64 db, {b2, %6};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\ntcgen05.mma.cta_group::1.kind::f16 [%0], dl, db, %4, t;\n"
+                 "mov.b64 da, {h3, %6};\nmov.b64 dl, {l3, %6};\nmov.b64 db, {b3, %6};\n"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, t;\ntcgen05.mma.cta_group::1.kind::f16 [%0], dl, db, %4, t;\n}"
+                 ::"r"(tmem_d), "r"(h_lo), "r"(l_lo), "r"(b_lo), "r"(idesc), "r"(accumulate_first), "r"(UMMA_DESC_HI) : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
@@ -142,6 +160,19 @@ inline bool make_map(CUtensorMap *tm, void *base, long long rows, int cols, int 
     const cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 3-D tensor map of rows [n_rows][n_pos][cols] bf16: box of 64 columns x 64 positions x 2 rows, 128-byte swizzle
+inline bool make_map_rows(CUtensorMap *tm, void *base, long long n_rows, int n_pos, int cols)
+{
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)n_pos, (cuuint64_t)n_rows};
+    const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * 2 * (cuuint64_t)n_pos};
+    const cuuint32_t box[3] = {(cuuint32_t)TC_BK, 64, 2};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
