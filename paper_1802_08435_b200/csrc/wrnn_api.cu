@@ -701,7 +701,9 @@ static int subscale_dependent_impl(wrnn_model *m, int32_t n_frames, int32_t hop,
 static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float *frames, int n_frames, int hop, int lag, long long L, int B, uint64_t seed, float *v,
                               float *hst, int16_t *hist, uint8_t *cp, uint8_t *fp, cudaStream_t s)
 {
-    constexpr int N = 64;
+    // The stepping calls take five clusters at most (up to five rows in one each, ten two by two, sixteen by up to four: 3.3, 3.7, 4.4 us per step), which
+    // leaves the network 68 SMs: 44.7 ms for 16 x 6,000 positions; 46.8 with six, 48.2 with four where its products could use the room.
+    constexpr int N = 64, STEP_CLUSTERS = 5;
     if (!subnet_ring_fits(net, lag)) return -1;
     const int D = m->cond_dim, H = m->H, most = (int)std::min<long long>(B, (L + lag - 1) / lag + 1);
     for (int n = 1; n <= most; ++n)
@@ -727,7 +729,7 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
         if (n_lo > n_hi) continue;                                          // (a gap between rows: lag > L)
         for (int e = 0; e < 2; ++e)                                         // every stepping call of two blocks ago and before
             if (stepped[e] >= 0 && stepped[e] <= k - 2 && cudaStreamWaitEvent(sn, subnet_event(net, 2 + e), 0) != cudaSuccess) rc = WRNN_ERR_CUDA;
-        if (rc == WRNN_OK) rc = subnet_ring_run(net, hist, frames, n_frames, hop, L, n_lo, n_hi - n_lo + 1, t, lag, v, m->wait_limit_ns(), sn);
+        if (rc == WRNN_OK) rc = subnet_ring_run(net, hist, frames, n_frames, hop, L, n_lo, n_hi - n_lo + 1, t, lag, v, m->n_sms - 16 * STEP_CLUSTERS, m->wait_limit_ns(), sn);
         if (t < 0 || rc != WRNN_OK) continue;
         const int r_lo = n_lo, r_hi = (int)std::min<long long>(B - 1, t / lag), rows = r_hi - r_lo + 1;
         if (rows < 1) continue;
@@ -748,8 +750,7 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
             a.c_in = a.c_st_out = cp + r0; a.f_in = a.f_st_out = fp + r0;
             a.out = hist + (size_t)r0 * L + p0;
             a.row_lag = lag; a.out_pitch = L - lag;
-            // leave the SMs that the network's widest product takes, twelve per pair of rows, free where four rows per cluster allow that
-            a.clusters = std::max(1, (m->n_sms - 12 * ((rows + 1) / 2)) / 16);
+            a.clusters = STEP_CLUSTERS;
             rc = run_steps(m, a, st);
         }
         if (cudaEventRecord(subnet_event(net, 2 + (k & 1)), st) != cudaSuccess) rc = WRNN_ERR_CUDA;

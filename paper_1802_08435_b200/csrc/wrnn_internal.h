@@ -167,7 +167,7 @@ int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps);        // act
 bool subnet_ring_fits(const wrnn_subscale_net *n, int lag);
 int subnet_ring_reserve(wrnn_subscale_net *n);
 int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows, long long t0, int lag,
-                    float *v, unsigned long long limit_ns, cudaStream_t s);
+                    float *v, int free_sms, unsigned long long limit_ns, cudaStream_t s);
 int subnet_clear_status(wrnn_subscale_net *n, cudaStream_t s);
 cudaStream_t subnet_side(const wrnn_subscale_net *n, int i);              // 0: the network's, 1: the stepping calls'
 cudaEvent_t subnet_event(const wrnn_subscale_net *n, int i);

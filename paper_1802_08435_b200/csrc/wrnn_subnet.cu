@@ -102,20 +102,22 @@ template <int N>
 __device__ __forceinline__ void sn_tmem_ld(uint32_t a, float (&r)[N])
 {
     if constexpr (N == 32) tmem_ld32(a, r);
+    else if constexpr (N == 8) tmem_ld8(a, r);
     else tmem_ld16(a, reinterpret_cast<uint32_t (&)[16]>(r));
 }
 
-// RING: a tile of 128 is 64 positions of each of two rows.  SPLIT (convolution of three taps): a cluster of three CTAs, one per tap, shares a
-// tile -- twelve k-blocks one after the other instead of 36, each of which takes 715 cycles of shared-memory traffic (44 KB in, 56 KB out to the
-// MMAs); each adds up a third of the channels.
-template <int BN, int MODE, int STAGES, bool RING, bool SPLIT = false>
+// RING: a tile of 128 is 64 positions of each of two rows.  NS (convolution): a cluster of NS CTAs shares a tile, each with 1 / NS of the k-blocks
+// -- of which it has 36 one after the other, each 715 cycles of shared-memory traffic (44 KB in, 56 KB out to the MMAs) -- and adds up 1 / NS of the
+// channels.
+template <int BN, int MODE, int STAGES, bool RING, int NS = 1>
 __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                                                                     const __grid_constant__ CUtensorMap tmW, const SubnetGemmParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tap = SPLIT ? (int)blockIdx.x % 3 : 0, nt = SPLIT ? (int)blockIdx.x / 3 : (int)blockIdx.x, mt = blockIdx.y, seg = blockIdx.z;
-    static_assert(!SPLIT || (MODE == SN_CONV && RING && BN == 96), "a third of the channels is a chunk of 32");
+    const int me = (int)blockIdx.x % NS, nt = (int)blockIdx.x / NS, mt = blockIdx.y, seg = blockIdx.z;       // (me: rank in the cluster)
+    static_assert(NS == 1 || (MODE == SN_CONV && RING && NS <= 3), "only these");
+    constexpr int CT = BN / NS, XS = CT * 4 + 16;               // channels that a CTA finishes; bytes of a row of sums that it is sent
     constexpr uint32_t A_BYTES = SN_BM * TC_BK * 2, W_BYTES = BN * TC_BK * 2, STAGE_BYTES = 2 * A_BYTES + W_BYTES;
     constexpr int TMEM_COLS = BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
     __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], done, part;
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     if (tid == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(smem_u32(&full[i]), 3); mbar_init(smem_u32(&empty[i]), 1); }
         mbar_init(smem_u32(&done), 1);
-        if (SPLIT) { mbar_init(smem_u32(&part), 1); mbar_expect_tx(smem_u32(&part), 2 * SN_BM * 128); }
+        if (NS > 1) { mbar_init(smem_u32(&part), 1); mbar_expect_tx(smem_u32(&part), (NS - 1) * SN_BM * CT * 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     }
     for (int i = tid; i < BN; i += SN_THREADS) s_bias[i] = MODE != SN_OUT ? __ldg(p.bias + nt * BN + i) : i < p.cond_dim ? __ldg(p.b_out + i) : 0.f;
     tc_fence_before();
-    if (SPLIT) cluster_sync_all();                              // every peer's barrier is initialised before anyone sends
+    if (NS > 1) cluster_sync_all();                              // every peer's barrier is initialised before anyone sends
     else __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
@@ -147,7 +149,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
     // clusters of a stepping call from starting.)
     if (warp != 3) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    const int nkb = (SPLIT ? 1 : p.taps) * p.n_kb_tap;
+    const int nkb = p.taps * p.n_kb_tap / NS;
     const int arow0 = seg * p.n_alloc + mt * SN_BM;          // first activation row (position) of this tile
     bool ok = true;
     if ((warp == 0 || warp == 2 || warp == 3) && lane == 0) {
@@ -156,8 +158,9 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
         const int op = warp == 0 ? 0 : warp - 1;                // high parts, low parts, weights
         const CUtensorMap *tm = op == 0 ? &tmAh : op == 1 ? &tmAl : &tmW;
         const uint32_t off = op * A_BYTES, bytes = op < 2 ? A_BYTES : W_BYTES;
-        const int y0 = op < 2 ? (RING ? (p.a_slot0 + tap * p.dil) & (SN_RING - 1) : arow0) : p.w_row0 + tap * p.w_tap_rows + nt * BN, ystep = op < 2 ? p.dil : p.w_tap_rows;
-        int st = 0, ph = 1, kc = 0, y = y0;
+        const int ystep = op < 2 ? p.dil : p.w_tap_rows, tap0 = me * nkb / p.n_kb_tap;
+        int st = 0, ph = 1, kc = (me * nkb - tap0 * p.n_kb_tap) * TC_BK, y = (op < 2 ? (RING ? p.a_slot0 : arow0) : p.w_row0 + nt * BN) + tap0 * ystep;
+        if (RING && op < 2) y &= SN_RING - 1;
         for (int kb = 0; kb < nkb; ++kb) {
             if (!mbar_wait(smem_u32(&empty[st]), ph, p.limit_ns)) { ok = false; break; }
             const uint32_t fb = smem_u32(&full[st]);
@@ -200,9 +203,9 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
         auto slot = [&](int i) { return (s0 + i) & (SN_RING - 1); };
         auto frow = [&](int i) { return RING ? slot(i) : i; };
         auto prow = [&](int i) { return RING && MODE == SN_RES ? slot(i) : i; };
-        constexpr int CH = (SPLIT ? 32 : BN) / 2, CC = CH % 32 ? 16 : 32;                  // channels that this warp finishes, in chunks of so many
-        const size_t fbase = (RING ? (size_t)r * SN_RING : (size_t)seg * p.n_alloc + j0) * p.C_out + nt * BN + 32 * tap + CH * cg;
-        const size_t pbase = (!RING ? (size_t)seg * p.n_alloc + j0 : MODE == SN_CONV ? (size_t)r * 64 + j0 : (size_t)r * (SN_RING + 64)) * p.C_out + nt * BN + 32 * tap + CH * cg;
+        constexpr int CH = CT / 2, CC = CH % 32 == 0 ? 32 : CH % 16 == 0 ? 16 : 8;                  // channels that this warp finishes, in chunks of so many
+        const size_t fbase = (RING ? (size_t)r * SN_RING : (size_t)seg * p.n_alloc + j0) * p.C_out + nt * BN + CT * me + CH * cg;
+        const size_t pbase = (!RING ? (size_t)seg * p.n_alloc + j0 : MODE == SN_CONV ? (size_t)r * 64 + j0 : (size_t)r * (SN_RING + 64)) * p.C_out + nt * BN + CT * me + CH * cg;
         constexpr int FS = CH * 4 + 16, PS = CH * 2 + 16;       // bytes of a slab's row: fp32, a part
         // a pass of the warp over N 16-byte pieces per row: f(row, piece)
         auto pieces = [&](auto N_C, auto &&f) {
@@ -237,32 +240,33 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
         __syncwarp();
         if (mbar_wait(smem_u32(&done), 0, p.limit_ns)) {
             tc_fence_after();
-            const uint32_t xslab = ring0 + STAGES * STAGE_BYTES;                // sums of the other two taps (SPLIT): [2][128 positions][36 floats]
-            if (SPLIT)
+            const uint32_t xslab = ring0 + STAGES * STAGE_BYTES + (32 * q + lane) * XS + 4 * CH * cg;   // this lane's row of the sums of the others (NS > 1)
 #pragma unroll 1
-                for (int k = 1; k < 3; ++k) {                                   // a third to each of the others: the one of tap t has it in slot (t' - t - 1) mod 3
-                    const int to = (tap + k) % 3;
-                    float acc[16];
-                    sn_tmem_ld<16>(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * to + 16 * cg), acc);
-                    tmem_wait_ld();
-                    const uint32_t a = map_to_rank(xslab + ((2 - k) * SN_BM + 32 * q + lane) * 144 + 64 * cg, (unsigned)to), b = map_to_rank(smem_u32(&part), (unsigned)to);
+            for (int k = 1; k < NS; ++k) {                                      // their share to each of the others: theirs of CTA (me + 1 + n) mod NS is in slot n
+                const int to = (me + k) % NS;
+                const uint32_t a = map_to_rank(xslab + (NS - 1 - k) * SN_BM * XS, (unsigned)to), b = map_to_rank(smem_u32(&part), (unsigned)to);
 #pragma unroll
-                    for (int c = 0; c < 16; c += 4) st_async_v4(a + 4 * c, acc[c], acc[c + 1], acc[c + 2], acc[c + 3], b);
+                for (int c0 = 0; c0 < CH; c0 += CC) {
+                    float acc[CC];
+                    sn_tmem_ld<CC>(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(CT * to + CH * cg + c0), acc);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < CC; c += 4) st_async_v4(a + 4 * (c0 + c), acc[c], acc[c + 1], acc[c + 2], acc[c + 3], b);
                 }
-            const bool here = !SPLIT || mbar_wait(smem_u32(&part), 0, p.limit_ns);
+            }
+            const bool here = NS == 1 || mbar_wait(smem_u32(&part), 0, p.limit_ns);
             ok = here;
 #pragma unroll 1
             for (int c0 = 0; c0 < CH; c0 += CC) {
                 float acc[CC];
-                sn_tmem_ld<CC>(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(c0 + CH * cg + 32 * tap), acc);
+                sn_tmem_ld<CC>(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(CT * me + CH * cg + c0), acc);
                 tmem_wait_ld();
-                if (SPLIT && here) {
-                    // tap 0 + tap 1 + tap 2, whoever adds
-                    const uint32_t x0 = xslab + (32 * q + lane) * 144 + 64 * cg, x1 = x0 + SN_BM * 144;      // taps (tap + 1) % 3, (tap + 2) % 3
+                if (NS > 1 && here) {
+                    // in the order of the CTAs, whoever adds
 #pragma unroll
                     for (int c = 0; c < CC; c += 4) {
-                        const float4 a = sn_lds(x0 + 4 * c), b = sn_lds(x1 + 4 * c);
-                        auto sum = [&](float own, float n1, float n2) { return tap == 0 ? (own + n1) + n2 : tap == 1 ? (n2 + own) + n1 : (n1 + n2) + own; };
+                        const float4 a = sn_lds(xslab + 4 * (c0 + c)), b = NS > 2 ? sn_lds(xslab + SN_BM * XS + 4 * (c0 + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        auto sum = [&](float own, float n1, float n2) { return NS == 2 ? own + n1 : me == 0 ? (own + n1) + n2 : me == 1 ? (n2 + own) + n1 : (n1 + n2) + own; };
                         acc[c] = sum(acc[c], a.x, b.x); acc[c + 1] = sum(acc[c + 1], a.y, b.y); acc[c + 2] = sum(acc[c + 2], a.z, b.z); acc[c + 3] = sum(acc[c + 3], a.w, b.w);
                     }
                 }
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
 #pragma unroll
                     for (int c = 0; c < CC; c += 4) {
                         float4 x = sn_lds(f4 + 4 * c);
-                        const float4 b = *reinterpret_cast<const float4 *>(s_bias + 32 * tap + CH * cg + c0 + c);
+                        const float4 b = *reinterpret_cast<const float4 *>(s_bias + CT * me + CH * cg + c0 + c);
                         x.x += acc[c] + b.x; x.y += acc[c + 1] + b.y; x.z += acc[c + 2] + b.z; x.w += acc[c + 3] + b.w;
                         sn_sts(f4 + 4 * c, x);
                     }
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
                 }
 #pragma unroll
                 for (int c = 0; c < CC; c += 4) {
-                    const float4 b = *reinterpret_cast<const float4 *>(s_bias + 32 * tap + CH * cg + c0 + c);
+                    const float4 b = *reinterpret_cast<const float4 *>(s_bias + CT * me + CH * cg + c0 + c);
                     float4 x = {0.f, 0.f, 0.f, 0.f};
                     if (MODE == SN_RES) {
                         x = sn_lds(f4 + 4 * c);
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(SN_THREADS, 1) subnet_gemm_kernel(const __grid
         } else ok = false;
     }
     if (!ok && atomicCAS(&p.status->code, DEV_OK, DEV_TIMEOUT) == DEV_OK) { p.status->cta = blockIdx.x; p.status->step = blockIdx.y; p.status->phase = 20 + MODE; }
-    if (SPLIT) cluster_sync_all();                              // nobody leaves while a peer may still send to it
+    if (NS > 1) cluster_sync_all();                              // nobody leaves while a peer may still send to it
     else __syncthreads();
     if (warp == 1) {
         tc_fence_after();
@@ -460,7 +464,7 @@ static void pdl_launch(K kernel, dim3 grid, int smem, cudaStream_t s, const CUte
 // stages, and a slab of fp32 values for the epilogue of all but the convolution
 template <int BN, int ST> constexpr int sn_smem(bool slab) { return ST * (2 * SN_BM * TC_BK * 2 + BN * TC_BK * 2) + 1024 + (slab ? 2 * SN_BM * (BN * 2 + 16) : 0); }
 constexpr int SN_SMEM_CONV = sn_smem<SN_BN_CONV, SN_ST_CONV>(false), SN_SMEM_RES = sn_smem<SN_BN_RES, SN_ST_RES>(true), SN_SMEM_OUT = sn_smem<SN_BN_OUT, SN_ST_OUT>(true);
-constexpr int SN_SMEM_SPLIT = SN_SMEM_CONV + 2 * SN_BM * 144;
+constexpr int sn_smem_split(int ns) { return SN_SMEM_CONV + (ns - 1) * SN_BM * (SN_BN_CONV / ns * 4 + 16); }
 
 // The whole network for the segments of one call: v[seg][n_steps][cond_dim] (the conditioning vectors the stepping call
 // of these rows consumes).  Segment b is row r_lo + b from position p_lo - b * lag on.
@@ -547,7 +551,7 @@ bool subnet_ring_fits(const wrnn_subscale_net *n, int lag)
 // The next 64 positions: rows r_lo .. r_lo + n_rows - 1, row r from position t0 - r * lag on (t0 a multiple of 64; a row starts at
 // -64 ceil(reach / 64)).  v[B][64][cond_dim]; what belongs to positions below 0 or at and beyond L is not written.
 int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows, long long t0, int lag,
-                    float *v, unsigned long long limit_ns, cudaStream_t s)
+                    float *v, int free_sms, unsigned long long limit_ns, cudaStream_t s)
 {
     const size_t fl = (size_t)n->B * SN_RING * n->res_ch, pl = (size_t)n->B * (SN_RING + 64) * n->res_ch;       // a layer of the rings
     subnet_input_kernel<true><<<dim3(64 / SN_IN_POS, n_rows), 256, 0, s>>>(hist, n->W_in, n->b_in, n->B, L, n->res_ch, r_lo, t0 + n->reach, lag, 0, 64, n->rf, n->rh, n->rl);
@@ -564,10 +568,16 @@ int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *fram
         p.n_kb_tap = n->res_ch / TC_BK; p.taps = n->taps; p.dil = d; p.w_row0 = l * n->taps * n->conv_ch; p.w_tap_rows = n->conv_ch;
         p.a_idx0 = l * n->B + r_lo; p.a_slot0 = (int)((t0 + reach) & (SN_RING - 1));
         p.C_out = n->conv_ch; p.bias = n->b_conv + (size_t)l * n->conv_ch; p.oh = n->bh; p.ol = n->bl; p.relu_parts = 0;
-        if (n->taps == 3)
-            pdl_launch(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, true>, dim3(3 * (n->conv_ch / SN_BN_CONV), tiles, 1), SN_SMEM_SPLIT, s, n->tmRh, n->tmRl, n->tmWc, p, 3);
-        else
-            pdl_launch(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true>, dim3(n->conv_ch / SN_BN_CONV, tiles, 1), SN_SMEM_CONV, s, n->tmRh, n->tmRl, n->tmWc, p);
+        // as many CTAs per tile as find an SM beside the stepping call (and share the k-blocks evenly)
+        const int n_tiles = n->conv_ch / SN_BN_CONV, kbs = n->taps * p.n_kb_tap;
+        const int ns = 3 * n_tiles * tiles <= free_sms && kbs % 3 == 0 ? 3 : 2 * n_tiles * tiles <= free_sms && kbs % 2 == 0 ? 2 : 1;
+        auto conv = [&](auto NS_C) {
+            constexpr int NS = decltype(NS_C)::value;
+            pdl_launch(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, NS>, dim3(NS * n_tiles, tiles, 1), sn_smem_split(NS), s, n->tmRh, n->tmRl, n->tmWc, p, NS);
+        };
+        if (ns == 3) conv(std::integral_constant<int, 3>{});
+        else if (ns == 2) conv(std::integral_constant<int, 2>{});
+        else conv(std::integral_constant<int, 1>{});
         p.n_kb_tap = n->conv_ch / TC_BK; p.taps = 1; p.dil = 0; p.w_row0 = l * n->res_ch; p.w_tap_rows = 0;
         p.a_idx0 = r_lo; p.a_slot0 = 0; p.relu_parts = l == n->n_layers - 1;
         p.C_out = n->res_ch; p.bias = n->b_res + (size_t)l * n->res_ch; p.oh = n->rh + (l + 1) * pl; p.ol = n->rl + (l + 1) * pl;
@@ -636,7 +646,7 @@ extern "C" int wrnn_subscale_net_create(const wrnn_subscale_net_params *q, wrnn_
     auto allow = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess; };
     constexpr int sc = SN_SMEM_CONV, sr = SN_SMEM_RES, so = SN_SMEM_OUT;
     ok = ok && allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, false>, sc) && allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true>, sc) &&
-         allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, true>, SN_SMEM_SPLIT) &&
+         allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, 2>, sn_smem_split(2)) && allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, 3>, sn_smem_split(3)) &&
          allow(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, false>, sr) && allow(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, true>, sr) &&
          allow(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, false>, so) && allow(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, true>, so);
     if (!ok) { cudaGetLastError(); wrnn_subscale_net_destroy(n); return WRNN_ERR_NOMEM; }
