@@ -128,8 +128,8 @@ static bool use_resident(const wrnn_model *m, int batch)
 }
 
 // Rows of a dense H = 896 model: the kernels that hold the whole model in one cluster, up to four rows per cluster (seven clusters at a
-// time) in the one, five to fourteen in the other, more of either in waves of clusters.  us per step of the two at 28 rows: 4.38 / 4.59, at 8:
-// 3.72 / 4.52; of the second and the cluster-partitioned kernel: 29 rows 4.65 / 25, 56: 4.8 / 25.2, 98: 6.9 / 25.8, 168: 13.7 / 28.8, 224: 19.3 /
+// time) in the one, five to fourteen in the other, more of either in waves of clusters.  us per step of the two at 28 rows: 4.30 / 4.59, at 8:
+// 3.69 / 4.52; of the second and the cluster-partitioned kernel: 29 rows 4.65 / 25, 56: 4.8 / 25.2, 98: 6.9 / 25.8, 168: 13.7 / 28.8, 224: 19.3 /
 // 31.1, 256: 20.4 / 32.2, 336: 27.6 / 34.
 constexpr int RESCL_BF16_ROWS = 28;
 // (beyond, the grid-phased kernel)

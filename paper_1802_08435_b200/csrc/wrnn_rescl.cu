@@ -7,7 +7,7 @@
 // step.  A bf16 model is 6.1 MB; the shared memory of a 16-CTA cluster is 3.6 MB, but its tensor memory is another 4.2 MB.  With
 // the model inside one cluster every exchange is an all-gather through distributed shared memory (measured here: 420 cycles +
 // 0.87 per byte and receiver, against 1,000 - 1,500 cycles for the same through L2 and across the chip), clusters never meet, and
-// seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.33, 8 rows 3.69, 28 rows 4.38
+// seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.27, 8 rows 3.69, 28 rows 4.30
 // (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 28; more rows of a bf16 model: wrnn_resrows.cu); fp32 5.1 to 6.9, with where the streamed weights lie, up to 7
 // rows and 6.2 to 7.1 up to 14 (7.4 at one row, 55 and more at several); fused 3.5 (4.54).
 //
@@ -88,7 +88,7 @@ struct ResClPack {
     ClScales sc;
 };
 
-// ROWS: most rows of a cluster: 1 or 4; fp32 weights 1 or 2.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate; MODE 2:
+// ROWS: rows of a cluster: 1, 3 (two: sent as they are) or 4 (three or four); fp32 weights 1 or 2.  MODE 0: plain sampling; MODE 1: forced symbols, dumps, phase stamps and the self-test predicate; MODE 2:
 // these and the checks.
 // Warps 0..7 are the chain: hidden layer, logits, then (one row of the batch each) draw and gates, and all sends.  Warps 8..15
 // multiply the rows of R in the background, while the chain waits for exchanges.
@@ -487,29 +487,40 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         const float hn = fmaf(u, half_g ? hF : hC, (1.0f - u) * e);
         if (half_g) hF = hn; else hC = hn;
         if (gater) {
-            __half *d = reinterpret_cast<__half *>(ystage + (st_d * 7 + (lane >> 2)) * 16) + (lane & 3);
+            __half *d = reinterpret_cast<__half *>(ystage + ((lane >> 2) * IR + (ONE ? 0 : st_d)) * 16) + (lane & 3);
             const float x = hn * CL_STATE;
             const __half hi = __float2half_rn(x);
             d[0] = hi;
             d[4] = __float2half_rn(x - __half2float(hi));
             if (DBG) { dbg_v[0] = u; dbg_v[1] = r; dbg_v[2] = e; dbg_v[3] = hn; }
         }
+        if (ROWS == 4) fence_proxy_async_cta();
     };
     // three rows of a group travel as four: 48-byte runs in the receivers' images are slower than 64-byte ones (21 rows: 4.74 us
     // per step with three, 4.52 with four)
     const int nsend = (nrc & 3) == 3 ? nrc + 1 : nrc;
-    // warps 0..7: the staged state values of this CTA's units -> images in the cluster's CTAs, two each
+    // warps 0..7: the staged state values of this CTA's units -> images in the cluster's CTAs, two each.  Three or four rows: as one copy, which keeps the load /
+    // store pipe free for the background warps (16 rows 4.24 -> 4.15, 28 rows 4.39 -> 4.31 us per step; one row 3.32 -> 3.44, two 3.70 -> 3.81: not they).
+    // (The staged values are overwritten when logits have come that depend on what every CTA made of these copies.)
+    constexpr uint32_t SLICE = 7 * 16 * IR;
+    constexpr bool BULK = ROWS == 4;
+    const uint32_t dyb = map_to_rank(sbase, (unsigned)((warp & 7) + 8 * (lane & 1))) - sbase;
     auto send_y = [&](int half_g, long long s) {
-        if (bad || (ONE ? lane >= 14 : !pc_on) || (DBG && (int)s == skip_at)) return;
-        const uint32_t a = sbase + (uint32_t)(X0 + half_g * XSTR) + pc_off, bar = smem_u32(&xy[half_g]);
-        if ((ONE || pc_a < nsend) && store_ok(pc_off, 16, CS_IMG)) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(ystage + ((ONE ? 0 : pc_a) * 7 + pc_quad) * 16);
+        if constexpr (BULK) {
+            if (bad || lane >= 2 || (DBG && (int)s == skip_at) || !store_ok(rank * SLICE, SLICE, CS_IMG)) return;
+            cl_copy_bulk(sbase + (uint32_t)(X0 + half_g * XSTR) + rank * SLICE + dyb, smem_u32(ystage), SLICE, smem_u32(&xy[half_g]) + dyb);
+        } else {
+            if (bad || (ONE ? lane >= 14 : !pc_on) || (DBG && (int)s == skip_at)) return;
+            const uint32_t a = sbase + (uint32_t)(X0 + half_g * XSTR) + pc_off, bar = smem_u32(&xy[half_g]);
+            if ((ONE || pc_a < nsend) && store_ok(pc_off, 16, CS_IMG)) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(ystage + (pc_quad * IR + (ONE ? 0 : pc_a)) * 16);
 #pragma unroll
-            for (int k = 0; k < (ONE ? 1 : 2); ++k) cl_st_async16(a + dy[k], v, bar + dy[k]);
+                for (int k = 0; k < (ONE ? 1 : 2); ++k) cl_st_async16(a + dy[k], v, bar + dy[k]);
+            }
         }
     };
     const int n_draw = 32 * nrc;                                         // threads of the drawing warps
-    const unsigned ybytes = (unsigned)(nsend * CK * 4), lbytes = FUSED ? 256u : (unsigned)(nrc * 1024);
+    const unsigned qbytes = (unsigned)(nsend * CK * 4), ybytes = BULK ? CCS * SLICE : qbytes, lbytes = FUSED ? 256u : (unsigned)(nrc * 1024);
 
     // ---- warp 7 prepares, one row per lane, what the draws of a half-step need: the uniform and the conditioning frame (the
     // same for both halves of a step), tracked without a division per step
@@ -583,7 +594,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         const unsigned yuse = (n - 1) >> 1, quse = n - 1;
         const uint32_t xin = sbase + (uint32_t)(X0 + in * XSTR), qin = sbase + (uint32_t)Q0;
         if (tid == 0 && !bad) {
-            mbar_arrive_expect(smem_u32(&xq), ybytes);
+            mbar_arrive_expect(smem_u32(&xq), qbytes);
             mbar_arrive_expect(smem_u32(&xl), lbytes);
             if (!last) mbar_arrive_expect(smem_u32(&xy[half]), ybytes);
         }
@@ -841,7 +852,7 @@ static const void *cl_kernel_of(int nr, int mode, int kind)
 #define CL_K(R, K) (mode == 2 ? (const void *)resident_cluster_kernel<R, 2, K> : mode ? (const void *)resident_cluster_kernel<R, 1, K> : (const void *)resident_cluster_kernel<R, 0, K>)
     if (kind == CL_FUSED) return CL_K(1, CL_FUSED);
     if (kind == CL_F32) return nr == 1 ? CL_K(1, CL_F32) : CL_K(2, CL_F32);
-    return nr == 1 ? CL_K(1, CL_BF16) : CL_K(4, CL_BF16);
+    return nr == 1 ? CL_K(1, CL_BF16) : nr == 2 ? CL_K(3, CL_BF16) : CL_K(4, CL_BF16);
 #undef CL_K
 }
 
@@ -863,7 +874,7 @@ int rescl_prepare(wrnn_model *m)
     ResClPack k;
     { const char *d = getenv("WRNN_DEBUG"); k.checked = d && d[0] == '1'; }
     k.kind = m->variant == 1 ? CL_FUSED : m->dtype == WRNN_F32 ? CL_F32 : CL_BF16;
-    for (int nr : {1, 2})
+    for (int nr : {1, 2, 4})
         for (int mode = 0; mode < (k.checked ? 3 : 2); ++mode) {
             const void *f = cl_kernel_of(nr, mode, k.kind);
             if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess || !allow_smem(f, m->device, mode == 2 ? cl_checked_smem(k.kind) : cl_launch_smem(k.kind))) {
