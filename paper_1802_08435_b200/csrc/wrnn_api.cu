@@ -240,7 +240,7 @@ static int run_steps(wrnn_model *m, StepArgs &a, cudaStream_t s)
     int rc = WRNN_OK;
     if (!a.g) {
         if (!ensure_g(m, (size_t)a.batch * nf * 3 * m->H)) return fail(m, WRNN_ERR_NOMEM, "conditioning scratch allocation failed");
-        rc = cond_project(m, a.cond, a.batch, nf, m->g, s);
+        rc = cond_project(m, a.cond, a.batch, nf, m->g, m->status, s);
         if (rc != WRNN_OK) return fail(m, rc, "conditioning projection launch failed");
     }
     if (use_resrows(m, a.batch)) return resrows_run(m, a, s);
@@ -734,7 +734,7 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
         const int r_lo = n_lo, r_hi = (int)std::min<long long>(B - 1, t / lag), rows = r_hi - r_lo + 1;
         if (rows < 1) continue;
         float *g = m->g + (k & 1) * gn;
-        rc = cond_project(m, v + (size_t)r_lo * N * D, rows, N, g, sn);
+        rc = cond_project(m, v + (size_t)r_lo * N * D, rows, N, g, nullptr, sn);
         if (rc == WRNN_OK && !follow(st, (int)(k & 1), sn, net)) rc = WRNN_ERR_CUDA;
         // the oldest row may end inside the block: all rows up to there, then the others
         const long long left = L - (t - (long long)r_lo * lag);

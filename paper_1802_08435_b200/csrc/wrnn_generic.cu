@@ -263,12 +263,20 @@ __global__ void __launch_bounds__(512, 1) generic_step_kernel(const GenericParam
 // pairs -- a chunk of 128 steps of 16 rows -- at 107 us).  The sum over D runs in the same order whatever NP.
 // Few pairs: NP per block, four rows of the gates per thread (their weights of an input are one load), the weights of the next eight inputs
 // on their way while these are multiplied: bound by the latency of the loads.
+// What every projection does besides: clear the status word of the stepping call that follows it (one launch less), and let that call's clusters start
+// (they bring their weights on chip and wait for this grid before they read what it writes): 120 steps of one row 411 -> 407 us per call.
+__device__ __forceinline__ void cond_begin(DevStatus *status)
+{
+    if (status && (blockIdx.x | blockIdx.y | threadIdx.x) == 0) *status = DevStatus{DEV_OK, 0, 0, 0};
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 constexpr int COND_THREADS = 128;
 template <int NP>
 __global__ void __launch_bounds__(COND_THREADS) cond_project_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT,
                                                                     const float *__restrict__ b_gate, float *__restrict__ g, int G, int D,
-                                                                    long long n_pairs)
+                                                                    long long n_pairs, DevStatus *status)
 {
+    cond_begin(status);
     // blockIdx.y strides over the (row of the batch, frame) pairs, so no grid dimension limits their number
     extern __shared__ __align__(16) float fr[];              // [D][NP]
     const int row = 4 * (blockIdx.x * COND_THREADS + threadIdx.x);           // (G = 3 H, H a multiple of eight)
@@ -323,11 +331,12 @@ __global__ void __launch_bounds__(COND_THREADS) cond_project_kernel(const float 
 
 // Many pairs: a tile of 64 pairs x 128 rows per block, weights and frames of 32 inputs at a time in shared memory, eight pairs x four rows per thread --
 // three 16-byte loads for 32 products (a value of a frame is the same for a whole warp).  With every weight read from L2 by every block of 16
-// pairs, 1,024 pairs took 31 us at H = 896; @@FIG@@ now.
+// pairs, 1,024 pairs took 31 us at H = 896; 17.7 now.
 constexpr int COND_TP = 64, COND_TR = 128, COND_TD = 32;
 __global__ void __launch_bounds__(256) cond_project_tile_kernel(const float *__restrict__ cond, const float *__restrict__ W_condT, const float *__restrict__ b_gate,
-                                                                float *__restrict__ g, int G, int D, long long n_pairs)
+                                                                float *__restrict__ g, int G, int D, long long n_pairs, DevStatus *status)
 {
+    cond_begin(status);
     __shared__ __align__(16) float sw[COND_TD][COND_TR], sx[COND_TD][COND_TP + 4];
     const int tid = threadIdx.x, lane = tid & 31, pg = tid >> 5;                 // rows row0 + 4 lane .., pairs k0 + 8 pg ..
     const int row0 = blockIdx.x * COND_TR, row = row0 + 4 * lane;
@@ -382,32 +391,33 @@ __global__ void __launch_bounds__(256) cond_project_tile_kernel(const float *__r
 
 // Tiles from 256 pairs on (84 blocks at H = 896 and more); below, as many pairs per block as leave the chip two blocks per SM, one in short calls.
 // The sums are the same in all of them.
-static void cond_project_launch(const float *cond, const float *W_condT, const float *b_gate, float *g, int G, int D, long long n_pairs, cudaStream_t s)
+static void cond_project_launch(const float *cond, const float *W_condT, const float *b_gate, float *g, int G, int D, long long n_pairs, DevStatus *status, cudaStream_t s)
 {
     auto few = [&](auto NP_C) {
         constexpr int NP = decltype(NP_C)::value;
         const dim3 grid((G + 4 * COND_THREADS - 1) / (4 * COND_THREADS), (unsigned)std::min<long long>((n_pairs + NP - 1) / NP, 65535));
-        cond_project_kernel<NP><<<grid, COND_THREADS, (size_t)NP * D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+        cond_project_kernel<NP><<<grid, COND_THREADS, (size_t)NP * D * sizeof(float), s>>>(cond, W_condT, b_gate, g, G, D, n_pairs, status);
     };
     if (n_pairs >= 256)
-        cond_project_tile_kernel<<<dim3((G + COND_TR - 1) / COND_TR, (unsigned)std::min<long long>((n_pairs + COND_TP - 1) / COND_TP, 65535)), 256, 0, s>>>(cond, W_condT, b_gate, g, G, D, n_pairs);
+        cond_project_tile_kernel<<<dim3((G + COND_TR - 1) / COND_TR, (unsigned)std::min<long long>((n_pairs + COND_TP - 1) / COND_TP, 65535)), 256, 0, s>>>(cond, W_condT, b_gate, g, G, D, n_pairs, status);
     else if (n_pairs >= 100 && (size_t)4 * D * sizeof(float) <= 48 * 1024) few(std::integral_constant<int, 4>{});
     else few(std::integral_constant<int, 1>{});
 }
 
-__global__ void cond_bias_only_kernel(const float *__restrict__ b_gate, float *__restrict__ g, int G, int batch)
+__global__ void cond_bias_only_kernel(const float *__restrict__ b_gate, float *__restrict__ g, int G, int batch, DevStatus *status)
 {
+    cond_begin(status);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < G * batch) g[i] = b_gate ? b_gate[i % G] : 0.f;
 }
 
-int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, float *g, cudaStream_t s)
+int cond_project(wrnn_model *m, const float *cond, int batch, int n_frames, float *g, DevStatus *status, cudaStream_t s)
 {
     const int G = 3 * m->H;
     if (m->cond_dim == 0) {
-        cond_bias_only_kernel<<<(G * batch + 255) / 256, 256, 0, s>>>(m->b_gate, g, G, batch);
+        cond_bias_only_kernel<<<(G * batch + 255) / 256, 256, 0, s>>>(m->b_gate, g, G, batch, status);
     } else {
-        cond_project_launch(cond, m->W_condT, m->b_gate, g, G, m->cond_dim, (long long)batch * n_frames, s);
+        cond_project_launch(cond, m->W_condT, m->b_gate, g, G, m->cond_dim, (long long)batch * n_frames, status, s);
     }
     ++g_launches;
     return cudaGetLastError() == cudaSuccess ? WRNN_OK : WRNN_ERR_CUDA;
@@ -641,10 +651,10 @@ extern "C" int wrnn_sample_noalloc(wrnn_model *m, const wrnn_cond *cond, int64_t
 
     // conditioning projection into the fixed array
     if (m->cond_dim == 0) {
-        cond_bias_only_kernel<<<(unsigned)((G * B + 255) / 256), 256, 0, s>>>(m->b_gate, g, (int)G, batch);
+        cond_bias_only_kernel<<<(unsigned)((G * B + 255) / 256), 256, 0, s>>>(m->b_gate, g, (int)G, batch, nullptr);
     } else {
         const long long n_pairs = (long long)(B * nf);
-        cond_project_launch(a.cond, m->W_condT, m->b_gate, g, (int)G, m->cond_dim, n_pairs, s);
+        cond_project_launch(a.cond, m->W_condT, m->b_gate, g, (int)G, m->cond_dim, n_pairs, nullptr, s);
     }
     ++g_launches;
     if (cudaGetLastError() != cudaSuccess) { m->err = "conditioning projection launch failed"; return WRNN_ERR_CUDA; }

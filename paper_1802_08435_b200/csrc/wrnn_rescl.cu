@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
         wide = __syncthreads_or(wide);
         tc_fence_after();
         if (wide) {
+            cl_await_projection();
             if (tid < nrc) {
                 if (FUSED) { s_sym[0][tid] = p.a_in ? p.a_in[0] : 0x8000; s_sym[1][tid] = p.b_in ? p.b_in[0] : 0x8000; }
                 else { s_sym[0][tid] = p.c_in ? p.c_in[row0 + tid] : 128; s_sym[1][tid] = p.f_in ? p.f_in[row0 + tid] : 0; }
@@ -190,6 +191,7 @@ __global__ void __launch_bounds__(512, 1) resident_cluster_kernel(const __grid_c
             }
         }
         cl_load_tmem(s_tmem, blob + CB_SMEM, warp, lane);
+        cl_await_projection();
         // images of the initial state
         if (p.h_in)
             for (int i = tid; i < nrc * H; i += 512) {
@@ -993,12 +995,12 @@ int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     cl_fill_params(m, a, k.sc, &p);
     p.nr = nr; p.blob = k.d_blob; p.stream = k.d_stream;
     p.prof = m->prof_enabled ? k.d_prof : nullptr;
-    if (!a.g && cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     if (k.checked) { const char *poke = getenv("WRNN_DEBUG_POKE"); p.poke = poke && poke[0] == '1'; }
     const bool dbg = cl_wants_dumps(m, p);
-    cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg; cudaLaunchAttribute at[2];
     p.smem_bytes = (unsigned)(k.checked ? cl_checked_smem(k.kind) : cl_launch_smem(k.kind));
-    cl_fill_launch(n_clusters, p.smem_bytes, &cfg, at, s);
+    // (a lone cluster: several that start while blocks of the projection still run end up on other SMs, and 16 rows take 4.21 instead of 4.15 us per step)
+    cl_fill_launch(n_clusters, p.smem_bytes, &cfg, at, s, !a.g && n_clusters == 1);
     void *args[] = {&p};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, cl_kernel_of(nr, k.checked ? 2 : dbg, k.kind), args);
     if (e != cudaSuccess) {

@@ -103,6 +103,8 @@ __device__ __forceinline__ void cl_tmem_ld8(uint32_t c, uint32_t (&r)[8])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(c));
 }
+// before anything that the projection of this call writes (g, the status word) is used
+__device__ __forceinline__ void cl_await_projection() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The weights of a CTA, once per launch: 390 KB, bound by the loads in flight.  Shared memory: bulk copies (one thread), which the caller awaits
 // on `bar`; a CTA has them in flight while its warps fill tensor memory.  (One row, 120 steps: 2 us less per call than with a 16-byte piece per
 // thread and round trip, 418 -> 416 us; a fresh fp32 model's 1,200 steps 6.13 -> 6.00 ms.)
@@ -334,7 +336,8 @@ bool cl_wants_dumps(const wrnn_model *m, const ClParams &p)
     return m->dbg_skip_cta >= 0 || p.prof || p.c_forced || p.f_forced || p.c_out || p.f_out || p.a_forced || p.b_forced || p.a_out || p.b_out || p.dbg_gates ||
            p.dbg_h || p.dbg_logits;
 }
-void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s)
+// `early`: behind the projection of this call, which it may overlap (at: two attributes)
+void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at, cudaStream_t s, bool early = false)
 {
     std::memset(cfg, 0, sizeof(*cfg));
     cfg->gridDim = dim3(n_clusters * CCS);
@@ -343,8 +346,9 @@ void cl_fill_launch(int n_clusters, size_t smem, cudaLaunchConfig_t *cfg, cudaLa
     cfg->stream = s;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CCS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    if (early) { at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[1].val.programmaticStreamSerializationAllowed = 1; }
     cfg->attrs = at;
-    cfg->numAttrs = 1;
+    cfg->numAttrs = early ? 2 : 1;
 }
 }  // namespace
 

@@ -751,7 +751,6 @@ int resrows_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
     rw_geometry(k, a.batch, &p.nr, &n_clusters);
     p.blob = k.d_blob;
     p.prof = m->prof_enabled ? k.d_prof : nullptr;
-    if (!a.g && cudaMemsetAsync(m->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     if (k.checked) { const char *poke = getenv("WRNN_DEBUG_POKE"); p.poke = poke && poke[0] == '1'; }
     cudaLaunchConfig_t cfg; cudaLaunchAttribute at[1];
     p.smem_bytes = (unsigned)rw_launch_smem(p.nr, k.checked);
