@@ -380,21 +380,27 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
             q.pr += r_row(st[i], half_g * 3 * CU + CU + gu);
             q.ae = r_row(st[i], half_g * 3 * CU + 2 * CU + gu);
         };
-        auto gates_and_stage = [&](int half_g, int drawn, const GatePre &q, int i) {
+        auto gates = [&](int half_g, int drawn, const GatePre &q, int i) {
             const float *Iu = sI + (half_g * 3 * CU + gu) * 3 + 1 + half_g, *Ir = Iu + CU * 3, *Ie = Ir + CU * 3;
             const float x = scale8(drawn);
             const float u = cl_sigmoid(fmaf(*Iu, x, q.pu)), r = cl_sigmoid(fmaf(*Ir, x, q.pr));
             const float e = cl_tanh(fmaf(r, q.ae, fmaf(*Ie, x, q.pe)));
             const float hn = fmaf(u, half_g ? hF[i] : hC[i], (1.0f - u) * e);
             if (half_g) hF[i] = hn; else hC[i] = hn;
-            if (unit_on && on[i]) {
-                __half *d = reinterpret_cast<__half *>(ystage + img_off(7 * rank + (lane >> 2), row[i]) - 7 * rank * QSTR) + (lane & 3);
-                const float v = hn * CL_STATE;
-                const __half hi = __float2half_rn(v);
-                d[0] = hi;
-                d[4] = __float2half_rn(v - __half2float(hi));
-                if (DBG) { const int k = DBG ? i : 0; dbg_v[k][0] = u; dbg_v[k][1] = r; dbg_v[k][2] = e; dbg_v[k][3] = hn; }
-            }
+            if (DBG) { const int k = DBG ? i : 0; dbg_v[k][0] = u; dbg_v[k][1] = r; dbg_v[k][2] = e; dbg_v[k][3] = hn; }
+        };
+        // all rows' values are there before the first is staged, and one fence is for all of them: row by row the second one waits for the
+        // first one's stores and fence (64 rows 6.63 -> 6.52, 256 rows 20.33 -> 20.05 us per step)
+        auto stage = [&](int half_g) {
+#pragma unroll
+            for (int i = 0; i < NG; ++i)
+                if (unit_on && on[i]) {
+                    __half *d = reinterpret_cast<__half *>(ystage + img_off(7 * rank + (lane >> 2), row[i]) - 7 * rank * QSTR) + (lane & 3);
+                    const float v = (half_g ? hF[i] : hC[i]) * CL_STATE;
+                    const __half hi = __float2half_rn(v);
+                    d[0] = hi;
+                    d[4] = __float2half_rn(v - __half2float(hi));
+                }
             fence_proxy_async_cta();
         };
         // the new state values of this CTA's units -> images in four CTAs of the cluster (the staged values are overwritten when symbols have
@@ -421,8 +427,9 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
                 for (int gate = 0; gate < 3; ++gate) gv[gate] = __ldg(g + gate * H);
                 GatePre gp = gates_prepare(0, gv, i);
                 gates_add_r(0, gp, i);
-                gates_and_stage(0, f_prev[i], gp, i);
+                gates(0, f_prev[i], gp, i);
             }
+        stage(0);
         __syncthreads();
         cl_cluster_wait();
         send_y(0, 0);
@@ -591,8 +598,12 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
             for (int i = 0; i < NG; ++i) {
                 const int fed = (int)s_sym[half][8 * pipe + st[i]] & 255;
                 if (!half) gates_add_r(half, gp[i], i);
-                if (!last) gates_and_stage(half, fed, gp[i], i);
                 if (half) c_prev[i] = fed; else f_prev[i] = fed;
+            }
+            if (!last) {
+#pragma unroll
+                for (int i = 0; i < NG; ++i) gates(half, half ? c_prev[i] : f_prev[i], gp[i], i);
+                stage(half);
             }
             STAMP(8 * half + 7);
             if (!last) {
