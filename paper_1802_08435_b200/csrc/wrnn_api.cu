@@ -413,6 +413,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             wrnn_destroy(m);
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
+        rescl_packed(m);
         m->err.clear();
         *out = m;
         return WRNN_OK;
@@ -457,6 +458,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
     }
+    rescl_packed(m);
     m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call
     noalloc_warm(dev);
     *out = m;

@@ -71,6 +71,7 @@ struct Sparse1Pack;    // the same inside one cluster
 struct ResF32Pack;     // per-CTA fp32 weight shards of the single-stream fp32 resident kernel (opaque here)
 struct ResClPack;      // per-CTA weights of the cluster-resident kernel (opaque here)
 struct ResRowsPack;    // the same of its form for many rows
+struct ClHalf;         // fp16 matrices that both are packed from
 struct BcPack;         // per-CTA weight slices and stacked activation images of the cluster-partitioned multi-row kernel
 
 }  // namespace wrnn
@@ -110,6 +111,7 @@ struct wrnn_model {
     wrnn::ResF32Pack *resf32 = nullptr;
     wrnn::ResClPack *rescl = nullptr;
     wrnn::ResRowsPack *resrows = nullptr;
+    wrnn::ClHalf *half = nullptr;     // while the model is created
     int prof_cl = 0;                  // the last call with phase timing ran on the cluster-resident kernel (2: on its form for many rows)
     // wrnn_selftest_lost_word: bound of every device-side wait (0 = the default of two seconds) and the CTA / step whose
     // publication (or operand load) is withheld (-1 = none)
@@ -232,6 +234,7 @@ void pack_tile(const std::vector<std::vector<uint16_t>> &rows, int K, uint16_t *
 int rescl_supported(const wrnn_model *m, int batch);
 int rescl_prepare(wrnn_model *m);
 void rescl_destroy(wrnn_model *m);
+void rescl_packed(wrnn_model *m);        // gives up what only the packers of the cluster-resident kernels need
 int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
 int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int rescl_phase_cycles(const wrnn_model *m, long long *out16);

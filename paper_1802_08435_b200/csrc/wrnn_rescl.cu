@@ -894,8 +894,9 @@ int rescl_prepare(wrnn_model *m)
     // below 2^-28 of the largest one, where at most 2^-39 of that is lost; fp32 weights as two parts (2^-23 of a weight)
     const bool w2 = k.kind == CL_F32;
     const int NP = w2 ? 2 : 1, NIN = cl_nin(k.kind), LR = cl_rows(k.kind);
-    HalfMatrix R(m->hR, NP), O[4] = {{m->hO1, NP}, {m->hO3, NP}, {m->hO2, NP}, {m->hO4, NP}};
-    k.sc = ClScales(m, R, O);
+    m->half = new ClHalf(m, NP);
+    const HalfMatrix &R = m->half->R, *O = m->half->O;
+    k.sc = m->half->sc;
     const size_t smem_bytes = cl_blob_smem(k.kind), cta_bytes = smem_bytes + CB_TMEM;
     std::vector<uint8_t> stream(w2 ? CCS * CB_STREAM : 0, 0);
     std::vector<uint8_t> blob(CCS * cta_bytes, 0);
@@ -962,8 +963,15 @@ int rescl_prepare(wrnn_model *m)
     return WRNN_OK;
 }
 
+void rescl_packed(wrnn_model *m)
+{
+    delete m->half;
+    m->half = nullptr;
+}
+
 void rescl_destroy(wrnn_model *m)
 {
+    rescl_packed(m);
     if (!m->rescl) return;
     cudaFree(m->rescl->d_blob); cudaFree(m->rescl->d_stream); cudaFree(m->rescl->d_prof);
     delete m->rescl;

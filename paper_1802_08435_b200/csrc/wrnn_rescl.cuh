@@ -17,21 +17,6 @@
 
 namespace wrnn {
 
-namespace {
-constexpr int CK = 448;                  // H / 2
-constexpr int CU = 28;                   // state units of one half, hidden-layer rows per CTA
-constexpr int CL = 16;                   // logits rows per CTA
-constexpr int CCS = 16;                  // CTAs per cluster
-constexpr int CK8 = CK / 8, CQ = CK / 4; // groups of eight and of four values of a half
-constexpr int CRT = 9, CRS = 6 * CU - 16 * CRT;             // of the 168 rows of R: tiles of 16 in tensor memory, the 24 rows left in shared memory
-constexpr int CPR = 6 * CU;              // rows of R of a CTA
-constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
-constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: nine tiles of R as A fragments, four registers each
-constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
-enum { CL_BF16 = 0, CL_F32 = 1, CL_FUSED = 2 };                // kinds of model: bf16 weights, fp32 weights, the Fused Subscale WaveRNN 2x (bf16)
-__host__ __device__ constexpr int cl_nin(int kind) { return kind == CL_FUSED ? 12 : 3; }
-__host__ __device__ constexpr int cl_rows(int kind) { return kind == CL_FUSED ? 4 : CL; }       // logits rows per CTA in use
-
 // What the power-of-two scaled operands are divided by again: 2^-14 over the power of two in R, in the hidden layers and logits rows; the
 // one of the hidden-layer values ([0] coarse half)
 struct ClScales {
@@ -50,6 +35,27 @@ struct ClScales {
         }
     }
 };
+// A model's matrices as fp16 parts, for the packers of both kernels while it is created
+struct ClHalf {
+    HalfMatrix R, O[4];                      // O1, O3, O2, O4
+    ClScales sc;
+    ClHalf(const wrnn_model *m, int np) : R(m->hR, np), O{{m->hO1, np}, {m->hO3, np}, {m->hO2, np}, {m->hO4, np}}, sc(m, R, O) {}
+};
+
+namespace {
+constexpr int CK = 448;                  // H / 2
+constexpr int CU = 28;                   // state units of one half, hidden-layer rows per CTA
+constexpr int CL = 16;                   // logits rows per CTA
+constexpr int CCS = 16;                  // CTAs per cluster
+constexpr int CK8 = CK / 8, CQ = CK / 4; // groups of eight and of four values of a half
+constexpr int CRT = 9, CRS = 6 * CU - 16 * CRT;             // of the 168 rows of R: tiles of 16 in tensor memory, the 24 rows left in shared memory
+constexpr int CPR = 6 * CU;              // rows of R of a CTA
+constexpr size_t CW_R2 = 2 * CK8 * CRS * 16;                 // 24 rows of R as core matrices [k / 8][3][8][16 B]
+constexpr int CTC = 2 * 7 * CRT * 4;                         // columns of tensor memory: nine tiles of R as A fragments, four registers each
+constexpr size_t CB_TMEM = (size_t)CTC * 128 * 4;
+enum { CL_BF16 = 0, CL_F32 = 1, CL_FUSED = 2 };                // kinds of model: bf16 weights, fp32 weights, the Fused Subscale WaveRNN 2x (bf16)
+__host__ __device__ constexpr int cl_nin(int kind) { return kind == CL_FUSED ? 12 : 3; }
+__host__ __device__ constexpr int cl_rows(int kind) { return kind == CL_FUSED ? 4 : CL; }       // logits rows per CTA in use
 
 struct ClParams {
     int batch, nr;              // rows of the call, rows per cluster

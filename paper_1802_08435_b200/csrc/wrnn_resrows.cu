@@ -684,8 +684,9 @@ int resrows_prepare(wrnn_model *m)
         }
     }
     // fp16 weights, every matrix scaled by a power of two (see rescl_prepare)
-    HalfMatrix R(m->hR, 1), O[4] = {{m->hO1, 1}, {m->hO3, 1}, {m->hO2, 1}, {m->hO4, 1}};
-    k.sc = ClScales(m, R, O);
+    if (!m->half) m->half = new ClHalf(m, 1);
+    const HalfMatrix &R = m->half->R, *O = m->half->O;
+    k.sc = m->half->sc;
     const size_t cta_bytes = RB_SMEM + CB_TMEM;
     std::vector<uint8_t> blob(CCS * cta_bytes, 0);
     parallel_for(CCS, [&](int rank) {
