@@ -652,10 +652,10 @@ static const void *rw_kernel_of(int rows, int mode)
 #undef RW_K
 }
 
-// Rows per cluster and clusters of a batch: waves of clusters of up to eight rows (4.63 to 4.82 us per step, 5 to 8 rows) or of up to fourteen
-// (6.63 to 6.90 us, 9 to 14 rows), whichever all waves together take less time with, evenly filled: with seven clusters at a time 6.8 against 9.6 us
+// Rows per cluster and clusters of a batch: waves of clusters of up to eight rows (4.60 to 4.75 us per step, 5 to 8 rows) or of up to fourteen
+// (6.52 to 6.74 us, 9 to 14 rows), whichever all waves together take less time with, evenly filled: with seven clusters at a time 6.7 against 9.5 us
 // from 64 to 98 rows, 9.6 against 13.6 to 112, 13.7 against 14.3 to 168 and 19.2 to 196, 19.2 against 20.1 to 224, 20.4 against 24 to 280.  (57 to
-// 63 rows, nine per cluster, would take 6.6 instead of 9.3; they stay two waves, the launch that wrnn_launch_info has always stated at 57 rows.)
+// 63 rows, nine per cluster, would take 6.5 instead of 9.3; they stay two waves, the launch that wrnn_launch_info has always stated at 57 rows.)
 static void rw_geometry(const ResRowsPack &k, int batch, int *nr, int *n_clusters)
 {
     const int c = k.max_clusters, few = (batch + 8 * c - 1) / (8 * c), many = (batch + RM * c - 1) / (RM * c);
