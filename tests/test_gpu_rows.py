@@ -59,3 +59,21 @@ def test_rows_kernel(rows, monkeypatch):
         assert np.array_equal(_free_run(torch, B, m, cond, 30, rows, SEED, **kw), whole)
     finally:
         B.wrnn_destroy(m)
+
+
+def test_rows_kernel_staggered():
+    """Dependent rows on the staggered schedule with up to forty of them under way at once: every draw against the oracle conditioned on the device's
+    samples."""
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    from tests.test_gpu_subscale_dep import _case, _gpu_run
+    rows, L, F, chunk = 40, 360, 4, 4
+    w, V, b, frames = _case(896, rows, L, F, scale=1.0)
+    m = B.wrnn_create(w, "bf16", max_batch=rows)
+    try:
+        got = orc.fold(_gpu_run(torch, B, m, frames, V, b, F, chunk, 8, rows, L), rows)
+        want, _, mg = orc.subscale_dependent_run(orc.OracleModel(w, "bf16"), frames, V, b, rows, L, synth.HOP, SEED, forced=got, teacher=True)
+        for g, r, k in zip(pu._split(got), pu._split(want), (0, 1)):
+            assert pu.check_indices(g, r, mg[:, :, k])[1] == 0
+    finally:
+        B.wrnn_destroy(m)
