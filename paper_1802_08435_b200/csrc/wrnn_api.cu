@@ -712,7 +712,7 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
         if (!use_rescl(m, n) && !use_resrows(m, n)) return -1;
     const size_t gn = (size_t)B * N * 3 * H;
     // (where the rings find no room, the calls one by one, which need less)
-    if (subnet_ring_reserve(net) != WRNN_OK || !ensure_g(m, 2 * gn)) return -1;
+    if (subnet_ring_reserve(net, s) != WRNN_OK || !ensure_g(m, 2 * gn)) return -1;
     const cudaStream_t sn = subnet_side(net, 0), st = subnet_side(net, 1);
     const auto follow = [](cudaStream_t to, int e, cudaStream_t from, wrnn_subscale_net *q) {
         return cudaEventRecord(subnet_event(q, e), from) == cudaSuccess && cudaStreamWaitEvent(to, subnet_event(q, e), 0) == cudaSuccess;
@@ -794,7 +794,7 @@ int wrnn_sample_subscale_net(wrnn_model *m, wrnn_subscale_net *net, const float 
                                    [&](const int16_t *hist, float *v, long long L, int r_a, int n_rows, long long p_lo, int n) {
                                        return subnet_run(net, hist, frames, n_frames, hop, L, r_a, n_rows, p_lo, lag, n, v, m->wait_limit_ns(), s);
                                    },
-                                   [&](int n_rows, int n_steps) { return subnet_reserve(net, n_rows, n_steps); },
+                                   [&](int n_rows, int n_steps) { return subnet_reserve(net, n_rows, n_steps, s); },
                                    [&](long long L, float *v, float *hst, int16_t *hist, uint8_t *cp, uint8_t *fp) {
                                        // (v holds B x chunk vectors: two chunks of 64 positions and more, a chunk of 64 and more)
                                        if (chunk < 64) return -1;

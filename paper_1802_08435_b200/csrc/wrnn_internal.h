@@ -165,10 +165,10 @@ int subscale_cond_launch(const int16_t *hist, const float *frames, const float *
 // wrnn_subnet.cu: the masked dilated conditioning network on the tensor cores, for the segments of one stepping call
 int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows,
                long long p_lo, int lag, int n_steps, float *v, unsigned long long limit_ns, cudaStream_t s);
-int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps);        // activations for calls of up to that many rows and steps
+int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps, cudaStream_t s);        // activations for calls of up to that many rows and steps
 // the same in blocks of 64 positions for a whole staggered generation, on rings (see wrnn_subnet.cu)
 bool subnet_ring_fits(const wrnn_subscale_net *n, int lag);
-int subnet_ring_reserve(wrnn_subscale_net *n);
+int subnet_ring_reserve(wrnn_subscale_net *n, cudaStream_t s);
 int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows, long long t0, int lag,
                     float *v, int free_sms, unsigned long long limit_ns, cudaStream_t s);
 int subnet_clear_status(wrnn_subscale_net *n, cudaStream_t s);

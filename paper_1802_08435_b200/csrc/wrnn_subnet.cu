@@ -419,8 +419,9 @@ static void free_acts(wrnn_subscale_net *n)
 }
 
 // activation tensors for n_seg segments of n_pos positions (grown on demand; synchronises when it grows; a schedule of calls reserves
-// what its largest one takes, see subnet_reserve)
-static int ensure_acts(wrnn_subscale_net *n, int n_seg, int n_pos)
+// what its largest one takes, see subnet_reserve).  Zeroed in the order of stream s, on which the call runs: the default stream's order means
+// nothing to a stream that does not block with it.
+static int ensure_acts(wrnn_subscale_net *n, int n_seg, int n_pos, cudaStream_t s)
 {
     const int n_alloc = ((n_pos + SN_BM - 1) / SN_BM) * SN_BM + SN_BM;       // tiles are whole, taps may reach one tile further
     if (n_seg <= n->n_seg && n_alloc <= n->n_alloc) return WRNN_OK;
@@ -432,9 +433,11 @@ static int ensure_acts(wrnn_subscale_net *n, int n_seg, int n_pos)
         cudaMalloc((void **)&n->al, rows * n->conv_ch * 2) != cudaSuccess) {
         cudaGetLastError(); free_acts(n); n->err = "activation buffers of the conditioning network do not fit"; return WRNN_ERR_NOMEM;
     }
-    cudaMemset(n->xh, 0, rows * n->res_ch * 2); cudaMemset(n->xl, 0, rows * n->res_ch * 2);
-    cudaMemset(n->ah, 0, rows * n->conv_ch * 2); cudaMemset(n->al, 0, rows * n->conv_ch * 2);
-    cudaMemset(n->xf, 0, rows * n->res_ch * 4);
+    if (cudaMemsetAsync(n->xh, 0, rows * n->res_ch * 2, s) != cudaSuccess || cudaMemsetAsync(n->xl, 0, rows * n->res_ch * 2, s) != cudaSuccess ||
+        cudaMemsetAsync(n->ah, 0, rows * n->conv_ch * 2, s) != cudaSuccess || cudaMemsetAsync(n->al, 0, rows * n->conv_ch * 2, s) != cudaSuccess ||
+        cudaMemsetAsync(n->xf, 0, rows * n->res_ch * 4, s) != cudaSuccess) {
+        cudaGetLastError(); free_acts(n); n->err = "activation buffers of the conditioning network could not be cleared"; return WRNN_ERR_CUDA;
+    }
     if (!make_map(&n->tmXh, n->xh, (long long)rows, n->res_ch, SN_BM) || !make_map(&n->tmXl, n->xl, (long long)rows, n->res_ch, SN_BM) ||
         !make_map(&n->tmAh, n->ah, (long long)rows, n->conv_ch, SN_BM) || !make_map(&n->tmAl, n->al, (long long)rows, n->conv_ch, SN_BM)) {
         free_acts(n); n->err = "tensor map encoding failed"; return WRNN_ERR_CUDA;
@@ -473,7 +476,7 @@ int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, i
 {
     if (n_rows <= 0 || n_steps <= 0) return WRNN_OK;
     const int n0 = n_steps + n->reach;                       // positions of x_0 a segment needs
-    int rc = ensure_acts(n, n_rows, n0);
+    int rc = ensure_acts(n, n_rows, n0, s);
     if (rc != WRNN_OK) return rc;
     if (cudaMemsetAsync(n->status, 0, sizeof(DevStatus), s) != cudaSuccess) return WRNN_ERR_CUDA;
     subnet_input_kernel<false><<<dim3((n0 + SN_IN_POS - 1) / SN_IN_POS, n_rows), 256, 0, s>>>(hist, n->W_in, n->b_in, n->B, L, n->res_ch, r_lo, p_lo, lag, n->n_alloc, n0, n->xf, n->xh, n->xl);
@@ -517,7 +520,8 @@ static void free_rings(wrnn_subscale_net *n)
     for (cudaEvent_t &e : n->ev) { if (e) cudaEventDestroy(e); e = nullptr; }
 }
 
-int subnet_ring_reserve(wrnn_subscale_net *n)
+// (zeroed in the order of stream s, which the streams of the network and of the stepping calls follow)
+int subnet_ring_reserve(wrnn_subscale_net *n, cudaStream_t s)
 {
     if (n->rf) return WRNN_OK;
     // (a pair of rows beyond an odd last one is read, not used: one row more)
@@ -526,9 +530,9 @@ int subnet_ring_reserve(wrnn_subscale_net *n)
     cudaDeviceGetStreamPriorityRange(&least, &greatest);
     bool ok = cudaMalloc((void **)&n->rf, rows * SN_RING * n->res_ch * 4) == cudaSuccess && cudaMalloc((void **)&n->rh, part_rows * n->res_ch * 2) == cudaSuccess &&
               cudaMalloc((void **)&n->rl, part_rows * n->res_ch * 2) == cudaSuccess && cudaMalloc((void **)&n->bh, conv_rows * n->conv_ch * 2) == cudaSuccess &&
-              cudaMalloc((void **)&n->bl, conv_rows * n->conv_ch * 2) == cudaSuccess && cudaMemset(n->rf, 0, rows * SN_RING * n->res_ch * 4) == cudaSuccess &&
-              cudaMemset(n->rh, 0, part_rows * n->res_ch * 2) == cudaSuccess && cudaMemset(n->rl, 0, part_rows * n->res_ch * 2) == cudaSuccess &&
-              cudaMemset(n->bh, 0, conv_rows * n->conv_ch * 2) == cudaSuccess && cudaMemset(n->bl, 0, conv_rows * n->conv_ch * 2) == cudaSuccess;
+              cudaMalloc((void **)&n->bl, conv_rows * n->conv_ch * 2) == cudaSuccess && cudaMemsetAsync(n->rf, 0, rows * SN_RING * n->res_ch * 4, s) == cudaSuccess &&
+              cudaMemsetAsync(n->rh, 0, part_rows * n->res_ch * 2, s) == cudaSuccess && cudaMemsetAsync(n->rl, 0, part_rows * n->res_ch * 2, s) == cudaSuccess &&
+              cudaMemsetAsync(n->bh, 0, conv_rows * n->conv_ch * 2, s) == cudaSuccess && cudaMemsetAsync(n->bl, 0, conv_rows * n->conv_ch * 2, s) == cudaSuccess;
     ok = ok && make_map_rows(&n->tmRh, n->rh, (long long)(rows + n->B + 1), SN_RING + 64, n->res_ch) && make_map_rows(&n->tmRl, n->rl, (long long)(rows + n->B + 1), SN_RING + 64, n->res_ch) &&
          make_map_rows(&n->tmBh, n->bh, n->B + 1, 64, n->conv_ch) && make_map_rows(&n->tmBl, n->bl, n->B + 1, 64, n->conv_ch);
     // the stepping calls first: a cluster of theirs needs sixteen free SMs of one part of the chip, a product of the network any
@@ -594,7 +598,7 @@ int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *fram
 }
 int subnet_clear_status(wrnn_subscale_net *n, cudaStream_t s) { return cudaMemsetAsync(n->status, 0, sizeof(DevStatus), s) == cudaSuccess ? WRNN_OK : WRNN_ERR_CUDA; }
 
-int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps) { return ensure_acts(n, n_rows, n_steps + n->reach); }
+int subnet_reserve(wrnn_subscale_net *n, int n_rows, int n_steps, cudaStream_t s) { return ensure_acts(n, n_rows, n_steps + n->reach, s); }
 int subnet_reach(const wrnn_subscale_net *n) { return n->reach; }
 int subnet_B(const wrnn_subscale_net *n) { return n->B; }
 int subnet_cond_dim(const wrnn_subscale_net *n) { return n->cond_dim; }

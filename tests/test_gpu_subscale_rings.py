@@ -60,3 +60,35 @@ def test_rings(rows, L, chunk, lag, net):
     finally:
         B.wrnn_subscale_net_destroy(q)
         B.wrnn_destroy(m)
+
+
+@pytest.mark.parametrize("chunk", [64, 32])
+def test_first_call_of_a_network_on_a_stream_of_its_own(chunk):
+    """A network makes its workspaces at its first call and clears them in the order of that call's stream: what waits on the default stream,
+    with which the streams here do not block, neither holds the clearing back nor lets it fall into the call.  With rings and without."""
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    rows, L = 6, 900
+    nw = synth.make_subscale_net(rows)
+    frames = torch.from_numpy(synth.make_cond(rows, rows * L // synth.HOP + 2, synth.COND_DIM)).cuda()
+    m = B.wrnn_create(synth.make_weights(896), "bf16", max_batch=rows)
+
+    def first(stream, busy=0):
+        q, out = B.wrnn_subscale_net_create(nw), torch.zeros(rows * L, dtype=torch.int16, device="cuda:0")
+        try:
+            torch.cuda.synchronize()
+            if busy:
+                torch.cuda._sleep(busy)
+            B.wrnn_sample_subscale_net(m, q, frames, F, chunk, 256, rows * L, SEED, out, stream=stream)
+            torch.cuda.synchronize()
+            assert B.wrnn_poll_status(m) == 0 and B.wrnn_subscale_net_status(q) == 0
+            return out.cpu().numpy()
+        finally:
+            B.wrnn_subscale_net_destroy(q)
+
+    try:
+        want, side = first(None), torch.cuda.Stream()               # (the model's own workspaces are made here)
+        for busy in (0, 1_000_000, 4_000_000, 10_000_000):          # clocks: up to 5 ms, half of a call
+            assert np.array_equal(first(side, busy), want)
+    finally:
+        B.wrnn_destroy(m)
