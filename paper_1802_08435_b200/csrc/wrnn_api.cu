@@ -309,6 +309,20 @@ static void subscale_schedule(int B, long long L, int chunk, int lag, std::vecto
     }
 }
 
+// A model that is there: its uploads and cleared buffers are in the default stream's order (copies from pageable memory return when they are
+// staged), which streams that do not block with it do not follow, so that it is waited for here.
+static int created(wrnn_model *m, wrnn_model **out)
+{
+    if (cudaStreamSynchronize(0) != cudaSuccess) {
+        const std::string why = cudaGetErrorString(cudaGetLastError());
+        wrnn_destroy(m);
+        return fail(nullptr, WRNN_ERR_CUDA, "upload failed: " + why);
+    }
+    m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call
+    *out = m;
+    return WRNN_OK;
+}
+
 }  // namespace wrnn
 
 using namespace wrnn;
@@ -414,9 +428,7 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
             return fail(nullptr, rc, "resident kernel unavailable: " + why);
         }
         rescl_packed(m);
-        m->err.clear();
-        *out = m;
-        return WRNN_OK;
+        return created(m, out);
     }
     if (p->kernel == WRNN_KERNEL_AUTO || p->kernel == WRNN_KERNEL_SPARSE) {
         const int rc = sparse_prepare(m);
@@ -459,10 +471,8 @@ int wrnn_create(const wrnn_params *p, int32_t max_batch, wrnn_model **out)
         }
     }
     rescl_packed(m);
-    m->err.clear();             // reasons why optional kernels were not prepared are not errors of this call
     noalloc_warm(dev);
-    *out = m;
-    return WRNN_OK;
+    return created(m, out);
 }
 
 void wrnn_destroy(wrnn_model *m)

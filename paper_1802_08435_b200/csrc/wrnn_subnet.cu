@@ -653,6 +653,8 @@ extern "C" int wrnn_subscale_net_create(const wrnn_subscale_net_params *q, wrnn_
          allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, 2>, sn_smem_split(2)) && allow(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, true, 3>, sn_smem_split(3)) &&
          allow(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, false>, sr) && allow(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, true>, sr) &&
          allow(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, false>, so) && allow(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, true>, so);
+    // (uploads and the cleared status word are in the default stream's order, which not every caller's stream follows)
+    ok = ok && cudaStreamSynchronize(0) == cudaSuccess;
     if (!ok) { cudaGetLastError(); wrnn_subscale_net_destroy(n); return WRNN_ERR_NOMEM; }
     *out = n;
     return WRNN_OK;

@@ -409,3 +409,23 @@ def test_checked_form_of_the_default_kernels(env, monkeypatch, case, region):
         finally:
             B.wrnn_destroy(m)
     assert np.array_equal(*outs)
+
+
+@pytest.mark.parametrize("H,dtype,rows,kernel", [(896, "bf16", 1, "AUTO"), (896, "bf16", 32, "AUTO"), (896, "f32", 2, "AUTO"), (128, "bf16", 11, "BATCHED"), (128, "bf16", 11, "BCLUSTER"),
+                                                 (64, "bf16", 3, "GENERIC")])
+def test_a_new_model_is_whole_on_any_stream(env, H, dtype, rows, kernel):
+    """Creation returns when the weights and cleared buffers are there: the first call, on a stream that does not block with the default
+    stream, draws what a later one draws."""
+    torch, B = env
+    w, cond, side = synth.make_weights(H), torch.from_numpy(synth.make_cond(rows, 2)).cuda(), torch.cuda.Stream()
+    for _ in range(3):
+        outs = [torch.zeros((rows, 20), dtype=torch.int16, device="cuda:0") for _ in range(2)]
+        torch.cuda.synchronize()
+        m = B.wrnn_create(w, dtype, max_batch=rows, kernel=getattr(B, "WRNN_KERNEL_" + kernel))
+        try:
+            for out in outs:
+                B.wrnn_sample(m, cond, 20, rows, SEED, out, stream=side)
+                side.synchronize()
+            assert B.wrnn_poll_status(m) == 0 and torch.equal(*outs)
+        finally:
+            B.wrnn_destroy(m)
