@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
         };
         // ---- prologue: coarse gates of step 0 (the background warps have multiplied R by the initial state)
         const bool lead = w4 == 0 && lane == 0;
-        if (lead) mbar_arrive_expect(smem_u32(&xyp[0]), ybytes);
+        if (lead && rows) mbar_arrive_expect(smem_u32(&xyp[0]), ybytes);
         __syncthreads();
         // The products read the images of the initial state, over which the peers store their first one: nobody sends before
         // every CTA has arrived here (the loop needs nothing of the kind: whoever sends has received something from everybody)
@@ -432,7 +432,9 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
         stage(0);
         __syncthreads();
         cl_cluster_wait();
-        send_y(0, 0);
+        // a pipe without rows sends nothing: it would not wait for what it is sent, and the cluster barrier at the end does not hold a CTA back
+        // until a copy into it has landed
+        if (rows) send_y(0, 0);
         if (DBG) dump_gates(0, 0);
 
         // Half-step n = 2 s + 1 is the coarse half of step s (input y_c(s): coarse head -> c_s, then the fine gates of step s),

@@ -61,6 +61,28 @@ def test_rows_kernel(rows, monkeypatch):
         B.wrnn_destroy(m)
 
 
+# last clusters of one row, whose second pipe has none: 31 -> 5 rows per cluster (7 clusters), 131 -> 10 (14), 183 -> 14 (14)
+@pytest.mark.parametrize("rows", [31, 131, 183])
+def test_rows_kernel_pipe_without_rows(rows):
+    """A pipe without rows takes part in nothing, in calls as short as one step: these draw what one call draws."""
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    cond, n = synth.make_cond(rows, 2), 30
+    m = B.wrnn_create(synth.make_weights(896), "bf16", max_batch=rows)
+    try:
+        per = -(-rows // (B.wrnn_launch_info(m, rows)["n_ctas"] // 16))
+        assert rows % per == 1
+        whole, cond_d = _free_run(torch, B, m, cond, n, rows, SEED), torch.from_numpy(cond).cuda()
+        for _ in range(3):
+            st, out = _state(torch, rows), torch.zeros((n, rows, 1), dtype=torch.int16, device="cuda:0")
+            for i in range(n):
+                B.wrnn_sample(m, cond_d, 1, rows, SEED, out[i], step0=i, **st)
+            torch.cuda.synchronize()
+            assert B.wrnn_poll_status(m) == 0 and np.array_equal(out.cpu().numpy()[:, :, 0].T, whole)
+    finally:
+        B.wrnn_destroy(m)
+
+
 def test_rows_kernel_staggered():
     """Dependent rows on the staggered schedule with up to forty of them under way at once: every draw against the oracle conditioned on the device's
     samples."""
