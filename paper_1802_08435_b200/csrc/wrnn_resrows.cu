@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
                 im[0] = __float2half_rn(x);
                 im[4] = __float2half_rn(x - __half2float(im[0]));
             }
+        fence_proxy_async_cta();                                         // before bulk copies of the peers go over what this CTA wrote
     }
     bool bad = !mbar_wait(smem_u32(&xw), 0, p.limit_ns);                 // this thread gave up: it skips waits and sends from here on
     if (bad && atomicCAS(&p.status->code, DEV_OK, DEV_TIMEOUT) == DEV_OK) { p.status->cta = blockIdx.x; p.status->step = 0; p.status->phase = 9; }
