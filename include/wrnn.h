@@ -367,7 +367,10 @@ int wrnn_fs2_sample_host(wrnn_model *m, const float *cond_host, int32_t n_frames
  * plain fp32 row products, and 2 / 8 a second chip-wide wait (the hidden layer crosses L2 there).
  * The cluster-resident kernel (the default for a dense H = 896 model) has eight phases per half, fine half in entries 0..7
  * and coarse half in 8..15, of the first CTA's first warp: wait for the state half; hidden-layer products; hidden-layer
- * sums and send; wait for the hidden layer; logits products; logits sums and send; draw; gates.
+ * sums and send; wait for the hidden layer; logits products; logits sums and send; draw; gates.  Its form for many rows (29 to
+ * 336) has instead: wait for the state half; hidden-layer products; hidden-layer sums; wait for the recurrent products of the
+ * half-step before; logits products and their send; what of the gates does not depend on the draw; wait for the symbol (the sums of
+ * the logits and the draw, in the CTA that draws the row); gates.
  * wrnn_phase_names writes the sixteen names that belong to the last profiled call, comma-separated, into buf (HOST, cap bytes).
  * The stamps cost the stamped warp, which is on the critical path of the whole chip, some tens of cycles each, so they
  * are taken only while wrnn_phase_profile(m, 1) is in effect (default off); wrnn_phase_cycles then reports the last

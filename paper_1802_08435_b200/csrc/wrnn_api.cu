@@ -1017,7 +1017,10 @@ int wrnn_phase_names(wrnn_model *m, char *buf, int32_t cap)
     // per half: warp 0 of CTA 0 (wait, products, sums and sends), then its first drawing warp
     const char *cl = "F.wait_y,F.hid_products,F.hid_sums_send,F.wait_q,F.log_products,F.log_sums_send,F.draw,F.gates,"
                      "C.wait_y,C.hid_products,C.hid_sums_send,C.wait_q,C.log_products,C.log_sums_send,C.draw,C.gates";
-    const char *src = m->prof_cl ? cl : first;
+    // the same warp of the form for many rows, whose logits are summed where a row is drawn
+    const char *rows = "F.wait_y,F.hid_products,F.hid_sums,F.wait_background,F.log_products_send,F.gates_prepare,F.wait_symbol,F.gates,"
+                       "C.wait_y,C.hid_products,C.hid_sums,C.wait_background,C.log_products_send,C.gates_prepare,C.wait_symbol,C.gates";
+    const char *src = m->prof_cl == 2 ? rows : m->prof_cl ? cl : first;
     std::snprintf(buf, (size_t)cap, "%s", src);
     return WRNN_OK;
 }

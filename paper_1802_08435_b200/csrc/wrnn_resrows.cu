@@ -520,8 +520,9 @@ __global__ void __launch_bounds__(512, 1) rows_cluster_kernel(const __grid_const
             uint4 lv[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) lv[i] = wL[half][(8 * w4 + i) * 32 + lane];
-            cl_bar_sync(2 + BAR, 256);   // the background warps are done with the last half-step, and go on
             STAMP(8 * half + 2);
+            cl_bar_sync(2 + BAR, 256);   // the background warps are done with the last half-step, and go on
+            STAMP(8 * half + 3);
             // ---- this CTA's part of the logits: warp w has logits 64 w .. 64 w + 63 of all rows, in two pairs of tiles of which a lane holds four
             // consecutive ones (quad 8 v + 2 g, or 8 v + 2 (g - 4) + 1, of pair v)
             {

@@ -83,6 +83,26 @@ def test_rows_kernel_pipe_without_rows(rows):
         B.wrnn_destroy(m)
 
 
+@pytest.mark.parametrize("rows", [37, 98])
+def test_rows_kernel_phases(rows):
+    """The stamps of the first warp have names of their own, all of them are taken, and they neither change what is drawn nor exceed the call."""
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    cond, n = synth.make_cond(rows, 3), 240
+    m = B.wrnn_create(synth.make_weights(896), "bf16", max_batch=rows)
+    try:
+        plain = _free_run(torch, B, m, cond, n, rows, SEED)
+        B.wrnn_phase_profile(m, True)
+        assert np.array_equal(_free_run(torch, B, m, cond, n, rows, SEED), plain)
+        cycles, names = B.wrnn_phase_cycles(m), B.wrnn_phase_names(m)
+        phases = ["wait_y", "hid_products", "hid_sums", "wait_background", "log_products_send", "gates_prepare", "wait_symbol", "gates"]
+        assert names == [h + p for h in ("F.", "C.") for p in phases]
+        print("\n[phases] %d rows, cycles per step: %s" % (rows, ", ".join("%s %.0f" % (k, c / n) for k, c in zip(names, cycles))))
+        assert min(cycles) > 0 and 2000 * n < sum(cycles) < 40000 * n, cycles
+    finally:
+        B.wrnn_destroy(m)
+
+
 def test_rows_kernel_staggered():
     """Dependent rows on the staggered schedule with up to forty of them under way at once: every draw against the oracle conditioned on the device's
     samples."""
