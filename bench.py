@@ -219,6 +219,14 @@ def step_floor(ctx, wl, info, Hh, alg_bytes, us_per_step, note):
     if wl.batch == 1 and info["n_ctas"] > 16:
         return "latency_floor", latency_floor(ctx, info, Hh, alg_bytes, us_per_step, note)
     floor_us = 6 * (0.33 if wl.H == 2048 else 0.25)
+    per = -(-wl.batch // (info["n_ctas"] // 16))
+    if per > 4:
+        # five to fourteen rows per cluster, in operand images of 8, 12 or 14: what each row past the first adds to the two gathers of a state
+        # half at 16 bytes per cycle, in every wave of seven clusters
+        image, waves = (8 if per <= 8 else 12 if per <= 12 else 14), -(-info["n_ctas"] // (16 * 7))
+        floor_us = waves * (floor_us + 2 * (image - 1) * 2 * wl.H / 16 / 1965)
+        return "chain_floor", {"floor_us_per_step": floor_us, "frac_of_floor": floor_us / us_per_step,
+                               "note": "the exchanges of a 16-CTA cluster of %d rows per step, in %d wave(s) of clusters; weights stay on chip and are read beside them" % (per, waves)}
     return "chain_floor", {"floor_us_per_step": floor_us, "frac_of_floor": floor_us / us_per_step,
                            "note": "six all-gathers inside a 16-CTA cluster per step, one stream's; weights stay on chip and are read beside them"}
 
@@ -245,7 +253,7 @@ def roofline(ctx, wl, info, model, n_steps, ms_per_step, cond_bytes, out_bytes):
         roof = {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                 "frac": ach / peaks["bf16_tflops_sustained"], "traffic": traffic, "traffic_note": traffic_note,
                 "peak_source": peaks["source"] + " sustained", "algorithmic_flops_per_step": flops}
-        if info["kernel"] == 2:      # the cluster-resident kernel stamps the phases of its first CTA's first warp
+        if info["kernel"] == 2:      # a cluster-resident kernel stamps the phases of its first CTA's first warp
             pc = B.wrnn_phase_cycles(model)
             names = B.wrnn_phase_names(model)
             roof["phase_cycles_per_step"] = {k: round(v / n_steps, 1) for k, v in zip(names, pc)}

@@ -60,10 +60,11 @@ typedef enum { WRNN_F32 = 0, WRNN_BF16 = 1 } wrnn_dtype;
 typedef enum {
     WRNN_KERNEL_AUTO = 0,       /* the fastest one that supports the model and batch          */
     WRNN_KERNEL_GENERIC = 1,    /* weights streamed from L2 every step; any shape; bring-up path */
-    WRNN_KERNEL_RESIDENT = 2,   /* persistent kernel, weights resident in shared memory (one row; 2 to 16 rows of a dense bf16 H = 896 model) */
+    WRNN_KERNEL_RESIDENT = 2,   /* persistent kernel, weights resident on chip (one row; several of a dense H = 896 model: by default */
+                                /* up to 336 rows with bf16 weights and any number with fp32 ones, by name 16 and one)            */
     WRNN_KERNEL_BATCHED = 3,    /* tensor-pipe contractions over all rows (dense bf16, >= 2 rows)  */
     WRNN_KERNEL_SPARSE = 4,     /* block-sparse model resident in 16-CTA clusters (one row)        */
-    WRNN_KERNEL_BCLUSTER = 5    /* rows dealt to 16-CTA clusters (dense bf16, >= 2 rows): each with the whole model, H = 896 by default; tcgen05 contractions otherwise and by name */
+    WRNN_KERNEL_BCLUSTER = 5    /* rows dealt to 16-CTA clusters, tcgen05 contractions (dense bf16, >= 2 rows) */
 } wrnn_kernel;
 
 /*

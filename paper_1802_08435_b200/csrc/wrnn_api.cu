@@ -134,8 +134,6 @@ static bool use_resident(const wrnn_model *m, int batch)
 constexpr int RESCL_BF16_ROWS = 28;
 // (beyond, the grid-phased kernel)
 constexpr int RESROWS_MOST = 336;
-// up to here its launches are stated as those of a resident kernel, then as those of the family that deals rows to clusters
-constexpr int RESROWS_RESIDENT = 224;
 static bool use_rescl(const wrnn_model *m, int batch)
 {
     if (m->kernel != WRNN_KERNEL_AUTO && m->kernel != WRNN_KERNEL_RESIDENT) return false;
@@ -954,7 +952,7 @@ int wrnn_launch_info(wrnn_model *m, int32_t batch, int32_t *kernel, int32_t *n_c
 {
     if (!m || batch < 1 || batch > m->max_batch) return WRNN_ERR_INVALID_ARG;
     if (use_resrows(m, batch)) {
-        if (kernel) *kernel = batch <= RESROWS_RESIDENT ? WRNN_KERNEL_RESIDENT : WRNN_KERNEL_BCLUSTER;
+        if (kernel) *kernel = WRNN_KERNEL_RESIDENT;
         return resrows_launch_info(m, batch, n_ctas, n_threads, smem_bytes, weight_bytes_per_step);
     }
     if (use_rescl(m, batch)) {

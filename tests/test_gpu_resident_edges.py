@@ -353,10 +353,10 @@ def test_resident_by_name_refuses_more_rows_than_it_says(env, dtype, most):
         B.wrnn_destroy(m)
 
 
-@pytest.mark.parametrize("H,rows,kernel", [(896, 224, "RESIDENT"), (896, 225, "BCLUSTER"), (896, 336, "BCLUSTER"), (896, 340, "BATCHED"), (1024, 224, "BCLUSTER"), (1024, 230, "BATCHED")])
+@pytest.mark.parametrize("H,rows,kernel", [(896, 224, "RESIDENT"), (896, 225, "RESIDENT"), (896, 336, "RESIDENT"), (896, 340, "BATCHED"), (1024, 224, "BCLUSTER"), (1024, 230, "BATCHED")])
 def test_large_batches_run_on_the_tensor_core_kernels(env, H, rows, kernel):
-    """The lines of the dispatch for many rows of a dense bf16 model: waves of the cluster-resident kernel, the cluster-partitioned
-    kernel, and the grid-phased one where the rows do not fit the clusters.  A few rows against the oracle."""
+    """The lines of the dispatch for many rows of a dense bf16 model: waves of the cluster-resident kernel of many rows, for other H the
+    cluster-partitioned kernel, and the grid-phased one where the rows do not fit the clusters.  A few rows against the oracle."""
     torch, B = env
     w = synth.make_weights(H)
     cond = synth.make_cond(rows, 4)
@@ -366,6 +366,26 @@ def test_large_batches_run_on_the_tensor_core_kernels(env, H, rows, kernel):
         out = _free_run(torch, B, m, cond, 20, rows, SEED, row_offset_mul=1)
         chk = pu.oracle_on_gpu_stream(orc.OracleModel(w, "bf16"), cond, [0, rows // 2, rows - 1], out, SEED, row_offset_mul=1)
         assert chk["idx_bad"] == 0, chk
+    finally:
+        B.wrnn_destroy(m)
+
+
+@pytest.mark.parametrize("rows", [225, 256, 336])
+def test_cluster_partitioned_kernel_at_many_rows(env, rows):
+    """The cluster-partitioned tcgen05 kernel by name, at H = 896 and as many rows as its clusters take (several lane quadrants, ragged and full):
+    rows on both sides of the cluster boundaries, every draw and the final state against the oracle forced on the device's samples."""
+    torch, B = env
+    w, cond = synth.make_weights(896), synth.make_cond(rows, 4)
+    m = B.wrnn_create(w, "bf16", max_batch=rows, kernel=B.WRNN_KERNEL_BCLUSTER)
+    try:
+        info = B.wrnn_launch_info(m, rows)
+        assert info["kernel"] == B.WRNN_KERNEL_BCLUSTER
+        st = _state(torch, rows)
+        out = _free_run(torch, B, m, cond, 40, rows, SEED, row_offset_mul=1, **st)
+        per = -(-rows // (info["n_ctas"] // 16))
+        some = sorted({0, per - 1, per, 2 * per, rows // 2, rows - per, rows - 1})
+        chk = pu.oracle_on_gpu_stream(orc.OracleModel(w, "bf16"), cond, some, out, SEED, row_offset_mul=1, h_final=st["h"].cpu().numpy())
+        assert chk["idx_bad"] == 0 and chk["h_final_err"] < pu.TOL["bf16"], chk
     finally:
         B.wrnn_destroy(m)
 
