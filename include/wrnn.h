@@ -256,8 +256,8 @@ int wrnn_subscale_schedule(int32_t B, int64_t L, int32_t chunk, int32_t lag, int
  * call; the matrices are rounded to bf16 (nearest even), biases stay fp32:
  *     W_in [res_ch][B], b_in [res_ch]; W_conv [n_layers][taps][conv_ch][res_ch], b_conv [n_layers][conv_ch];
  *     W_res [n_layers][res_ch][conv_ch], b_res [n_layers][res_ch]; W_out [cond_dim][res_ch], b_out [cond_dim].
- * The products run on the tensor cores (tiles of 128 positions): conv_ch must be a multiple of 192, res_ch of 128,
- * B <= 64, cond_dim <= 64, every dilation <= 64; other shapes return WRNN_ERR_UNSUPPORTED.
+ * The products run on the tensor cores (tiles of 128 positions and 96 channels): conv_ch and res_ch must be multiples of 96, others
+ * return WRNN_ERR_UNSUPPORTED; B <= 64, n_layers <= 64, taps <= 8, cond_dim <= 64, every dilation <= 64, else WRNN_ERR_INVALID_ARG.
  */
 typedef struct wrnn_subscale_net wrnn_subscale_net;     /* opaque; owns its device memory */
 typedef struct {

@@ -469,6 +469,9 @@ template <int BN, int ST> constexpr int sn_smem(bool slab) { return ST * (2 * SN
 constexpr int SN_SMEM_CONV = sn_smem<SN_BN_CONV, SN_ST_CONV>(false), SN_SMEM_RES = sn_smem<SN_BN_RES, SN_ST_RES>(true), SN_SMEM_OUT = sn_smem<SN_BN_OUT, SN_ST_OUT>(true);
 constexpr int sn_smem_split(int ns) { return SN_SMEM_CONV + (ns - 1) * SN_BM * (SN_BN_CONV / ns * 4 + 16); }
 
+// k-blocks of a product over so many channels: beyond the last channel both operands' boxes are filled with zeros
+static int sn_kbs(int channels) { return (channels + TC_BK - 1) / TC_BK; }
+
 // The whole network for the segments of one call: v[seg][n_steps][cond_dim] (the conditioning vectors the stepping call
 // of these rows consumes).  Segment b is row r_lo + b from position p_lo - b * lag on.
 int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, int n_frames, int hop, long long L, int r_lo, int n_rows,
@@ -490,19 +493,19 @@ int subnet_run(wrnn_subscale_net *n, const int16_t *hist, const float *frames, i
         need -= (n->taps - 1) * d;                           // positions of a_l and x_{l+1}
         const int mtiles = (need + SN_BM - 1) / SN_BM;
         // a_l = relu(conv): K = taps x res_ch, N = conv_ch
-        p.n_kb_tap = n->res_ch / TC_BK; p.taps = n->taps; p.dil = d; p.w_row0 = l * n->taps * n->conv_ch; p.w_tap_rows = n->conv_ch;
+        p.n_kb_tap = sn_kbs(n->res_ch); p.taps = n->taps; p.dil = d; p.w_row0 = l * n->taps * n->conv_ch; p.w_tap_rows = n->conv_ch;
         p.n_pos = need; p.C_out = n->conv_ch; p.bias = n->b_conv + (size_t)l * n->conv_ch; p.oh = n->ah; p.ol = n->al; p.xf = nullptr; p.relu_parts = 0;
         pdl_launch(subnet_gemm_kernel<SN_BN_CONV, SN_CONV, SN_ST_CONV, false>, dim3(n->conv_ch / SN_BN_CONV, mtiles, n_rows), SN_SMEM_CONV, s,
                    n->tmXh, n->tmXl, n->tmWc, p);
         // x_{l+1} = x_l + W_res a_l + b_res: K = conv_ch, N = res_ch
-        p.n_kb_tap = n->conv_ch / TC_BK; p.taps = 1; p.dil = 0; p.w_row0 = l * n->res_ch; p.w_tap_rows = 0;
+        p.n_kb_tap = sn_kbs(n->conv_ch); p.taps = 1; p.dil = 0; p.w_row0 = l * n->res_ch; p.w_tap_rows = 0;
         p.C_out = n->res_ch; p.bias = n->b_res + (size_t)l * n->res_ch; p.oh = n->xh; p.ol = n->xl; p.xf = p.xf_out = n->xf; p.relu_parts = l == n->n_layers - 1;
         pdl_launch(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, false>, dim3(n->res_ch / SN_BN_RES, mtiles, n_rows), SN_SMEM_RES, s,
                    n->tmAh, n->tmAl, n->tmWr, p);
         g_launches += 2;
     }
     // v = frames + W_out relu(x_last) + b_out
-    p.n_kb_tap = n->res_ch / TC_BK; p.taps = 1; p.dil = 0; p.w_row0 = 0; p.w_tap_rows = 0; p.n_pos = n_steps; p.C_out = 0; p.bias = nullptr;
+    p.n_kb_tap = sn_kbs(n->res_ch); p.taps = 1; p.dil = 0; p.w_row0 = 0; p.w_tap_rows = 0; p.n_pos = n_steps; p.C_out = 0; p.bias = nullptr;
     p.v = v; p.n_steps = n_steps; p.cond_dim = n->cond_dim; p.frames = frames; p.n_frames = n_frames; p.hop = hop; p.Bsub = n->B; p.b_out = n->b_out;
     pdl_launch(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, false>, dim3(1, (n_steps + SN_BM - 1) / SN_BM, n_rows), SN_SMEM_OUT, s,
                n->tmXh, n->tmXl, n->tmWo, p);
@@ -569,7 +572,7 @@ int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *fram
         const int d = n->dilation[l];
         reach -= (n->taps - 1) * d;
         p.reach = reach;
-        p.n_kb_tap = n->res_ch / TC_BK; p.taps = n->taps; p.dil = d; p.w_row0 = l * n->taps * n->conv_ch; p.w_tap_rows = n->conv_ch;
+        p.n_kb_tap = sn_kbs(n->res_ch); p.taps = n->taps; p.dil = d; p.w_row0 = l * n->taps * n->conv_ch; p.w_tap_rows = n->conv_ch;
         p.a_idx0 = l * n->B + r_lo; p.a_slot0 = (int)((t0 + reach) & (SN_RING - 1));
         p.C_out = n->conv_ch; p.bias = n->b_conv + (size_t)l * n->conv_ch; p.oh = n->bh; p.ol = n->bl; p.relu_parts = 0;
         // as many CTAs per tile as find an SM beside the stepping call (and share the k-blocks evenly)
@@ -582,13 +585,13 @@ int subnet_ring_run(wrnn_subscale_net *n, const int16_t *hist, const float *fram
         if (ns == 3) conv(std::integral_constant<int, 3>{});
         else if (ns == 2) conv(std::integral_constant<int, 2>{});
         else conv(std::integral_constant<int, 1>{});
-        p.n_kb_tap = n->conv_ch / TC_BK; p.taps = 1; p.dil = 0; p.w_row0 = l * n->res_ch; p.w_tap_rows = 0;
+        p.n_kb_tap = sn_kbs(n->conv_ch); p.taps = 1; p.dil = 0; p.w_row0 = l * n->res_ch; p.w_tap_rows = 0;
         p.a_idx0 = r_lo; p.a_slot0 = 0; p.relu_parts = l == n->n_layers - 1;
         p.C_out = n->res_ch; p.bias = n->b_res + (size_t)l * n->res_ch; p.oh = n->rh + (l + 1) * pl; p.ol = n->rl + (l + 1) * pl;
         p.xf = n->rf + l * fl; p.xf_out = p.relu_parts ? nullptr : n->rf + (l + 1) * fl;
         pdl_launch(subnet_gemm_kernel<SN_BN_RES, SN_RES, SN_ST_RES, true>, dim3(n->res_ch / SN_BN_RES, tiles, 1), SN_SMEM_RES, s, n->tmBh, n->tmBl, n->tmWr, p);
     }
-    p.n_kb_tap = n->res_ch / TC_BK; p.taps = 1; p.dil = 0; p.w_row0 = 0; p.w_tap_rows = 0; p.C_out = 0; p.bias = nullptr;
+    p.n_kb_tap = sn_kbs(n->res_ch); p.taps = 1; p.dil = 0; p.w_row0 = 0; p.w_tap_rows = 0; p.C_out = 0; p.bias = nullptr;
     p.a_idx0 = n->n_layers * n->B + r_lo; p.a_slot0 = (int)(t0 & (SN_RING - 1)); p.reach = 0;
     p.v = v; p.n_steps = 64; p.cond_dim = n->cond_dim; p.frames = frames; p.n_frames = n_frames; p.hop = hop; p.Bsub = n->B; p.b_out = n->b_out;
     pdl_launch(subnet_gemm_kernel<SN_BN_OUT, SN_OUT, SN_ST_OUT, true>, dim3(1, tiles, 1), SN_SMEM_OUT, s, n->tmRh, n->tmRl, n->tmWo, p);
@@ -620,7 +623,7 @@ extern "C" int wrnn_subscale_net_create(const wrnn_subscale_net_params *q, wrnn_
         return WRNN_ERR_INVALID_ARG;
     if (q->B < 1 || q->B > 64 || q->n_layers < 1 || q->n_layers > 64 || q->taps < 1 || q->taps > 8 || q->cond_dim < 1 || q->cond_dim > 64)
         return WRNN_ERR_INVALID_ARG;
-    // the tensor-core tiling: whole 64-wide k-blocks and whole channel tiles
+    // the tensor-core tiling: whole channel tiles
     if (q->conv_ch < SN_BN_CONV || q->conv_ch % SN_BN_CONV || q->res_ch < SN_BN_RES || q->res_ch % SN_BN_RES) return WRNN_ERR_UNSUPPORTED;
     int dev = 0;
     cudaDeviceProp prop;

@@ -52,6 +52,40 @@ def test_conditioning_vectors_against_the_oracle(env, B_rows, L, dil):
         Bn.wrnn_subscale_net_destroy(net)
 
 
+# channel counts that are no whole number of 64-wide k-blocks, among whole ones
+@pytest.mark.parametrize("conv_ch,res_ch", [(96, 288), (288, 96), (96, 96), (192, 480)])
+def test_channels_beyond_whole_k_blocks(env, conv_ch, res_ch):
+    """Every channel takes part in the products, whatever is left over beyond the last whole k-block: the conditioning vectors, and the draws of a
+    generation on rings, against the oracle."""
+    torch, Bn = env
+    B_rows, L = 5, 150
+    nw = synth.make_subscale_net(B_rows, conv_ch=conv_ch, res_ch=res_ch, dilations=(1, 5, 11))
+    rng = np.random.default_rng(7)
+    hist = rng.integers(-32768, 32767, size=(B_rows, L)).astype(np.int16)
+    frames = synth.make_cond(B_rows, (B_rows * L) // synth.HOP + 2, synth.COND_DIM)
+    net, w = Bn.wrnn_subscale_net_create(nw), synth.make_weights(896)
+    m = Bn.wrnn_create(w, "bf16", max_batch=B_rows)
+    try:
+        h_d, f_d = torch.from_numpy(hist).cuda(), torch.from_numpy(frames).cuda()
+        for row in range(B_rows):
+            v = torch.zeros((L, synth.COND_DIM), dtype=torch.float32, device="cuda:0")
+            Bn.wrnn_subscale_net_conditioning(net, h_d, f_d, row, v)
+            torch.cuda.synchronize()
+            ref = frames[row][(B_rows * np.arange(L) + row) // synth.HOP] + sn.SubscaleNet(nw).conditioning(hist, row)
+            assert pu.rel_err(v.cpu().numpy(), ref) < 1e-4
+        out = torch.zeros(B_rows * L, dtype=torch.int16, device="cuda:0")
+        Bn.wrnn_sample_subscale_net(m, net, f_d, 128, 64, 256, B_rows * L, SEED, out)
+        torch.cuda.synchronize()
+        assert Bn.wrnn_poll_status(m) == 0 and Bn.wrnn_subscale_net_status(net) == 0
+        got = orc.fold(out.cpu().numpy(), B_rows)
+        want, _, mg = sn.subscale_net_run(orc.OracleModel(w, "bf16"), sn.SubscaleNet(nw), frames, L, synth.HOP, SEED, forced=got, teacher=True)
+        for g, r, k in zip(pu._split(got), pu._split(want), (0, 1)):
+            assert pu.check_indices(g, r, mg[:, :, k])[1] == 0
+    finally:
+        Bn.wrnn_subscale_net_destroy(net)
+        Bn.wrnn_destroy(m)
+
+
 @pytest.mark.parametrize("H,dtype,B_rows,L,chunk,kernel", [(64, "bf16", 5, 96, 32, "generic"), (896, "bf16", 16, 384, 128, "auto")])
 def test_generation_through_the_network(env, H, dtype, B_rows, L, chunk, kernel):
     torch, Bn = env
