@@ -169,7 +169,7 @@ __device__ __noinline__ long long cl_wide_steps(const ClParams &p, int row0, int
         float acc = 0.f;
         for (int c = lane; c < cols / 4; c += 32) {
             const size_t at = ((size_t)(row >> 2) * (cols / 4) + c) * 16 + 4 * (row & 3);
-            const float4 v = __ldcg(reinterpret_cast<const float4 *>(x) + c);
+            const float4 v = make_float4(__ldcg(x + 4 * c), __ldcg(x + 4 * c + 1), __ldcg(x + 4 * c + 2), __ldcg(x + 4 * c + 3));       // (a caller's state: floats at any address)
             float4 w;
             if (KIND == CL_F32) w = __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(M) + at));
             else {

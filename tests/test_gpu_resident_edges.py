@@ -228,6 +228,37 @@ def test_error_against_64_bits(env, dtype, rows):
         assert all(e <= b for e, b in zip(err, bound)), (err, bound)
 
 
+@pytest.mark.parametrize("case,rows", [("bf16", 1), ("bf16", 6), ("bf16", 30), ("f32", 3), ("fused", 1)])
+def test_states_at_any_address(env, case, rows):
+    """A caller's state is an array of floats: one that starts between two 16-byte boundaries gives what an aligned one gives, also where it is
+    so large that the cluster takes plain steps."""
+    torch, B = env
+    n, fused = 20, case == "fused"
+    w = synth.make_weights(896, **(dict(n_inputs=12, n_logits=64) if fused else {}))
+    cond = torch.from_numpy(synth.make_cond(rows, 2)).cuda()
+    m = B.wrnn_create(w, "f32" if case == "f32" else "bf16", max_batch=rows, variant=1 if fused else 0)
+    h0 = torch.from_numpy(np.random.default_rng(3).uniform(-0.9, 0.9, (rows, 896)).astype(np.float32)).cuda()
+    try:
+        for big in (0.5, 30.0):
+            h0[rows // 2, 7] = big
+            got = []
+            for shift in (0, 1, 3):
+                h = torch.zeros(rows * 896 + 4, device="cuda:0")[shift:shift + rows * 896].view(rows, 896)
+                assert h.data_ptr() % 16 == 4 * shift
+                h.copy_(h0)
+                out = torch.zeros((2 if fused else rows, n), dtype=torch.int16, device="cuda:0")
+                if fused:
+                    B.wrnn_fs2_sample(m, cond, n, SEED, out, h=h)
+                else:
+                    B.wrnn_sample(m, cond, n, rows, SEED, out, h=h)
+                torch.cuda.synchronize()
+                assert B.wrnn_poll_status(m) == 0
+                got.append((out.cpu(), h.cpu()))
+            assert all(torch.equal(a, b) for g in got[1:] for a, b in zip(g, got[0]))
+    finally:
+        B.wrnn_destroy(m)
+
+
 def test_first_subscale_call_costs_little_more_than_the_next(env):
     """A staggered schedule starts with one active row and adds one per lag: its workspaces are made for the largest call at once, not
     regrown (with a device synchronisation each time) on the way.  Best of three fresh models, room for the kernels' first loads."""
