@@ -518,7 +518,10 @@ __global__ void __launch_bounds__(BC_THREADS, 1) bcluster_step_kernel(const __gr
                     // row bl of the group is drawn by warp bl / 16 of CTA bl % 16: the logits go straight into its shared memory
                     const unsigned dst = map_to_rank(smem_addr(s_log + (bl >> 4) * 256 + r0), (unsigned)(bl & 15));
                     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "f"(o.x), "f"(o.y), "f"(o.z), "f"(o.w) : "memory");
-                    if (DBG && p.dbg_logits) *reinterpret_cast<float4 *>(p.dbg_logits + (((size_t)s * p.batch + gb) * 2 + head) * 256 + r0) = o;
+                    if (DBG && p.dbg_logits) {                           // (a caller's array: floats at any address)
+                        float *d = p.dbg_logits + (((size_t)s * p.batch + gb) * 2 + head) * 256 + r0;
+                        d[0] = o.x; d[1] = o.y; d[2] = o.z; d[3] = o.w;
+                    }
                 }
             }
             CSTAMP(8 + 8 * head);

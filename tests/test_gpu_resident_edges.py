@@ -259,6 +259,28 @@ def test_states_at_any_address(env, case, rows):
         B.wrnn_destroy(m)
 
 
+@pytest.mark.parametrize("H,rows,kernel", [(128, 11, "BCLUSTER"), (128, 11, "BATCHED"), (896, 3, "AUTO"), (896, 30, "AUTO"), (64, 2, "GENERIC")])
+def test_dumps_at_any_address(env, H, rows, kernel):
+    """Gates, states and logits are written as floats, wherever the caller's arrays start."""
+    torch, B = env
+    n, dev = 12, "cuda:0"
+    cond = torch.from_numpy(synth.make_cond(rows, 2)).cuda()
+    forced = torch.from_numpy(np.random.default_rng(4).integers(0, 256, (2, rows, n)).astype(np.uint8)).cuda()
+    m = B.wrnn_create(synth.make_weights(H), "bf16", max_batch=rows, kernel=getattr(B, "WRNN_KERNEL_" + kernel))
+    try:
+        got = []
+        for shift in (0, 1):
+            d = [torch.zeros(n * rows * k + 4, device=dev)[shift:shift + n * rows * k].view(n, rows, k) for k in (3 * H, H, 512)]
+            c, f = torch.zeros_like(forced[0]), torch.zeros_like(forced[1])
+            B.wrnn_step_teacher_forced(m, cond, n, rows, SEED, forced[0], forced[1], c, f, dbg_gates=d[0], dbg_h=d[1], dbg_logits=d[2].view(n, rows, 2, 256))
+            torch.cuda.synchronize()
+            assert B.wrnn_poll_status(m) == 0
+            got.append([x.cpu() for x in (*d, c, f)])
+        assert all(torch.equal(a, b) for a, b in zip(*got)) and got[0][2].abs().min() > 0
+    finally:
+        B.wrnn_destroy(m)
+
+
 def test_first_subscale_call_costs_little_more_than_the_next(env):
     """A staggered schedule starts with one active row and adds one per lag: its workspaces are made for the largest call at once, not
     regrown (with a device synchronisation each time) on the way.  Best of three fresh models, room for the kernels' first loads."""
