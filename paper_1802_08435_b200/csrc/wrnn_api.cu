@@ -719,8 +719,8 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
     for (int n = 1; n <= most; ++n)
         if (!use_rescl(m, n) && !use_resrows(m, n)) return -1;
     const size_t gn = (size_t)B * N * 3 * H;
-    // (where the rings find no room, the calls one by one, which need less)
-    if (subnet_ring_reserve(net, s) != WRNN_OK || !ensure_g(m, 2 * gn)) return -1;
+    // (where the rings find no room, the calls one by one, which need less; the rings come last, so that none are kept beside these)
+    if (!ensure_g(m, 2 * gn) || subnet_ring_reserve(net, s) != WRNN_OK) return -1;
     const cudaStream_t sn = subnet_side(net, 0), st = subnet_side(net, 1);
     const auto follow = [](cudaStream_t to, int e, cudaStream_t from, wrnn_subscale_net *q) {
         return cudaEventRecord(subnet_event(q, e), from) == cudaSuccess && cudaStreamWaitEvent(to, subnet_event(q, e), 0) == cudaSuccess;
