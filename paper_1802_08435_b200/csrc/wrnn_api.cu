@@ -152,6 +152,12 @@ static bool use_resrows(const wrnn_model *m, int batch)
     return !(off && off[0] == '1');
 }
 
+// 16-CTA clusters that a stepping call of so many rows has on the chip at a time (one of the two kernels above takes it)
+static int stepping_clusters(const wrnn_model *m, int batch, int limit)
+{
+    return use_resrows(m, batch) ? resrows_clusters(m, batch) : rescl_clusters(m, batch, limit);
+}
+
 static bool use_resf32(const wrnn_model *m, int batch)
 {
     if (m->kernel == WRNN_KERNEL_GENERIC || m->kernel == WRNN_KERNEL_BATCHED || m->kernel == WRNN_KERNEL_BCLUSTER) return false;
@@ -739,7 +745,10 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
         if (n_lo > n_hi) continue;                                          // (a gap between rows: lag > L)
         for (int e = 0; e < 2; ++e)                                         // every stepping call of two blocks ago and before
             if (stepped[e] >= 0 && stepped[e] <= k - 2 && cudaStreamWaitEvent(sn, subnet_event(net, 2 + e), 0) != cudaSuccess) rc = WRNN_ERR_CUDA;
-        if (rc == WRNN_OK) rc = subnet_ring_run(net, hist, frames, n_frames, hop, L, n_lo, n_hi - n_lo + 1, t, lag, v, m->n_sms - 16 * STEP_CLUSTERS, m->wait_limit_ns(), sn);
+        // more than 20 bf16 rows, or ten fp32 ones, take more than five clusters: what is left is what a convolution of the network may be split
+        // over (192 channels, all rows under way: 28 rows 66.1 -> 64.5, 40 rows 104.0 -> 100.3 ms; 384 channels are not split there anyway)
+        const int sms = 16 * std::max(STEP_CLUSTERS, stepping_clusters(m, std::min(n_hi - n_lo + 1, most), STEP_CLUSTERS));
+        if (rc == WRNN_OK) rc = subnet_ring_run(net, hist, frames, n_frames, hop, L, n_lo, n_hi - n_lo + 1, t, lag, v, m->n_sms - sms, m->wait_limit_ns(), sn);
         if (t < 0 || rc != WRNN_OK) continue;
         const int r_lo = n_lo, r_hi = (int)std::min<long long>(B - 1, t / lag), rows = r_hi - r_lo + 1;
         if (rows < 1) continue;

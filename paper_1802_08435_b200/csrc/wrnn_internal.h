@@ -57,7 +57,8 @@ struct StepArgs {
     long long out_pitch;
     // projected conditioning [batch][n_frames][3H] that is there already (null: projected from cond by this call), with a status word that is cleared
     const float *g;
-    int clusters;            // at most so many 16-CTA clusters at a time, where that is possible (0: as many as there are)
+    int clusters;            // at most so many 16-CTA clusters at a time, where four rows per cluster (two with fp32 weights) allow it; 0, and
+                             // always more than four rows per cluster: as many as there are
     // fused subscale variant: 16-bit samples of parts A and B in place of the bytes above (batch 1)
     const uint16_t *a_in, *b_in; uint16_t *a_st_out, *b_st_out;
     const uint16_t *a_forced, *b_forced;         // [n_steps] or null
@@ -238,6 +239,7 @@ void rescl_packed(wrnn_model *m);        // gives up what only the packers of th
 int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
 int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int rescl_phase_cycles(const wrnn_model *m, long long *out16);
+int rescl_clusters(const wrnn_model *m, int batch, int clusters);        // on the chip at a time, with StepArgs.clusters = clusters
 
 // wrnn_resrows.cu: five to fourteen rows per cluster (bf16)
 int resrows_prepare(wrnn_model *m);
@@ -245,6 +247,7 @@ void resrows_destroy(wrnn_model *m);
 int resrows_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_threads, int *smem, int64_t *weight_bytes);
 int resrows_run(wrnn_model *m, const StepArgs &a, cudaStream_t s);
 int resrows_phase_cycles(const wrnn_model *m, long long *out16);
+int resrows_clusters(const wrnn_model *m, int batch);
 
 // wrnn_resf32.cu: the same role for dense fp32 models (every matrix sharded chip-wide, nothing replicated)
 int resf32_supported(const wrnn_model *m, int batch, std::string *why);

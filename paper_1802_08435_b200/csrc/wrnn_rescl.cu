@@ -995,6 +995,13 @@ int rescl_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thread
     return WRNN_OK;
 }
 
+int rescl_clusters(const wrnn_model *m, int batch, int clusters)
+{
+    int nr, n_clusters;
+    cl_geometry(*m->rescl, batch, clusters, &nr, &n_clusters);
+    return std::min(n_clusters, m->rescl->max_clusters);
+}
+
 int rescl_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
 {
     const ResClPack &k = *m->rescl;

@@ -758,6 +758,13 @@ int resrows_launch_info(const wrnn_model *m, int batch, int *n_ctas, int *n_thre
     return WRNN_OK;
 }
 
+int resrows_clusters(const wrnn_model *m, int batch)
+{
+    int nr, n_clusters;
+    rw_geometry(*m->resrows, batch, &nr, &n_clusters);
+    return std::min(n_clusters, m->resrows->max_clusters);
+}
+
 int resrows_run(wrnn_model *m, const StepArgs &a, cudaStream_t s)
 {
     const ResRowsPack &k = *m->resrows;

@@ -92,3 +92,36 @@ def test_first_call_of_a_network_on_a_stream_of_its_own(chunk):
             assert np.array_equal(first(side, busy), want)
     finally:
         B.wrnn_destroy(m)
+
+
+@pytest.mark.parametrize("dtype,rows,conv_ch", [("bf16", 30, 192), ("f32", 12, 96)])
+def test_rings_with_all_rows_under_way(dtype, rows, conv_ch):
+    """Rows that follow one another closely enough for all of them to be under way at once: every count of rows per cluster, up to the kernel of many
+    rows, and more clusters than the schedule leaves for the stepping otherwise.  The draws of rows spread over the schedule against the oracle
+    forced on the device's samples."""
+    import torch
+    from concurrent.futures import ThreadPoolExecutor
+    from paper_1802_08435_b200 import binding as B
+    lag = 128
+    L = lag * (rows - 1) + 90
+    w, nw = synth.make_weights(896), synth.make_subscale_net(rows, conv_ch=conv_ch, res_ch=96, taps=1, dilations=(1, 1))
+    frames = synth.make_cond(rows, rows * L // synth.HOP + 2, synth.COND_DIM)
+    m, q = B.wrnn_create(w, dtype, max_batch=rows), B.wrnn_subscale_net_create(nw)
+    try:
+        out = torch.zeros(rows * L, dtype=torch.int16, device="cuda:0")
+        B.wrnn_sample_subscale_net(m, q, torch.from_numpy(frames).cuda(), 64, 64, lag, rows * L, SEED, out)
+        torch.cuda.synchronize()
+        assert B.wrnn_poll_status(m) == 0 and B.wrnn_subscale_net_status(q) == 0
+    finally:
+        B.wrnn_subscale_net_destroy(q)
+        B.wrnn_destroy(m)
+    got, om, net = orc.fold(out.cpu().numpy(), rows), orc.OracleModel(w, dtype), sn.SubscaleNet(nw)
+
+    def wrong(s):
+        c, f = pu._split(got[s])
+        cond = frames[s][(rows * np.arange(L) + s) // synth.HOP] + net.conditioning(got, s)
+        r = om.run(cond[None], L, 1, SEED, hop=1, stream0=s, c_forced=c, f_forced=f)
+        return [pu.check_indices(x, y[0], r.margins[0, :, k])[1] for x, y, k in ((c, r.c_out, 0), (f, r.f_out, 1))]
+
+    with ThreadPoolExecutor(pu.NCPU) as ex:
+        assert all(n == [0, 0] for n in ex.map(wrong, sorted({0, 1, rows // 3, rows // 2, rows - 2, rows - 1})))
