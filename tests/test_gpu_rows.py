@@ -14,9 +14,9 @@ pytestmark = pytest.mark.gpu
 SEED = synth.SEED_SAMPLING
 
 
-# rows -> rows per cluster (clusters): 29 -> 5 (6, the last one 4), 43 -> 7 (7, the last one 1: a pipe without rows), 70 -> 10 (7), 85 -> 13 (7, 7),
-# 98 -> 14 (7), 225 -> 11 (21, 5)
-@pytest.mark.parametrize("rows", [29, 43, 70, 85, 98, 225])
+# rows -> rows per cluster (clusters): 29 -> 5 (6, the last one 4), 43 -> 7 (7, the last one 1: a pipe without rows), 70 -> 10 (7), 78 -> 12 (7, 6),
+# 85 -> 13 (7, 7), 98 -> 14 (7), 225 -> 11 (21, 5)
+@pytest.mark.parametrize("rows", [29, 43, 70, 78, 85, 98, 225])
 def test_rows_kernel(rows, monkeypatch):
     """Teacher-forced against the oracle; a call in pieces, down to single steps, equals one call; the checked form draws the same samples; the
     errors against 64 bits stay below those of the kernel before it (2-norms 0.92e-7 gates, 1.75e-7 state, 2.30e-7 logits)."""
@@ -99,6 +99,69 @@ def test_rows_kernel_phases(rows):
         assert names == [h + p for h in ("F.", "C.") for p in phases]
         print("\n[phases] %d rows, cycles per step: %s" % (rows, ", ".join("%s %.0f" % (k, c / n) for k, c in zip(names, cycles))))
         assert min(cycles) > 0 and 2000 * n < sum(cycles) < 40000 * n, cycles
+    finally:
+        B.wrnn_destroy(m)
+
+
+@pytest.mark.parametrize("rows,big", [(43, 30.0), (78, 1e6), (98, 30.0)])
+def test_rows_kernel_large_states(rows, big):
+    """A row whose state is beyond what the operand images hold, in a cluster of seven, twelve and fourteen rows: its cluster takes plain steps until
+    it has come back, and every row -- those beside it in either pipe, those of the other clusters -- follows the oracle in gates, states, logits, draws
+    and the final state; so does a row that comes back after the first step.  (The large row itself in its first gates, within the rounding of its sums.)"""
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    n, H, dev = 24, 896, "cuda:0"
+    w, cond = synth.make_weights(H), synth.make_cond(rows, 2)
+    h0 = np.tanh(np.random.default_rng(5).standard_normal((rows, H))).astype(np.float32)
+    odd, back = rows // 2, 1                                             # (clusters of their own)
+    h0[odd, ::7] *= np.float32(big)
+    h0[back, int(np.argmin(np.diag(w["R"][:H])))] = big                  # a unit that its own update gate takes back at once
+    ref = orc.OracleModel(w, "bf16").run(cond, n, rows, SEED, dump=True, h=h0, threads=pu.NCPU)
+    z = lambda *s: torch.zeros(s, dtype=torch.float32, device=dev)
+    m = B.wrnn_create(w, "bf16", max_batch=rows)
+    try:
+        per = -(-rows // (B.wrnn_launch_info(m, rows)["n_ctas"] // 16))
+        assert odd // per != back // per
+        h, c, f = torch.from_numpy(h0).to(dev), torch.from_numpy(ref.c_out).to(dev), torch.from_numpy(ref.f_out).to(dev)
+        d, co, fo = (z(n, rows, 3 * H), z(n, rows, H), z(n, rows, 2, 256)), torch.zeros_like(c), torch.zeros_like(f)
+        B.wrnn_step_teacher_forced(m, torch.from_numpy(cond).to(dev), n, rows, SEED, c, f, co, fo, dbg_gates=d[0], dbg_h=d[1], dbg_logits=d[2], h=h)
+        torch.cuda.synchronize()
+        assert B.wrnn_poll_status(m) == 0, B.wrnn_last_error(m)
+    finally:
+        B.wrnn_destroy(m)
+    got = [x.cpu().numpy().reshape(n, rows, -1) for x in d] + [h.cpu().numpy()[None]]
+    want = [np.asarray(x).reshape(n, rows, -1) for x in (ref.gates, ref.hs, ref.logits)] + [np.asarray(ref.h)[None]]
+    rest = [b for b in range(rows) if b != odd]
+    for g, r in zip(got, want):
+        assert np.isfinite(g).all() and pu.rel_err(g[:, rest], r[:, rest]) < pu.TOL["bf16"]
+    for x, y, k in ((co, ref.c_out, 0), (fo, ref.f_out, 1)):
+        assert pu.check_indices(x.cpu().numpy()[rest], y[rest], ref.margins[rest][:, :, k])[1] == 0
+    # sums of fp32 terms, (terms) x 2^-24 x sum |term|; gates of slope one at most
+    bound = H * 2.0 ** -24 * (np.abs(w["R"]).astype(np.float64) @ np.abs(h0[odd]).astype(np.float64)).max()
+    assert np.abs(got[0][0, odd] - want[0][0, odd]).max() < pu.TOL["bf16"] + bound
+
+
+@pytest.mark.parametrize("rows", [78, 98])
+def test_rows_kernel_lost_word(rows):
+    """The wider forms (pipes of six and seven rows) when a CTA of every cluster withholds the state it publishes at one step: the waits that depend on
+    it run out, the call reports where and returns, and the model works again."""
+    import re
+    import torch
+    from paper_1802_08435_b200 import binding as B
+    cond, n, at = synth.make_cond(rows, 2), 60, 23
+    m = B.wrnn_create(synth.make_weights(896), "bf16", max_batch=rows)
+    try:
+        ref = _free_run(torch, B, m, cond, n, rows, SEED)
+        n_ctas = B.wrnn_launch_info(m, rows)["n_ctas"]
+        B.wrnn_selftest_lost_word(m, 4_000_000, n_ctas // 2, at)
+        out = torch.zeros((rows, n), dtype=torch.int16, device="cuda:0")
+        B.wrnn_sample(m, torch.from_numpy(cond).cuda(), n, rows, SEED, out)
+        torch.cuda.synchronize()
+        assert B.wrnn_poll_status(m) == B.WRNN_ERR_TIMEOUT
+        cta, step, _ = (int(x) for x in re.search(r"at cta (-?\d+), step (-?\d+), phase (-?\d+)", B.wrnn_last_error(m)).groups())
+        assert 0 <= cta < n_ctas and at <= step <= at + 1, B.wrnn_last_error(m)
+        B.wrnn_selftest_lost_word(m, 0, -1, -1)
+        assert np.array_equal(_free_run(torch, B, m, cond, n, rows, SEED), ref)
     finally:
         B.wrnn_destroy(m)
 
