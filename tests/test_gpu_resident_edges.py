@@ -228,6 +228,46 @@ def test_error_against_64_bits(env, dtype, rows):
         assert all(e <= b for e, b in zip(err, bound)), (err, bound)
 
 
+@pytest.mark.parametrize("case,rows", [("bf16", 1), ("bf16", 16), ("bf16", 37), ("f32", 1), ("fused", 1)])
+def test_captured_calls(env, case, rows):
+    """A call in a graph -- a lone cluster is launched beside the projection of its frames there too -- and pieces that hand the state on from one
+    call to the next: every replay draws what the calls draw."""
+    torch, B = env
+    n, fused, dev = 30, case == "fused", "cuda:0"
+    w = synth.make_weights(896, **(dict(n_inputs=12, n_logits=64) if fused else {}))
+    cond = torch.from_numpy(synth.make_cond(rows, 2)).cuda()
+    m = B.wrnn_create(w, "f32" if case == "f32" else "bf16", max_batch=rows, variant=1 if fused else 0)
+    out = torch.zeros((3, 2 if fused else rows, n), dtype=torch.int16, device=dev)
+    st = {} if fused else _state(torch, rows)
+    h0 = torch.zeros((rows, 896), device=dev)
+
+    def calls():
+        if fused:
+            h0.zero_()
+            for i in range(3):
+                B.wrnn_fs2_sample(m, cond, n, SEED, out[i], h=h0, step0=n * i)
+            return
+        st["h"].zero_(), st["c_prev"].fill_(128), st["f_prev"].zero_()
+        for i in range(3):
+            B.wrnn_sample(m, cond, n, rows, SEED, out[i], step0=n * i, **st)
+
+    try:
+        calls()
+        torch.cuda.synchronize()
+        want = out.clone()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            calls()
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert B.wrnn_poll_status(m) == 0 and torch.equal(out, want)
+        del graph
+    finally:
+        B.wrnn_destroy(m)
+
+
 @pytest.mark.parametrize("case,rows", [("bf16", 1), ("bf16", 6), ("bf16", 30), ("f32", 3), ("fused", 1)])
 def test_states_at_any_address(env, case, rows):
     """A caller's state is an array of floats: one that starts between two 16-byte boundaries gives what an aligned one gives, also where it is
