@@ -275,14 +275,20 @@ int wrnn_subscale_net_conditioning(wrnn_subscale_net *net, const int16_t *hist, 
                                    int32_t row, int64_t L, float *v, void *cuda_stream);
 int wrnn_subscale_net_status(wrnn_subscale_net *net);
 /* wrnn_sample_subscale_dependent with this network in place of the one-layer convolution: B = the network's B; F >= the
- * network's reach; lag a multiple of chunk and >= F + chunk.  Per chunk the network is evaluated for chunk + reach positions
- * of every active row (the positions ahead are recomputed by the next chunk).  Asynchronous on cuda_stream. */
+ * network's reach; lag a multiple of chunk and >= F + chunk.  Asynchronous on cuda_stream; one call in flight per network.
+ * Two ways of doing it, by the arguments.  Where lag is a multiple of 128, lag - reach >= 128, chunk >= 64, every
+ * (taps - 1) dilation <= 64 and the model a dense one of H = 896 whose rows under way the resident family takes (left to AUTO: up to 336 if its weights
+ * are bf16), the network works ahead of the stepping, on streams of its own that are joined to cuda_stream, in blocks of 64 positions whatever the
+ * chunk, and computes every position once; for this it keeps the last positions of every layer and row until it is destroyed, some 1,280
+ * bytes per layer, row and residual channel (169 MB for 16 rows of ten layers and 768 channels).  Otherwise (a lag of 192, say), and
+ * where there is no room for that, one stepping call after the other at about half the rate: per chunk the network is evaluated for
+ * chunk + reach positions of every active row, the positions ahead again for the next chunk.  The two agree within rounding. */
 int wrnn_sample_subscale_net(wrnn_model *m, wrnn_subscale_net *net, const float *frames, int32_t n_frames, int32_t hop, int32_t F,
                              int32_t chunk, int32_t lag, int64_t n_total, uint64_t seed, int16_t *out, void *cuda_stream);
 
 /* One stepping call of the staggered schedule on caller-owned buffers: rows r_lo .. r_lo + n_rows - 1 of the B sub-tensors
- * advance n_steps positions, row b of the call from position p_lo - b * lag on (the unit wrnn_sample_subscale_net is made of,
- * exposed so that the sub-tensors can be spread over several devices, each generating some rows and passing the samples on one
+ * advance n_steps positions, row b of the call from position p_lo - b * lag on (a chunk of wrnn_sample_subscale_net where that
+ * goes one call after the other, exposed so that the sub-tensors can be spread over several devices, each generating some rows and passing the samples on one
  * way, online: Section 5.3's closing paragraph).  hist: DEVICE int16 [B][L], read for the rows below r_lo + n_rows (positions up
  * to F ahead must be there) and written in place for the rows of the call; h [B][H], c_prev / f_prev [B]: DEVICE carry state
  * of all rows, read and written for the rows of the call (start from h = 0, c_prev = 128, f_prev = 0).  n_rows <= max_batch.

@@ -128,9 +128,9 @@ static bool use_resident(const wrnn_model *m, int batch)
 }
 
 // Rows of a dense H = 896 model: the kernels that hold the whole model in one cluster, up to four rows per cluster (seven clusters at a
-// time) in the one, five to fourteen in the other, more of either in waves of clusters.  us per step of the two at 28 rows: 4.30 / 4.59, at 8:
-// 3.69 / 4.52; of the second and the cluster-partitioned kernel: 29 rows 4.65 / 25, 56: 4.8 / 25.2, 98: 6.9 / 25.8, 168: 13.7 / 28.8, 224: 19.3 /
-// 31.1, 256: 20.4 / 32.2, 336: 27.6 / 34.
+// time) in the one, five to fourteen in the other, more of either in waves of clusters.  us per step of the two at 28 rows: 4.28 / 4.59, at 8:
+// 3.65 / 4.52; of the second and the cluster-partitioned kernel: 29 rows 4.56 / 25.2, 56: 4.74 / 25.0, 98: 6.72 / 25.1, 168: 13.2 / 28.6, 224: 19.0 /
+// 31.0, 256: 20.0 / 32.2, 336: 26.4 / 34.2.
 constexpr int RESCL_BF16_ROWS = 28;
 // (beyond, the grid-phased kernel)
 constexpr int RESROWS_MOST = 336;
@@ -718,7 +718,8 @@ static int subscale_net_whole(wrnn_model *m, wrnn_subscale_net *net, const float
                               float *hst, int16_t *hist, uint8_t *cp, uint8_t *fp, cudaStream_t s)
 {
     // The stepping calls take five clusters at most (up to five rows in one each, ten two by two, sixteen by up to four: 3.3, 3.7, 4.4 us per step), which
-    // leaves the network 68 SMs: 44.7 ms for 16 x 6,000 positions; 46.8 with six, 48.2 with four where its products could use the room.
+    // leaves the network 68 SMs: 44.7 ms for 16 x 6,000 positions when this was chosen (43.4 now); 46.8 with six, 48.2 with four where its products
+    // could use the room.
     constexpr int N = 64, STEP_CLUSTERS = 5;
     if (!subnet_ring_fits(net, lag)) return -1;
     const int D = m->cond_dim, H = m->H, most = (int)std::min<long long>(B, (L + lag - 1) / lag + 1);

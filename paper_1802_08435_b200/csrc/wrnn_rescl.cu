@@ -8,8 +8,8 @@
 // the model inside one cluster every exchange is an all-gather through distributed shared memory (measured here: 420 cycles +
 // 0.87 per byte and receiver, against 1,000 - 1,500 cycles for the same through L2 and across the chip), clusters never meet, and
 // seven of them advance seven times as many rows in the same time.  us per step: 1 to 7 rows 3.27, 8 rows 3.69, 28 rows 4.30
-// (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 28; more rows of a bf16 model: wrnn_resrows.cu); fp32 5.1 to 6.9, with where the streamed weights lie, up to 7
-// rows and 6.2 to 7.1 up to 14 (7.4 at one row, 55 and more at several); fused 3.5 (4.54).
+// (the kernels before: 4.73 at one row, 5.6 at 8, 9.5 at 16, 25 at 28; more rows of a bf16 model: wrnn_resrows.cu); fp32 5.0 up to 7
+// rows and 6.0 up to 14, with several models alive up to 0.9 more, with where the streamed weights lie (7.4 at one row, 55 and more at several); fused 3.5 (4.54).
 //
 // Per CTA (rank r of its cluster): state units 28 r .. 28 r + 27 of both halves with their 168 rows of R, rows 28 r .. of O1
 // and O3, rows 16 r .. of O2 and O4.
