@@ -244,8 +244,9 @@ def roofline(ctx, wl, info, model, n_steps, ms_per_step, cond_bytes, out_bytes):
     g_bytes = wl.batch * (wl.n_frames if wl.n_frames else 1) * 3 * H * 4
     traffic = (wbytes + cond_bytes + 2 * g_bytes + out_bytes) if resident else None
     traffic_note = ("computed: resident weight bytes loaded once per launch (%d) + conditioning (%d) + projected gate offsets "
-                    "written and read (%d) + samples (%d); does not grow with the number of steps; the ncu captures in "
-                    "profiles/ measured the same quantity" % (wbytes, cond_bytes, 2 * g_bytes, out_bytes)) if resident else \
+                    "written and read (%d) + samples (%d); the weights' share does not grow with the number of steps%s" % (
+                        wbytes, cond_bytes, 2 * g_bytes, out_bytes,
+                        "; the ncu captures in profiles/ measured the same quantity" if wl.batch == 1 else "")) if resident else \
                    "weights are re-read from L2 every step; DRAM traffic not modelled"
     if wl.batch >= 2:
         flops = 2.0 * wl.batch * (3 * H * H + 2 * Hh * Hh + 2 * 256 * Hh)
