@@ -30,7 +30,7 @@ def _state(torch, batch, H=896):
 def test_calls_of_one_step_equal_one_call(env, dtype, batch):
     """Every call multiplies R by the state that it is given before the CTAs of a cluster exchange their first new one, and a CTA that
     is ahead must not store that over the state that another one still reads.  Calls of one step are nothing but this: all forms of
-    the cluster-resident kernel (one, up to four, up to eight rows per cluster), against one call."""
+    the cluster-resident kernels (one, up to four, up to eight rows per cluster), against one call."""
     torch, B = env
     n = 60
     cond = synth.make_cond(batch, 2)

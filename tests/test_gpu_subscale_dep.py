@@ -44,7 +44,7 @@ def _gpu_run(torch, Bn, m, frames, V, b, F, chunk, lag, B_rows, L, hop=synth.HOP
 
 @pytest.mark.parametrize("H,dtype,B_rows,L,F,chunk,kernel", [
     (32, "f32", 4, 90, 6, 3, "generic"), (64, "bf16", 5, 64, 8, 8, "generic"), (896, "bf16", 16, 300, 32, 32, "generic"),
-    (896, "bf16", 16, 300, 32, 32, "auto"),      # four or more active rows advance together on the multi-stream resident kernel
+    (896, "bf16", 16, 300, 32, 32, "auto"),      # four or more active rows advance together on the cluster-resident kernel
     (896, "bf16", 16, 300, 32, 32, "bcluster"),  # the same on the cluster-partitioned kernel (lone rows on the any-shape kernel)
 ])
 def test_staggered_schedule_and_oracle(env, H, dtype, B_rows, L, F, chunk, kernel):
