@@ -413,7 +413,7 @@ int wrnn_selftest_bounded_wait(int64_t limit_ns, int32_t *code, int32_t *cta, in
  * CTA `cta` withholds at step `step` (relative to the call) what it would hand to the other CTAs: the state values it
  * publishes (shared-memory-resident and sparse kernels), one operand load of its own tensor pipeline (cluster-partitioned
  * kernel), or its arrivals at the grid barrier (any-shape and grid-phased kernels); limit_ns (0 = the default of two
- * seconds, at most two seconds) bounds every device-side wait of the launch.  The waits that depend on the missing piece
+ * seconds, at most two seconds; less than a millisecond counts as one) bounds every device-side wait of the launch.  The waits that depend on the missing piece
  * run out, the first CTA to give up records WRNN_ERR_TIMEOUT with (cta, step, phase), every CTA leaves through its normal
  * exit and wrnn_poll_status reports it.  cta = -1 restores normal operation (limit_ns still applies).  Host only. */
 int wrnn_selftest_lost_word(wrnn_model *m, int64_t limit_ns, int32_t cta, int64_t step);

@@ -119,7 +119,9 @@ struct wrnn_model {
     unsigned long long dbg_limit_ns = 0;
     int dbg_skip_cta = -1;
     long long dbg_skip_step = -1;
-    unsigned long long wait_limit_ns() const { return dbg_limit_ns ? dbg_limit_ns : 2000000000ull; }
+    // At least a millisecond: waits are also for a CTA's own copies in flight (weights, operands), some microseconds, and one that gave up on them
+    // could leave before they land in its shared memory.
+    unsigned long long wait_limit_ns() const { return dbg_limit_ns ? std::max(dbg_limit_ns, 1000000ull) : 2000000000ull; }
     bool prof_enabled = false;      // wrnn_phase_profile: the resident kernels stamp their phases
     wrnn::BatchedPack *batched = nullptr;
     wrnn::SparsePack *sparse_pack = nullptr;

@@ -228,6 +228,22 @@ def test_error_against_64_bits(env, dtype, rows):
         assert all(e <= b for e, b in zip(err, bound)), (err, bound)
 
 
+@pytest.mark.parametrize("rows", [1, 16, 37])
+def test_short_wait_limits_leave_copies_their_time(env, rows):
+    """A wait covers the copies that bring a CTA's own weights on chip: a limit below what these take, which a caller may ask for, does not let
+    the CTA leave before they have landed.  Nothing is withheld here, so the call ends as any other."""
+    torch, B = env
+    cond = synth.make_cond(rows, 2)
+    m = B.wrnn_create(synth.make_weights(896), "bf16", max_batch=rows)
+    try:
+        want = _free_run(torch, B, m, cond, 20, rows, SEED)
+        for limit in (1, 1000):
+            B.wrnn_selftest_lost_word(m, limit, -1, -1)
+            assert np.array_equal(_free_run(torch, B, m, cond, 20, rows, SEED), want) and B.wrnn_poll_status(m) == 0
+    finally:
+        B.wrnn_destroy(m)
+
+
 @pytest.mark.parametrize("case,rows", [("bf16", 1), ("bf16", 16), ("bf16", 37), ("f32", 1), ("fused", 1)])
 def test_captured_calls(env, case, rows):
     """A call in a graph -- a lone cluster is launched beside the projection of its frames there too -- and pieces that hand the state on from one
